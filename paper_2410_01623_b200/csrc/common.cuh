@@ -21,7 +21,7 @@ struct MatScalars {
   float lambda;       // limiter factor of the latest step
   float norm_scaled;  // ||S|| before the limiter
   float k_min, k_max;
-  float pad;          // bias factor sqrt(1-b2^s)/(1-b1^s) of the running step (tensor-core path)
+  float pad;          // bias factor sqrt(1-b2^s)/(1-b1^s) of the next step, s = t + 1
   long long t;        // steps taken
 };
 static_assert(sizeof(MatScalars) == 32, "MatScalars layout");
@@ -36,10 +36,10 @@ struct MatDev {
   float* V;           // l x r
   MatScalars* sc;
   float* Rt;          // scratch: l x r fp32 low-rank gradient (transposed layout)
-  float* Xt;          // scratch: l x r fp32, first N then X = a_low N - a_res lambda k R
+  float* Xt;          // scratch: l x r fp32 N
   float* kvec;        // scratch: l factors
   float* part;        // scratch: partial sums of ||S||^2
-  float* aux;         // scratch: 2 l floats, ||N_l||^2 and ||R_l||^2 (matrix-level factor only)
+  float* aux;         // scratch: ||N_l||^2, then ||R_l||^2; engine 0: l floats of each per tile of r
   __nv_bfloat16* Nb;  // scratch of the tensor-core path: l x r bf16 N
   __nv_bfloat16* Rb;  //   "      l x r bf16 R
   __nv_bfloat16* Xb;  //   "      l x r bf16 X
@@ -51,7 +51,7 @@ struct MatDev {
   int m, n, r;
   int left;           // 1: m <= n (left projection), 0: right projection
   int bf16;           // storage type of W, G, P
-  int engine;         // 0 CUDA-core fp32, 1 tcgen05 bf16
+  int engine;         // 0 fp32 precision, any size (step_simt.cu), 1 bf16 (step_tc.cu)
   int l, d;
 };
 
@@ -67,6 +67,11 @@ enum HyperMode : unsigned {
   HYPER_PSI_ADAGRAD = 16u,     // base optimizer: Adagrad instead of Adam
   HYPER_ONLY_SCALING = 32u,    // Fira-only-scaling: W <- W - lr phi(R) G (no P N term, S = G diag k)
 };
+
+// sqrt(1 - b2^s) / (1 - b1^s) (Eq. 4), in double.
+__host__ __device__ inline float bias_factor(float beta1, float beta2, long long s) {
+  return (float)(sqrt(1.0 - pow((double)beta2, (double)s)) / (1.0 - pow((double)beta1, (double)s)));
+}
 
 enum DeviceStatusBits : unsigned {
   DEV_STATUS_TIMEOUT = 1u,

@@ -8,7 +8,6 @@
 #include <new>
 
 #include "context.cuh"
-#include "simt_gemm.cuh"
 #include "step_tc.cuh"
 
 namespace fira {
@@ -92,7 +91,7 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
     if (d.ld == 0) d.ld = d.n;
     const size_t ll = std::max(d.m, d.n), r = d.r;
     L.offK[i] = w; w += align_up(ll * 4);
-    L.offAux[i] = w; w += align_up(2 * ll * 4);
+    L.offAux[i] = w; w += align_up(2 * (L.engine[i] == 0 ? simt_tiles(d.r) : 1) * ll * 4);
     if (L.engine[i] == 0) {
       const size_t tiles = (size_t)simt_tiles(d.m) * simt_tiles(d.n);
       L.offRt[i] = w; w += align_up(ll * r * 4);
@@ -242,24 +241,21 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
   };
   {
     const std::vector<int>& lst = c->simt_list;
-    std::vector<int> pt{0}, rs{0}, wt{0}, np;
+    std::vector<int> pt{0}, wt{0}, np;
     for (int i : lst) {
       const MatDev& mt = c->mats[i];
       pt.push_back(pt.back() + simt_tiles(mt.l) * simt_tiles(mt.r));
-      rs.push_back(rs.back() + mt.l);
       const int tiles = simt_tiles(mt.m) * simt_tiles(mt.n);
       wt.push_back(wt.back() + tiles);
       np.push_back(tiles);
     }
-    const size_t o_list = push_block(lst), o_pt = push_block(pt), o_rs = push_block(rs),
-                 o_wt = push_block(wt), o_np = push_block(np);
+    const size_t o_list = push_block(lst), o_pt = push_block(pt), o_wt = push_block(wt), o_np = push_block(np);
     c->simt.mats = c->mats_dev;
     c->simt.list = c->ints_dev + o_list; c->simt.nlist = (int)lst.size();
     c->simt.proj_tile_start = c->ints_dev + o_pt; c->simt.proj_tiles = pt.back();
-    c->simt.row_start = c->ints_dev + o_rs; c->simt.rows_total = rs.back();
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
     c->simt.npart = c->ints_dev + o_np;
-    c->simt.h_proj_tile_start = pt; c->simt.h_row_start = rs; c->simt.h_w_tile_start = wt;
+    c->simt.h_proj_tile_start = pt; c->simt.h_w_tile_start = wt;
   }
   fira_status ts = tc_build_plan(c, ints);
   if (ts != FIRA_OK) { tc_destroy_plan(c); delete c; return ts; }
@@ -272,7 +268,7 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
   // ||S_prev|| = -1 marks "unset"
   MatScalars init;
   memset(&init, 0, sizeof(init));
-  init.prev_norm = -1.f; init.lambda = 1.f;
+  init.prev_norm = -1.f; init.lambda = 1.f; init.pad = bias_factor(hp->beta1, hp->beta2, 1);
   for (int i = 0; i < count && ce == cudaSuccess; ++i)
     ce = cudaMemcpyAsync(c->mats[i].sc, &init, sizeof(MatScalars), cudaMemcpyHostToDevice, c->stream);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(c->mats_dev, c->mats.data(), sizeof(MatDev) * count, cudaMemcpyHostToDevice, c->stream);
@@ -306,7 +302,8 @@ static fira_status set_pointers(fira_ctx* c, void* const* W_dev, const void* con
 // to one sub-range of each); returns the number of launches or -1.
 static int launch_range(fira_ctx* c, const Hyper& h, int i0, int i1, bool whole) {
   if (whole) {
-    int launches = launch_simt_step(c->simt, h, c->status_dev, c->stream, &c->timer);
+    const int launches = launch_simt_step(c->simt, h, c->status_dev, c->stream, &c->timer);
+    if (launches < 0) return -1;
     if (c->simt.nlist == 0) c->timer.mark(c->stream);
     const int tcl = launch_tc_step(c, h);
     return tcl < 0 ? -1 : launches + tcl;
@@ -317,7 +314,10 @@ static int launch_range(fira_ctx* c, const Hyper& h, int i0, int i1, bool whole)
   };
   int qa, qb, launches = 0;
   sub(c->simt_list, qa, qb);
-  if (qb > qa) launches += launch_simt_step(c->simt, h, c->status_dev, c->stream, &c->timer, qa, qb);
+  if (qb > qa) {
+    launches = launch_simt_step(c->simt, h, c->status_dev, c->stream, &c->timer, qa, qb);
+    if (launches < 0) return -1;
+  }
   sub(c->tc_list, qa, qb);
   if (qb > qa) {
     const int tcl = launch_tc_step(c, h, qa, qb);
@@ -575,6 +575,7 @@ fira_status fira_set_state(fira_ctx* c, int32_t idx, const float* M_dev, const f
   memset(&sc, 0, sizeof(sc));
   sc.prev_norm = norm_prev < 0.f ? -1.f : norm_prev;
   sc.lambda = 1.f;
+  sc.pad = bias_factor(c->hp.beta1, c->hp.beta2, t + 1);
   sc.t = t;
   FIRA_CUDA(cudaMemcpyAsync(mt.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
   FIRA_CUDA(cudaStreamSynchronize(c->stream));
@@ -625,7 +626,7 @@ fira_status fira_enable_phase_timing(fira_ctx* c, int32_t enable) {
   if (enable && tm.events.empty()) {
     tm.events.resize((size_t)FIRA_TIMING_MAX_STEPS * (FIRA_TIMING_MAX_PHASES + 1));
     for (auto& ev : tm.events) FIRA_CUDA(cudaEventCreate(&ev));
-    if (c->simt.nlist) for (int i = 0; i < 6; ++i) tm.names.push_back(kSimtPhaseNames[i]);
+    if (c->simt.nlist) for (int i = 0; i < SIMT_PHASES; ++i) tm.names.push_back(kSimtPhaseNames[i]);
     if (!c->tc_list.empty()) {
       const char* nm[8];
       const int k = tc_phase_names(nm);

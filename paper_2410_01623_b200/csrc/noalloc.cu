@@ -19,14 +19,17 @@
 #include <mutex>
 
 #include "context.cuh"
-#include "simt_gemm.cuh"
+#include "step_simt.cuh"
 
 namespace fira {
 
 namespace {
 
-constexpr size_t kNoAllocScratchBytes = 8u << 20;   // 8 MiB
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
+constexpr size_t kNoAllocScratchBytes = 8u << 20;   // 8 MiB: what a caller's matrix may take
+// The row sums of matrices whose rank spans several tiles come behind it.  Such a matrix has r > 128, so
+// l r <= 2^20 (N and R fill the 8 MiB) bounds them: 2 l ceil(r / 128) floats < 2 * 2^20 * (1 / 128 + 1 / 129).
+constexpr size_t kRowSumBytes = 144u << 10;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + kRowSumBytes];
 
 constexpr int kMaxDevices = 64;
 // Device addresses of g_noalloc_scratch, one per device, resolved on first use.  In
@@ -78,8 +81,8 @@ Carve carve(int m, int n, int r) {
   return c;
 }
 
-// The schedule arrays of a one-matrix list: [list(1)] [proj_start(2)] [row_start(2)] [w_start(2)] [npart(1)].
-struct NoAllocInts { int v[8]; };
+// The schedule arrays of a one-matrix list: [list(1)] [proj_start(2)] [w_start(2)] [npart(1)].
+struct NoAllocInts { int v[6]; };
 
 // Writes this call's tables into the array (it still holds the previous call's; everything else
 // that a step reads there is rewritten by the step's own kernels before it is read).  The matrix
@@ -87,12 +90,13 @@ struct NoAllocInts { int v[8]; };
 // once the call has returned.  Also moves the two state scalars from the caller's memory into the
 // MatScalars block that the step kernels use.
 __global__ void k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, int* ints_out,
-                                const float* norm_prev, const long long* t) {
+                                const float* norm_prev, const long long* t, float beta1, float beta2) {
   *mats_out = mt;
-  for (int i = 0; i < 8; ++i) ints_out[i] = ints.v[i];
+  for (int i = 0; i < 6; ++i) ints_out[i] = ints.v[i];
   MatScalars* sc = mt.sc;
   sc->prev_norm = (*norm_prev < 0.f) ? -1.f : *norm_prev;
-  sc->lambda = 1.f; sc->norm_scaled = 0.f; sc->k_min = 0.f; sc->k_max = 0.f; sc->pad = 0.f;
+  sc->lambda = 1.f; sc->norm_scaled = 0.f; sc->k_min = 0.f; sc->k_max = 0.f;
+  sc->pad = bias_factor(beta1, beta2, *t + 1);
   sc->t = *t;
 }
 __global__ void k_noalloc_store_scalars(const MatScalars* sc, float* norm_prev, long long* t) {
@@ -145,6 +149,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   mt.Xt = reinterpret_cast<float*>(base + cv.off_xt);
   mt.kvec = reinterpret_cast<float*>(base + cv.off_k);
   mt.part = reinterpret_cast<float*>(base + cv.off_part);
+  mt.aux = reinterpret_cast<float*>(base + kNoAllocScratchBytes);
   mt.m = desc->m; mt.n = desc->n; mt.r = desc->r;
   mt.ld = desc->ld ? desc->ld : desc->n;
   mt.left = desc->m <= desc->n;
@@ -154,20 +159,19 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
 
   const int ptiles = simt_tiles(mt.l) * simt_tiles(mt.r);
   const int wtiles = simt_tiles(mt.m) * simt_tiles(mt.n);
-  const NoAllocInts ints = {{0, 0, ptiles, 0, mt.l, 0, wtiles, wtiles}};
+  const NoAllocInts ints = {{0, 0, ptiles, 0, wtiles, wtiles}};
   int* ints_dev = reinterpret_cast<int*>(base + cv.off_ints);
   // sticky across calls until fira_noalloc_poll() reads it (zero when the library is loaded)
   unsigned* status_dev = reinterpret_cast<unsigned*>(base + cv.off_status);
 
   k_noalloc_setup<<<1, 1, 0, st>>>(mt, ints, reinterpret_cast<MatDev*>(base + cv.off_mats), ints_dev,
-                                   norm_prev_dev, reinterpret_cast<const long long*>(t_dev));
+                                   norm_prev_dev, reinterpret_cast<const long long*>(t_dev), hp->beta1, hp->beta2);
   SimtPlan pl;
   pl.mats = reinterpret_cast<const MatDev*>(base + cv.off_mats);
   pl.list = ints_dev; pl.nlist = 1;
   pl.proj_tile_start = ints_dev + 1; pl.proj_tiles = ptiles;
-  pl.row_start = ints_dev + 3; pl.rows_total = mt.l;
-  pl.w_tile_start = ints_dev + 5; pl.w_tiles = wtiles;
-  pl.npart = ints_dev + 7;
+  pl.w_tile_start = ints_dev + 3; pl.w_tiles = wtiles;
+  pl.npart = ints_dev + 5;
   Hyper h;
   h.beta1 = hp->beta1; h.beta2 = hp->beta2; h.eps = hp->eps;
   h.lr = lr < 0.f ? hp->lr : lr;
@@ -176,7 +180,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   h.mode = 0;
   h.gamma = hp->gamma;
   PhaseTimer no_timer;
-  launch_simt_step(pl, h, status_dev, st, &no_timer);
+  if (launch_simt_step(pl, h, status_dev, st, &no_timer) < 0) return FIRA_ERR_CUDA;
   k_noalloc_store_scalars<<<1, 1, 0, st>>>(mt.sc, norm_prev_dev, reinterpret_cast<long long*>(t_dev));
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -7,14 +7,14 @@
 // barrier.
 #pragma once
 #include "common.cuh"
+#include "step_simt.cuh"
 
 namespace fira {
 
 constexpr int TM = 64, TN = 64, TK = 16;    // the Q = 1 tile
 constexpr int GEMM_THREADS = 256;
-constexpr int SIMT_Q = 2;                   // tile factor of the step and refresh products (128 x 128)
-constexpr int SIMT_TILE = 64 * SIMT_Q;
-inline int simt_tiles(long long extent) { return (int)((extent + SIMT_TILE - 1) / SIMT_TILE); }
+constexpr int SIMT_Q = 2;                   // tile factor of the refresh products (128 x 128)
+static_assert(SIMT_TILE == 64 * SIMT_Q, "one tile size");
 
 // Row (or column) of accumulator index x within a tile: quadrant x / 4, then the thread's 4.
 __device__ __forceinline__ int tile_coord(int t16, int x) { return (x >> 2) * 64 + t16 * 4 + (x & 3); }

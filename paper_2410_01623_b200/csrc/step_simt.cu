@@ -1,18 +1,25 @@
-// fp32 CUDA-core kernels of the Fira step (Algorithm 1's loop body), grouped over
-// a list of matrices: one launch per phase covers every matrix of the list.
+// Kernels of the Fira step (Algorithm 1's loop body) in fp32 precision, grouped over a list of
+// matrices of any size and pitch: one launch per phase covers every matrix of the list.
 //
 // Phases (l = unprojected index, d = projected index, Pi = the d x r projection):
-//   1. project      Rt[l][j]   = sum_d G(d,l) Pi[d][j]                      (R = P^T G)
-//   2. adam_rows    M,V update, N, k_l = ||N_l|| / (||R_l|| + eps)           (Eq. 2-4, Eq. 11)
-//   3. back_project mode NORM:   part = sum (k_l (G - Pi R))^2               (||S||, literal residual)
-//   4. finalize     lambda, ||S_prev||, t                                    (Eq. 12)
-//   5. form_x       Xt = a_low N - a_res lambda k_l R
-//   6. back_project mode UPDATE: W -= lr (Pi X + a_res lambda k_l G)
-// Phase 6 uses the identity alpha (P N + lambda (G - P R) diag k) =
-// P (alpha N - alpha lambda R diag k) + alpha lambda G diag k, so that the update
-// needs one product instead of two.
+//   1. project      R[l][j] = sum_d G(d,l) Pi[d][j]  (R = P^T G); epilogue: M, V update, N (Eq. 2-4) and the
+//                   row sums ||N_l||^2, ||R_l||^2 of which k_l = ||N_l|| / (||R_l|| + eps) is made (Eq. 11)
+//   2. norm         D = Pi R; part = sum (k_l (G - D))^2                   (||S||, literal residual)
+//   3. finalize     lambda, ||S_prev||, t                                  (Eq. 12)
+//   4. update       D = Pi X with X = a_low N - a_res lambda k_l R; W -= lr (D + a_res lambda k_l G)
+// Phase 4 uses the identity alpha (P N + lambda (G - P R) diag k) =
+// P (alpha N - alpha lambda R diag k) + alpha lambda G diag k, so that the update needs one product
+// instead of two; X is formed while the product loads N and R.
+//
+// The products are the 128 x 128 tile products of split_gemm.cuh: fp32 precision on the tensor cores.  Every
+// epilogue takes the finished tile from shared memory, one warp per row, so that all traffic with
+// global memory runs along rows.
+//
+// Measured (56 fp32 matrices of 8 layers 512 / 1376, r = 128; one 512 x 1376 matrix): see each kernel.
+#include <atomic>
+
 #include "common.cuh"
-#include "simt_gemm.cuh"
+#include "split_gemm.cuh"
 #include "step_simt.cuh"
 
 namespace fira {
@@ -21,256 +28,330 @@ namespace {
 
 __device__ __forceinline__ int simt_tiles_dev(int extent) { return (extent + SIMT_TILE - 1) / SIMT_TILE; }
 
-// ---------------------------------------------------------------- phase 1
+// Four entries of a row per lane: the neighbours 4 lane .. 4 lane + 3 where a row's groups of four are
+// aligned (VEC), lane, lane + 32, ... otherwise; either way a warp's access is contiguous.
+template <bool VEC>
+__device__ __forceinline__ int lane_col(int lane, int c) { return VEC ? 4 * lane + c : lane + 32 * c; }
+
+template <bool VEC>
+__device__ __forceinline__ void load_row(const float* p, int lane, int n, float (&v)[4]) {
+  if (VEC) {
+    const float4 u = 4 * lane < n ? *reinterpret_cast<const float4*>(p + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = lane + 32 * c < n ? p[lane + 32 * c] : 0.f;
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void load_row(const __nv_bfloat16* p, int lane, int n, float (&v)[4]) {
+  if (VEC) {
+    const uint2 u = 4 * lane < n ? *reinterpret_cast<const uint2*>(p + 4 * lane) : make_uint2(0u, 0u);
+    v[0] = __uint_as_float(u.x << 16); v[1] = __uint_as_float(u.x & 0xffff0000u);
+    v[2] = __uint_as_float(u.y << 16); v[3] = __uint_as_float(u.y & 0xffff0000u);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = lane + 32 * c < n ? __bfloat162float(p[lane + 32 * c]) : 0.f;
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void store_row(float* p, int lane, int n, const float (&v)[4]) {
+  if (VEC) {
+    if (4 * lane < n) *reinterpret_cast<float4*>(p + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) if (lane + 32 * c < n) p[lane + 32 * c] = v[c];
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void store_row(__nv_bfloat16* p, int lane, int n, const float (&v)[4]) {
+  if (VEC) {
+    if (4 * lane < n) {
+      const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+      uint2 u;
+      u.x = *reinterpret_cast<const unsigned*>(&a); u.y = *reinterpret_cast<const unsigned*>(&b);
+      *reinterpret_cast<uint2*>(p + 4 * lane) = u;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) if (lane + 32 * c < n) p[lane + 32 * c] = __float2bfloat16_rn(v[c]);
+  }
+}
+// n entries per row (a multiple of 4 from an aligned start, or any number), rows `pitch` entries apart
 template <typename T>
-__device__ __forceinline__ void project_tile(const MatDev& mt, int tile, float (*As)[SIMT_TILE + 4],
-                                             float (*Bs)[SIMT_TILE + 4]) {
-  const int rt = simt_tiles_dev(mt.r);
-  const int i0 = (tile / rt) * SIMT_TILE, j0 = (tile % rt) * SIMT_TILE;
-  float acc[4 * SIMT_Q][4 * SIMT_Q] = {};
-  const T* G = static_cast<const T*>(mt.G);
-  const T* P = static_cast<const T*>(mt.P);
-  // A(i = l, k = d): G[d][l] when left, G[l][d] when right.
-  const long long sAi = mt.left ? 1 : mt.ld, sAk = mt.left ? mt.ld : 1;
-  gemm_tile<SIMT_Q, T, T>(G, sAi, sAk, P, mt.r, 1, mt.l, mt.r, mt.d, i0, j0, acc, As, Bs);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+__device__ __forceinline__ bool rows_vec(const T* base, long long pitch, int n) {
+  return pitch % 4 == 0 && n % 4 == 0 && reinterpret_cast<unsigned long long>(base) % (4 * sizeof(T)) == 0;
+}
+
+constexpr int ROWS_AT_ONCE = 4;                 // rows of a warp whose loads are in flight together
+constexpr int WARP_ROWS = SIMT_TILE / (split::THREADS / 32);
+
+// ---------------------------------------------------------------- phase 1
+// Rows of the finished tile R: Adam (Eq. 2-4), N and R to scratch, row sums.
+template <bool VEC>
+__device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, const float* C, const Hyper& hp, float bias) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = min(SIMT_TILE, mt.r - j0);
+  const int nrt = simt_tiles_dev(mt.r), q = j0 / SIMT_TILE;
+  const bool momentum = !(hp.mode & (HYPER_PSI_RMSPROP | HYPER_PSI_ADAGRAD));
+  for (int x = 0; x < WARP_ROWS; x += ROWS_AT_ONCE) {
+    float m[ROWS_AT_ONCE][4], v[ROWS_AT_ONCE][4];
 #pragma unroll
-  for (int x = 0; x < 4 * SIMT_Q; ++x) {
-    const int i = i0 + tile_coord(ty, x);
-    if (i >= mt.l) continue;
+    for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+      const int l = l0 + warp * WARP_ROWS + x + y;
+      const long long at = (long long)l * mt.r + j0;
+      load_row<VEC>(mt.V + at, lane, l < mt.l ? n : 0, v[y]);
+      load_row<VEC>(mt.M + at, lane, l < mt.l && momentum ? n : 0, m[y]);
+    }
 #pragma unroll
-    for (int y = 0; y < 4 * SIMT_Q; ++y) {
-      const int j = j0 + tile_coord(tx, y);
-      if (j < mt.r) mt.Rt[(long long)i * mt.r + j] = acc[x][y];
+    for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+      const int row = warp * WARP_ROWS + x + y, l = l0 + row;
+      if (l >= mt.l) continue;
+      const long long at = (long long)l * mt.r + j0;
+      float rv[4], nv[4], nn = 0.f, rn = 0.f;
+      load_row<VEC>(C + row * split::C_LD, lane, n, rv);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (hp.mode & HYPER_PSI_RMSPROP) {
+          v[y][c] = hp.beta2 * v[y][c] + (1.f - hp.beta2) * rv[c] * rv[c];
+          nv[c] = rv[c] / (sqrtf(v[y][c]) + hp.eps);
+        } else if (hp.mode & HYPER_PSI_ADAGRAD) {
+          v[y][c] = v[y][c] + rv[c] * rv[c];
+          nv[c] = rv[c] / (sqrtf(v[y][c]) + hp.eps);
+        } else {
+          m[y][c] = hp.beta1 * m[y][c] + (1.f - hp.beta1) * rv[c];
+          v[y][c] = hp.beta2 * v[y][c] + (1.f - hp.beta2) * rv[c] * rv[c];
+          nv[c] = bias * m[y][c] / (sqrtf(v[y][c]) + hp.eps);
+        }
+        nn = fmaf(nv[c], nv[c], nn);            // (entries past the row's end are zeros throughout)
+        rn = fmaf(rv[c], rv[c], rn);
+      }
+      if (momentum) store_row<VEC>(mt.M + at, lane, n, m[y]);
+      store_row<VEC>(mt.V + at, lane, n, v[y]);
+      store_row<VEC>(mt.Xt + at, lane, n, nv);
+      store_row<VEC>(mt.Rt + at, lane, n, rv);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        nn += __shfl_xor_sync(0xffffffffu, nn, o);
+        rn += __shfl_xor_sync(0xffffffffu, rn, o);
+      }
+      if (lane == 0) {
+        if (hp.mode & HYPER_NO_SCALING) mt.kvec[l] = 1.f;
+        else if (nrt == 1 && !(hp.mode & HYPER_MATRIX_SCALING)) mt.kvec[l] = sqrtf(nn) / (sqrtf(rn) + hp.eps);
+        else { mt.aux[(long long)q * mt.l + l] = nn; mt.aux[(long long)(nrt + q) * mt.l + l] = rn; }
+      }
     }
   }
 }
 
-__global__ void __launch_bounds__(GEMM_THREADS, 2)
+template <typename T>
+__device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, unsigned char* smem, split::Ctl* ctl) {
+  // A(i = l, k = d): G[d][l] when left, G[l][d] when right.
+  split::Operand<T> a(static_cast<const T*>(mt.G), mt.left ? 1 : mt.ld, mt.left ? mt.ld : 1, mt.l, mt.d, l0);
+  split::Operand<T> b(static_cast<const T*>(mt.P), 1, mt.r, mt.r, mt.d, j0);
+  return split::tile_product<true>(a, b, mt.d, mt.r - j0, smem, ctl);
+}
+
+__global__ void __launch_bounds__(split::THREADS, 2)
 k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
-          const int* __restrict__ tile_start, int first) {
-  __shared__ __align__(16) float As[TK][SIMT_TILE + 4];
-  __shared__ __align__(16) float Bs[TK][SIMT_TILE + 4];
+          const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  split::Ctl* ctl = reinterpret_cast<split::Ctl*>(smem + split::STAGES * split::STAGE_BYTES);
   const int gt = blockIdx.x + first;
   const int p = find_matrix(tile_start, nlist, gt);
   const MatDev mt = mats[list[p]];
-  const int tile = gt - tile_start[p];
-  if (mt.bf16) project_tile<__nv_bfloat16>(mt, tile, As, Bs);
-  else project_tile<float>(mt, tile, As, Bs);
+  const int tile = gt - tile_start[p], rt = simt_tiles_dev(mt.r);
+  const int l0 = (tile / rt) * SIMT_TILE, j0 = (tile % rt) * SIMT_TILE;
+  split::begin(ctl);
+  const bool ok = mt.bf16 ? project_tile<__nv_bfloat16>(mt, l0, j0, smem, ctl) : project_tile<float>(mt, l0, j0, smem, ctl);
+  if (ok) {
+    const float bias = mt.sc->pad;
+    if (mt.r % 4 == 0) adam_rows<true>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
+    else adam_rows<false>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
+  }
+  split::end(ctl, status);
 }
 
-// ---------------------------------------------------------------- phase 2
-// One warp per unprojected index l.  N goes to Xt.
-__global__ void __launch_bounds__(256)
-k_adam_rows(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
-            const int* __restrict__ row_start, int first_row, int rows_total, Hyper hp) {
-  const int warps_per_block = blockDim.x >> 5;
-  const int lane = threadIdx.x & 31;
-  const int row = first_row + blockIdx.x * warps_per_block + (threadIdx.x >> 5);
-  if (row >= rows_total) return;
-  const int p = find_matrix(row_start, nlist, row);
-  const MatDev mt = mats[list[p]];
-  const int l = row - row_start[p];
-  // bias correction sqrt(1 - b2^s) / (1 - b1^s), s = t + 1, in double
-  const double s = (double)(mt.sc->t + 1);
-  const float bias = (float)(sqrt(1.0 - pow((double)hp.beta2, s)) / (1.0 - pow((double)hp.beta1, s)));
-  const long long base = (long long)l * mt.r;
-  float nn = 0.f, rn = 0.f;
-  // four entries per lane at a time, their loads before their stores (see back_tile)
-  for (int jq = lane; jq < mt.r; jq += 128) {
-    float rv4[4], m4[4], v4[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = jq + 32 * u;
-      const bool in = j < mt.r;
-      rv4[u] = in ? mt.Rt[base + j] : 0.f;
-      v4[u] = in ? mt.V[base + j] : 0.f;
-      m4[u] = (in && !(hp.mode & (HYPER_PSI_RMSPROP | HYPER_PSI_ADAGRAD))) ? mt.M[base + j] : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = jq + 32 * u;
-      if (j >= mt.r) continue;
-      const float rv = rv4[u];
-      float vv, nv;
-      if (hp.mode & HYPER_PSI_RMSPROP) {
-        vv = hp.beta2 * v4[u] + (1.f - hp.beta2) * rv * rv;
-        nv = rv / (sqrtf(vv) + hp.eps);
-      } else if (hp.mode & HYPER_PSI_ADAGRAD) {
-        vv = v4[u] + rv * rv;
-        nv = rv / (sqrtf(vv) + hp.eps);
-      } else {
-        const float mv = hp.beta1 * m4[u] + (1.f - hp.beta1) * rv;
-        vv = hp.beta2 * v4[u] + (1.f - hp.beta2) * rv * rv;
-        mt.M[base + j] = mv;
-        nv = bias * mv / (sqrtf(vv) + hp.eps);
-      }
-      mt.V[base + j] = vv;
-      mt.Xt[base + j] = nv;
-      nn = fmaf(nv, nv, nn);
-      rn = fmaf(rv, rv, rn);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nn += __shfl_xor_sync(0xffffffffu, nn, o);
-    rn += __shfl_xor_sync(0xffffffffu, rn, o);
-  }
-  if (lane == 0) {
-    if (hp.mode & HYPER_MATRIX_SCALING) {        // the factor comes from the whole matrix: k_finalize
-      mt.aux[l] = nn; mt.aux[mt.l + l] = rn; mt.kvec[l] = 1.f;
-    } else if (hp.mode & HYPER_NO_SCALING) {
-      mt.kvec[l] = 1.f;
-    } else {
-      mt.kvec[l] = sqrtf(nn) / (sqrtf(rn) + hp.eps);
-    }
-  }
-}
-
-// ---------------------------------------------------------------- phases 3 and 6
+// ---------------------------------------------------------------- phases 2 and 4
 enum { MODE_NORM = 0, MODE_UPDATE = 1 };
 
-template <typename T, int MODE>
-__device__ __forceinline__ void back_tile(const MatDev& mt, int tile, float lr, float a_res,
-                                          float (*As)[SIMT_TILE + 4], float (*Bs)[SIMT_TILE + 4], float* red) {
-  const int ct = simt_tiles_dev(mt.n);
-  const int i0 = (tile / ct) * SIMT_TILE, j0 = (tile % ct) * SIMT_TILE;
-  float acc[4 * SIMT_Q][4 * SIMT_Q] = {};
-  const T* P = static_cast<const T*>(mt.P);
-  const float* X = (MODE == MODE_NORM) ? mt.Rt : mt.Xt;
-  const long long r = mt.r;
-  if (mt.left) {
-    // D[d][l] = sum_j Pi[d][j] X[l][j]
-    gemm_tile<SIMT_Q, T, float>(P, r, 1, X, 1, r, mt.m, mt.n, mt.r, i0, j0, acc, As, Bs);
-  } else {
-    // D[l][d] = sum_j X[l][j] Pi[d][j]
-    gemm_tile<SIMT_Q, float, T>(X, r, 1, P, 1, r, mt.m, mt.n, mt.r, i0, j0, acc, As, Bs);
+// The factor k_l from the row sums, where more than one tile of R holds parts of the row.
+__device__ __forceinline__ float row_factor(const MatDev& mt, int l, const Hyper& hp) {
+  const int nrt = simt_tiles_dev(mt.r);
+  float nn = 0.f, rn = 0.f;
+  for (int q = 0; q < nrt; ++q) { nn += mt.aux[(long long)q * mt.l + l]; rn += mt.aux[(long long)(nrt + q) * mt.l + l]; }
+  return sqrtf(nn) / (sqrtf(rn) + hp.eps);
+}
+
+// ks[x] <- the factor of the tile's column (left) or row (right) x.  The first phase that asks makes them
+// from the row sums and leaves them in the k table for the phases that follow.
+template <int MODE>
+__device__ __forceinline__ void tile_factors(const MatDev& mt, int i0, int j0, int tile, const Hyper& hp, float* ks) {
+  const bool ones = MODE == MODE_NORM && (hp.mode & (HYPER_NO_SCALING | HYPER_MATRIX_SCALING));
+  const bool from_sums = MODE == MODE_NORM && !ones && simt_tiles_dev(mt.r) > 1;
+  if ((int)threadIdx.x < tile) {
+    const int l = (mt.left ? j0 : i0) + threadIdx.x;
+    float k = 0.f;
+    if (l < mt.l) {
+      k = ones ? 1.f : from_sums ? row_factor(mt, l, hp) : mt.kvec[l];
+      if (from_sums && (mt.left ? i0 : j0) == 0) mt.kvec[l] = k;
+    }
+    ks[threadIdx.x] = k;
   }
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+}
+
+// Rows of the finished tile D.  ks[]: the factors of the tile's columns (left) or rows (right).
+template <typename T, int MODE, bool VEC>
+__device__ __forceinline__ float back_rows(const MatDev& mt, int i0, int j0, const float* C, const float* ks, float lr, float cres) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = min(SIMT_TILE, mt.n - j0);
   const T* G = static_cast<const T*>(mt.G);
   T* W = static_cast<T*>(mt.W);
-  const float lam = (MODE == MODE_UPDATE) ? mt.sc->lambda : 1.f;
-  float ss = 0.f;
-  // Two rows of the thread's entries at a time: every load of the pair first, then the arithmetic
-  // and the stores.  (Written element by element, each load of G and W would wait for the store
-  // before it, since the compiler cannot tell that they never overlap.)
+  float kc[4], ss = 0.f;
 #pragma unroll
-  for (int xb = 0; xb < 4 * SIMT_Q; xb += 2) {
-    float g[2][4 * SIMT_Q], w[2][4 * SIMT_Q], kf[2][4 * SIMT_Q];
+  for (int c = 0; c < 4; ++c) kc[c] = mt.left ? ks[lane_col<VEC>(lane, c)] : 0.f;
+  for (int x = 0; x < WARP_ROWS; x += ROWS_AT_ONCE) {
+    float g[ROWS_AT_ONCE][4], w[ROWS_AT_ONCE][4];
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      const int i = i0 + tile_coord(ty, xb + x);
-#pragma unroll
-      for (int y = 0; y < 4 * SIMT_Q; ++y) {
-        const int j = j0 + tile_coord(tx, y);
-        const bool in = i < mt.m && j < mt.n;
-        const long long off = (long long)i * mt.ld + j;
-        kf[x][y] = in ? mt.kvec[mt.left ? j : i] : 0.f;
-        g[x][y] = in ? to_float<T>(G[off]) : 0.f;
-        w[x][y] = (MODE == MODE_UPDATE && in) ? to_float<T>(W[off]) : 0.f;
-      }
+    for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+      const int i = i0 + warp * WARP_ROWS + x + y;
+      const long long at = (long long)i * mt.ld + j0;
+      load_row<VEC>(G + at, lane, i < mt.m ? n : 0, g[y]);
+      if (MODE == MODE_UPDATE) load_row<VEC>(W + at, lane, i < mt.m ? n : 0, w[y]);
     }
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      const int i = i0 + tile_coord(ty, xb + x);
+    for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+      const int row = warp * WARP_ROWS + x + y, i = i0 + row;
       if (i >= mt.m) continue;
+      float dv[4];
+      load_row<VEC>(C + row * split::C_LD, lane, n, dv);
+      const float kr = mt.left ? 0.f : ks[row];
 #pragma unroll
-      for (int y = 0; y < 4 * SIMT_Q; ++y) {
-        const int j = j0 + tile_coord(tx, y);
-        if (j >= mt.n) continue;
+      for (int c = 0; c < 4; ++c) {
+        const float kf = mt.left ? kc[c] : kr;
         if (MODE == MODE_NORM) {
-          const float sv = kf[x][y] * (g[x][y] - acc[xb + x][y]);
+          const float sv = kf * (g[y][c] - dv[c]);          // (zero past the row's end)
           ss = fmaf(sv, sv, ss);
         } else {
-          W[(long long)i * mt.ld + j] =
-              from_float<T>(w[x][y] - lr * (acc[xb + x][y] + a_res * lam * kf[x][y] * g[x][y]));
+          w[y][c] = w[y][c] - lr * (dv[c] + cres * kf * g[y][c]);
         }
       }
-    }
-  }
-  if (MODE == MODE_NORM) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float tot = 0.f;
-      for (int w = 0; w < GEMM_THREADS / 32; ++w) tot += red[w];
-      mt.part[tile] = tot;
-    }
-  }
-}
-
-template <int MODE>
-__global__ void __launch_bounds__(GEMM_THREADS, 2)
-k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
-               const int* __restrict__ tile_start, int first, float lr, float a_res) {
-  __shared__ __align__(16) float As[TK][SIMT_TILE + 4];
-  __shared__ __align__(16) float Bs[TK][SIMT_TILE + 4];
-  __shared__ float red[GEMM_THREADS / 32];
-  const int gt = blockIdx.x + first;
-  const int p = find_matrix(tile_start, nlist, gt);
-  const MatDev mt = mats[list[p]];
-  const int tile = gt - tile_start[p];
-  if (mt.bf16) back_tile<__nv_bfloat16, MODE>(mt, tile, lr, a_res, As, Bs, red);
-  else back_tile<float, MODE>(mt, tile, lr, a_res, As, Bs, red);
-}
-
-// ---------------------------------------------------------------- phase 5
-__global__ void __launch_bounds__(256)
-k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
-         const int* __restrict__ row_start, int first_row, int rows_total, float a_low, float a_res) {
-  const int lane = threadIdx.x & 31;
-  const int row = first_row + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= rows_total) return;
-  const int p = find_matrix(row_start, nlist, row);
-  const MatDev mt = mats[list[p]];
-  const int l = row - row_start[p];
-  const float c = a_res * mt.sc->lambda * mt.kvec[l];
-  const long long base = (long long)l * mt.r;
-  for (int jq = lane; jq < mt.r; jq += 128) {    // four entries per lane, loads before stores
-    float n4[4], r4[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = jq + 32 * u;
-      n4[u] = j < mt.r ? mt.Xt[base + j] : 0.f;
-      r4[u] = j < mt.r ? mt.Rt[base + j] : 0.f;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = jq + 32 * u;
-      if (j < mt.r) mt.Xt[base + j] = a_low * n4[u] - c * r4[u];
-    }
-  }
-}
-
-// ---------------------------------------------------------------- Fira-only-scaling
-// W <- W - lr phi(R) G: no product.  One block per tile x tile block of W; rows are walked by the
-// warps, columns by the lanes (coalesced along the rows of G and W).
-template <typename T, int UPDATE>
-__device__ __forceinline__ float scaled_gradient_tile(const MatDev& mt, int i0, int j0, int tile, float c) {
-  const T* G = static_cast<const T*>(mt.G);
-  T* W = static_cast<T*>(mt.W);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i1 = min(i0 + tile, mt.m), j1 = min(j0 + tile, mt.n);
-  float ss = 0.f;
-  for (int i = i0 + warp; i < i1; i += 8) {
-    const float krow = mt.left ? 0.f : mt.kvec[i];
-    for (int j = j0 + lane; j < j1; j += 32) {
-      const float kf = mt.left ? mt.kvec[j] : krow;
-      const long long off = (long long)i * mt.ld + j;
-      const float g = to_float<T>(G[off]);
-      if (UPDATE) W[off] = from_float<T>(to_float<T>(W[off]) - c * kf * g);
-      else { const float sv = kf * g; ss = fmaf(sv, sv, ss); }
+      if (MODE == MODE_UPDATE) store_row<VEC>(W + (long long)i * mt.ld + j0, lane, n, w[y]);
     }
   }
   return ss;
 }
 
+template <typename T, int MODE>
+__device__ __forceinline__ bool back_product(const MatDev& mt, int i0, int j0, float a_low, float cres,
+                                             unsigned char* smem, split::Ctl* ctl) {
+  // left: D[d][l] = sum_j Pi[d][j] X[l][j]; right: D[l][d] = sum_j X[l][j] Pi[d][j]
+  const int cols = mt.n - j0;
+  split::Operand<T> p(static_cast<const T*>(mt.P), mt.r, 1, mt.d, mt.r, mt.left ? i0 : j0);
+  p.along_x = false; p.ld = mt.r;               // (r = 1 would count as contiguous along d)
+  const int x0 = mt.left ? j0 : i0;
+  if (MODE == MODE_NORM) {
+    split::Operand<float> x(mt.Rt, mt.r, 1, mt.l, mt.r, x0);
+    x.along_x = false; x.ld = mt.r;
+    return mt.left ? split::tile_product<false>(p, x, mt.r, cols, smem, ctl) : split::tile_product<false>(x, p, mt.r, cols, smem, ctl);
+  } else {
+    split::CombinedOperand x(mt.Xt, mt.Rt, mt.r, mt.l, mt.r, x0, mt.kvec, a_low, cres);
+    return mt.left ? split::tile_product<false>(p, x, mt.r, cols, smem, ctl) : split::tile_product<false>(x, p, mt.r, cols, smem, ctl);
+  }
+}
+
+template <typename T, int MODE>
+__device__ __forceinline__ float back_tile(const MatDev& mt, int i0, int j0, const Hyper& hp, unsigned char* smem,
+                                           split::Ctl* ctl, float* ks) {
+  const float cres = MODE == MODE_UPDATE ? hp.a_res * mt.sc->lambda : 0.f;
+  tile_factors<MODE>(mt, i0, j0, SIMT_TILE, hp, ks);
+  if (!back_product<T, MODE>(mt, i0, j0, hp.a_low, cres, smem, ctl)) return 0.f;
+  const float* C = reinterpret_cast<const float*>(smem);
+  const bool vec = rows_vec(static_cast<const T*>(mt.G), mt.ld, mt.n) && rows_vec(static_cast<const T*>(mt.W), mt.ld, mt.n);
+  return vec ? back_rows<T, MODE, true>(mt, i0, j0, C, ks, hp.lr, cres) : back_rows<T, MODE, false>(mt, i0, j0, C, ks, hp.lr, cres);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(split::THREADS, 2)
+k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
+               const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ float ks[SIMT_TILE];
+  split::Ctl* ctl = reinterpret_cast<split::Ctl*>(smem + split::STAGES * split::STAGE_BYTES);
+  const int gt = blockIdx.x + first;
+  const int p = find_matrix(tile_start, nlist, gt);
+  const MatDev mt = mats[list[p]];
+  const int tile = gt - tile_start[p], ct = simt_tiles_dev(mt.n);
+  const int i0 = (tile / ct) * SIMT_TILE, j0 = (tile % ct) * SIMT_TILE;
+  split::begin(ctl);
+  float ss = mt.bf16 ? back_tile<__nv_bfloat16, MODE>(mt, i0, j0, hp, smem, ctl, ks)
+                     : back_tile<float, MODE>(mt, i0, j0, hp, smem, ctl, ks);
+  if (MODE == MODE_NORM) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((threadIdx.x & 31) == 0) ctl->red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      float tot = 0.f;
+      for (int w = 0; w < split::THREADS / 32; ++w) tot += ctl->red[w];
+      mt.part[tile] = tot;
+    }
+  }
+  split::end(ctl, status);
+}
+
+// ---------------------------------------------------------------- Fira-only-scaling
+// W <- W - lr phi(R) G: no product.  One block per tile x tile elements of W, a warp per row.
+template <typename T, int UPDATE, bool VEC>
+__device__ __forceinline__ float scaled_gradient_rows(const MatDev& mt, int i0, int j0, int tile, const float* ks, float c) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const T* G = static_cast<const T*>(mt.G);
+  T* W = static_cast<T*>(mt.W);
+  float ss = 0.f;
+  for (int jc = 0; jc < tile && j0 + jc < mt.n; jc += 128) {
+    const int n = min(128, mt.n - j0 - jc);
+    float kc[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) kc[q] = mt.left ? ks[jc + lane_col<VEC>(lane, q)] : 0.f;
+    for (int x = warp * ROWS_AT_ONCE; x < tile; x += 8 * ROWS_AT_ONCE) {
+      float g[ROWS_AT_ONCE][4], w[ROWS_AT_ONCE][4];
+#pragma unroll
+      for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+        const int i = i0 + x + y;
+        const long long at = (long long)i * mt.ld + j0 + jc;
+        load_row<VEC>(G + at, lane, i < mt.m ? n : 0, g[y]);
+        if (UPDATE) load_row<VEC>(W + at, lane, i < mt.m ? n : 0, w[y]);
+      }
+#pragma unroll
+      for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+        const int i = i0 + x + y;
+        if (i >= mt.m) continue;
+        const float kr = mt.left ? 0.f : ks[x + y];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float kf = mt.left ? kc[q] : kr;
+          if (UPDATE) w[y][q] = w[y][q] - c * kf * g[y][q];
+          else { const float sv = kf * g[y][q]; ss = fmaf(sv, sv, ss); }
+        }
+        if (UPDATE) store_row<VEC>(W + (long long)i * mt.ld + j0 + jc, lane, n, w[y]);
+      }
+    }
+  }
+  return ss;
+}
+
+template <typename T, int UPDATE>
+__device__ __forceinline__ float scaled_gradient_tile(const MatDev& mt, int i0, int j0, int tile, const float* ks, float c) {
+  const bool vec = rows_vec(static_cast<const T*>(mt.G), mt.ld, mt.n) && rows_vec(static_cast<const T*>(mt.W), mt.ld, mt.n);
+  return vec ? scaled_gradient_rows<T, UPDATE, true>(mt, i0, j0, tile, ks, c)
+             : scaled_gradient_rows<T, UPDATE, false>(mt, i0, j0, tile, ks, c);
+}
+
 template <int UPDATE>
 __global__ void __launch_bounds__(256)
 k_scaled_gradient(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
-                  const int* __restrict__ tile_start, int first, int tile, float lr, float a_res) {
+                  const int* __restrict__ tile_start, int first, int tile, Hyper hp) {
+  __shared__ float ks[256];
   __shared__ float red[8];
   const int gt = blockIdx.x + first;
   const int p = find_matrix(tile_start, nlist, gt);
@@ -278,9 +359,11 @@ k_scaled_gradient(const MatDev* __restrict__ mats, const int* __restrict__ list,
   const int t = gt - tile_start[p];
   const int ct = (mt.n + tile - 1) / tile;
   const int i0 = (t / ct) * tile, j0 = (t % ct) * tile;
-  const float c = UPDATE ? lr * a_res * mt.sc->lambda : 0.f;
-  float ss = mt.bf16 ? scaled_gradient_tile<__nv_bfloat16, UPDATE>(mt, i0, j0, tile, c)
-                     : scaled_gradient_tile<float, UPDATE>(mt, i0, j0, tile, c);
+  tile_factors<UPDATE ? MODE_UPDATE : MODE_NORM>(mt, i0, j0, tile, hp, ks);
+  __syncthreads();
+  const float c = UPDATE ? hp.lr * hp.a_res * mt.sc->lambda : 0.f;
+  float ss = mt.bf16 ? scaled_gradient_tile<__nv_bfloat16, UPDATE>(mt, i0, j0, tile, ks, c)
+                     : scaled_gradient_tile<float, UPDATE>(mt, i0, j0, tile, ks, c);
   if (!UPDATE) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -297,13 +380,13 @@ k_scaled_gradient(const MatDev* __restrict__ mats, const int* __restrict__ list,
 }  // namespace
 
 void launch_scaled_gradient(const MatDev* mats, const int* list, int nlist, const int* tile_start, int first,
-                            int tiles, int tile, int update, float lr, float a_res, cudaStream_t st) {
+                            int tiles, int tile, int update, const Hyper& hp, cudaStream_t st) {
   if (tiles <= 0) return;
-  if (update) k_scaled_gradient<1><<<tiles, 256, 0, st>>>(mats, list, nlist, tile_start, first, tile, lr, a_res);
-  else k_scaled_gradient<0><<<tiles, 256, 0, st>>>(mats, list, nlist, tile_start, first, tile, lr, a_res);
+  if (update) k_scaled_gradient<1><<<tiles, 256, 0, st>>>(mats, list, nlist, tile_start, first, tile, hp);
+  else k_scaled_gradient<0><<<tiles, 256, 0, st>>>(mats, list, nlist, tile_start, first, tile, hp);
 }
 
-// ---------------------------------------------------------------- phase 4
+// ---------------------------------------------------------------- phase 3
 __global__ void __launch_bounds__(256)
 k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
            const int* __restrict__ npart_of, Hyper hp, unsigned* __restrict__ status) {
@@ -311,6 +394,8 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   __shared__ float smin[256], smax[256];
   const MatDev mt = mats[list[blockIdx.x]];
   const int npart = npart_of[blockIdx.x];
+  // the bias factor sqrt(1 - b2^s) / (1 - b1^s) of the NEXT step, in double, while the others add up
+  if (threadIdx.x == 255) mt.sc->pad = bias_factor(hp.beta1, hp.beta2, mt.sc->t + 2);
   double acc = 0.0;
   for (int i = threadIdx.x; i < npart; i += 256) acc += (double)mt.part[i];
   // Matrix-level factor (Eq. 9): the phases before ran with k = 1, so `part` holds ||G - P R||^2;
@@ -319,7 +404,8 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   if (hp.mode & HYPER_MATRIX_SCALING) {
     __shared__ double sn[256], sr[256];
     double an = 0.0, ar = 0.0;
-    for (int i = threadIdx.x; i < mt.l; i += 256) { an += (double)mt.aux[i]; ar += (double)mt.aux[mt.l + i]; }
+    const long long sums = (long long)(mt.engine == 0 ? (mt.r + SIMT_TILE - 1) / SIMT_TILE : 1) * mt.l;   // one or more per row
+    for (long long i = threadIdx.x; i < sums; i += 256) { an += (double)mt.aux[i]; ar += (double)mt.aux[sums + i]; }
     sn[threadIdx.x] = an; sr[threadIdx.x] = ar;
     __syncthreads();
     for (int o = 128; o > 0; o >>= 1) {
@@ -372,52 +458,57 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   }
 }
 
-const char* const kSimtPhaseNames[6] = {"k_project", "k_adam_rows", "k_back_project<norm>",
-                                        "k_finalize", "k_form_x", "k_back_project<update>"};
+const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_back_project<norm>", "k_finalize", "k_back_project<update>"};
+
+// The products' shared memory is above the default limit: a per-device, per-kernel setting.
+static bool allow_smem() {
+  static std::atomic<bool> done[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
+  if (e == cudaSuccess && !done[dev].load()) {
+    const void* kernels[3] = {(const void*)k_project, (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
+    for (const void* k : kernels)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
+    if (e == cudaSuccess) done[dev].store(true);
+  }
+  if (e != cudaSuccess) set_error(std::string("step kernels, shared memory: ") + cudaGetErrorString(e));
+  return e == cudaSuccess;
+}
 
 int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, cudaStream_t st,
                      PhaseTimer* tm, int qa, int qb) {
   if (pl.nlist == 0) return 0;
-  // the sub-range [qa, qb) of the list: first tile / row and their counts from the host copies of
-  // the prefix arrays; the kernels still search the whole arrays with absolute indices
-  int pt0 = 0, pt1 = pl.proj_tiles, r0 = 0, r1 = pl.rows_total, wt0 = 0, wt1 = pl.w_tiles, nq = pl.nlist;
+  if (!allow_smem()) return -1;
+  // the sub-range [qa, qb) of the list: first tile and their counts from the host copies of the
+  // prefix arrays; the kernels still search the whole arrays with absolute indices
+  int pt0 = 0, pt1 = pl.proj_tiles, wt0 = 0, wt1 = pl.w_tiles, nq = pl.nlist;
   if (qb >= 0) {
     if (qa >= qb) return 0;
     pt0 = pl.h_proj_tile_start[qa]; pt1 = pl.h_proj_tile_start[qb];
-    r0 = pl.h_row_start[qa]; r1 = pl.h_row_start[qb];
     wt0 = pl.h_w_tile_start[qa]; wt1 = pl.h_w_tile_start[qb];
     nq = qb - qa;
   } else {
     qa = 0;
   }
+  constexpr int TH = split::THREADS, SM = split::SMEM_BYTES;
+  const bool only_scaling = hp.mode & HYPER_ONLY_SCALING;     // W <- W - lr phi(R) G: no back-projection
   tm->mark(st);
-  k_project<<<pt1 - pt0, GEMM_THREADS, 0, st>>>(pl.mats, pl.list, pl.nlist, pl.proj_tile_start, pt0);
+  k_project<<<pt1 - pt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.proj_tile_start, pt0, hp, status_dev);
   tm->mark(st);
-  const int row_blocks = (r1 - r0 + 7) / 8;
-  k_adam_rows<<<row_blocks, 256, 0, st>>>(pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp);
-  tm->mark(st);
-  if (hp.mode & HYPER_ONLY_SCALING) {
-    // W <- W - lr phi(R) G: the norm of the scaled gradient, the limiter, the element-wise update
-    launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 0, 0.f, hp.a_res, st);
-    tm->mark(st);
-    k_finalize<<<nq, 256, 0, st>>>(pl.mats, pl.list + qa, nq, pl.npart + qa, hp, status_dev);
-    tm->mark(st);
-    tm->mark(st);
-    launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 1, hp.lr, hp.a_res, st);
-    tm->mark(st);
-    return 5;
-  }
-  k_back_project<MODE_NORM><<<wt1 - wt0, GEMM_THREADS, 0, st>>>(pl.mats, pl.list, pl.nlist,
-                                                                pl.w_tile_start, wt0, 0.f, hp.a_res);
+  if (only_scaling)
+    launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 0, hp, st);
+  else
+    k_back_project<MODE_NORM><<<wt1 - wt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev);
   tm->mark(st);
   k_finalize<<<nq, 256, 0, st>>>(pl.mats, pl.list + qa, nq, pl.npart + qa, hp, status_dev);
   tm->mark(st);
-  k_form_x<<<row_blocks, 256, 0, st>>>(pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp.a_low, hp.a_res);
+  if (only_scaling)
+    launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 1, hp, st);
+  else
+    k_back_project<MODE_UPDATE><<<wt1 - wt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev);
   tm->mark(st);
-  k_back_project<MODE_UPDATE><<<wt1 - wt0, GEMM_THREADS, 0, st>>>(pl.mats, pl.list, pl.nlist,
-                                                                  pl.w_tile_start, wt0, hp.lr, hp.a_res);
-  tm->mark(st);
-  return 6;
+  return 4;
 }
 
 }  // namespace fira

@@ -817,7 +817,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     // W <- W - lr phi(R) G: no back-projection; the element-wise update works on the caller's W and
     // G in place (whatever their pitch), so nothing is copied back from the aligned copies
     tm->mark(st);
-    launch_scaled_gradient(mats, pl->list, pl->nlist, pl->k2_start, k2a, k2n, 2 * BM, 1, hp.lr, hp.a_res, st);
+    launch_scaled_gradient(mats, pl->list, pl->nlist, pl->k2_start, k2a, k2n, 2 * BM, 1, hp, st);
     tm->mark(st);
     tm->mark(st);
     return srn ? 6 : 5;

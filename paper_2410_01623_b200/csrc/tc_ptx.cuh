@@ -289,6 +289,18 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_
   return d;
 }
 
+// The same without swizzle: the operand is made of 8 x 16-byte core matrices (128 contiguous bytes).
+//   K-major: rows of a core matrix along M/N; LBO = distance of core matrices along K, SBO along M/N.
+//   MN-major: rows of a core matrix along K (eight M/N elements each); LBO along K, SBO along M/N.
+__device__ __forceinline__ uint64_t make_smem_desc_plain(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+
 // Instruction descriptor of kind::f16 with bf16 operands and fp32 accumulation:
 // c_format (bits 4-5) = 1 (f32), a_format (7-9) = b_format (10-12) = 1 (bf16),
 // a_major (15), b_major (16): 0 = K-major, 1 = MN-major; N >> 3 at bits 17-22,
