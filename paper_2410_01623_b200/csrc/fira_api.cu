@@ -59,6 +59,8 @@ int engine_for(const fira_hparams& hp, const fira_matrix_desc& d) {
   return tc_supported(d) ? 1 : 0;
 }
 
+constexpr size_t REFRESH_SMALL_LIST_BYTES = (size_t)512 << 20;
+
 Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_t count) {
   Layout L;
   size_t so = 0;
@@ -82,7 +84,7 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
   L.off_tcmaps = wo; wo += tc_tables_bytes(hp, descs, count);
   L.off_work = wo;
   size_t w = 0;
-  size_t refresh_max = 0;
+  size_t refresh_max = 0, refresh_all = 0;
   L.offRt.assign(count, 0); L.offXt.assign(count, 0); L.offK.assign(count, 0); L.offPart.assign(count, 0);
   L.offNb.assign(count, 0); L.offRb.assign(count, 0); L.offXb.assign(count, 0);
   L.offColpart.assign(count, 0); L.offGs.assign(count, 0); L.offWs.assign(count, 0); L.offAux.assign(count, 0);
@@ -109,10 +111,14 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
         L.offWs[i] = w; w += align_up((size_t)d.m * lds * 2);
       }
     }
-    refresh_max = std::max(refresh_max, refresh_bytes_per_matrix(d));
+    const size_t rb = refresh_bytes_per_matrix(d);
+    refresh_max = std::max(refresh_max, rb);
+    refresh_all += rb;
   }
   L.step_work_bytes = w;
-  L.refresh_min_bytes = refresh_max;
+  // room for the largest matrix; small models get room for all of theirs, so that one pass takes the whole
+  // list (one matrix of theirs does not fill the chip)
+  L.refresh_min_bytes = std::max(refresh_max, std::min(refresh_all, REFRESH_SMALL_LIST_BYTES));
   L.scratch_bytes = L.off_work + std::max(L.step_work_bytes, L.refresh_min_bytes);
   return L;
 }

@@ -12,9 +12,8 @@
 // The paper calls a library SVD here; the iteration converges to the same subspace
 // at the rate (sigma_{r+1}/sigma_r)^2 per round.
 //
-// Everything runs on the CUDA cores in fp32, except for bf16 matrices of tensor-core size with
-// TMA-readable rows.  For those every product of the iteration is a job of the step's projection
-// kernel in its plain-output mode (fp32 accumulation in tensor memory):
+// Products.  bf16 matrices of tensor-core size with TMA-readable rows use the step's projection kernel in
+// its plain-output mode (fp32 accumulation in tensor memory):
 //   * A Z and A^T Y: G is exact in bf16; the iterate is rounded to bf16, and in the last round it is
 //     split into a bf16 high part and a bf16 remainder (two k-segments), so that the basis that is
 //     kept carries no bf16 rounding of the iterate;
@@ -22,9 +21,13 @@
 //     that is kept both operands are fp32 matrices split into two bf16 parts, three k-segments
 //     (hi hi + hi lo + lo hi), which is good to about 2^-16: enough for CholeskyQR, whose second pass
 //     removes what the first left; for the intermediate iterates plain bf16 operands (one segment):
-//     the next product rounds the iterate to bf16 anyway, and all it asks is a well-conditioned one;
-//   * L^-T itself comes from the triangular-solve kernel applied to the identity (r x r, fp32).
-// Only the Cholesky factorisation and that small solve stay on the CUDA cores.
+//     the next product rounds the iterate to bf16 anyway, and all it asks is a well-conditioned one.
+// Every other matrix (fp32, odd pitches, small or odd ranks) is iterated in fp32 precision: G, Y, Z and L^-T
+// are kept as bf16 parts (three, or one for a bf16 G) and multiplied by the part products of
+// part_gemm.cu, which also leave their results as parts; only the Gram matrix is needed as fp32.  On the
+// CUDA cores these products were 90 % of the refresh of a list with odd-width matrices.
+// L^-T comes from the triangular-solve kernel applied to the identity (r x r, fp32); the Cholesky
+// factorisation and that small solve run on the CUDA cores.
 //
 // Random numbers: Philox4x32-10 (Salmon et al., "Parallel random numbers: as easy
 // as 1, 2, 3", SC'11), keyed by the caller's seed, turned into normals by the
@@ -32,7 +35,9 @@
 #include <algorithm>
 
 #include "context.cuh"
+#include "part_gemm.cuh"
 #include "simt_gemm.cuh"
+#include "split_gemm.cuh"
 #include "step_tc.cuh"
 
 namespace fira {
@@ -42,11 +47,15 @@ namespace {
 struct RefreshMat {
   const void* G;
   void* P;
-  float* Y;   // d x r
-  float* Z;   // l x r
   float* C;   // r x r
-  float* U;            // r x r: L^-T (tc only)
-  __nv_bfloat16* Yb;   // bf16 high parts of Y, Z, U: operands of the tensor-core products (tc only)
+  float* U;   // r x r: L^-T
+  // matrices iterated in fp32 precision: everything as bf16 parts; the two buffers of an iterate hold it
+  // before and after its orthonormalisation
+  PartMatrix Gp, Y0, Y1, Z0, Z1, Up;
+  // matrices whose products run on the step's projection kernel (tc)
+  float* Y;            // d x r
+  float* Z;            // l x r
+  __nv_bfloat16* Yb;   // bf16 high parts of Y, Z, U: operands of the tensor-core products
   __nv_bfloat16* Zb;
   __nv_bfloat16* Ub;
   __nv_bfloat16* Yl;   // bf16 remainders: X - bf16(X)
@@ -54,18 +63,11 @@ struct RefreshMat {
   __nv_bfloat16* Ul;
   float* out32;        // optional copy of the kept basis in fp32, before it is rounded for storage
   float* info;         // a few floats of the Cholesky factorisation (pivot floor)
-  int tc;              // every product of this matrix runs on the tensor cores
+  int tc;
   long long ld;
   int d, l, r;
   int left, bf16;
   unsigned long long key;
-};
-
-struct GemmDesc {
-  const void* A; long long sAi, sAk; int a_bf16;
-  const float* B; long long sBk, sBj;
-  float* C; long long sCi;
-  int I, J, K;
 };
 
 // ------------------------------------------------------------------ Philox4x32-10
@@ -104,39 +106,37 @@ k_gauss(const RefreshMat* __restrict__ rm) {
     const float v[4] = {ra * c0, ra * s0, rb * c1, rb * s1};
     for (int e = 0; e < 4; ++e) {
       const long long idx = q * 4 + e;
-      if (idx < total) m.Z[idx] = v[e];
+      if (idx >= total) break;
+      if (m.tc) { m.Z[idx] = v[e]; continue; }
+      uint32_t h, mid, lo;
+      split::split3(v[e], 0.f, h, mid, lo);
+      __nv_bfloat16_raw* o = reinterpret_cast<__nv_bfloat16_raw*>(m.Z1.base) + idx / m.r * m.Z1.pitch + idx % m.r;
+      o[0].x = (unsigned short)h; o[m.Z1.part_stride].x = (unsigned short)mid; o[2 * m.Z1.part_stride].x = (unsigned short)lo;
     }
   }
 }
 
-// ------------------------------------------------------------------ grouped product
-__global__ void __launch_bounds__(GEMM_THREADS, 2)
-k_rgemm(const GemmDesc* __restrict__ descs, int ndesc, const int* __restrict__ tile_start) {
-  __shared__ __align__(16) float As[TK][SIMT_TILE + 4];
-  __shared__ __align__(16) float Bs[TK][SIMT_TILE + 4];
-  const int p = find_matrix(tile_start, ndesc, blockIdx.x);
-  const GemmDesc g = descs[p];
-  const int tile = blockIdx.x - tile_start[p];
-  const int jt = (g.J + SIMT_TILE - 1) / SIMT_TILE;
-  const int i0 = (tile / jt) * SIMT_TILE, j0 = (tile % jt) * SIMT_TILE;
-  float acc[4 * SIMT_Q][4 * SIMT_Q] = {};
-  if (g.a_bf16)
-    gemm_tile<SIMT_Q, __nv_bfloat16, float>((const __nv_bfloat16*)g.A, g.sAi, g.sAk, g.B, g.sBk, g.sBj,
-                                    g.I, g.J, g.K, i0, j0, acc, As, Bs);
-  else
-    gemm_tile<SIMT_Q, float, float>((const float*)g.A, g.sAi, g.sAk, g.B, g.sBk, g.sBj, g.I, g.J, g.K,
-                            i0, j0, acc, As, Bs);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int x = 0; x < 4 * SIMT_Q; ++x) {
-    const int i = i0 + tile_coord(ty, x);
-    if (i >= g.I) continue;
-#pragma unroll
-    for (int y = 0; y < 4 * SIMT_Q; ++y) {
-      const int j = j0 + tile_coord(tx, y);
-      if (j < g.J) g.C[(long long)i * g.sCi + j] = acc[x][y];
-    }
+// ------------------------------------------------------------------ parts
+// What is kept as parts: G (which = 0, once) and L^-T (which = 1).  Eight neighbours per thread; the columns
+// between a matrix's width and its pitch become zeros.
+template <typename T>
+__device__ __forceinline__ void to_parts(const T* src, long long ld, const PartMatrix& p) {
+  const bool vec = ld * (long long)sizeof(T) % 16 == 0 && reinterpret_cast<unsigned long long>(src) % 16 == 0;
+  const long long per_row = p.pitch / 8, units = p.rows * per_row;
+  for (long long u = (long long)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += (long long)gridDim.x * blockDim.x) {
+    const long long i = u / per_row, j = u % per_row * 8;
+    split::Frag<T> f;
+    split::load_frag(src + i * ld + j, (int)(p.cols - j), vec, f);
+    split::store_parts(reinterpret_cast<unsigned char*>(p.base + i * p.pitch + j), f, p.part_stride * 2);
   }
+}
+__global__ void __launch_bounds__(256)
+k_to_parts(const RefreshMat* __restrict__ rm, int which) {
+  const RefreshMat& m = rm[blockIdx.y];
+  if (m.tc) return;
+  if (which == 1) to_parts(m.U, m.r, m.Up);
+  else if (m.bf16) to_parts((const __nv_bfloat16*)m.G, m.ld, m.Gp);
+  else to_parts((const float*)m.G, m.ld, m.Gp);
 }
 
 // ------------------------------------------------------------------ Cholesky
@@ -346,13 +346,11 @@ k_chol_update(const RefreshMat* __restrict__ rm, int J0, int nt) {
   }
 }
 
-// ------------------------------------------------------------------ X <- X L^-T
-// One block per tile of 64 rows of X (rows x r, in place).  For each 64-wide
-// block column J: X_J = (X_J - X_{<J} L[J, <J]^T) L_JJ^-T.
-// tri: X starts as the identity (the solve that produces L^-T itself).  The result is upper
-// triangular and stays so on the way, so a row tile starts at its own diagonal block and its
-// products run over the columns from there on: a third of the work.
-struct TrsmDesc { float* X; const float* L; int rows, r; int tri; };
+// ------------------------------------------------------------------ X <- X L^-T, X the identity: L^-T itself
+// One block per tile of 64 rows of X (r x r, in place).  For each 64-wide block column J:
+// X_J = (X_J - X_{<J} L[J, <J]^T) L_JJ^-T.  The result is upper triangular and stays so on the way, so a
+// row tile starts at its own diagonal block and its products run over the columns from there on.
+struct TrsmDesc { float* X; const float* L; int r; };
 
 __global__ void __launch_bounds__(GEMM_THREADS)
 k_trsm_rows(const TrsmDesc* __restrict__ descs, int ndesc, const int* __restrict__ tile_start) {
@@ -366,25 +364,25 @@ k_trsm_rows(const TrsmDesc* __restrict__ descs, int ndesc, const int* __restrict
   const int I0 = (blockIdx.x - tile_start[p]) * TM;
   const int r = t.r;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int K0 = t.tri ? I0 : 0;               // first column of X that can be non-zero in these rows
+  const int K0 = I0;                           // first column of X that can be non-zero in these rows
   for (int J0 = K0; J0 < r; J0 += CB) {
     const int jb = min(CB, r - J0);
     float acc[4][4] = {};
-    gemm_tile<1, float, float>(t.X + K0, r, 1, t.L + K0, 1, r, t.rows, J0 + jb, J0 - K0, I0, J0, acc, As, Bs);
+    gemm_tile<1, float, float>(t.X + K0, r, 1, t.L + K0, 1, r, r, J0 + jb, J0 - K0, I0, J0, acc, As, Bs);
     float xin[4][4];
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
       for (int y = 0; y < 4; ++y) {
         const int il = ty * 4 + x, jl = tx * 4 + y;
-        xin[x][y] = (I0 + il < t.rows && jl < jb) ? __ldcg(t.X + (long long)(I0 + il) * r + J0 + jl) : 0.f;
+        xin[x][y] = (I0 + il < r && jl < jb) ? __ldcg(t.X + (long long)(I0 + il) * r + J0 + jl) : 0.f;
       }
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
       for (int y = 0; y < 4; ++y) {
         const int il = ty * 4 + x, jl = tx * 4 + y;
-        DT[CB + il][jl] = (I0 + il < t.rows && jl < jb) ? xin[x][y] - acc[x][y] : 0.f;
+        DT[CB + il][jl] = (I0 + il < r && jl < jb) ? xin[x][y] - acc[x][y] : 0.f;
       }
 #pragma unroll
     for (int e = tid; e < CB * CB; e += GEMM_THREADS) {
@@ -409,7 +407,7 @@ k_trsm_rows(const TrsmDesc* __restrict__ descs, int ndesc, const int* __restrict
     __syncthreads();
     for (int e = tid; e < TM * CB; e += GEMM_THREADS) {
       const int i = e / CB, j = e % CB;
-      if (I0 + i < t.rows && j < jb) t.X[(long long)(I0 + i) * r + J0 + j] = DT[CB + i][j];
+      if (I0 + i < r && j < jb) t.X[(long long)(I0 + i) * r + J0 + j] = DT[CB + i][j];
     }
     __syncthreads();                           // the next block column's product reads these columns
   }
@@ -417,13 +415,20 @@ k_trsm_rows(const TrsmDesc* __restrict__ descs, int ndesc, const int* __restrict
 
 __global__ void __launch_bounds__(256)
 k_store_projection(const RefreshMat* __restrict__ rm) {
-  const RefreshMat m = rm[blockIdx.y];
+  const RefreshMat& m = rm[blockIdx.y];
   const long long total = (long long)m.d * m.r;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
-    if (m.bf16) ((__nv_bfloat16*)m.P)[i] = __float2bfloat16_rn(m.Y[i]);
-    else ((float*)m.P)[i] = m.Y[i];
-    if (m.out32) m.out32[i] = m.Y[i];
+    float y;
+    if (m.tc) {
+      y = m.Y[i];
+    } else {                                   // the sum of the parts is the fp32 number they were made of
+      const __nv_bfloat16* p = m.Y0.base + i / m.r * m.Y0.pitch + i % m.r;
+      y = __bfloat162float(p[0]) + (__bfloat162float(p[m.Y0.part_stride]) + __bfloat162float(p[2 * m.Y0.part_stride]));
+    }
+    if (m.bf16) ((__nv_bfloat16*)m.P)[i] = __float2bfloat16_rn(y);
+    else ((float*)m.P)[i] = y;
+    if (m.out32) m.out32[i] = y;
   }
 }
 
@@ -458,8 +463,7 @@ k_split_bf16(const RefreshMat* __restrict__ rm, int which, int with_lo) {
 // U <- identity (r x r); the triangular-solve kernel then turns it into L^-T.
 __global__ void __launch_bounds__(256)
 k_identity(const RefreshMat* __restrict__ rm) {
-  const RefreshMat m = rm[blockIdx.y];
-  if (!m.tc) return;
+  const RefreshMat& m = rm[blockIdx.y];
   const long long total = (long long)m.r * m.r;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x)
@@ -469,7 +473,7 @@ k_identity(const RefreshMat* __restrict__ rm) {
 // descriptor tables of a chunk: per-matrix entries plus alignment slack
 constexpr size_t TABLE_PER_MATRIX = 1024;
 constexpr size_t TABLE_SLACK = 16 * 1024;
-static_assert(sizeof(RefreshMat) + 4 * sizeof(GemmDesc) + 3 * sizeof(TrsmDesc) + 10 * sizeof(int) <= TABLE_PER_MATRIX, "table allowance");
+static_assert(sizeof(RefreshMat) + sizeof(TrsmDesc) + sizeof(int) <= TABLE_PER_MATRIX, "table allowance");
 
 }  // namespace
 
@@ -512,13 +516,63 @@ static TcGemmJob refresh_job(const fira_matrix_desc& dsc, int kind) {
   return j;
 }
 
-static size_t refresh_data_bytes(const fira_matrix_desc& d) {
-  const size_t dd = std::min(d.m, d.n), ll = std::max(d.m, d.n), r = d.r;
-  size_t b = align_up(dd * r * 4) + align_up(ll * r * 4) + align_up(r * r * 4) + 256;
-  if (refresh_on_tc(d)) {
-    b += align_up(r * r * 4) + 2 * (align_up(dd * r * 2) + align_up(ll * r * 2) + align_up(r * r * 2));
-    for (int k = 0; k < JOB_KINDS; ++k) { const TcGemmJob j = refresh_job(d, k); b += tc_gemm_table_bytes(&j, 1); }
+// The part products of a matrix that is iterated in fp32 precision.
+enum { PART_AZ = 0, PART_ATY, PART_GRAM_Y, PART_APPLY_Y, PART_GRAM_Y2, PART_APPLY_Y2, PART_GRAM_Z, PART_APPLY_Z, PART_KINDS };
+
+static PartGemm part_job(const RefreshMat& m, int kind) {
+  PartGemm g;
+  auto gram = [&](const PartMatrix& x) { g.a = g.b = x; g.a_t = true; g.c = m.C; g.ldc = m.r; g.lower = true; };
+  auto apply = [&](const PartMatrix& x, const PartMatrix& y) { g.a = x; g.b = m.Up; g.upper_b = true; g.out = y; };
+  switch (kind) {
+    case PART_AZ: g.a = m.Gp; g.a_t = !m.left; g.b = m.Z1; g.out = m.Y0; break;
+    case PART_ATY: g.a = m.Gp; g.a_t = m.left; g.b = m.Y1; g.out = m.Z0; break;
+    case PART_GRAM_Y: gram(m.Y0); break;
+    case PART_APPLY_Y: apply(m.Y0, m.Y1); break;
+    case PART_GRAM_Y2: gram(m.Y1); break;
+    case PART_APPLY_Y2: apply(m.Y1, m.Y0); break;
+    case PART_GRAM_Z: gram(m.Z0); break;
+    default: apply(m.Z0, m.Z1); break;
   }
+  return g;
+}
+
+// The matrix's buffers, carved from base (null: only their sizes count); *end_out: what follows.
+static RefreshMat carve_refresh(const fira_matrix_desc& dsc, char* base, size_t* bytes_out) {
+  RefreshMat m{};
+  size_t off = 0;
+  auto take = [&](size_t bytes) { char* p = base ? base + off : nullptr; off += align_up(bytes); return p; };
+  m.ld = dsc.ld ? dsc.ld : dsc.n;
+  m.d = std::min(dsc.m, dsc.n); m.l = std::max(dsc.m, dsc.n); m.r = dsc.r;
+  m.left = dsc.m <= dsc.n; m.bf16 = dsc.dtype == FIRA_BF16;
+  m.tc = refresh_on_tc(dsc) ? 1 : 0;
+  const size_t d = m.d, l = m.l, r = m.r;
+  m.C = (float*)take(r * r * 4);
+  m.U = (float*)take(r * r * 4);
+  m.info = (float*)take(256);
+  if (m.tc) {
+    m.Y = (float*)take(d * r * 4);
+    m.Z = (float*)take(l * r * 4);
+    m.Yb = (__nv_bfloat16*)take(d * r * 2); m.Yl = (__nv_bfloat16*)take(d * r * 2);
+    m.Zb = (__nv_bfloat16*)take(l * r * 2); m.Zl = (__nv_bfloat16*)take(l * r * 2);
+    m.Ub = (__nv_bfloat16*)take(r * r * 2); m.Ul = (__nv_bfloat16*)take(r * r * 2);
+  } else {
+    auto parts = [&](long long rows, long long cols, int n) { return part_matrix(take(part_matrix_bytes(rows, cols, n)), rows, cols, n); };
+    m.Gp = parts(dsc.m, dsc.n, m.bf16 ? 1 : 3);
+    m.Y0 = parts(d, r, 3); m.Y1 = parts(d, r, 3);
+    m.Z0 = parts(l, r, 3); m.Z1 = parts(l, r, 3);
+    m.Up = parts(r, r, 3);
+  }
+  *bytes_out = off;
+  return m;
+}
+
+static size_t refresh_data_bytes(const fira_matrix_desc& d) {
+  size_t b = 0;
+  const RefreshMat m = carve_refresh(d, nullptr, &b);
+  if (m.tc)
+    for (int k = 0; k < JOB_KINDS; ++k) { const TcGemmJob j = refresh_job(d, k); b += tc_gemm_table_bytes(&j, 1); }
+  else
+    for (int k = 0; k < PART_KINDS; ++k) { const PartGemm g = part_job(m, k); b += part_gemm_table_bytes(&g, 1); }
   return b;
 }
 
@@ -565,37 +619,18 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
     for (int a = 0; a < nm; ++a) {
       const int idx = which[pos + a];
       const MatDev& mt = c->mats[idx];
-      RefreshMat rm;
-      memset(&rm, 0, sizeof(rm));
+      size_t bytes = 0;
+      RefreshMat rm = carve_refresh(c->descs[idx], tg.work_base + offs[a], &bytes);
       rm.G = G_dev[idx]; rm.P = tg.P_out ? tg.P_out[idx] : mt.P;
       rm.out32 = basis_out ? basis_out[idx] : nullptr;
-      char* base = tg.work_base + offs[a];
-      const size_t r = mt.r;
-      rm.Y = (float*)base; base += align_up((size_t)mt.d * r * 4);
-      rm.Z = (float*)base; base += align_up((size_t)mt.l * r * 4);
-      rm.C = (float*)base; base += align_up(r * r * 4);
-      rm.info = (float*)base; base += 256;
-      rm.tc = refresh_on_tc(c->descs[idx]) ? 1 : 0;
-      if (rm.tc) {
-        rm.U = (float*)base; base += align_up(r * r * 4);
-        rm.Yb = (__nv_bfloat16*)base; base += align_up((size_t)mt.d * r * 2);
-        rm.Yl = (__nv_bfloat16*)base; base += align_up((size_t)mt.d * r * 2);
-        rm.Zb = (__nv_bfloat16*)base; base += align_up((size_t)mt.l * r * 2);
-        rm.Zl = (__nv_bfloat16*)base; base += align_up((size_t)mt.l * r * 2);
-        rm.Ub = (__nv_bfloat16*)base; base += align_up(r * r * 2);
-        rm.Ul = (__nv_bfloat16*)base; base += align_up(r * r * 2);
-      }
-      data_end = std::max(data_end, (size_t)(base - tg.work_base));
-      rm.ld = mt.ld; rm.d = mt.d; rm.l = mt.l; rm.r = mt.r; rm.left = mt.left; rm.bf16 = mt.bf16;
+      data_end = std::max(data_end, offs[a] + bytes);
       rm.key = seed * 0x9E3779B97F4A7C15ull + (unsigned long long)idx * 0xD1B54A32D192ED03ull + 1ull;
       rms.push_back(rm);
     }
-    // ---- descriptor tables of the CUDA-core kernels: AZ->Y, A^T Y->Z, Y^T Y->C, Z^T Z->C, trsm(Y), trsm(Z)
-    // for the matrices that stay there; trsm(U) for the others
-    std::vector<GemmDesc> gAZ, gAtY, gYY, gZZ;
-    std::vector<TrsmDesc> tY, tZ, tU;
-    std::vector<int> sAZ{0}, sAtY{0}, sYY{0}, sTY{0}, sTZ{0}, sTU{0};
-    auto tiles = [](int I, int J) { return simt_tiles(I) * simt_tiles(J); };
+    // ---- descriptor tables: the products' jobs, the triangular solves
+    std::vector<TrsmDesc> tU;
+    std::vector<int> sTU{0};
+    std::vector<PartGemm> pjobs[PART_KINDS];
     std::vector<TcGemmJob> jobs[JOB_KINDS];
     for (size_t a = 0; a < rms.size(); ++a) {
       const RefreshMat& m = rms[a];
@@ -617,26 +652,10 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
           }
           jobs[k].push_back(j);
         }
-        tU.push_back(TrsmDesc{m.U, m.C, m.r, m.r, 1}); sTU.push_back(sTU.back() + (m.r + TM - 1) / TM);
-        continue;
+      } else {
+        for (int k = 0; k < PART_KINDS; ++k) pjobs[k].push_back(part_job(m, k));
       }
-      GemmDesc g;
-      // Y[d][j] = sum_l A(d,l) Z[l][j]
-      g.A = m.G; g.a_bf16 = m.bf16;
-      g.sAi = m.left ? m.ld : 1; g.sAk = m.left ? 1 : m.ld;
-      g.B = m.Z; g.sBk = m.r; g.sBj = 1; g.C = m.Y; g.sCi = m.r; g.I = m.d; g.J = m.r; g.K = m.l;
-      gAZ.push_back(g); sAZ.push_back(sAZ.back() + tiles(g.I, g.J));
-      // Z[l][j] = sum_d A(d,l) Y[d][j]
-      g.sAi = m.left ? 1 : m.ld; g.sAk = m.left ? m.ld : 1;
-      g.B = m.Y; g.C = m.Z; g.I = m.l; g.K = m.d;
-      gAtY.push_back(g); sAtY.push_back(sAtY.back() + tiles(g.I, g.J));
-      // C = Y^T Y and C = Z^T Z
-      g.a_bf16 = 0; g.sAi = 1; g.sAk = m.r; g.sBk = m.r; g.sBj = 1; g.C = m.C; g.sCi = m.r; g.I = m.r; g.J = m.r;
-      g.A = m.Y; g.B = m.Y; g.K = m.d; gYY.push_back(g);
-      g.A = m.Z; g.B = m.Z; g.K = m.l; gZZ.push_back(g);
-      sYY.push_back(sYY.back() + tiles(m.r, m.r));
-      tY.push_back(TrsmDesc{m.Y, m.C, m.d, m.r, 0}); sTY.push_back(sTY.back() + (m.d + TM - 1) / TM);
-      tZ.push_back(TrsmDesc{m.Z, m.C, m.l, m.r, 0}); sTZ.push_back(sTZ.back() + (m.l + TM - 1) / TM);
+      tU.push_back(TrsmDesc{m.U, m.C, m.r}); sTU.push_back(sTU.back() + (m.r + TM - 1) / TM);
     }
     char* tp = tg.work_base + align_up(data_end);
     cudaError_t cerr = cudaSuccess;
@@ -650,22 +669,11 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
       return dst;
     };
     const RefreshMat* rm_dev = (const RefreshMat*)put(rms.data(), rms.size() * sizeof(RefreshMat));
-    const GemmDesc* dAZ = (const GemmDesc*)put(gAZ.data(), gAZ.size() * sizeof(GemmDesc));
-    const GemmDesc* dAtY = (const GemmDesc*)put(gAtY.data(), gAtY.size() * sizeof(GemmDesc));
-    const GemmDesc* dYY = (const GemmDesc*)put(gYY.data(), gYY.size() * sizeof(GemmDesc));
-    const GemmDesc* dZZ = (const GemmDesc*)put(gZZ.data(), gZZ.size() * sizeof(GemmDesc));
-    const TrsmDesc* dTY = (const TrsmDesc*)put(tY.data(), tY.size() * sizeof(TrsmDesc));
-    const TrsmDesc* dTZ = (const TrsmDesc*)put(tZ.data(), tZ.size() * sizeof(TrsmDesc));
     const TrsmDesc* dTU = (const TrsmDesc*)put(tU.data(), tU.size() * sizeof(TrsmDesc));
-    const int* dsAZ = (const int*)put(sAZ.data(), sAZ.size() * sizeof(int));
-    const int* dsAtY = (const int*)put(sAtY.data(), sAtY.size() * sizeof(int));
-    const int* dsYY = (const int*)put(sYY.data(), sYY.size() * sizeof(int));
-    const int* dsTY = (const int*)put(sTY.data(), sTY.size() * sizeof(int));
-    const int* dsTZ = (const int*)put(sTZ.data(), sTZ.size() * sizeof(int));
     const int* dsTU = (const int*)put(sTU.data(), sTU.size() * sizeof(int));
     if (cerr != cudaSuccess) { set_error(std::string("refresh tables: ") + cudaGetErrorString(cerr)); return FIRA_ERR_CUDA; }
     // tables of the tensor-core jobs (tensor maps and tile records), after the others
-    const int ntc = (int)jobs[0].size(), nsimt = nm - ntc;
+    const int ntc = (int)jobs[0].size(), nparts = nm - ntc;
     char* tab[JOB_KINDS] = {};
     int jtiles[JOB_KINDS] = {};
     if (ntc) {
@@ -680,15 +688,27 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
         tp += bytes;
       }
     }
+    char* ptab[PART_KINDS] = {};
+    int ptiles[PART_KINDS] = {};
+    if (nparts)
+      for (int k = 0; k < PART_KINDS; ++k) {
+        const size_t bytes = part_gemm_table_bytes(pjobs[k].data(), nparts);
+        if ((size_t)(tp + bytes - tg.work_base) > tg.work_bytes) {
+          set_error("scratch buffer too small for the projection refresh"); return FIRA_ERR_WORKSPACE_TOO_SMALL;
+        }
+        ptab[k] = tp;
+        const fira_status ps = part_gemm_prepare(pjobs[k].data(), nparts, ptab[k], bytes, &ptiles[k], st);
+        if (ps != FIRA_OK) return ps;
+        tp += bytes;
+      }
+    auto part_product = [&](int k) { return nparts ? part_gemm_run(ptab[k], nparts, ptiles[k], c->status_dev, st) : FIRA_OK; };
     int rmax = 0;
     for (const RefreshMat& m : rms) rmax = std::max(rmax, m.r);
     const dim3 ew_grid(296, nm);      // element-wise helpers: every matrix of the chunk, tc ones act
     // A Z -> Y and A^T Y -> Z.  precise: the iterate enters with its bf16 remainder as a second k-segment.
     auto product = [&](bool az, bool precise) -> fira_status {
-      if (nsimt) {
-        if (az) k_rgemm<<<sAZ.back(), GEMM_THREADS, 0, st>>>(dAZ, nsimt, dsAZ);
-        else k_rgemm<<<sAtY.back(), GEMM_THREADS, 0, st>>>(dAtY, nsimt, dsAtY);
-      }
+      const fira_status ps = part_product(az ? PART_AZ : PART_ATY);
+      if (ps != FIRA_OK) return ps;
       if (ntc) {
         k_split_bf16<<<ew_grid, 256, 0, st>>>(rm_dev, az ? 1 : 0, precise ? 1 : 0);
         const int k = az ? (precise ? JOB_AZ_SPLIT : JOB_AZ) : (precise ? JOB_ATY_SPLIT : JOB_ATY);
@@ -704,7 +724,8 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
       const int kg = y ? (precise ? JOB_GRAM_Y : JOB_GRAM_Y1) : (precise ? JOB_GRAM_Z : JOB_GRAM_Z1);
       const int ka = y ? (precise ? JOB_APPLY_Y : JOB_APPLY_Y1) : (precise ? JOB_APPLY_Z : JOB_APPLY_Z1);
       for (int pass = 0; pass < passes; ++pass) {
-        if (nsimt) k_rgemm<<<sYY.back(), GEMM_THREADS, 0, st>>>(y ? dYY : dZZ, nsimt, dsYY);
+        fira_status ps = part_product(!y ? PART_GRAM_Z : pass == 0 ? PART_GRAM_Y : PART_GRAM_Y2);
+        if (ps != FIRA_OK) return ps;
         if (ntc) {
           k_split_bf16<<<ew_grid, 256, 0, st>>>(rm_dev, y ? 0 : 1, precise ? 1 : 0);
           const fira_status gs = tc_gemm_run(c, tab[kg], ntc, jtiles[kg], st);
@@ -718,13 +739,12 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
             k_chol_update<<<nm * (nt * (nt + 1) / 2), GEMM_THREADS, 0, st>>>(rm_dev, J0, nt);
           }
         }
-        if (nsimt) {
-          if (y) k_trsm_rows<<<sTY.back(), GEMM_THREADS, 0, st>>>(dTY, nsimt, dsTY);
-          else k_trsm_rows<<<sTZ.back(), GEMM_THREADS, 0, st>>>(dTZ, nsimt, dsTZ);
-        }
+        k_identity<<<ew_grid, 256, 0, st>>>(rm_dev);
+        k_trsm_rows<<<sTU.back(), GEMM_THREADS, 0, st>>>(dTU, nm, dsTU);      // U = L^-T
+        if (nparts) k_to_parts<<<ew_grid, 256, 0, st>>>(rm_dev, 1);
+        ps = part_product(!y ? PART_APPLY_Z : pass == 0 ? PART_APPLY_Y : PART_APPLY_Y2);
+        if (ps != FIRA_OK) return ps;
         if (ntc) {
-          k_identity<<<ew_grid, 256, 0, st>>>(rm_dev);
-          k_trsm_rows<<<sTU.back(), GEMM_THREADS, 0, st>>>(dTU, ntc, dsTU);      // U = L^-T
           k_split_bf16<<<ew_grid, 256, 0, st>>>(rm_dev, 2, precise ? 1 : 0);
           const fira_status as = tc_gemm_run(c, tab[ka], ntc, jtiles[ka], st);
           if (as != FIRA_OK) return as;
@@ -732,6 +752,7 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
       }
       return FIRA_OK;
     };
+    if (nparts) k_to_parts<<<ew_grid, 256, 0, st>>>(rm_dev, 0);
     k_gauss<<<ew_grid, 256, 0, st>>>(rm_dev);
     fira_status prs = product(true, iters == 0);
     if (prs == FIRA_OK) prs = orth(true, iters == 0 ? 2 : 1, iters == 0);

@@ -110,15 +110,15 @@ __device__ __forceinline__ void load_frag(const __nv_bfloat16* p, int n, bool ve
     f.u = make_uint4(x[0], x[1], x[2], x[3]);
   }
 }
-__device__ __forceinline__ void store_parts(unsigned char* p, const Frag<float>& f) {
+__device__ __forceinline__ void store_parts(unsigned char* p, const Frag<float>& f, long long part_bytes = PART_BYTES) {
   uint32_t h[4], m[4], l[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) split3(f.v[2 * i], f.v[2 * i + 1], h[i], m[i], l[i]);
   *reinterpret_cast<uint4*>(p) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(p + PART_BYTES) = make_uint4(m[0], m[1], m[2], m[3]);
-  *reinterpret_cast<uint4*>(p + 2 * PART_BYTES) = make_uint4(l[0], l[1], l[2], l[3]);
+  *reinterpret_cast<uint4*>(p + part_bytes) = make_uint4(m[0], m[1], m[2], m[3]);
+  *reinterpret_cast<uint4*>(p + 2 * part_bytes) = make_uint4(l[0], l[1], l[2], l[3]);
 }
-__device__ __forceinline__ void store_parts(unsigned char* p, const Frag<__nv_bfloat16>& f) {
+__device__ __forceinline__ void store_parts(unsigned char* p, const Frag<__nv_bfloat16>& f, long long = 0) {
   *reinterpret_cast<uint4*>(p) = f.u;
 }
 

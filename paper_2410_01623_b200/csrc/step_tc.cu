@@ -30,13 +30,12 @@
 // bf16) deep per pipeline stage; two accumulators of 256 tensor-memory columns alternate so
 // that the epilogue of one tile overlaps the products of the next; all epilogue traffic
 // moves through TMA boxes in shared memory.
-#include <cuda.h>
-
 #include <algorithm>
 
 #include "context.cuh"
 #include "step_tc.cuh"
 #include "tc_ptx.cuh"
+#include "tma_encode.cuh"
 
 namespace fira {
 
@@ -350,40 +349,14 @@ k_selftest_bounded_wait(unsigned* status, const uint32_t* never_raised, uint32_t
 }
 
 // ============================================================================ host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (fn) return fn;
-  void* sym = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres) != cudaSuccess ||
-      qres != cudaDriverEntryPointSuccess)
-    return nullptr;
-  fn = reinterpret_cast<EncodeTiledFn>(sym);
-  return fn;
-}
-
 // bf16 row-major matrix [rows][cols] with leading dimension ld; box = box_c x box_r.
 bool encode_map(CUtensorMap* out, const void* base, long long rows, long long cols, long long ld,
                 int box_c, int box_r, int mode = 0) {
   // mode 0: bf16, 128-byte swizzle; 1: fp32, 128-byte swizzle; 2: bf16, 64-byte swizzle
-  const bool fp32 = mode == 1;
-  EncodeTiledFn fn = get_encode_fn();
-  if (!fn) { set_error("cuTensorMapEncodeTiled is not available"); return false; }
-  const cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  const cuuint64_t gstr[1] = {(cuuint64_t)ld * (fp32 ? 4 : 2)};
-  const cuuint32_t box[2] = {(cuuint32_t)box_c, (cuuint32_t)box_r};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = fn(out, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                        const_cast<void*>(base), gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        mode == 2 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed with code " + std::to_string((int)r)); return false; }
-  return true;
+  const unsigned long long extent[2] = {(unsigned long long)cols, (unsigned long long)rows};
+  const unsigned long long stride[1] = {(unsigned long long)ld * (mode == 1 ? 4 : 2)};
+  const unsigned box[2] = {(unsigned)box_c, (unsigned)box_r};
+  return encode_tiled(out, base, mode == 1, 2, extent, stride, box, mode == 2 ? 64 : 128);
 }
 
 // The same matrix seen as [cols / 64 chunks][rows][64]: one box brings `nchunk` adjacent
@@ -391,22 +364,39 @@ bool encode_map(CUtensorMap* out, const void* base, long long rows, long long co
 // layout of an MN-major operand).  Needs cols % 64 == 0: the chunk dimension has no ragged edge.
 bool encode_map_chunked(CUtensorMap* out, const void* base, long long rows, long long cols, long long ld,
                         int box_r, int nchunk) {
-  EncodeTiledFn fn = get_encode_fn();
-  if (!fn) { set_error("cuTensorMapEncodeTiled is not available"); return false; }
-  const cuuint64_t gdim[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
-  const cuuint64_t gstr[2] = {(cuuint64_t)ld * 2, 128};
-  const cuuint32_t box[3] = {64, (cuuint32_t)box_r, (cuuint32_t)nchunk};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstr, box, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled (chunked) failed with code " + std::to_string((int)r)); return false; }
-  return true;
+  const unsigned long long extent[3] = {64, (unsigned long long)rows, (unsigned long long)(cols / 64)};
+  const unsigned long long stride[2] = {(unsigned long long)ld * 2, 128};
+  const unsigned box[3] = {64, (unsigned)box_r, (unsigned)nchunk};
+  return encode_tiled(out, base, false, 3, extent, stride, box, 128);
 }
 
 int host_tile_bn(int r) { return (r % 256 == 0) ? 256 : 128; }
 
 }  // namespace
+
+bool encode_tiled(CUtensorMap* out, const void* base, bool fp32, int rank, const unsigned long long* extent,
+                  const unsigned long long* stride_bytes, const unsigned* box, int swizzle_bytes) {
+  typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static const EncodeTiledFn fn = [] {
+    void* sym = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool found = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) == cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess;
+    return reinterpret_cast<EncodeTiledFn>(found ? sym : nullptr);
+  }();
+  if (!fn) { set_error("cuTensorMapEncodeTiled is not available"); return false; }
+  cuuint64_t dims[4], strides[3];
+  cuuint32_t boxes[4], ones[4] = {1, 1, 1, 1};
+  for (int i = 0; i < rank; ++i) { dims[i] = extent[i]; boxes[i] = box[i]; if (i) strides[i - 1] = stride_bytes[i - 1]; }
+  const CUresult r = fn(out, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank,
+                        const_cast<void*>(base), dims, strides, boxes, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed with code " + std::to_string((int)r)); return false; }
+  return true;
+}
 
 struct TcPlan {
   std::vector<TcMaps> maps;          // host image, one entry per matrix of the tc list
