@@ -287,10 +287,16 @@ bool encode_operand(CUtensorMap* map, const PartMatrix& p, bool rows_contiguous,
   return encode_tiled(map, p.base, false, 3, extent, stride, box, 64);
 }
 
+long long depth_of(const PartGemm& g) { return g.a_t ? g.a.rows : g.a.cols; }
+
+// The tiles of a row of tiles are neighbours (they share the rows of A in L2), forth and back in turn: where B is
+// triangular their lengths differ, and every pair gets some of each.
 void tiles_of(const PartGemm& g, int job, std::vector<TileDev>& out) {
-  const long long I = g.a_t ? g.a.cols : g.a.rows, K = g.a_t ? g.a.rows : g.a.cols, J = g.b_t ? g.b.rows : g.b.cols;
-  for (int i0 = 0; i0 < I; i0 += PM)
-    for (int j0 = 0; j0 < J; j0 += PN) {
+  const long long I = g.a_t ? g.a.cols : g.a.rows, K = depth_of(g), J = g.b_t ? g.b.rows : g.b.cols;
+  const int nj = (int)((J + PN - 1) / PN);
+  for (int i0 = 0, row = 0; i0 < I; i0 += PM, ++row)
+    for (int q = 0; q < nj; ++q) {
+      const int j0 = (row % 2 ? nj - 1 - q : q) * PN;
       if (g.lower && j0 >= i0 + PM) continue;
       const long long k = g.upper_b ? std::min<long long>(K, j0 + PN) : K;
       out.push_back(TileDev{job, i0, j0, (int)((k + PK - 1) / PK)});
@@ -317,10 +323,12 @@ fira_status part_gemm_prepare(const PartGemm* jobs, int njobs, char* table_dev, 
     j.out = g.out.base; j.pitch = g.out.pitch; j.part_stride = g.out.part_stride;
     j.I = (int)(g.a_t ? g.a.cols : g.a.rows); j.J = (int)(g.b_t ? g.b.rows : g.b.cols);
     j.shape = g.a.parts | (g.b.parts << 2) | (g.a_t ? 16 : 0) | (g.b_t ? 32 : 0);
-    tiles_of(g, q, td);
   }
-  // the longest tiles first: what is left over at the end of the list is short
-  std::stable_sort(td.begin(), td.end(), [](const TileDev& x, const TileDev& y) { return x.nk > y.nk; });
+  // the matrices with the longest products first: what is left over at the end of the list is short
+  std::vector<int> order((size_t)njobs);
+  for (int q = 0; q < njobs; ++q) order[q] = q;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return depth_of(jobs[x]) > depth_of(jobs[y]); });
+  for (int q : order) tiles_of(jobs[q], q, td);
   const size_t off = align_up(sizeof(JobDev) * (size_t)njobs);
   if (off + align_up(sizeof(TileDev) * td.size()) > table_bytes) { set_error("part products: table area too small"); return FIRA_ERR_WORKSPACE_TOO_SMALL; }
   cudaError_t e = cudaMemcpyAsync(table_dev, jd.data(), sizeof(JobDev) * jd.size(), cudaMemcpyHostToDevice, st);

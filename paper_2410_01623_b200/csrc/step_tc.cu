@@ -639,18 +639,29 @@ fira_status tc_gemm_prepare(fira_ctx* c, const TcGemmJob* jobs, int njobs, char*
       }
       if (gb && !encode_map_chunked(mb, gb, D, j.r, j.r, 64, bn / 128)) return FIRA_ERR_CUDA;
     }
-    if (!encode_map(&mp.em, j.C, L, j.r, j.r, K1_ECOLS, K1_EROWS, 1)) return FIRA_ERR_CUDA;
+    if (j.C) {
+      if (!encode_map(&mp.em, j.C, L, j.r, j.r, K1_ECOLS, K1_EROWS, 1)) return FIRA_ERR_CUDA;
+    } else {
+      if (!encode_map(&mp.en, j.hi, L, j.r, j.r, K1_ECOLS, K1_EROWS, 2)) return FIRA_ERR_CUDA;
+      if (j.lo && !encode_map(&mp.er, j.lo, L, j.r, j.r, K1_ECOLS, K1_EROWS, 2)) return FIRA_ERR_CUDA;
+    }
     const int nseg = j.nseg > 1 ? j.nseg : 1;
     const int nkb_seg = (D + BK - 1) / BK;
     if (nseg > 3 || ((j.asel >> nseg) != 0) || ((j.bsel >> nseg) != 0) || (j.asel && !j.G_lo) || (j.bsel && !j.B_lo)) {
       set_error("internal: bad k-segments of a refresh product"); return FIRA_ERR_INVALID_ARG;
     }
+    // the r-tiles of one row of tiles are neighbours (they share the panel of A in L2), forth and back in turn: where
+    // B is triangular their lengths differ, and every pair gets some of each
     for (int l0 = 0; l0 < L; l0 += 2 * BM)
-      for (int r0 = 0; r0 < j.r; r0 += bn) {
+      for (int q0 = 0; q0 < j.r; q0 += bn) {
+        const int r0 = (l0 / (2 * BM)) % 2 ? j.r - bn - q0 : q0;
+        if (j.lower && r0 >= l0 + 2 * BM) continue;
+        const int nkb = j.upper_b ? std::min(nkb_seg, (r0 + bn + BK - 1) / BK) : nkb_seg;
         ProjTileDesc d;
-        d.colpart = reinterpret_cast<float*>(seg_word(nkb_seg, j.asel, j.bsel)); d.slot = q; d.l0 = l0; d.r0 = r0;
-        d.nkb = nseg * nkb_seg; d.L = L;
-        d.bn_left = bn | ((j.r / bn) << 16) | (j.mn_major ? (int)0x80000000 : 0) | (chunked ? PROJ_A_CHUNKED : 0);
+        d.colpart = reinterpret_cast<float*>(seg_word(nkb, j.asel, j.bsel)); d.slot = q; d.l0 = l0; d.r0 = r0;
+        d.nkb = nseg * nkb; d.L = L;
+        d.bn_left = bn | ((j.r / bn) << 16) | (j.mn_major ? (int)0x80000000 : 0) | (chunked ? PROJ_A_CHUNKED : 0) |
+                    (j.C ? 0 : PROJ_OUT_BF16) | (!j.C && j.lo ? PROJ_OUT_REMAINDER : 0);
         tiles.push_back(d);
       }
   }

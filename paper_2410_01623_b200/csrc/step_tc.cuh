@@ -44,11 +44,16 @@ int tc_phase_names(const char** out);
 // the same output; segment s takes A from G (bit s of asel clear) or G_lo (set) and B from B (bsel
 // clear) or B_lo (set).  G_lo / B_lo have the shapes and pitches of G / B.  For an fp32 matrix
 // X = X_hi + X_lo (two bf16 parts), segments (hi,hi), (hi,lo), (lo,hi) give X Y to about 2^-16.
+// The result: C (fp32, pitch r), or, if C is null, its bf16 rounding in hi and (if not null) the bf16 remainder in lo.
+// lower: only the tiles that meet the lower triangle of the result are wanted.  upper_b: B is upper
+// triangular, column j needs k <= j only.
 struct TcGemmJob {
   const void* G; long long ld; int m, n; int mn_major;
   const void* B; float* C; int r;
   const void* G_lo; const void* B_lo;
   int nseg; unsigned asel, bsel;
+  void* hi; void* lo;
+  int lower, upper_b;
 };
 // Device bytes of the tables (tensor maps, tile records) of a job list.
 size_t tc_gemm_table_bytes(const TcGemmJob* jobs, int njobs);

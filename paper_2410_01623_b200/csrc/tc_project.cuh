@@ -91,12 +91,16 @@ struct ProjTileDesc {
   int slot;            // index into the tensor-map table and the fast-scalar table
   int l0, r0;          // first unprojected index / first rank index of the tile
   int nkb;             // k-blocks: ceil(d / 64)
-  int bn_left;         // bits 0-15: BN (128 or 256); 16-23: r / BN; 29: the epilogue forms X; 30: G comes as one chunked box; 31: left
+  int bn_left;         // bits 0-15: BN (128 or 256); 16-23: r / BN; 27, 28: see PROJ_OUT_*; 29: the epilogue forms X;
+                       // 30: G comes as one chunked box; 31: left
   int L;               // number of unprojected indices of the matrix
 };
 static_assert(sizeof(ProjTileDesc) == 32, "ProjTileDesc layout");
 constexpr int PROJ_A_CHUNKED = 1 << 30;
 constexpr int PROJ_FUSE_X = 1 << 29;      // bn_left: this tile's epilogue forms X itself (FUSE_X kernels only)
+// EPI_PLAIN: the result is stored as bf16 (through the map en), with the bf16 remainder (er) beside it; neither bit
+// set: as fp32 (em).
+constexpr int PROJ_OUT_BF16 = 1 << 28, PROJ_OUT_REMAINDER = 1 << 27;
 // Which matrices take that route.  The second sweep lengthens the epilogue and the exchange makes the
 // pairs of a row of tiles wait for the slowest of them.  Measured on the step: one r-tile per row (no
 // exchange, 350M list, r = 256): -8 %; long products (7B list, d = 4096, four r-tiles): -6 to -7 %;
@@ -155,7 +159,7 @@ __device__ __forceinline__ ProjTileDesc load_desc(const ProjTileDesc* __restrict
 }
 
 // EPI_ADAM: the step's kernel as described above.  EPI_PLAIN: the same product with the accumulator
-// written out as it is, C[l][j] (fp32, through the `em` map): the products A^T Y and A Z of the
+// written out as it is, C[l][j] (fp32), or as the bf16 operands of the next product: the products of the
 // projection refresh.  Then no M/V boxes are loaded, the output box of a row half is built in that
 // half's N/R buffer, and the loader and the G^2 warps have nothing to do.
 enum { EPI_ADAM = 0, EPI_PLAIN = 1 };
@@ -450,6 +454,9 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
                 ptx::tma_store_2d(&mp->en, srn, j, row);
                 ptx::tma_store_2d(&mp->er, srn + K1_HBOX_BYTES, j, row);
               }
+            } else if (d.bn_left & PROJ_OUT_BF16) {
+              ptx::tma_store_2d(&mp->en, srn, j, row);
+              if (d.bn_left & PROJ_OUT_REMAINDER) ptx::tma_store_2d(&mp->er, srn + K1_HBOX_BYTES, j, row);
             } else {
               ptx::tma_store_2d(&mp->em, srn, j, row);      // the fp32 output box sits in the N/R buffer
             }
@@ -544,7 +551,23 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
         }
         unsigned char* mb = mvbuf + (size_t)mv * K1_MVBUF_BYTES;
         unsigned char* vb = mb + K1_FBOX_BYTES;
-        if (EPI == EPI_PLAIN) {
+        if (EPI == EPI_PLAIN && (d.bn_left & PROJ_OUT_BF16)) {
+#pragma unroll
+          for (int qq = 0; qq < QN; ++qq) {
+            float v[8], rest[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(rr[8 * qq + e]);
+            const uint4 hi = pack8_bf16(v);
+            const uint32_t h = hrow + (((uint32_t)(q0 + qq) ^ hsw) << 4);
+            *reinterpret_cast<uint4*>(nb + h) = hi;
+            if (d.bn_left & PROJ_OUT_REMAINDER) {
+              unpack8_bf16(hi, rest);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) rest[e] = v[e] - rest[e];
+              *reinterpret_cast<uint4*>(rb + h) = pack8_bf16(rest);
+            }
+          }
+        } else if (EPI == EPI_PLAIN) {
           // 32 fp32 values of this row: eight 16-byte slots of a 128-byte row, slot ^= row % 8
 #pragma unroll
           for (int qq = 0; qq < 8 / EG; ++qq) {
