@@ -28,32 +28,44 @@ __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast
 // Eight steps of factor_subblock on rows whose last W entries are still to be done.  a: lane i's row i, moved left by
 // one entry per step, so that the loop body is the same for every step (unrolled over all 32 steps one warp waits for
 // its instructions: 20 us per sub-block instead of 4); t: lane j's column j of the identity on its way to the inverse,
-// moved the same way.  Both take the same values of the factor's column, handed round by shuffles.
+// moved the same way.  Both take the entries of the factor's column below the pivot from `column` (the first of them,
+// on which the next pivot waits, by a shuffle).
 template <int W>
-__device__ __forceinline__ void factor_steps(float (&a)[SB], float (&t)[SB], int k0, float* S, float* X, int n,
-                                             float floor_pivot, bool& bad) {
+__device__ __forceinline__ void factor_steps(float (&a)[SB], float (&t)[SB], int k0, float* S, float* X, float* column,
+                                             int n, float floor_pivot, bool& bad) {
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int k = k0; k < k0 + 8; ++k) {
     float pv = __shfl_sync(0xffffffffu, a[0], k);
-    if (k < n && (!(pv > floor_pivot) || !isfinite(pv))) { bad = true; pv = floor_pivot; }
+    if (k < n && !(pv > floor_pivot && pv < INFINITY)) { bad = true; pv = floor_pivot; }
     float s = rsqrtf(pv);
     s = s * (1.5f - 0.5f * pv * s * s);         // one Newton step: to working precision
     const float l = lane == k ? pv * s : a[0] * s, x = t[0] * s;
+    float* c = column + (k & 1) * SB;           // (two in turn: nobody is more than a step behind)
+    if (lane > k) c[lane - k - 1] = l;
     S[lane * FP + k] = lane >= k ? l : 0.f;
     X[k * FP + lane] = x;
+    const float next = __shfl_sync(0xffffffffu, l, k + 1);
+    a[0] = a[1] - l * next;
+    t[0] = t[1] - next * x;
+    __syncwarp();
 #pragma unroll
-    for (int j = 1; j < W; ++j) {               // (entries past the row's end never come to the front)
-      const float v = __shfl_sync(0xffffffffu, l, k + j);
-      a[j - 1] = a[j] - l * v;
-      t[j - 1] = t[j] - v * x;
+    for (int j = 0; j < W; j += 4) {            // (entries past the row's end never come to the front)
+      const float4 v = ld4(c + j);
+      const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (j + q > 0 && j + q < W - 1) {
+          a[j + q] = a[j + q + 1] - l * w[q];
+          t[j + q] = t[j + q + 1] - w[q] * x;
+        }
     }
   }
 }
 
 // One warp: Cholesky factor of the SB x SB block at S (pitch FP) in place and its inverse at X.
 // n of its rows are the matrix's, the others the identity's.
-__device__ __forceinline__ void factor_subblock(float* S, float* X, int n, float floor_pivot, bool& bad) {
+__device__ __forceinline__ void factor_subblock(float* S, float* X, float* column, int n, float floor_pivot, bool& bad) {
   const int lane = threadIdx.x & 31;
   float a[SB], t[SB];
 #pragma unroll
@@ -64,16 +76,17 @@ __device__ __forceinline__ void factor_subblock(float* S, float* X, int n, float
     for (int q = 0; q < 4; ++q) t[j + q] = j + q == lane ? 1.f : 0.f;
   }
   __syncwarp();
-  factor_steps<32>(a, t, 0, S, X, n, floor_pivot, bad);
-  factor_steps<24>(a, t, 8, S, X, n, floor_pivot, bad);
-  factor_steps<16>(a, t, 16, S, X, n, floor_pivot, bad);
-  factor_steps<8>(a, t, 24, S, X, n, floor_pivot, bad);
+  factor_steps<32>(a, t, 0, S, X, column, n, floor_pivot, bad);
+  factor_steps<24>(a, t, 8, S, X, column, n, floor_pivot, bad);
+  factor_steps<16>(a, t, 16, S, X, column, n, floor_pivot, bad);
+  factor_steps<8>(a, t, 24, S, X, column, n, floor_pivot, bad);
 }
 
-// Products of 32 columns, four per thread, in shared memory (pitch FP).  Thread: rows row + 32 x, x < NX.
+// Products in shared memory (pitch FP), NX blocks of 32 x 32, four neighbours of a row of every block per thread.
 //   by_rows:  acc[x][y] = sum_k P[row + 32 x][k] Q[col + 8 y][k]      (col = lane % 8)
-//   otherwise acc[x][y] = sum_k P[row + 32 x][k] Q[k][4 col + y]
-// Four of k at a time, all loads 16 bytes and free of bank conflicts: 3 + 4 of them for 48 multiply-adds.
+//   otherwise acc[x][y] = sum_k P[row][k] Q[k][32 x + 4 col + y]
+// Four of k at a time, all loads 16 bytes and free of bank conflicts: for three blocks 7 or 13 of them for 48
+// multiply-adds.
 template <int NX, bool BY_ROWS>
 __device__ __forceinline__ void small_product(float (&acc)[3][4], const float* P, const float* Q, int depth) {
   const int col = threadIdx.x & 7, row = threadIdx.x >> 3;
@@ -83,21 +96,31 @@ __device__ __forceinline__ void small_product(float (&acc)[3][4], const float* P
     for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
 #pragma unroll 2
   for (int k = 0; k < depth; k += 4) {
-    float p[NX][4], q[4][4];                    // q[y][kk]
+    if (BY_ROWS) {
+      float4 p[NX], q[4];
 #pragma unroll
-    for (int x = 0; x < NX; ++x) { const float4 v = ld4(P + (row + 32 * x) * FP + k); p[x][0] = v.x; p[x][1] = v.y; p[x][2] = v.z; p[x][3] = v.w; }
+      for (int x = 0; x < NX; ++x) p[x] = ld4(P + (row + 32 * x) * FP + k);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float4 v = BY_ROWS ? ld4(Q + (col + 8 * u) * FP + k) : ld4(Q + (k + u) * FP + 4 * col);
-      if (BY_ROWS) { q[u][0] = v.x; q[u][1] = v.y; q[u][2] = v.z; q[u][3] = v.w; }
-      else { q[0][u] = v.x; q[1][u] = v.y; q[2][u] = v.z; q[3][u] = v.w; }
-    }
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk)
+      for (int y = 0; y < 4; ++y) q[y] = ld4(Q + (col + 8 * y) * FP + k);
 #pragma unroll
       for (int x = 0; x < NX; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] = fmaf(p[x][kk], q[y][kk], acc[x][y]);
+        for (int y = 0; y < 4; ++y)
+          acc[x][y] = fmaf(p[x].w, q[y].w, fmaf(p[x].z, q[y].z, fmaf(p[x].y, q[y].y, fmaf(p[x].x, q[y].x, acc[x][y]))));
+    } else {
+      const float4 p = ld4(P + row * FP + k);
+      const float pk[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+      for (int x = 0; x < NX; ++x)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float4 q = ld4(Q + (k + u) * FP + 32 * x + 4 * col);
+          acc[x][0] = fmaf(pk[u], q.x, acc[x][0]);
+          acc[x][1] = fmaf(pk[u], q.y, acc[x][1]);
+          acc[x][2] = fmaf(pk[u], q.z, acc[x][2]);
+          acc[x][3] = fmaf(pk[u], q.w, acc[x][3]);
+        }
+    }
   }
 }
 template <bool BY_ROWS>
@@ -112,6 +135,7 @@ __global__ void __launch_bounds__(FACTOR_THREADS)
 k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsigned* __restrict__ status) {
   extern __shared__ __align__(16) float fsm[];
   __shared__ float red[FACTOR_THREADS / 32];
+  __shared__ __align__(16) float column[2 * SB];
   float* S = fsm;                               // the block, later its factor
   float* X = fsm + NB * FP;                     // the factor's inverse
   const RefreshMat& m = rm[blockIdx.x];
@@ -135,17 +159,39 @@ k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsig
     mean_diag = m.info[0];
   }
   const float shift = shift_rel * mean_diag, floor_pivot = fmaxf(1e-30f, 1e-12f * mean_diag);
-#pragma unroll 16
-  for (int e = tid; e < NB * NB; e += FACTOR_THREADS) {
-    const int i = e / NB, j = e % NB;
-    S[i * FP + j] = (j <= i && i < nb) ? C[(long long)i * r + j] + (i == j ? shift : 0.f) : (i == j ? 1.f : 0.f);
-    X[i * FP + j] = 0.f;
+  // eight groups of four entries per thread at a time, their loads before their stores to shared memory
+  const bool vec = r % 4 == 0;
+#pragma unroll 1
+  for (int h = 0; h < NB * NB / 4; h += 8 * FACTOR_THREADS) {
+    float v[8][4];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = h + q * FACTOR_THREADS + tid, i = e / (NB / 4), j = e % (NB / 4) * 4;
+      if (vec && i < nb && j < nb) {
+        const float4 u = __ldcg(reinterpret_cast<const float4*>(C + (long long)i * r + j));
+        v[q][0] = u.x; v[q][1] = u.y; v[q][2] = u.z; v[q][3] = u.w;
+      } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[q][c] = i < nb && j + c < nb ? __ldcg(C + (long long)i * r + j + c) : (i == j + c ? 1.f : 0.f);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = h + q * FACTOR_THREADS + tid, i = e / (NB / 4), j = e % (NB / 4) * 4;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {             // the lower triangle, shifted
+        if (j + c > i) v[q][c] = 0.f;
+        else if (j + c == i && i < nb) v[q][c] += shift;
+      }
+      *reinterpret_cast<float4*>(S + i * FP + j) = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
+      *reinterpret_cast<float4*>(X + i * FP + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
   __syncthreads();
   bool bad = false;
   const int col = tid & 7, row = tid >> 3;
   for (int b = 0; b < NB; b += SB) {
-    if (warp == 0) factor_subblock(S + b * FP + b, X + b * FP + b, nb - b, floor_pivot, bad);
+    if (warp == 0) factor_subblock(S + b * FP + b, X + b * FP + b, column, nb - b, floor_pivot, bad);
     __syncthreads();
     const int lo = b + SB, below = (NB - lo) / SB;
     float acc[3][4];
@@ -159,15 +205,11 @@ k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsig
         if (x < below) S[(lo + row + 32 * x) * FP + b + col + 8 * y] = acc[x][y];
     // X[b + j][i] = -sum_k X[b + j][b + k] T[k][i] with T[j][i] = sum_k S[b + j][k] X[k][i], over the columns
     // i < b; T takes the place of the row block of S that it is made of
-    float t[3][4];
-    for (int c = 0; c < b; c += SB) {
-      small_product<false>(1, acc, S + b * FP, X + c, b);
-#pragma unroll
-      for (int y = 0; y < 4; ++y) t[c / SB][y] = acc[0][y];
-    }
+    small_product<false>(b / SB, acc, S + b * FP, X, b);
     __syncthreads();
-    for (int c = 0; c < b; c += SB)
-      *reinterpret_cast<float4*>(S + (b + row) * FP + c + 4 * col) = make_float4(t[c / SB][0], t[c / SB][1], t[c / SB][2], t[c / SB][3]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (c * SB < b) *reinterpret_cast<float4*>(S + (b + row) * FP + c * SB + 4 * col) = make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
     // the rest of the block: S[i][j] -= sum_k S[i][b + k] S[j][b + k], 32 columns at a time
     for (int c = 0; c < below; ++c) {
       small_product<true>(below, acc, S + lo * FP + b, S + (lo + SB * c) * FP + b, SB);
@@ -180,10 +222,10 @@ k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsig
         }
     }
     __syncthreads();
-    for (int c = 0; c < b; c += SB) {
-      small_product<false>(1, acc, X + b * FP + b, S + b * FP + c, SB);
-      *reinterpret_cast<float4*>(X + (b + row) * FP + c + 4 * col) = make_float4(-acc[0][0], -acc[0][1], -acc[0][2], -acc[0][3]);
-    }
+    small_product<false>(b / SB, acc, X + b * FP + b, S + b * FP, SB);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (c * SB < b) *reinterpret_cast<float4*>(X + (b + row) * FP + c * SB + 4 * col) = make_float4(-acc[c][0], -acc[c][1], -acc[c][2], -acc[c][3]);
     __syncthreads();
   }
   if (bad && lane == 0) atomicOr(status, DEV_STATUS_NONFINITE);

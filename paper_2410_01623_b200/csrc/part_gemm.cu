@@ -104,6 +104,45 @@ __device__ __forceinline__ void store_result(const JobDev& jb, int i, int j, con
   }
 }
 
+// MMAs of one slab.  An operand along its rows: 64-element chunks of 32 k-rows (4 KiB), 16 k-rows of 128 bytes per
+// step; along k: 64-byte rows.
+template <int PA, int PB, bool A_MN, bool B_MN>
+__device__ __forceinline__ void issue_slab(uint32_t main, uint32_t small, uint32_t slab, bool fresh, bool first) {
+  constexpr uint64_t mn = ptx::smem_desc_constant(ptx::LAYOUT_SW128, PK * 128, 1024);
+  constexpr uint64_t km = ptx::smem_desc_constant(ptx::LAYOUT_SW64, 0, 512);
+  const uint32_t idesc = ptx::make_idesc_bf16(PM, PN, A_MN, B_MN);
+  uint64_t a = (A_MN ? mn : km) + (slab >> 4), b = (B_MN ? mn : km) + ((slab + 3 * A_PART) >> 4);
+  uint32_t acc = !first;
+#pragma unroll
+  for (int s = 0; s < PK / 16; ++s, a += (A_MN ? 2048 : 32) / 16, b += (B_MN ? 2048 : 32) / 16) {
+    ptx::umma_bf16_pair(main, a, b, idesc, s ? 1u : !fresh);
+#pragma unroll
+    for (int q = 2; q >= 1; --q)
+#pragma unroll
+      for (int p = 0; p <= q; ++p)
+        if (p < PA && q - p < PB) {
+          ptx::umma_bf16_pair(small, a + p * (A_PART / 16), b + (q - p) * (B_PART / 16), idesc, acc);
+          acc = 1u;
+        }
+  }
+}
+template <int PA, int PB>
+__device__ __forceinline__ void issue_slab(int shape, uint32_t main, uint32_t small, uint32_t slab, bool fresh, bool first) {
+  if (shape & 16) {
+    if (shape & 32) issue_slab<PA, PB, true, false>(main, small, slab, fresh, first);
+    else issue_slab<PA, PB, true, true>(main, small, slab, fresh, first);
+  } else {
+    if (shape & 32) issue_slab<PA, PB, false, false>(main, small, slab, fresh, first);
+    else issue_slab<PA, PB, false, true>(main, small, slab, fresh, first);
+  }
+}
+__device__ __forceinline__ void issue(int shape, uint32_t main, uint32_t small, uint32_t slab, bool fresh, bool first) {
+  if ((shape & 15) == 15) issue_slab<3, 3>(shape, main, small, slab, fresh, first);
+  else if ((shape & 15) == 13) issue_slab<1, 3>(shape, main, small, slab, fresh, first);
+  else if ((shape & 15) == 7) issue_slab<3, 1>(shape, main, small, slab, fresh, first);
+  else issue_slab<1, 1>(shape, main, small, slab, fresh, first);
+}
+
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
 k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, int ntiles, unsigned* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -169,9 +208,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
       const uint32_t tmem = ctl->tmem_base;
       for (int t = pair; t < ntiles && ok; t += npairs, ++tile) {
         const TileDev d = load_tile(tiles + t);
-        const int shape = jobs[d.job].shape, pa = shape & 3, pb = (shape >> 2) & 3;
-        const bool a_mn = shape & 16, b_mn = !(shape & 32);
-        const uint32_t idesc = ptx::make_idesc_bf16(PM, PN, a_mn, b_mn);
+        const int shape = jobs[d.job].shape;
         const uint32_t small = tmem + 2 * PN + (tile & 1) * PN;
         if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->small_empty[tile & 1]), ((tile >> 1) & 1) ^ 1u, abort_flag)) break;
         for (int k = 0; k < d.nk; ++k) {
@@ -180,26 +217,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
           if (fresh && !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->main_empty[mb]), ((piece >> 1) & 1) ^ 1u, abort_flag)) { ok = false; break; }
           if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag)) { ok = false; break; }
           ptx::tc_fence_after();
-          const uint32_t sa = slabs + stage * PG_STAGE_BYTES, sb = sa + 3 * A_PART;
-#pragma unroll
-          for (int s = 0; s < PK / 16; ++s) {
-            uint64_t ad[3], bd[3];
-#pragma unroll
-            for (int p = 0; p < 3; ++p) {
-              // along rows: 64-element chunks of 32 k-rows (4 KiB), 16 k-rows of 128 bytes per step; along k: 64-byte rows
-              ad[p] = a_mn ? ptx::make_smem_desc(sa + p * A_PART + s * 2048, PK * 128, 1024)
-                           : ptx::make_smem_desc_sw64(sa + p * A_PART + s * 32, 512);
-              bd[p] = b_mn ? ptx::make_smem_desc(sb + p * B_PART + s * 2048, PK * 128, 1024)
-                           : ptx::make_smem_desc_sw64(sb + p * B_PART + s * 32, 512);
-            }
-            ptx::umma_bf16_pair(tmem + mb * PN, ad[0], bd[0], idesc, !(fresh && s == 0));
-            uint32_t acc = (k | s) ? 1u : 0u;
-#pragma unroll
-            for (int q = 2; q >= 1; --q)
-#pragma unroll
-              for (int p = 0; p <= q; ++p)
-                if (p < pa && q - p < pb) { ptx::umma_bf16_pair(small, ad[p], bd[q - p], idesc, acc); acc = 1u; }
-          }
+          issue(shape, tmem + mb * PN, small, slabs + stage * PG_STAGE_BYTES, fresh, k == 0);
           ptx::umma_commit_pair(ptx::smem_u32(&ctl->empty[stage]), 3);
           if (++stage == PG_STAGES) { stage = 0; phase ^= 1u; }
           if ((k + 1) % PG_PROMOTE == 0 || k + 1 == d.nk) {      // (covers the small products so far as well)

@@ -227,26 +227,35 @@ __device__ __forceinline__ void end(Ctl* ctl, unsigned* status) {
 
 // MMAs of one slab, issued by one thread: `steps` of 16 along k, the main product into column 0 of the
 // block's tensor memory, the small ones behind it.
-template <int PA, int PB>
-__device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, bool a_x, bool b_x, int n, int steps,
-                                           bool first, bool fresh_main) {
-  const uint32_t idesc = ptx::make_idesc_bf16(TILE, n, a_x, b_x);
-  const uint32_t a_lbo = a_x ? 128 : K_LBO, a_sbo = a_x ? X_SBO : 128, a_step = a_x ? 256 : 2 * K_LBO;
-  const uint32_t b_lbo = b_x ? 128 : K_LBO, b_sbo = b_x ? X_SBO : 128, b_step = b_x ? 256 : 2 * K_LBO;
-  for (int k = 0; k < steps; ++k) {
-    uint64_t ad[PA], bd[PB];
-#pragma unroll
-    for (int i = 0; i < PA; ++i) ad[i] = ptx::make_smem_desc_plain(slab + i * PART_BYTES + k * a_step, a_lbo, a_sbo);
-#pragma unroll
-    for (int i = 0; i < PB; ++i)
-      bd[i] = ptx::make_smem_desc_plain(slab + OPERAND_BYTES + i * PART_BYTES + k * b_step, b_lbo, b_sbo);
-    ptx::umma_bf16(tmem, ad[0], bd[0], idesc, !(fresh_main && k == 0));
-    bool acc = !(first && k == 0);
+template <int PA, int PB, bool A_X, bool B_X>
+__device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, int n, int steps, bool first, bool fresh_main) {
+  const uint32_t idesc = ptx::make_idesc_bf16(TILE, n, A_X, B_X);
+  constexpr uint64_t along_x = ptx::smem_desc_constant(ptx::LAYOUT_PLAIN, 128, X_SBO);
+  constexpr uint64_t along_k = ptx::smem_desc_constant(ptx::LAYOUT_PLAIN, K_LBO, 128);
+  constexpr int a_step = (A_X ? 256 : 2 * K_LBO) / 16, b_step = (B_X ? 256 : 2 * K_LBO) / 16;
+  uint64_t a = (A_X ? along_x : along_k) + (slab >> 4), b = (B_X ? along_x : along_k) + ((slab + OPERAND_BYTES) >> 4);
+  uint32_t acc_main = !fresh_main, acc = !first;
+  for (int k = 0; k < steps; ++k, a += a_step, b += b_step) {
+    ptx::umma_bf16(tmem, a, b, idesc, acc_main);
 #pragma unroll
     for (int s = 2; s >= 1; --s)                // i + j = 2, then 1: the smallest first
 #pragma unroll
       for (int i = 0; i <= s; ++i)
-        if (i < PA && s - i < PB) { ptx::umma_bf16(tmem + TILE, ad[i], bd[s - i], idesc, acc); acc = true; }
+        if (i < PA && s - i < PB) {
+          ptx::umma_bf16(tmem + TILE, a + i * (PART_BYTES / 16), b + (s - i) * (PART_BYTES / 16), idesc, acc);
+          acc = 1;
+        }
+    acc_main = 1;
+  }
+}
+template <int PA, int PB>
+__device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, bool a_x, bool b_x, int n, int steps, bool first, bool fresh_main) {
+  if (a_x) {
+    if (b_x) issue_slab<PA, PB, true, true>(tmem, slab, n, steps, first, fresh_main);
+    else issue_slab<PA, PB, true, false>(tmem, slab, n, steps, first, fresh_main);
+  } else {
+    if (b_x) issue_slab<PA, PB, false, true>(tmem, slab, n, steps, first, fresh_main);
+    else issue_slab<PA, PB, false, false>(tmem, slab, n, steps, first, fresh_main);
   }
 }
 

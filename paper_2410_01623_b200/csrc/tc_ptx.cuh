@@ -298,25 +298,14 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr, uint32_t lbo_
 }
 
 // The same with a 64-byte swizzle (layout type 4), K-major: rows of 32 bf16 = 64 B along K, SBO = 512.
-__device__ __forceinline__ uint64_t make_smem_desc_sw64(uint32_t saddr, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-
-// The same without swizzle: the operand is made of 8 x 16-byte core matrices (128 contiguous bytes).
+// Without swizzle (type 0) the operand is made of 8 x 16-byte core matrices (128 contiguous bytes).
 //   K-major: rows of a core matrix along M/N; LBO = distance of core matrices along K, SBO along M/N.
 //   MN-major: rows of a core matrix along K (eight M/N elements each); LBO along K, SBO along M/N.
-__device__ __forceinline__ uint64_t make_smem_desc_plain(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
+// A descriptor is its constant part, which the layout fixes, plus the address in 16-byte units: a thread that issues
+// many MMAs adds offsets to it (building each one anew cost more than the MMAs of a 32-deep slab take).
+enum SmemLayout { LAYOUT_PLAIN = 0, LAYOUT_SW128 = 2, LAYOUT_SW64 = 4 };
+__device__ __forceinline__ constexpr uint64_t smem_desc_constant(SmemLayout layout, uint32_t lbo_bytes, uint32_t sbo_bytes) {
+  return ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)layout << 61);
 }
 
 // Instruction descriptor of kind::f16 with bf16 operands and fp32 accumulation:
