@@ -21,6 +21,8 @@
 
 #include <algorithm>
 #include <atomic>
+#include <functional>
+#include <queue>
 
 #include "part_gemm.cuh"
 #include "split_gemm.cuh"
@@ -32,11 +34,12 @@ namespace fira {
 namespace {
 
 constexpr int PM = 256, PN = 128, PK = 32;      // tile of a CTA pair, depth of a slab
-constexpr int PG_STAGES = 5;
+constexpr int PG_MAX_STAGES = 12;
+constexpr int PG_MAX_PAIRS = 127;               // (so many pairs of SMs at most)
 constexpr int PG_PROMOTE = split::PROMOTE / PK; // slabs between two readings of the main accumulator
 constexpr int A_PART = PM / 2 * PK * 2;         // bytes of one part of a slab in one CTA: 8 KiB
 constexpr int B_PART = PN / 2 * PK * 2;         // 4 KiB
-constexpr int PG_STAGE_BYTES = 3 * (A_PART + B_PART);
+constexpr int PG_SLAB_BYTES = 216 * 1024;       // for the slabs in flight: 6 of three parts each, 10 of one and three
 constexpr int PG_EPI_WARPS = 8;
 constexpr int PG_THREADS = 32 * (2 + PG_EPI_WARPS);
 constexpr int PG_TMEM = 512;
@@ -53,13 +56,13 @@ static_assert(sizeof(JobDev) % 64 == 0, "tensor maps must stay 64-byte aligned")
 struct TileDev { int job, i0, j0, nk; };
 
 struct PgCtl {
-  uint64_t full[PG_STAGES], empty[PG_STAGES];
+  uint64_t full[PG_MAX_STAGES], empty[PG_MAX_STAGES];
   uint64_t main_full[2], main_empty[2];         // a piece of the main product is complete / has been read
   uint64_t small_empty[2];                      // the small products of a tile have been read
   uint32_t tmem_base;
   int abort_flag;
 };
-constexpr size_t PG_SMEM_BYTES = (size_t)PG_STAGES * PG_STAGE_BYTES + sizeof(PgCtl);
+constexpr size_t PG_SMEM_BYTES = (size_t)PG_SLAB_BYTES + sizeof(PgCtl);
 static_assert(PG_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
 __device__ __forceinline__ TileDev load_tile(const TileDev* t) {
@@ -107,11 +110,11 @@ __device__ __forceinline__ void store_result(const JobDev& jb, int i, int j, con
 // MMAs of one slab.  An operand along its rows: 64-element chunks of 32 k-rows (4 KiB), 16 k-rows of 128 bytes per
 // step; along k: 64-byte rows.
 template <int PA, int PB, bool A_MN, bool B_MN>
-__device__ __forceinline__ void issue_slab(uint32_t main, uint32_t small, uint32_t slab, bool fresh, bool first) {
+__device__ __forceinline__ void issue_slab(uint32_t main, uint32_t small, uint32_t slab, int a_bytes, bool fresh, bool first) {
   constexpr uint64_t mn = ptx::smem_desc_constant(ptx::LAYOUT_SW128, PK * 128, 1024);
   constexpr uint64_t km = ptx::smem_desc_constant(ptx::LAYOUT_SW64, 0, 512);
   const uint32_t idesc = ptx::make_idesc_bf16(PM, PN, A_MN, B_MN);
-  uint64_t a = (A_MN ? mn : km) + (slab >> 4), b = (B_MN ? mn : km) + ((slab + 3 * A_PART) >> 4);
+  uint64_t a = (A_MN ? mn : km) + (slab >> 4), b = (B_MN ? mn : km) + ((slab + a_bytes) >> 4);
   uint32_t acc = !first;
 #pragma unroll
   for (int s = 0; s < PK / 16; ++s, a += (A_MN ? 2048 : 32) / 16, b += (B_MN ? 2048 : 32) / 16) {
@@ -127,32 +130,33 @@ __device__ __forceinline__ void issue_slab(uint32_t main, uint32_t small, uint32
   }
 }
 template <int PA, int PB>
-__device__ __forceinline__ void issue_slab(int shape, uint32_t main, uint32_t small, uint32_t slab, bool fresh, bool first) {
+__device__ __forceinline__ void issue_slab(int shape, uint32_t main, uint32_t small, uint32_t slab, int a_bytes, bool fresh, bool first) {
   if (shape & 16) {
-    if (shape & 32) issue_slab<PA, PB, true, false>(main, small, slab, fresh, first);
-    else issue_slab<PA, PB, true, true>(main, small, slab, fresh, first);
+    if (shape & 32) issue_slab<PA, PB, true, false>(main, small, slab, a_bytes, fresh, first);
+    else issue_slab<PA, PB, true, true>(main, small, slab, a_bytes, fresh, first);
   } else {
-    if (shape & 32) issue_slab<PA, PB, false, false>(main, small, slab, fresh, first);
-    else issue_slab<PA, PB, false, true>(main, small, slab, fresh, first);
+    if (shape & 32) issue_slab<PA, PB, false, false>(main, small, slab, a_bytes, fresh, first);
+    else issue_slab<PA, PB, false, true>(main, small, slab, a_bytes, fresh, first);
   }
 }
-__device__ __forceinline__ void issue(int shape, uint32_t main, uint32_t small, uint32_t slab, bool fresh, bool first) {
-  if ((shape & 15) == 15) issue_slab<3, 3>(shape, main, small, slab, fresh, first);
-  else if ((shape & 15) == 13) issue_slab<1, 3>(shape, main, small, slab, fresh, first);
-  else if ((shape & 15) == 7) issue_slab<3, 1>(shape, main, small, slab, fresh, first);
-  else issue_slab<1, 1>(shape, main, small, slab, fresh, first);
+__device__ __forceinline__ void issue(int shape, uint32_t main, uint32_t small, uint32_t slab, int a_bytes, bool fresh, bool first) {
+  if ((shape & 15) == 15) issue_slab<3, 3>(shape, main, small, slab, a_bytes, fresh, first);
+  else if ((shape & 15) == 13) issue_slab<1, 3>(shape, main, small, slab, a_bytes, fresh, first);
+  else if ((shape & 15) == 7) issue_slab<3, 1>(shape, main, small, slab, a_bytes, fresh, first);
+  else issue_slab<1, 1>(shape, main, small, slab, a_bytes, fresh, first);
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
-k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, int ntiles, unsigned* __restrict__ status) {
+k_part_gemm(const JobDev* __restrict__ jobs, const int* __restrict__ starts, const TileDev* __restrict__ tiles, int stages,
+            int a_bytes, int stage_bytes, unsigned* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  PgCtl* ctl = reinterpret_cast<PgCtl*>(smem + (size_t)PG_STAGES * PG_STAGE_BYTES);
+  PgCtl* ctl = reinterpret_cast<PgCtl*>(smem + PG_SLAB_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_ctarank();
-  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int first_tile = starts[blockIdx.x >> 1], end_tile = starts[(blockIdx.x >> 1) + 1];     // this pair's
   const bool smem_ok = (ptx::smem_u32(smem) & 1023u) == 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < PG_STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       ptx::mbar_init(ptx::smem_u32(&ctl->full[s]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl->empty[s]), 1);
     }
@@ -178,7 +182,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
   if (warp == 0) {
     if (lane == 0 && smem_ok) {
       int stage = 0; uint32_t phase = 0; bool ok = true;
-      for (int t = pair; t < ntiles && ok; t += npairs) {
+      for (int t = first_tile; t < end_tile && ok; ++t) {
         const TileDev d = load_tile(tiles + t);
         const JobDev* jb = jobs + d.job;
         const int shape = jb->shape, pa = shape & 3, pb = (shape >> 2) & 3;
@@ -186,17 +190,17 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
         for (int k = 0; k < d.nk; ++k) {
           if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->empty[stage]), phase ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t fb = ptx::map_to_cta(ptx::smem_u32(&ctl->full[stage]), 0);
-          const uint32_t sa = slabs + stage * PG_STAGE_BYTES, sb = sa + 3 * A_PART;
+          const uint32_t sa = slabs + stage * stage_bytes, sb = sa + a_bytes;
           if (rank == 0) ptx::mbar_expect_tx(ptx::smem_u32(&ctl->full[stage]), 2 * (pa * A_PART + pb * B_PART));
           if (shape & 16) ptx::tma_load_4d_pair(sa, &jb->a, fb, 0, k * PK, i0 >> 6, 0);
           else ptx::tma_load_3d_pair(sa, &jb->a, fb, k * PK, i0, 0);
           if (shape & 32) ptx::tma_load_3d_pair(sb, &jb->b, fb, k * PK, j0, 0);
           else ptx::tma_load_4d_pair(sb, &jb->b, fb, 0, k * PK, j0 >> 6, 0);
-          if (++stage == PG_STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
         }
       }
       if (!ok && rank == 0) {   // give copies in flight a bounded time to land
-        for (int s = 0; s < PG_STAGES; ++s)
+        for (int s = 0; s < stages; ++s)
           for (uint32_t it = 0; it < (1u << 16); ++it)
             if (ptx::mbar_try_wait_cluster(ptx::smem_u32(&ctl->full[s]), (s < stage) ? phase : (phase ^ 1u))) break;
       }
@@ -206,7 +210,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
       int stage = 0; uint32_t phase = 0; bool ok = true;
       int piece = 0, tile = 0;                  // running numbers of the main accumulator's uses and of the tiles
       const uint32_t tmem = ctl->tmem_base;
-      for (int t = pair; t < ntiles && ok; t += npairs, ++tile) {
+      for (int t = first_tile; t < end_tile && ok; ++t) {
         const TileDev d = load_tile(tiles + t);
         const int shape = jobs[d.job].shape;
         const uint32_t small = tmem + 2 * PN + (tile & 1) * PN;
@@ -217,14 +221,15 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
           if (fresh && !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->main_empty[mb]), ((piece >> 1) & 1) ^ 1u, abort_flag)) { ok = false; break; }
           if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag)) { ok = false; break; }
           ptx::tc_fence_after();
-          issue(shape, tmem + mb * PN, small, slabs + stage * PG_STAGE_BYTES, fresh, k == 0);
+          issue(shape, tmem + mb * PN, small, slabs + stage * stage_bytes, a_bytes, fresh, k == 0);
           ptx::umma_commit_pair(ptx::smem_u32(&ctl->empty[stage]), 3);
-          if (++stage == PG_STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == stages) { stage = 0; phase ^= 1u; }
           if ((k + 1) % PG_PROMOTE == 0 || k + 1 == d.nk) {      // (covers the small products so far as well)
             ptx::umma_commit_pair(ptx::smem_u32(&ctl->main_full[mb]), 3);
             ++piece;
           }
         }
+        ++tile;
       }
     }
   } else if (smem_ok) {
@@ -235,7 +240,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
     const uint32_t se[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[1]), 0)};
     int piece = 0, tile = 0;
     bool ok = true;
-    for (int t = pair; t < ntiles && ok; t += npairs, ++tile) {
+    for (int t = first_tile; t < end_tile && ok; ++t) {
       const TileDev d = load_tile(tiles + t);
       const JobDev& jb = jobs[d.job];
       const int npieces = (d.nk + PG_PROMOTE - 1) / PG_PROMOTE;
@@ -274,6 +279,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const TileDev* __restrict__ tiles, 
         __syncwarp();
       }
       if (lane == 0) ptx::mbar_arrive_cluster(se[tile & 1]);
+      ++tile;
       const int i = d.i0 + PM / 2 * (int)rank + 32 * quarter + lane;
       if (i < jb.I && d.j0 + c0 < jb.J) store_result(jb, i, d.j0 + c0, sum);
     }
@@ -323,10 +329,49 @@ void tiles_of(const PartGemm& g, int job, std::vector<TileDev>& out) {
 
 }  // namespace
 
+// SMs of the current device (0: error) once the kernel may use its shared memory there.
+static int prepared_sms() {
+  static std::atomic<int> sms_of_device[64];    // (the shared-memory limit is a per-device setting)
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
+  if (e == cudaSuccess && (sms = sms_of_device[dev].load()) == 0) {
+    e = cudaFuncSetAttribute(k_part_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) sms_of_device[dev].store(sms);
+  }
+  if (e != cudaSuccess) { set_error(std::string("part products: ") + cudaGetErrorString(e)); return 0; }
+  return sms;
+}
+
+// Deals the tiles out to `pairs` CTA pairs, in order (neighbours run side by side), each to the pair with the least work
+// so far; pair p gets those at starts[p] .. starts[p + 1] of the result.  A tile's end costs about as much as two slabs.
+static std::vector<TileDev> deal(const std::vector<TileDev>& tiles, int pairs, std::vector<int>& starts) {
+  typedef std::pair<long long, int> Load;
+  std::priority_queue<Load, std::vector<Load>, std::greater<Load>> load;
+  for (int p = 0; p < pairs; ++p) load.push({0, p});
+  std::vector<std::vector<TileDev>> of((size_t)pairs);
+  for (const TileDev& t : tiles) {
+    const Load l = load.top();
+    load.pop();
+    of[l.second].push_back(t);
+    load.push({l.first + t.nk + 2, l.second});
+  }
+  std::vector<TileDev> out;
+  starts.assign(1, 0);
+  for (const auto& v : of) {
+    out.insert(out.end(), v.begin(), v.end());
+    starts.push_back((int)out.size());
+  }
+  return out;
+}
+
+static size_t starts_bytes() { return align_up((PG_MAX_PAIRS + 1) * sizeof(int)); }
+
 size_t part_gemm_table_bytes(const PartGemm* jobs, int njobs) {
   std::vector<TileDev> t;
   for (int q = 0; q < njobs; ++q) tiles_of(jobs[q], q, t);
-  return align_up(sizeof(JobDev) * (size_t)njobs) + align_up(sizeof(TileDev) * t.size());
+  return align_up(sizeof(JobDev) * (size_t)njobs) + starts_bytes() + align_up(sizeof(TileDev) * t.size());
 }
 
 fira_status part_gemm_prepare(const PartGemm* jobs, int njobs, char* table_dev, size_t table_bytes, int* ntiles, cudaStream_t st) {
@@ -347,30 +392,32 @@ fira_status part_gemm_prepare(const PartGemm* jobs, int njobs, char* table_dev, 
   for (int q = 0; q < njobs; ++q) order[q] = q;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return depth_of(jobs[x]) > depth_of(jobs[y]); });
   for (int q : order) tiles_of(jobs[q], q, td);
-  const size_t off = align_up(sizeof(JobDev) * (size_t)njobs);
-  if (off + align_up(sizeof(TileDev) * td.size()) > table_bytes) { set_error("part products: table area too small"); return FIRA_ERR_WORKSPACE_TOO_SMALL; }
-  cudaError_t e = cudaMemcpyAsync(table_dev, jd.data(), sizeof(JobDev) * jd.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(table_dev + off, td.data(), sizeof(TileDev) * td.size(), cudaMemcpyHostToDevice, st);
-  if (e != cudaSuccess) { set_error(std::string("part products, tables: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
+  const int sms = prepared_sms();
+  if (!sms) return FIRA_ERR_CUDA;
   *ntiles = (int)td.size();
+  std::vector<int> starts;
+  td = deal(td, std::min(*ntiles, sms / 2), starts);
+  const size_t o_starts = align_up(sizeof(JobDev) * (size_t)njobs), o_tiles = o_starts + starts_bytes();
+  if (starts.size() > PG_MAX_PAIRS + 1 || o_tiles + align_up(sizeof(TileDev) * td.size()) > table_bytes) {
+    set_error("part products: table area too small"); return FIRA_ERR_WORKSPACE_TOO_SMALL;
+  }
+  cudaError_t e = cudaMemcpyAsync(table_dev, jd.data(), sizeof(JobDev) * jd.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(table_dev + o_starts, starts.data(), sizeof(int) * starts.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(table_dev + o_tiles, td.data(), sizeof(TileDev) * td.size(), cudaMemcpyHostToDevice, st);
+  if (e != cudaSuccess) { set_error(std::string("part products, tables: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }
 
-fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, unsigned* status_dev, cudaStream_t st) {
-  static std::atomic<int> sms_of_device[64];    // (the shared-memory limit is a per-device setting)
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
-  if (e == cudaSuccess && (sms = sms_of_device[dev].load()) == 0) {
-    e = cudaFuncSetAttribute(k_part_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_BYTES);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) sms_of_device[dev].store(sms);
-  }
-  if (e != cudaSuccess) { set_error(std::string("part products: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
+fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, int a_parts, int b_parts, unsigned* status_dev, cudaStream_t st) {
+  const int sms = prepared_sms();
+  if (!sms) return FIRA_ERR_CUDA;
   if (ntiles == 0) return FIRA_OK;
+  const int a_bytes = a_parts * A_PART, stage_bytes = a_bytes + b_parts * B_PART;
+  const char* starts = table_dev + align_up(sizeof(JobDev) * (size_t)njobs);
   k_part_gemm<<<2 * std::min(ntiles, sms / 2), PG_THREADS, PG_SMEM_BYTES, st>>>(
-      reinterpret_cast<const JobDev*>(table_dev),
-      reinterpret_cast<const TileDev*>(table_dev + align_up(sizeof(JobDev) * (size_t)njobs)), ntiles, status_dev);
+      reinterpret_cast<const JobDev*>(table_dev), reinterpret_cast<const int*>(starts),
+      reinterpret_cast<const TileDev*>(starts + starts_bytes()), std::min(PG_MAX_STAGES, PG_SLAB_BYTES / stage_bytes), a_bytes,
+      stage_bytes, status_dev);
   return FIRA_OK;
 }
 

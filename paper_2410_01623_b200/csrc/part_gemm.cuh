@@ -39,7 +39,7 @@ struct PartGemm {
 size_t part_gemm_table_bytes(const PartGemm* jobs, int njobs);
 // Builds the tables on the host and uploads them to table_dev (256-byte aligned) on the given stream.
 fira_status part_gemm_prepare(const PartGemm* jobs, int njobs, char* table_dev, size_t table_bytes, int* ntiles, cudaStream_t st);
-// One grouped launch over the prepared jobs.
-fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, unsigned* status_dev, cudaStream_t st);
+// One grouped launch over the prepared jobs.  a_parts, b_parts: the most parts that an operand of theirs has.
+fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, int a_parts, int b_parts, unsigned* status_dev, cudaStream_t st);
 
 }  // namespace fira

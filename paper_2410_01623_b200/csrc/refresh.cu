@@ -430,8 +430,11 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
         if (ps != FIRA_OK) return ps;
         tp += bytes;
       }
-    int rmax = 0;
-    for (const RefreshMat& m : rms) rmax = std::max(rmax, m.r);
+    int rmax = 0, gparts = 1;
+    for (const RefreshMat& m : rms) {
+      rmax = std::max(rmax, m.r);
+      if (!m.tc) gparts = std::max(gparts, m.Gp.parts);
+    }
     // element-wise helpers: blockIdx.y is the matrix, enough blocks for the largest of its kind (at most two per SM)
     long long gmax = 0, ymax = 0, zmax = 0;
     for (const RefreshMat& m : rms) {
@@ -445,7 +448,8 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
     const long long umax = (long long)rmax * rmax;
     auto run = [&](int tc_kind, int part_kind) -> fira_status {
       if (nparts) {
-        const fira_status ps = part_gemm_run(ptab[part_kind], nparts, ptiles[part_kind], c->status_dev, st);
+        const bool with_g = part_kind == PART_AZ || part_kind == PART_ATY;
+        const fira_status ps = part_gemm_run(ptab[part_kind], nparts, ptiles[part_kind], with_g ? gparts : 3, 3, c->status_dev, st);
         if (ps != FIRA_OK) return ps;
       }
       return ntc ? tc_gemm_run(c, tab[tc_kind], ntc, jtiles[tc_kind], st) : FIRA_OK;
