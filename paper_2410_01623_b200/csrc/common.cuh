@@ -37,15 +37,22 @@ struct MatDev {
   MatScalars* sc;
   float* Rt;          // scratch: l x r fp32 low-rank gradient (transposed layout)
   float* Xt;          // scratch: l x r fp32 N
+  __nv_bfloat16* Rp;  //   "      long lists (PartStepPlan): R and X as three bf16 parts [3][l][rp_pitch]
+  __nv_bfloat16* Xp;
+  __nv_bfloat16* Pp;  //   "      the projection as parts [3 or 1][d][pp_pitch]
+  float* step_bias;   //   "      this step's bias factor (k_finalize puts the next one into MatScalars)
+  int rp_pitch, pp_pitch;
+  int aux_slots;      // row sums per l in aux
+  int tma_proj;       // long lists: the projection is part_project.cu's (slots of 64 columns), otherwise k_project's (of 128)
   float* kvec;        // scratch: l factors
   float* part;        // scratch: partial sums of ||S||^2
-  float* aux;         // scratch: ||N_l||^2, then ||R_l||^2; engine 0: l floats of each per tile of r
+  float* aux;         // scratch: row sums [aux_slots][l] of ||N_l||^2, then of ||R_l||^2 (engine 0: one slot per tile of r)
   __nv_bfloat16* Nb;  // scratch of the tensor-core path: l x r bf16 N
   __nv_bfloat16* Rb;  //   "      l x r bf16 R
   __nv_bfloat16* Xb;  //   "      l x r bf16 X
   float* colpart;     //   "      per (r-tile, l) partial sums of N^2 and R^2, then per-l sums of G^2
-  __nv_bfloat16* Gs;  //   "      copies of G and W with 16-byte aligned rows (pitch lds), only when the
-  __nv_bfloat16* Ws;  //          caller's rows are not (odd widths): TMA needs aligned rows
+  void* Gs;           //   "      copies of G and W with 16-byte aligned rows (pitch lds), only when the
+  void* Ws;           //          caller's rows are not (odd widths): TMA needs aligned rows
   long long lds;
   long long ld;
   int m, n, r;
@@ -77,6 +84,9 @@ enum DeviceStatusBits : unsigned {
   DEV_STATUS_TIMEOUT = 1u,
   DEV_STATUS_NONFINITE = 2u,
 };
+
+// The base optimizers, as template parameters of the projection's epilogues (Adam: Eq. 2-4).
+enum { PSI_ADAM = 0, PSI_RMSPROP = 1, PSI_ADAGRAD = 2 };
 
 template <typename T>
 __device__ __forceinline__ float to_float(T v);

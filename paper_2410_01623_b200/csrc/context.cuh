@@ -35,7 +35,7 @@ struct fira_ctx {
   char* work_base = nullptr;             // per-matrix step scratch, reused by the refresh
   size_t work_bytes = 0;
 
-  fira::SimtPlan simt;                   // matrices on the fp32 CUDA-core kernels
+  fira::SimtPlan simt;                   // matrices on the kernels of fp32 precision
   fira::TcPlan* tc = nullptr;            // matrices on the tensor-core kernels
   std::vector<int> simt_list, tc_list;
   std::vector<long long> t_host;         // host mirror of every matrix's step count
@@ -43,6 +43,7 @@ struct fira_ctx {
   fira::HostPipe pipe;
   bool table_dirty = true;
   bool proj_weights_dirty = true;        // tensor-core path: column norms of the stored projections to be retaken
+  bool proj_parts_dirty = true;          // long lists of the fp32-precision engine: the stored projections to be split again
   int last_launches = 0;
 };
 
@@ -56,8 +57,11 @@ struct Layout {
   size_t off_mats = 0, off_status = 0, off_ints = 0, off_tcmaps = 0, off_work = 0;
   size_t ints_count = 0;
   // byte offsets per matrix inside the work area
-  std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux;
+  std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux, offRp, offXp, offPp, offBias;
   std::vector<int> engine;
+  bool parts = false;       // the fp32-precision engine's list is long
+  bool tma_proj = false;    // and its projection runs on part_project.cu
+  size_t off_parts = 0, off_proj_parts = 0;
   size_t step_work_bytes = 0, refresh_min_bytes = 0;
   size_t scratch_bytes = 0;
 };

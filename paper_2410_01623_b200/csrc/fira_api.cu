@@ -59,6 +59,15 @@ int engine_for(const fira_hparams& hp, const fira_matrix_desc& d) {
   return tc_supported(d) ? 1 : 0;
 }
 
+// Row pitch (elements) of the aligned copies of a matrix on the fp32-precision engine's long lists; 0: none needed.
+static long long part_staging_pitch(const fira_matrix_desc& d, uint32_t flags) {
+  if (d.dtype == FIRA_BF16) return tc_staging_pitch(d, flags);
+  return (d.ld ? d.ld : d.n) % 4 == 0 && d.n % 4 == 0 ? 0 : ((long long)d.n + 63) / 64 * 64;
+}
+
+// Row sums per l: one per tile of R, whose width depends on the kernels.
+static int aux_slots(const Layout& L, int i, int r) { return L.engine[i] == 1 ? 1 : L.tma_proj ? (r + 63) / 64 : simt_tiles(r); }
+
 constexpr size_t REFRESH_SMALL_LIST_BYTES = (size_t)512 << 20;
 
 Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_t count) {
@@ -79,26 +88,56 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
   size_t wo = 0;
   L.off_mats = wo; wo += align_up(sizeof(MatDev) * count);
   L.off_status = wo; wo += 256;
-  L.ints_count = 16 * (size_t)(count + 1);
+  L.ints_count = 20 * (size_t)(count + 1);
   L.off_ints = wo; wo += align_up(L.ints_count * sizeof(int));
   L.off_tcmaps = wo; wo += tc_tables_bytes(hp, descs, count);
+  // matrices of the fp32-precision engine: a long list keeps R, X and the projections as parts
+  {
+    std::vector<fira_matrix_desc> own;
+    int tiles = 0, ptiles = 0;
+    for (int i = 0; i < count; ++i)
+      if (L.engine[i] == 0) {
+        own.push_back(descs[i]);
+        tiles += part_step_tiles(descs[i].m, descs[i].n);
+        ptiles += part_project_tiles(std::max(descs[i].m, descs[i].n), descs[i].r);
+      }
+    L.parts = !own.empty() && simt_long_list(own);
+    L.tma_proj = L.parts;             // M and V move as TMA boxes: rows on 16-byte boundaries
+    for (const fira_matrix_desc& d : own) L.tma_proj = L.tma_proj && d.r % 4 == 0;
+    L.off_parts = wo;
+    if (L.parts) wo += part_step_table_bytes((int)own.size(), tiles);
+    L.off_proj_parts = wo;
+    if (L.tma_proj) wo += part_project_table_bytes((int)own.size(), ptiles);
+  }
   L.off_work = wo;
   size_t w = 0;
   size_t refresh_max = 0, refresh_all = 0;
   L.offRt.assign(count, 0); L.offXt.assign(count, 0); L.offK.assign(count, 0); L.offPart.assign(count, 0);
   L.offNb.assign(count, 0); L.offRb.assign(count, 0); L.offXb.assign(count, 0);
-  L.offColpart.assign(count, 0); L.offGs.assign(count, 0); L.offWs.assign(count, 0); L.offAux.assign(count, 0);
+  L.offColpart.assign(count, 0); L.offGs.assign(count, 0); L.offWs.assign(count, 0); L.offAux.assign(count, 0); L.offRp.assign(count, 0); L.offPp.assign(count, 0);
+  L.offXp.assign(count, 0); L.offBias.assign(count, 0);
   for (int i = 0; i < count; ++i) {
     fira_matrix_desc d = descs[i];
     if (d.ld == 0) d.ld = d.n;
     const size_t ll = std::max(d.m, d.n), r = d.r;
     L.offK[i] = w; w += align_up(ll * 4);
-    L.offAux[i] = w; w += align_up(2 * (L.engine[i] == 0 ? simt_tiles(d.r) : 1) * ll * 4);
+    L.offAux[i] = w; w += align_up(2 * aux_slots(L, i, d.r) * ll * 4);
     if (L.engine[i] == 0) {
-      const size_t tiles = (size_t)simt_tiles(d.m) * simt_tiles(d.n);
-      L.offRt[i] = w; w += align_up(ll * r * 4);
-      L.offXt[i] = w; w += align_up(ll * r * 4);
-      L.offPart[i] = w; w += align_up(tiles * 4);
+      const size_t tiles = (size_t)simt_tiles(d.m) * simt_tiles(d.n), sums = (size_t)part_step_tiles(d.m, d.n) * PART_SUMS_PER_TILE;
+      const size_t dd = std::min(d.m, d.n), pitch = part_rank_pitch(d.r);
+      if (L.parts) {
+        L.offRp[i] = w; w += align_up(3 * ll * pitch * 2);
+        L.offXp[i] = w; w += align_up(3 * ll * pitch * 2);
+        L.offPp[i] = w; w += align_up((d.dtype == FIRA_BF16 ? 1 : 3) * dd * part_pitch(d.r) * 2);
+        L.offBias[i] = w; w += 256;
+        const size_t bytes = (size_t)d.m * part_staging_pitch(d, hp.flags) * (d.dtype == FIRA_BF16 ? 2 : 4);
+        L.offGs[i] = w; w += align_up(bytes);
+        L.offWs[i] = w; w += align_up(bytes);
+      } else {
+        L.offRt[i] = w; w += align_up(ll * r * 4);
+        L.offXt[i] = w; w += align_up(ll * r * 4);
+      }
+      L.offPart[i] = w; w += align_up((L.parts ? std::max(tiles, sums) : tiles) * 4);
     } else {
       L.offNb[i] = w; w += align_up(ll * r * 2);
       L.offRb[i] = w; w += align_up(ll * r * 2);
@@ -220,9 +259,22 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
     mt.kvec = (float*)(c->work_base + L.offK[i]);
     mt.aux = (float*)(c->work_base + L.offAux[i]);
     mt.part = (float*)(c->work_base + L.offPart[i]);
+    mt.aux_slots = aux_slots(L, i, d.r);
+    mt.tma_proj = L.tma_proj && mt.engine == 0;
     if (mt.engine == 0) {
-      mt.Rt = (float*)(c->work_base + L.offRt[i]);
-      mt.Xt = (float*)(c->work_base + L.offXt[i]);
+      if (L.parts) {
+        mt.Rp = (__nv_bfloat16*)(c->work_base + L.offRp[i]);
+        mt.Pp = (__nv_bfloat16*)(c->work_base + L.offPp[i]);
+        mt.Xp = (__nv_bfloat16*)(c->work_base + L.offXp[i]);
+        mt.step_bias = (float*)(c->work_base + L.offBias[i]);
+        mt.rp_pitch = part_rank_pitch(d.r);
+        mt.pp_pitch = (int)part_pitch(d.r);
+        mt.lds = part_staging_pitch(c->descs[i], c->hp.flags);
+        if (mt.lds) { mt.Gs = c->work_base + L.offGs[i]; mt.Ws = c->work_base + L.offWs[i]; }
+      } else {
+        mt.Rt = (float*)(c->work_base + L.offRt[i]);
+        mt.Xt = (float*)(c->work_base + L.offXt[i]);
+      }
       c->simt_list.push_back(i);
     } else {
       mt.Nb = (__nv_bfloat16*)(c->work_base + L.offNb[i]);
@@ -231,8 +283,8 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
       mt.colpart = (float*)(c->work_base + L.offColpart[i]);
       mt.lds = tc_staging_pitch(c->descs[i], c->hp.flags);
       if (mt.lds) {
-        mt.Gs = (__nv_bfloat16*)(c->work_base + L.offGs[i]);
-        mt.Ws = (__nv_bfloat16*)(c->work_base + L.offWs[i]);
+        mt.Gs = c->work_base + L.offGs[i];
+        mt.Ws = c->work_base + L.offWs[i];
       }
       c->tc_list.push_back(i);
     }
@@ -247,23 +299,34 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
   };
   {
     const std::vector<int>& lst = c->simt_list;
-    std::vector<int> pt{0}, wt{0}, np;
+    std::vector<int> pt{0}, wt{0}, rs{0}, np, npt, sl, ss{0}, sp{0};
     for (int i : lst) {
       const MatDev& mt = c->mats[i];
       pt.push_back(pt.back() + simt_tiles(mt.l) * simt_tiles(mt.r));
       const int tiles = simt_tiles(mt.m) * simt_tiles(mt.n);
       wt.push_back(wt.back() + tiles);
-      np.push_back(tiles);
+      rs.push_back(rs.back() + mt.l);
+      npt.push_back(tiles);
+      if (mt.Gs) { sl.push_back(i); ss.push_back(ss.back() + mt.m); }
+      sp.push_back((int)sl.size());
+      np.push_back(L.parts ? part_step_tiles(mt.m, mt.n) * PART_SUMS_PER_TILE : tiles);
     }
-    const size_t o_list = push_block(lst), o_pt = push_block(pt), o_wt = push_block(wt), o_np = push_block(np);
+    const size_t o_list = push_block(lst), o_pt = push_block(pt), o_wt = push_block(wt), o_np = push_block(np),
+                 o_npt = push_block(npt), o_rs = push_block(rs), o_sl = push_block(sl), o_ss = push_block(ss);
     c->simt.mats = c->mats_dev;
     c->simt.list = c->ints_dev + o_list; c->simt.nlist = (int)lst.size();
     c->simt.proj_tile_start = c->ints_dev + o_pt; c->simt.proj_tiles = pt.back();
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
-    c->simt.npart = c->ints_dev + o_np;
+    c->simt.npart = c->ints_dev + o_np; c->simt.npart_tiles = c->ints_dev + o_npt;
+    c->simt.row_start = c->ints_dev + o_rs; c->simt.h_row_start = rs;
+    c->simt.stage_list = c->ints_dev + o_sl; c->simt.stage_start = c->ints_dev + o_ss;
+    c->simt.h_stage_pos = sp; c->simt.h_stage_start = ss;
     c->simt.h_proj_tile_start = pt; c->simt.h_w_tile_start = wt;
   }
-  fira_status ts = tc_build_plan(c, ints);
+  fira_status ts = FIRA_OK;
+  if (L.parts) ts = part_step_prepare(c->mats, c->simt_list, c->scratch_base + L.off_parts, &c->simt.parts, c->stream);
+  if (L.tma_proj && ts == FIRA_OK) ts = part_project_prepare(c->mats, c->simt_list, c->scratch_base + L.off_proj_parts, &c->simt.parts, c->stream);
+  if (ts == FIRA_OK) ts = tc_build_plan(c, ints);
   if (ts != FIRA_OK) { tc_destroy_plan(c); delete c; return ts; }
   if (ints.size() > c->ints_count) { set_error("internal: schedule arrays overflow"); tc_destroy_plan(c); delete c; return FIRA_ERR_INVALID_ARG; }
 
@@ -298,6 +361,7 @@ static fira_status set_pointers(fira_ctx* c, void* const* W_dev, const void* con
   if (ptr_changed) {
     c->table_dirty = true;
     fira_status s = tc_update_pointers(c);
+    if (s == FIRA_OK && c->simt.parts.table) s = part_step_update_pointers(c->mats, c->simt_list, &c->simt.parts, c->stream);
     if (s != FIRA_OK) return s;
   }
   if (c->table_dirty) { fira_status s = upload_table(c); if (s != FIRA_OK) return s; }
@@ -307,6 +371,10 @@ static fira_status set_pointers(fira_ctx* c, void* const* W_dev, const void* con
 // Enqueues the step of the matrices [i0, i1) (both engines' lists are ascending, so the range maps
 // to one sub-range of each); returns the number of launches or -1.
 static int launch_range(fira_ctx* c, const Hyper& h, int i0, int i1, bool whole) {
+  if (c->proj_parts_dirty) {          // the stored projections have changed since they were split
+    launch_split_projections(c->simt, c->mats, c->simt_list, c->stream);
+    c->proj_parts_dirty = false;
+  }
   if (whole) {
     const int launches = launch_simt_step(c->simt, h, c->status_dev, c->stream, &c->timer);
     if (launches < 0) return -1;
@@ -541,7 +609,7 @@ fira_status fira_set_projection(fira_ctx* c, int32_t idx, const void* P_dev) {
   const MatDev& mt = c->mats[idx];
   const size_t bytes = (size_t)mt.d * mt.r * (mt.bf16 ? 2 : 4);
   FIRA_CUDA(cudaMemcpyAsync(mt.P, P_dev, bytes, cudaMemcpyDeviceToDevice, c->stream));
-  c->proj_weights_dirty = true;
+  c->proj_weights_dirty = c->proj_parts_dirty = true;
   return FIRA_OK;
 }
 

@@ -150,6 +150,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   mt.kvec = reinterpret_cast<float*>(base + cv.off_k);
   mt.part = reinterpret_cast<float*>(base + cv.off_part);
   mt.aux = reinterpret_cast<float*>(base + kNoAllocScratchBytes);
+  mt.aux_slots = simt_tiles(desc->r);
   mt.m = desc->m; mt.n = desc->n; mt.r = desc->r;
   mt.ld = desc->ld ? desc->ld : desc->n;
   mt.left = desc->m <= desc->n;

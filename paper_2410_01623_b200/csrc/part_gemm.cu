@@ -24,21 +24,16 @@
 #include <functional>
 #include <queue>
 
-#include "part_gemm.cuh"
+#include "part_slab.cuh"
 #include "split_gemm.cuh"
-#include "tc_ptx.cuh"
-#include "tma_encode.cuh"
 
 namespace fira {
 
 namespace {
 
-constexpr int PM = 256, PN = 128, PK = 32;      // tile of a CTA pair, depth of a slab
 constexpr int PG_MAX_STAGES = 12;
 constexpr int PG_MAX_PAIRS = 127;               // (so many pairs of SMs at most)
 constexpr int PG_PROMOTE = split::PROMOTE / PK; // slabs between two readings of the main accumulator
-constexpr int A_PART = PM / 2 * PK * 2;         // bytes of one part of a slab in one CTA: 8 KiB
-constexpr int B_PART = PN / 2 * PK * 2;         // 4 KiB
 constexpr int PG_SLAB_BYTES = 216 * 1024;       // for the slabs in flight: 6 of three parts each, 10 of one and three
 constexpr int PG_EPI_WARPS = 8;
 constexpr int PG_THREADS = 32 * (2 + PG_EPI_WARPS);
@@ -105,45 +100,6 @@ __device__ __forceinline__ void store_result(const JobDev& jb, int i, int j, con
       store32(o + 2 * jb.part_stride + q, l);
     }
   }
-}
-
-// MMAs of one slab.  An operand along its rows: 64-element chunks of 32 k-rows (4 KiB), 16 k-rows of 128 bytes per
-// step; along k: 64-byte rows.
-template <int PA, int PB, bool A_MN, bool B_MN>
-__device__ __forceinline__ void issue_slab(uint32_t main, uint32_t small, uint32_t slab, int a_bytes, bool fresh, bool first) {
-  constexpr uint64_t mn = ptx::smem_desc_constant(ptx::LAYOUT_SW128, PK * 128, 1024);
-  constexpr uint64_t km = ptx::smem_desc_constant(ptx::LAYOUT_SW64, 0, 512);
-  const uint32_t idesc = ptx::make_idesc_bf16(PM, PN, A_MN, B_MN);
-  uint64_t a = (A_MN ? mn : km) + (slab >> 4), b = (B_MN ? mn : km) + ((slab + a_bytes) >> 4);
-  uint32_t acc = !first;
-#pragma unroll
-  for (int s = 0; s < PK / 16; ++s, a += (A_MN ? 2048 : 32) / 16, b += (B_MN ? 2048 : 32) / 16) {
-    ptx::umma_bf16_pair(main, a, b, idesc, s ? 1u : !fresh);
-#pragma unroll
-    for (int q = 2; q >= 1; --q)
-#pragma unroll
-      for (int p = 0; p <= q; ++p)
-        if (p < PA && q - p < PB) {
-          ptx::umma_bf16_pair(small, a + p * (A_PART / 16), b + (q - p) * (B_PART / 16), idesc, acc);
-          acc = 1u;
-        }
-  }
-}
-template <int PA, int PB>
-__device__ __forceinline__ void issue_slab(int shape, uint32_t main, uint32_t small, uint32_t slab, int a_bytes, bool fresh, bool first) {
-  if (shape & 16) {
-    if (shape & 32) issue_slab<PA, PB, true, false>(main, small, slab, a_bytes, fresh, first);
-    else issue_slab<PA, PB, true, true>(main, small, slab, a_bytes, fresh, first);
-  } else {
-    if (shape & 32) issue_slab<PA, PB, false, false>(main, small, slab, a_bytes, fresh, first);
-    else issue_slab<PA, PB, false, true>(main, small, slab, a_bytes, fresh, first);
-  }
-}
-__device__ __forceinline__ void issue(int shape, uint32_t main, uint32_t small, uint32_t slab, int a_bytes, bool fresh, bool first) {
-  if ((shape & 15) == 15) issue_slab<3, 3>(shape, main, small, slab, a_bytes, fresh, first);
-  else if ((shape & 15) == 13) issue_slab<1, 3>(shape, main, small, slab, a_bytes, fresh, first);
-  else if ((shape & 15) == 7) issue_slab<3, 1>(shape, main, small, slab, a_bytes, fresh, first);
-  else issue_slab<1, 1>(shape, main, small, slab, a_bytes, fresh, first);
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PG_THREADS, 1)
@@ -221,7 +177,7 @@ k_part_gemm(const JobDev* __restrict__ jobs, const int* __restrict__ starts, con
           if (fresh && !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->main_empty[mb]), ((piece >> 1) & 1) ^ 1u, abort_flag)) { ok = false; break; }
           if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag)) { ok = false; break; }
           ptx::tc_fence_after();
-          issue(shape, tmem + mb * PN, small, slabs + stage * stage_bytes, a_bytes, fresh, k == 0);
+          issue_parts(shape, tmem + mb * PN, small, slabs + stage * stage_bytes, a_bytes, fresh, k == 0);
           ptx::umma_commit_pair(ptx::smem_u32(&ctl->empty[stage]), 3);
           if (++stage == stages) { stage = 0; phase ^= 1u; }
           if ((k + 1) % PG_PROMOTE == 0 || k + 1 == d.nk) {      // (covers the small products so far as well)
@@ -243,41 +199,19 @@ k_part_gemm(const JobDev* __restrict__ jobs, const int* __restrict__ starts, con
     for (int t = first_tile; t < end_tile && ok; ++t) {
       const TileDev d = load_tile(tiles + t);
       const JobDev& jb = jobs[d.job];
-      const int npieces = (d.nk + PG_PROMOTE - 1) / PG_PROMOTE;
-      float sum[64];
+      float sum[64];                            // this thread's row of the product, columns c0 .. c0 + 63
 #pragma unroll
       for (int e = 0; e < 64; ++e) sum[e] = 0.f;
+      const int npieces = (d.nk + PG_PROMOTE - 1) / PG_PROMOTE;
       for (int p = 0; p < npieces; ++p, ++piece) {
         const int mb = piece & 1;
         if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->main_full[mb]), (piece >> 1) & 1, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t v[32];
-          __syncwarp();
-          ptx::tmem_ld_32x32b_x32(tmem + mb * PN + 32 * h, v);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 32; ++e) sum[32 * h + e] += __uint_as_float(v[e]);
-        }
-        ptx::tc_fence_before();
-        __syncwarp();
+        add_columns(sum, tmem + mb * PN);
         if (lane == 0) ptx::mbar_arrive_cluster(me[mb]);
       }
       if (!ok) break;
-      if ((jb.shape & 15) != 5) {               // some operand has more than one part
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t v[32];
-          __syncwarp();
-          ptx::tmem_ld_32x32b_x32(tmem + 2 * PN + (tile & 1) * PN + 32 * h, v);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 32; ++e) sum[32 * h + e] += __uint_as_float(v[e]);
-        }
-        ptx::tc_fence_before();
-        __syncwarp();
-      }
+      if ((jb.shape & 15) != 5) add_columns(sum, tmem + 2 * PN + (tile & 1) * PN);    // some operand has more than one part
       if (lane == 0) ptx::mbar_arrive_cluster(se[tile & 1]);
       ++tile;
       const int i = d.i0 + PM / 2 * (int)rank + 32 * quarter + lane;
@@ -294,21 +228,6 @@ k_part_gemm(const JobDev* __restrict__ jobs, const int* __restrict__ starts, con
     ptx::tmem_dealloc_pair(ctl->tmem_base, PG_TMEM);
   }
   if (threadIdx.x == 0 && ctl->abort_flag) atomicOr(status, DEV_STATUS_TIMEOUT);
-}
-
-// Map of an operand: rows_contiguous: the operand's rows (i of A, j of B) are contiguous in memory.
-bool encode_operand(CUtensorMap* map, const PartMatrix& p, bool rows_contiguous, int rows_box) {
-  const unsigned long long pitch = p.pitch * 2, part = p.part_stride * 2;
-  if (rows_contiguous) {
-    const unsigned long long extent[4] = {64, (unsigned long long)p.rows, (unsigned long long)(p.pitch / 64), (unsigned long long)p.parts};
-    const unsigned long long stride[3] = {pitch, 128, part};
-    const unsigned box[4] = {64, PK, (unsigned)rows_box / 64, (unsigned)p.parts};
-    return encode_tiled(map, p.base, false, 4, extent, stride, box, 128);
-  }
-  const unsigned long long extent[3] = {(unsigned long long)p.cols, (unsigned long long)p.rows, (unsigned long long)p.parts};
-  const unsigned long long stride[2] = {pitch, part};
-  const unsigned box[3] = {PK, (unsigned)rows_box, (unsigned)p.parts};
-  return encode_tiled(map, p.base, false, 3, extent, stride, box, 64);
 }
 
 long long depth_of(const PartGemm& g) { return g.a_t ? g.a.rows : g.a.cols; }

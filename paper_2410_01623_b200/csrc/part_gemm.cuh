@@ -8,7 +8,8 @@
 
 namespace fira {
 
-// A matrix as parts: row-major [parts][rows][pitch], pitch a multiple of 64 elements, 16-byte aligned.
+// A matrix as parts: row-major [parts][rows][pitch], 16-byte aligned, pitch a multiple of 8 elements, or of 64 where the
+// products need it along its rows.
 struct PartMatrix {
   __nv_bfloat16* base = nullptr;
   long long rows = 0, cols = 0, pitch = 0, part_stride = 0;
@@ -41,5 +42,36 @@ size_t part_gemm_table_bytes(const PartGemm* jobs, int njobs);
 fira_status part_gemm_prepare(const PartGemm* jobs, int njobs, char* table_dev, size_t table_bytes, int* ntiles, cudaStream_t st);
 // One grouped launch over the prepared jobs.  a_parts, b_parts: the most parts that an operand of theirs has.
 fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, int a_parts, int b_parts, unsigned* status_dev, cudaStream_t st);
+
+// ---- the three products of the fp32-precision step, with their epilogues, for long lists: the projection (part_project.cu),
+// D = Pi R and D = Pi X (part_back.cu); R, X and Pi are kept as parts.
+struct PartStepPlan {
+  const char* table = nullptr;      // device; null: the list is short, its products split their operands themselves
+  const char* proj_table = nullptr;
+  int njobs = 0;
+  std::vector<int> proj_start;      // 256 x 128 tiles of R, prefix sums over the list
+  std::vector<unsigned char> jobs;  // host image of the table's first part: the norm's jobs, then the update's
+  std::vector<int> tile_start;      // 256 x 128 tiles of W, prefix sums over the list
+  int deep = 0;                     // some rank exceeds PART_STEP_RANK
+};
+constexpr int PART_STEP_RANK = 256, PART_STEP_MAX_RANK = 512;
+constexpr int PART_SUMS_PER_TILE = 16;   // partial sums of ||S||^2 that a tile leaves
+inline int part_rank_pitch(int r) { return (r + 7) / 8 * 8; }
+inline int part_step_tiles(int m, int n) { return ((m + 255) / 256) * ((n + 127) / 128); }
+inline int part_project_tiles(int l, int r) { return ((l + 255) / 256) * ((r + 127) / 128); }
+// Whether the projection's epilogue forms X (for limiter factor 1): the plain step of a matrix whose row sums are complete
+// in one tile.
+__host__ __device__ inline bool part_forms_x(int r, const Hyper& hp) { return r <= 128 && hp.mode == 0; }
+size_t part_project_table_bytes(int njobs, int ntiles);
+fira_status part_project_prepare(const std::vector<MatDev>& mats, const std::vector<int>& list, char* table_dev, PartStepPlan* plan, cudaStream_t st);
+fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, const Hyper& hp, unsigned* status_dev, cudaStream_t st);
+size_t part_step_table_bytes(int njobs, int ntiles);
+// mats: the host copies of the problem table, list: the indices of this engine's matrices in it.
+fira_status part_step_prepare(const std::vector<MatDev>& mats, const std::vector<int>& list, char* table_dev, PartStepPlan* plan, cudaStream_t st);
+// Called when W / G pointers changed.
+fira_status part_step_update_pointers(const std::vector<MatDev>& mats, const std::vector<int>& list, PartStepPlan* plan, cudaStream_t st);
+// The norm (update = 0) or the update of the matrices [qa, qb) of the list.
+fira_status part_step_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, int update, const Hyper& hp,
+                          unsigned* status_dev, cudaStream_t st);
 
 }  // namespace fira

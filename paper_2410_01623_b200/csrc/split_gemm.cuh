@@ -74,12 +74,19 @@ template <typename T> struct Frag;
 template <> struct Frag<float> { float v[8]; };
 template <> struct Frag<__nv_bfloat16> { uint4 u; };
 
+// All eight, from an aligned address, unconditionally: a load in a branch is waited for at the branch's end.
+__device__ __forceinline__ void load_frag(const float* p, Frag<float>& f) {
+  const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
+  f.v[0] = a.x; f.v[1] = a.y; f.v[2] = a.z; f.v[3] = a.w;
+  f.v[4] = b.x; f.v[5] = b.y; f.v[6] = b.z; f.v[7] = b.w;
+}
+__device__ __forceinline__ void load_frag(const __nv_bfloat16* p, Frag<__nv_bfloat16>& f) {
+  f.u = *reinterpret_cast<const uint4*>(p);
+}
 // n (>= 0) of the eight elements exist, the others are zeros.
 __device__ __forceinline__ void load_frag(const float* p, int n, bool vec, Frag<float>& f) {
   if (vec && n >= 8) {
-    const float4 a = *reinterpret_cast<const float4*>(p), b = *reinterpret_cast<const float4*>(p + 4);
-    f.v[0] = a.x; f.v[1] = a.y; f.v[2] = a.z; f.v[3] = a.w;
-    f.v[4] = b.x; f.v[5] = b.y; f.v[6] = b.z; f.v[7] = b.w;
+    load_frag(p, f);
   } else {
 #pragma unroll
     for (int e = 0; e < 8; ++e) f.v[e] = e < n ? p[e] : 0.f;
@@ -142,12 +149,21 @@ struct Operand {
     const int e = threadIdx.x + THREADS * u;
     if (along_x) { x = e % (TILE / 8) * 8; k = e / (TILE / 8); } else { k = e % (BK / 8) * 8; x = e / (BK / 8); }
   }
+  // Whether every slab's loads are whole aligned units; rows past the matrix then read its last ones again, for rows of the
+  // result that nobody looks at.
+  __device__ __forceinline__ bool regular() const { return vec && (!along_x || X % 8 == 0) && K % BK == 0; }
+  template <bool REGULAR>
   __device__ __forceinline__ void load(int k0) {
 #pragma unroll
     for (int u = 0; u < UNITS; ++u) {
       int x, k;
       coords(u, x, k);
       x += x0; k += k0;
+      if (REGULAR) {
+        x = min(x, along_x ? X - 8 : X - 1);
+        load_frag(base + (along_x ? (long long)k * ld + x : (long long)x * ld + k), f[u]);
+        continue;
+      }
       const int n = along_x ? (k < K ? X - x : 0) : (x < X ? K - k : 0);
       load_frag(base + (along_x ? (long long)k * ld + x : (long long)x * ld + k), n, vec, f[u]);
     }
@@ -182,9 +198,11 @@ struct CombinedOperand {
       c[u] = x0 + x < X ? c_ * factor[x0 + x] : 0.f;
     }
   }
+  __device__ __forceinline__ bool regular() const { return n.regular() && r.regular(); }
+  template <bool REGULAR>
   __device__ __forceinline__ void load(int k0) {
-    n.load(k0);
-    r.load(k0);
+    n.template load<REGULAR>(k0);
+    r.template load<REGULAR>(k0);
   }
   __device__ __forceinline__ void store(unsigned char* part) const {
 #pragma unroll
@@ -259,26 +277,16 @@ __device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, bool a_
   }
 }
 
-// The tile A B over k < K into shared memory, row x of A at C[x * C_LD]; ends with a block barrier.
-// cols: columns of the tile that are wanted (the others hold garbage).  C overlays the slabs.
-// Returns false if a wait ran out (bounded as in tc_ptx.cuh); all threads take the same path even then.
-template <bool LONG_K, class A, class B>
-__device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsigned char* slabs, Ctl* ctl) {
-  constexpr bool SMALL = A::PARTS > 1 || B::PARTS > 1;
-  const int n = (min(cols, TILE) + 15) / 16 * 16;
+// The slabs of tile_product: loads one slab ahead, splits, issues; sum: pieces of the main product.
+template <bool LONG_K, bool REGULAR, class A, class B>
+__device__ __forceinline__ void product_slabs(A& a, B& b, int K, int n, unsigned char* slabs, Ctl* ctl, float (&sum)[LONG_K ? TILE / 2 : 1]) {
   const int ns = (K + BK - 1) / BK;
-  const int warp = threadIdx.x >> 5;
+  const int warp = threadIdx.x >> 5, c0 = (warp >> 2) * (TILE / 2);
   const uint32_t tmem = ctl->tmem_base;
-  const uint32_t lane_col = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * (TILE / 2);
-  const int c0 = (warp >> 2) * (TILE / 2);      // this thread: row 32 (warp % 4) + lane, columns c0 .. c0 + 63
-  float sum[LONG_K ? TILE / 2 : 1];
-  if (LONG_K) {
-#pragma unroll
-    for (int i = 0; i < TILE / 2; ++i) sum[LONG_K ? i : 0] = 0.f;
-  }
+  const uint32_t lane_col = tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0;
   bool fresh = true;
-  a.load(0);
-  b.load(0);
+  a.template load<REGULAR>(0);
+  b.template load<REGULAR>(0);
   for (int s = 0; s < ns; ++s) {
     unsigned char* slab = slabs + (s % STAGES) * STAGE_BYTES;
     const uint32_t done = ptx::smem_u32(&ctl->done[s % STAGES]);
@@ -286,7 +294,9 @@ __device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsign
     a.store(slab);
     b.store(slab + OPERAND_BYTES);
     ptx::fence_proxy_async_smem();
-    if (s + 1 < ns) { a.load((s + 1) * BK); b.load((s + 1) * BK); }
+    const int next = min(s + 1, ns - 1) * BK;   // (the last slab once more, unused)
+    a.template load<REGULAR>(next);
+    b.template load<REGULAR>(next);
     ptx::tc_fence_before();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -312,6 +322,26 @@ __device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsign
       fresh = true;
     }
   }
+}
+
+// The tile A B over k < K into shared memory, row x of A at C[x * C_LD]; ends with a block barrier.
+// cols: columns of the tile that are wanted (the others hold garbage).  C overlays the slabs.
+// Returns false if a wait ran out (bounded as in tc_ptx.cuh); all threads take the same path even then.
+template <bool LONG_K, class A, class B>
+__device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsigned char* slabs, Ctl* ctl) {
+  constexpr bool SMALL = A::PARTS > 1 || B::PARTS > 1;
+  const int n = (min(cols, TILE) + 15) / 16 * 16;
+  const int ns = (K + BK - 1) / BK;
+  const int warp = threadIdx.x >> 5;
+  const uint32_t lane_col = ctl->tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (warp >> 2) * (TILE / 2);
+  const int c0 = (warp >> 2) * (TILE / 2);      // this thread: row 32 (warp % 4) + lane, columns c0 .. c0 + 63
+  float sum[LONG_K ? TILE / 2 : 1];
+  if (LONG_K) {
+#pragma unroll
+    for (int i = 0; i < TILE / 2; ++i) sum[LONG_K ? i : 0] = 0.f;
+  }
+  if (a.regular() && b.regular()) product_slabs<LONG_K, true>(a, b, K, n, slabs, ctl, sum);
+  else product_slabs<LONG_K, false>(a, b, K, n, slabs, ctl, sum);
   // all MMAs: the last commit covers the earlier ones; nobody overwrites the slabs before everybody has seen it
   const int last = ns - 1;
   const bool ok = ptx::mbar_wait(ptx::smem_u32(&ctl->done[last % STAGES]), (last / STAGES) & 1, &ctl->abort_flag);

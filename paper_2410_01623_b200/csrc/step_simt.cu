@@ -16,6 +16,7 @@
 // global memory runs along rows.
 //
 // Measured (56 fp32 matrices of 8 layers 512 / 1376, r = 128; one 512 x 1376 matrix): see each kernel.
+#include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
@@ -77,6 +78,34 @@ __device__ __forceinline__ void store_row(__nv_bfloat16* p, int lane, int n, con
     for (int c = 0; c < 4; ++c) if (lane + 32 * c < n) p[lane + 32 * c] = __float2bfloat16_rn(v[c]);
   }
 }
+// The row's entries as three bf16 parts, `stride` elements apart.
+template <bool VEC>
+__device__ __forceinline__ void store_row_parts(__nv_bfloat16* p, long long stride, int lane, int n, const float (&v)[4]) {
+  uint32_t a[3], b[3];                          // parts of entries 0, 1 and of 2, 3
+  split::split3(v[0], v[1], a[0], a[1], a[2]);
+  split::split3(v[2], v[3], b[0], b[1], b[2]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (VEC) {
+      if (4 * lane < n) *reinterpret_cast<uint2*>(p + i * stride + 4 * lane) = make_uint2(a[i], b[i]);
+    } else {
+      unsigned short* q = reinterpret_cast<unsigned short*>(p + i * stride) + lane;
+      if (lane < n) q[0] = (unsigned short)a[i];
+      if (lane + 32 < n) q[32] = (unsigned short)(a[i] >> 16);
+      if (lane + 64 < n) q[64] = (unsigned short)b[i];
+      if (lane + 96 < n) q[96] = (unsigned short)(b[i] >> 16);
+    }
+  }
+}
+template <bool VEC>
+__device__ __forceinline__ void load_row_parts(const __nv_bfloat16* p, long long stride, int lane, int n, float (&v)[4]) {
+  float h[4], m[4], l[4];
+  load_row<VEC>(p, lane, n, h);
+  load_row<VEC>(p + stride, lane, n, m);
+  load_row<VEC>(p + 2 * stride, lane, n, l);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) v[c] = h[c] + (m[c] + l[c]);        // exact: the number that was split
+}
 // n entries per row (a multiple of 4 from an aligned start, or any number), rows `pitch` entries apart
 template <typename T>
 __device__ __forceinline__ bool rows_vec(const T* base, long long pitch, int n) {
@@ -88,12 +117,12 @@ constexpr int WARP_ROWS = SIMT_TILE / (split::THREADS / 32);
 
 // ---------------------------------------------------------------- phase 1
 // Rows of the finished tile R: Adam (Eq. 2-4), N and R to scratch, row sums.
-template <bool VEC>
+template <int PSI, bool VEC>
 __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, const float* C, const Hyper& hp, float bias) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = min(SIMT_TILE, mt.r - j0);
   const int nrt = simt_tiles_dev(mt.r), q = j0 / SIMT_TILE;
-  const bool momentum = !(hp.mode & (HYPER_PSI_RMSPROP | HYPER_PSI_ADAGRAD));
+  constexpr bool momentum = PSI == PSI_ADAM;
   for (int x = 0; x < WARP_ROWS; x += ROWS_AT_ONCE) {
     float m[ROWS_AT_ONCE][4], v[ROWS_AT_ONCE][4];
 #pragma unroll
@@ -112,24 +141,18 @@ __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, cons
       load_row<VEC>(C + row * split::C_LD, lane, n, rv);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        if (hp.mode & HYPER_PSI_RMSPROP) {
-          v[y][c] = hp.beta2 * v[y][c] + (1.f - hp.beta2) * rv[c] * rv[c];
-          nv[c] = rv[c] / (sqrtf(v[y][c]) + hp.eps);
-        } else if (hp.mode & HYPER_PSI_ADAGRAD) {
-          v[y][c] = v[y][c] + rv[c] * rv[c];
-          nv[c] = rv[c] / (sqrtf(v[y][c]) + hp.eps);
-        } else {
-          m[y][c] = hp.beta1 * m[y][c] + (1.f - hp.beta1) * rv[c];
-          v[y][c] = hp.beta2 * v[y][c] + (1.f - hp.beta2) * rv[c] * rv[c];
-          nv[c] = bias * m[y][c] / (sqrtf(v[y][c]) + hp.eps);
-        }
+        nv[c] = adam_direction<PSI>(hp, bias, rv[c], m[y][c], v[y][c]);
         nn = fmaf(nv[c], nv[c], nn);            // (entries past the row's end are zeros throughout)
         rn = fmaf(rv[c], rv[c], rn);
       }
       if (momentum) store_row<VEC>(mt.M + at, lane, n, m[y]);
       store_row<VEC>(mt.V + at, lane, n, v[y]);
-      store_row<VEC>(mt.Xt + at, lane, n, nv);
-      store_row<VEC>(mt.Rt + at, lane, n, rv);
+      if (!mt.Rp) {
+        store_row<VEC>(mt.Xt + at, lane, n, nv);
+        store_row<VEC>(mt.Rt + at, lane, n, rv);
+      } else {                                  // a long list whose ranks TMA cannot address
+        store_row_parts<VEC>(mt.Rp + (long long)l * mt.rp_pitch + j0, (long long)mt.l * mt.rp_pitch, lane, n, rv);
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         nn += __shfl_xor_sync(0xffffffffu, nn, o);
@@ -152,6 +175,7 @@ __device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, u
   return split::tile_product<true>(a, b, mt.d, mt.r - j0, smem, ctl);
 }
 
+template <int PSI>
 __global__ void __launch_bounds__(split::THREADS, 2)
 k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
           const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
@@ -166,8 +190,8 @@ k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
   const bool ok = mt.bf16 ? project_tile<__nv_bfloat16>(mt, l0, j0, smem, ctl) : project_tile<float>(mt, l0, j0, smem, ctl);
   if (ok) {
     const float bias = mt.sc->pad;
-    if (mt.r % 4 == 0) adam_rows<true>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
-    else adam_rows<false>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
+    if (mt.r % 4 == 0) adam_rows<PSI, true>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
+    else adam_rows<PSI, false>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
   }
   split::end(ctl, status);
 }
@@ -175,20 +199,12 @@ k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
 // ---------------------------------------------------------------- phases 2 and 4
 enum { MODE_NORM = 0, MODE_UPDATE = 1 };
 
-// The factor k_l from the row sums, where more than one tile of R holds parts of the row.
-__device__ __forceinline__ float row_factor(const MatDev& mt, int l, const Hyper& hp) {
-  const int nrt = simt_tiles_dev(mt.r);
-  float nn = 0.f, rn = 0.f;
-  for (int q = 0; q < nrt; ++q) { nn += mt.aux[(long long)q * mt.l + l]; rn += mt.aux[(long long)(nrt + q) * mt.l + l]; }
-  return sqrtf(nn) / (sqrtf(rn) + hp.eps);
-}
-
 // ks[x] <- the factor of the tile's column (left) or row (right) x.  The first phase that asks makes them
 // from the row sums and leaves them in the k table for the phases that follow.
 template <int MODE>
 __device__ __forceinline__ void tile_factors(const MatDev& mt, int i0, int j0, int tile, const Hyper& hp, float* ks) {
   const bool ones = MODE == MODE_NORM && (hp.mode & (HYPER_NO_SCALING | HYPER_MATRIX_SCALING));
-  const bool from_sums = MODE == MODE_NORM && !ones && simt_tiles_dev(mt.r) > 1;
+  const bool from_sums = MODE == MODE_NORM && !ones && !factors_ready(mt, hp);
   if ((int)threadIdx.x < tile) {
     const int l = (mt.left ? j0 : i0) + threadIdx.x;
     float k = 0.f;
@@ -300,6 +316,71 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
   split::end(ctl, status);
 }
 
+// ---------------------------------------------------------------- long lists
+// X = a_low N - a_res lambda k_l R as parts, one warp per row l; N from the updated moments, by the arithmetic that the
+// projection's epilogue used.  (r % 4 != 0: scalar accesses.)
+template <int PSI, bool VEC>
+__device__ __forceinline__ void form_x_row(const MatDev& mt, int l, const Hyper& hp, float bias, float c) {
+  const int lane = threadIdx.x & 31;
+  const long long stride = (long long)mt.l * mt.rp_pitch, at = (long long)l * mt.rp_pitch;
+  for (int j = 0; j < mt.r; j += 128) {
+    const int n = min(128, mt.r - j);
+    float m[4], v[4], rv[4], x[4];
+    load_row<VEC>(mt.M + (long long)l * mt.r + j, lane, n, m);
+    load_row<VEC>(mt.V + (long long)l * mt.r + j, lane, n, v);
+    load_row_parts<VEC>(mt.Rp + at + j, stride, lane, n, rv);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = hp.a_low * direction<PSI>(hp, bias, rv[q], m[q], v[q]) - c * rv[q];
+    store_row_parts<VEC>(mt.Xp + at + j, stride, lane, n, x);
+  }
+}
+constexpr int FORM_X_ROWS = 4;                  // per warp: what it costs to find the matrix is shared
+template <int PSI>
+__global__ void __launch_bounds__(256)
+k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist, const int* __restrict__ row_start, int first_row,
+         int rows_end, Hyper hp) {
+  int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * FORM_X_ROWS;
+  if (row >= rows_end) return;
+  int p = find_matrix(row_start, nlist, row);
+  const int end = min(row + FORM_X_ROWS, rows_end);
+  while (row < end) {
+    const MatDev& mt = mats[list[p]];
+    const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
+    const float lambda = mt.sc->lambda, c = hp.a_res * lambda, bias = *mt.step_bias;
+    if (mt.tma_proj && part_forms_x(mt.r, hp) && lambda == 1.f) {
+      // the projection's epilogue has formed it
+    } else if (mt.r % 4 == 0) {
+#pragma unroll 2
+      for (int l = l0; l < l1; ++l) form_x_row<PSI, true>(mt, l, hp, bias, c * mt.kvec[l]);
+    } else {
+      for (int l = l0; l < l1; ++l) form_x_row<PSI, false>(mt, l, hp, bias, c * mt.kvec[l]);
+    }
+    row += l1 - l0;
+    ++p;
+  }
+}
+
+// The projection's parts, eight neighbours per thread (blockIdx.y = matrix of the list).
+__global__ void __launch_bounds__(256)
+k_split_projection(const MatDev* __restrict__ mats, const int* __restrict__ list) {
+  const MatDev& mt = mats[list[blockIdx.y]];
+  const long long per_row = mt.pp_pitch / 8, units = mt.d * per_row, stride = 2ll * mt.d * mt.pp_pitch;
+  const bool vec = mt.r % 8 == 0;
+  for (long long u = blockIdx.x * 256ll + threadIdx.x; u < units; u += gridDim.x * 256ll) {
+    const long long i = u / per_row, j = u % per_row * 8;
+    unsigned char* out = reinterpret_cast<unsigned char*>(mt.Pp + i * mt.pp_pitch + j);
+    if (mt.bf16) {
+      split::Frag<__nv_bfloat16> f;
+      split::load_frag(static_cast<const __nv_bfloat16*>(mt.P) + i * mt.r + j, (int)(mt.r - j), vec, f);
+      split::store_parts(out, f);
+    } else {
+      split::Frag<float> f;
+      split::load_frag(static_cast<const float*>(mt.P) + i * mt.r + j, (int)(mt.r - j), vec, f);
+      split::store_parts(out, f, stride);
+    }
+  }
+}
+
 // ---------------------------------------------------------------- Fira-only-scaling
 // W <- W - lr phi(R) G: no product.  One block per tile x tile elements of W, a warp per row.
 template <typename T, int UPDATE, bool VEC>
@@ -395,7 +476,10 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   const MatDev mt = mats[list[blockIdx.x]];
   const int npart = npart_of[blockIdx.x];
   // the bias factor sqrt(1 - b2^s) / (1 - b1^s) of the NEXT step, in double, while the others add up
-  if (threadIdx.x == 255) mt.sc->pad = bias_factor(hp.beta1, hp.beta2, mt.sc->t + 2);
+  if (threadIdx.x == 255) {
+    if (mt.step_bias) *mt.step_bias = mt.sc->pad;
+    mt.sc->pad = bias_factor(hp.beta1, hp.beta2, mt.sc->t + 2);
+  }
   double acc = 0.0;
   for (int i = threadIdx.x; i < npart; i += 256) acc += (double)mt.part[i];
   // Matrix-level factor (Eq. 9): the phases before ran with k = 1, so `part` holds ||G - P R||^2;
@@ -404,7 +488,7 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   if (hp.mode & HYPER_MATRIX_SCALING) {
     __shared__ double sn[256], sr[256];
     double an = 0.0, ar = 0.0;
-    const long long sums = (long long)(mt.engine == 0 ? (mt.r + SIMT_TILE - 1) / SIMT_TILE : 1) * mt.l;   // one or more per row
+    const long long sums = (long long)mt.aux_slots * mt.l;
     for (long long i = threadIdx.x; i < sums; i += 256) { an += (double)mt.aux[i]; ar += (double)mt.aux[sums + i]; }
     sn[threadIdx.x] = an; sr[threadIdx.x] = ar;
     __syncthreads();
@@ -458,7 +542,25 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   }
 }
 
-const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_back_project<norm>", "k_finalize", "k_back_project<update>"};
+const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"};
+
+// Measured below.
+constexpr long long LONG_LIST_TILES = 256;
+bool simt_long_list(const std::vector<fira_matrix_desc>& list) {
+  long long tiles = 0;
+  for (const fira_matrix_desc& d : list) {
+    if (d.r > PART_STEP_MAX_RANK) return false;
+    tiles += (long long)simt_tiles(d.m) * simt_tiles(d.n);
+  }
+  return tiles >= LONG_LIST_TILES;
+}
+
+void launch_split_projections(const SimtPlan& pl, const std::vector<MatDev>& mats, const std::vector<int>& list, cudaStream_t st) {
+  if (!pl.parts.table) return;
+  long long units = 1;
+  for (int i : list) units = std::max(units, (long long)mats[i].d * mats[i].pp_pitch / 8);
+  k_split_projection<<<dim3((unsigned)std::min<long long>(64, (units + 255) / 256), (unsigned)list.size()), 256, 0, st>>>(pl.mats, pl.list);
+}
 
 // The products' shared memory is above the default limit: a per-device, per-kernel setting.
 static bool allow_smem() {
@@ -467,7 +569,7 @@ static bool allow_smem() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && !done[dev].load()) {
-    const void* kernels[3] = {(const void*)k_project, (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
+    const void* kernels[5] = {(const void*)k_project<PSI_ADAM>, (const void*)k_project<PSI_RMSPROP>, (const void*)k_project<PSI_ADAGRAD>, (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
     for (const void* k : kernels)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
     if (e == cudaSuccess) done[dev].store(true);
@@ -493,22 +595,43 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   }
   constexpr int TH = split::THREADS, SM = split::SMEM_BYTES;
   const bool only_scaling = hp.mode & HYPER_ONLY_SCALING;     // W <- W - lr phi(R) G: no back-projection
+  const bool parts = pl.parts.table && !only_scaling;          // (a long list's only-scaling step has no back-projection)
+  const int psi = psi_of(hp);
+  const int qe = qb >= 0 ? qb : pl.nlist;
+  const int s0 = pl.parts.table ? pl.h_stage_start[pl.h_stage_pos[qa]] : 0;
+  const int staged = pl.parts.table ? pl.h_stage_start[pl.h_stage_pos[qe]] - s0 : 0, nstage = pl.parts.table ? pl.h_stage_pos.back() : 0;
   tm->mark(st);
-  k_project<<<pt1 - pt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.proj_tile_start, pt0, hp, status_dev);
+  launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 0, st);
+  if (pl.parts.proj_table) {           // (also before only-scaling, which needs the row sums)
+    if (part_project_run(pl.parts, pl.mats, qa, qe, hp, status_dev, st) != FIRA_OK) return -1;
+  } else
+    (psi == PSI_ADAM ? k_project<PSI_ADAM> : psi == PSI_RMSPROP ? k_project<PSI_RMSPROP> : k_project<PSI_ADAGRAD>)
+        <<<pt1 - pt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.proj_tile_start, pt0, hp, status_dev);
   tm->mark(st);
   if (only_scaling)
     launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 0, hp, st);
-  else
+  else if (parts) {
+    if (part_step_run(pl.parts, pl.mats, qa, qe, 0, hp, status_dev, st) != FIRA_OK) return -1;
+  } else
     k_back_project<MODE_NORM><<<wt1 - wt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev);
   tm->mark(st);
-  k_finalize<<<nq, 256, 0, st>>>(pl.mats, pl.list + qa, nq, pl.npart + qa, hp, status_dev);
+  // (only-scaling leaves one partial sum per 128 x 128 tile whatever the list)
+  k_finalize<<<nq, 256, 0, st>>>(pl.mats, pl.list + qa, nq, (only_scaling ? pl.npart_tiles : pl.npart) + qa, hp, status_dev);
+  tm->mark(st);
+  if (parts) {
+    const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
+    (psi == PSI_ADAM ? k_form_x<PSI_ADAM> : psi == PSI_RMSPROP ? k_form_x<PSI_RMSPROP> : k_form_x<PSI_ADAGRAD>)<<<(r1 - r0 + 8 * FORM_X_ROWS - 1) / (8 * FORM_X_ROWS), 256, 0, st>>>(pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp);
+  }
   tm->mark(st);
   if (only_scaling)
     launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 1, hp, st);
-  else
+  else if (parts) {
+    if (part_step_run(pl.parts, pl.mats, qa, qe, 1, hp, status_dev, st) != FIRA_OK) return -1;
+    launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 1, st);
+  } else
     k_back_project<MODE_UPDATE><<<wt1 - wt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev);
   tm->mark(st);
-  return 4;
+  return 4 + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
 }
 
 }  // namespace fira

@@ -1,12 +1,39 @@
 // Launch interface of the grouped step kernels that work in fp32 precision (any size, type and pitch).
 #pragma once
 #include "common.cuh"
+#include "part_gemm.cuh"
 
 namespace fira {
 
 constexpr int SIMT_TILE = 128;              // tiles of R (l x r) and of W (m x n)
 inline int simt_tiles(long long extent) { return (int)((extent + SIMT_TILE - 1) / SIMT_TILE); }
-constexpr int SIMT_PHASES = 4;
+constexpr int SIMT_PHASES = 5;
+
+// The factor k_l from the row sums.
+__device__ __forceinline__ float row_factor(const MatDev& mt, int l, const Hyper& hp) {
+  float nn = 0.f, rn = 0.f;
+  for (int q = 0; q < mt.aux_slots; ++q) { nn += mt.aux[(long long)q * mt.l + l]; rn += mt.aux[(long long)(mt.aux_slots + q) * mt.l + l]; }
+  return sqrtf(nn) / (sqrtf(rn) + hp.eps);
+}
+
+// Whether the projection's epilogue has made the factors k_l itself: the row sums were complete in one tile.
+__device__ __forceinline__ bool factors_ready(const MatDev& mt, const Hyper& hp) {
+  return mt.tma_proj ? part_forms_x(mt.r, hp) : mt.r <= SIMT_TILE;
+}
+
+inline int psi_of(const Hyper& hp) { return hp.mode & HYPER_PSI_RMSPROP ? PSI_RMSPROP : hp.mode & HYPER_PSI_ADAGRAD ? PSI_ADAGRAD : PSI_ADAM; }
+// The direction N of one entry (Eq. 4, or the other base optimizer's) from its updated moments.
+template <int PSI>
+__device__ __forceinline__ float direction(const Hyper& hp, float bias, float r, float m, float v) {
+  return (PSI == PSI_ADAM ? bias * m : r) / (sqrtf(v) + hp.eps);
+}
+// Updates the moments of one entry (Eq. 2-3; M is left alone by RMSProp and Adagrad) and returns N.
+template <int PSI>
+__device__ __forceinline__ float adam_direction(const Hyper& hp, float bias, float r, float& m, float& v) {
+  v = PSI == PSI_ADAGRAD ? v + r * r : hp.beta2 * v + (1.f - hp.beta2) * r * r;
+  if (PSI == PSI_ADAM) m = hp.beta1 * m + (1.f - hp.beta1) * r;
+  return direction<PSI>(hp, bias, r, m, v);
+}
 
 // Device-resident schedule of one list of matrices.  `list` holds indices into
 // `mats`; the *_start arrays have nlist + 1 ascending entries (prefix sums).
@@ -18,11 +45,26 @@ struct SimtPlan {
   int proj_tiles = 0;
   const int* w_tile_start = nullptr;     // 128 x 128 tiles of W (m x n)
   int w_tiles = 0;
-  const int* npart = nullptr;            // partial sums per matrix (= its W tiles)
+  const int* npart = nullptr;            // partial sums of ||S||^2 per matrix
+  const int* row_start = nullptr;        // rows l (long lists)
+  const int* npart_tiles = nullptr;      // the same where there is one per 128 x 128 tile of W
+  PartStepPlan parts;                    // long lists: the products with the projection
+  std::vector<int> h_row_start;
+  // long lists: the matrices whose rows TMA cannot address; their G and W are worked on as copies with an aligned pitch
+  const int* stage_list = nullptr;
+  const int* stage_start = nullptr;      // rows m
+  std::vector<int> h_stage_pos, h_stage_start;   // staged matrices among the first q of the list; their rows
   // host copies of the two prefix arrays (needed only to step a sub-range of the list)
   std::vector<int> h_proj_tile_start, h_w_tile_start;
 };
 
+// Whether a list of these matrices (the ones of this engine) is long: its products with the projection then run on
+// parts (part_gemm.cu), which R, X and the projection are kept as.
+bool simt_long_list(const std::vector<fira_matrix_desc>& list);
+// Copies rows of staged matrices (MatDev Gs, Ws): dir 0 G and W in, 1 W out (step_tc.cu).
+void launch_stage(const MatDev* mats, const int* list, int nlist, const int* row_start, int first_row, int rows, int dir, cudaStream_t st);
+// Splits the stored projections into parts; to be called after they have changed.
+void launch_split_projections(const SimtPlan& pl, const std::vector<MatDev>& mats, const std::vector<int>& list, cudaStream_t st);
 // Enqueues the phases for the matrices [qa, qb) of the list (qb < 0: the whole list); returns
 // the number of launches (negative: error, message set).  MatScalars::pad has to hold the bias factor of
 // the step (bias_factor).

@@ -206,15 +206,17 @@ k_tc_stage(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   const int p = find_matrix(row_start, nlist, gr);
   const MatDev& mt = mats[list[p]];
   const long long i = gr - row_start[p];
-  const unsigned short* g = static_cast<const unsigned short*>(mt.G) + i * mt.ld;
-  unsigned short* w = static_cast<unsigned short*>(mt.W) + i * mt.ld;
-  unsigned short* gs = reinterpret_cast<unsigned short*>(mt.Gs) + i * mt.lds;
-  unsigned short* ws = reinterpret_cast<unsigned short*>(mt.Ws) + i * mt.lds;
+  const int w2 = mt.bf16 ? 1 : 2;                // an fp32 element is two of the two-byte units that move here
+  const int n = mt.n * w2;
+  const unsigned short* g = static_cast<const unsigned short*>(mt.G) + i * mt.ld * w2;
+  unsigned short* w = static_cast<unsigned short*>(mt.W) + i * mt.ld * w2;
+  unsigned short* gs = reinterpret_cast<unsigned short*>(mt.Gs) + i * mt.lds * w2;
+  unsigned short* ws = reinterpret_cast<unsigned short*>(mt.Ws) + i * mt.lds * w2;
   if (dir == 0) {
-    copy_row_to_aligned(gs, g, mt.n, i == 0);
-    copy_row_to_aligned(ws, w, mt.n, i == 0);
+    copy_row_to_aligned(gs, g, n, i == 0);
+    copy_row_to_aligned(ws, w, n, i == 0);
   } else {
-    copy_row_from_aligned(w, ws, mt.n, (int)mt.lds);
+    copy_row_from_aligned(w, ws, n, (int)mt.lds * w2);
   }
 }
 
@@ -392,10 +394,14 @@ bool encode_tiled(CUtensorMap* out, const void* base, bool fp32, int rank, const
   for (int i = 0; i < rank; ++i) { dims[i] = extent[i]; boxes[i] = box[i]; if (i) strides[i - 1] = stride_bytes[i - 1]; }
   const CUresult r = fn(out, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank,
                         const_cast<void*>(base), dims, strides, boxes, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                        swizzle_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled failed with code " + std::to_string((int)r)); return false; }
   return true;
+}
+
+void launch_stage(const MatDev* mats, const int* list, int nlist, const int* row_start, int first_row, int rows, int dir, cudaStream_t st) {
+  if (rows > 0) k_tc_stage<<<rows, 256, 0, st>>>(mats, list, nlist, row_start, first_row, dir);
 }
 
 struct TcPlan {
@@ -778,7 +784,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     k_tc_proj_weights<<<pl->wq_blocks, 256, 0, st>>>(mats, pl->list, pl->wq_off, pl->wq_blk, pl->nlist, pl->wq_dev);
     c->proj_weights_dirty = false;
   }
-  if (srn) k_tc_stage<<<srn, 256, 0, st>>>(mats, pl->stage_list, pl->nstage, pl->stage_start, sra, 0);
+  launch_stage(mats, pl->stage_list, pl->nstage, pl->stage_start, sra, srn, 0, st);
   tm->mark(st);
   k_tc_prep<<<nq, 32, 0, st>>>(mats, pl->list, qa, hp, pl->fast_dev);
   tm->mark(st);
@@ -842,7 +848,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     k_tc_back_project<4, 3><<<2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(4, 3), st>>>(
         pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev);
   tm->mark(st);
-  if (srn) k_tc_stage<<<srn, 256, 0, st>>>(mats, pl->stage_list, pl->nstage, pl->stage_start, sra, 1);
+  launch_stage(mats, pl->stage_list, pl->nstage, pl->stage_start, sra, srn, 1, st);
   tm->mark(st);
   return (srn ? 7 : 5) + (any_plain ? 1 : 0) + (any_fused ? 1 : 0);
 }

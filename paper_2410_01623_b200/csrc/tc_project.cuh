@@ -165,7 +165,6 @@ __device__ __forceinline__ ProjTileDesc load_desc(const ProjTileDesc* __restrict
 enum { EPI_ADAM = 0, EPI_PLAIN = 1 };
 // PSI: the base optimizer of the EPI_ADAM epilogue (0 Adam, Eq. 2-4; 1 RMSProp; 2 Adagrad: M is then
 // carried through unchanged).
-enum { PSI_ADAM = 0, PSI_RMSPROP = 1, PSI_ADAGRAD = 2 };
 
 template <int EPI, int PSI, int FUSE_X, int EG = 1>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(k1_threads(EG), 1)
