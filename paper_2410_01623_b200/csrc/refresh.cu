@@ -353,12 +353,14 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
   cudaStream_t st = tg.stream;
   size_t pos = 0;
   while (pos < which.size()) {
-    // ---- carve a chunk: as many matrices as fit (data regions first, then tables)
+    // ---- carve a chunk: as many matrices as fit (data regions first, then the tables of all)
     std::vector<size_t> offs;
-    size_t off = 0, q = pos;
+    size_t need = 0, off = 0, q = pos;
     for (; q < which.size(); ++q) {
-      const size_t data = refresh_data_bytes(c->descs[which[q]]);
-      if (off + data + (q - pos + 1) * TABLE_PER_MATRIX + TABLE_SLACK > tg.work_bytes) break;
+      size_t data = 0;
+      carve_refresh(c->descs[which[q]], nullptr, &data);
+      need += refresh_data_bytes(c->descs[which[q]]) + TABLE_PER_MATRIX;
+      if (need + TABLE_SLACK > tg.work_bytes) break;
       offs.push_back(off);
       off += data;
     }
