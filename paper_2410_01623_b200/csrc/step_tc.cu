@@ -13,7 +13,7 @@
 //   k_tc_form_x        X = a_low N - a_res lambda k_l R  (bf16).  In the plain step the projection
 //                      epilogue has written X for lambda = 1 already (see tc_project.cuh) and this
 //                      kernel only touches the matrices whose limiter acted (k_tc_fix_x):
-//                      X <- lambda X + (1 - lambda) a_low N, N rebuilt from the stored moments
+//                      X <- X + (1 - lambda) a_res k_l R, or the same with N from the stored moments
 //   k_tc_back_project  D = Pi X on the tensor cores; epilogue: W -= lr (D + a_res lambda k_l G)
 //
 // ||S_l||^2 = ||G_l - Pi R_l||^2 = ||G_l||^2 - 2 ||R_l||^2 + R_l^T (Pi^T Pi) R_l.  For orthonormal
@@ -288,12 +288,13 @@ k_tc_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int n
 }
 
 // The matrices whose X the projection epilogue has formed for lambda = 1 (FUSE_X): where the limiter
-// acted, X_lambda = a_low N - a_res lambda k_l R = lambda X + (1 - lambda) a_low N, with N rebuilt
-// from the moments that the epilogue stored, by the epilogue's own arithmetic and rounded to bf16
-// as it was there; the other matrices are left as they are.  blockIdx.y = matrix of the range, the
-// blocks of a matrix stride over its rows, one warp per row.
+// acted, X_lambda = a_low N - a_res lambda k_l R is X + (1 - lambda) a_res k_l R if the projection kept R (FUSE_X = 2), otherwise
+// lambda X + (1 - lambda) a_low N with N rebuilt from the moments that the epilogue stored, by the epilogue's
+// own arithmetic and rounded to bf16 as it was there; the other matrices are left as they are.
+// blockIdx.y = matrix of the range, the blocks of a matrix stride over its rows, one warp per row.  Bound by
+// memory.
 __global__ void __launch_bounds__(256)
-k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int first, float a_low, float eps,
+k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int first, float a_low, float a_res, float eps, int kept,
            float* __restrict__ fast) {
   const int p = first + blockIdx.y;
   const MatDev& mt = mats[list[p]];
@@ -303,9 +304,24 @@ k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int fi
   if (lambda == 1.f) return;
   const int lane = threadIdx.x & 31;
   const float bias = fast[2 * p];                      // this step's bias factor (k_tc_prep)
-  const float cn = (1.f - lambda) * a_low;
+  const float cn = (1.f - lambda) * a_low, cr = (1.f - lambda) * a_res;
   for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < mt.l; l += gridDim.x * 8) {
     const long long base = (long long)l * mt.r;
+    if (kept) {
+      const float c = cr * mt.kvec[l];
+#pragma unroll 2
+      for (int j = lane * 8; j < mt.r; j += 256) {
+        const uint4 xu = *reinterpret_cast<const uint4*>(mt.Xb + base + j);
+        const uint4 ru = *reinterpret_cast<const uint4*>(mt.Rb + base + j);
+        float xv[8], rv[8];
+        unpack8_bf16(xu, xv);
+        unpack8_bf16(ru, rv);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) xv[e] = fmaf(c, rv[e], xv[e]);
+        *reinterpret_cast<uint4*>(mt.Xb + base + j) = pack8_bf16(xv);
+      }
+      continue;
+    }
     for (int j = lane * 8; j < mt.r; j += 256) {
       const uint4 xu = *reinterpret_cast<const uint4*>(mt.Xb + base + j);
       const float4 m0 = *reinterpret_cast<const float4*>(mt.M + base + j), m1 = *reinterpret_cast<const float4*>(mt.M + base + j + 4);
@@ -721,13 +737,15 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   if (!pl || pl->nlist == 0) return 0;
   cudaStream_t st = c->stream;
   if (!pl->attrs_set) {
-    const void* k1s[4] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0>, (const void*)k_tc_project<EPI_ADAM, PSI_RMSPROP, 0>,
-                          (const void*)k_tc_project<EPI_ADAM, PSI_ADAGRAD, 0>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1>};
-    const void* k1g[2] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0, 2>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1, 2>};
+    const void* k1s[5] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0>, (const void*)k_tc_project<EPI_ADAM, PSI_RMSPROP, 0>,
+                          (const void*)k_tc_project<EPI_ADAM, PSI_ADAGRAD, 0>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1>,
+                          (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 2>};
+    const void* k1g[3] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0, 2>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1, 2>,
+                          (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 2, 2>};
     cudaError_t e1 = cudaSuccess;
-    for (int i = 0; i < 4 && e1 == cudaSuccess; ++i)
+    for (int i = 0; i < 5 && e1 == cudaSuccess; ++i)
       e1 = cudaFuncSetAttribute(k1s[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K1_SMEM_BYTES);
-    for (int i = 0; i < 2 && e1 == cudaSuccess; ++i)
+    for (int i = 0; i < 3 && e1 == cudaSuccess; ++i)
       e1 = cudaFuncSetAttribute(k1g[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k1_smem_bytes(2));
     cudaError_t e2 = cudaFuncSetAttribute(k_tc_back_project<5, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k2_smem_bytes(5, 2));
     if (e2 == cudaSuccess)
@@ -746,14 +764,14 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
       at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
       cfg.attrs = at; cfg.numAttrs = 1;
       int nclusters = 0;
-      const cudaError_t e3 = cudaOccupancyMaxActiveClusters(&nclusters, k1s[3], &cfg);
+      const cudaError_t e3 = cudaOccupancyMaxActiveClusters(&nclusters, k1s[4], &cfg);
       if (e3 != cudaSuccess || nclusters <= 0) {
         set_error(std::string("cudaOccupancyMaxActiveClusters: ") + cudaGetErrorString(e3));
         return -1;
       }
       pl->max_pairs_fused = std::min(nclusters, pl->num_sms / 2);
       cfg.blockDim = dim3(k1_threads(2)); cfg.dynamicSmemBytes = k1_smem_bytes(2);
-      const cudaError_t e4 = cudaOccupancyMaxActiveClusters(&nclusters, k1g[1], &cfg);
+      const cudaError_t e4 = cudaOccupancyMaxActiveClusters(&nclusters, k1g[2], &cfg);
       if (e4 != cudaSuccess || nclusters <= 0) {
         set_error(std::string("cudaOccupancyMaxActiveClusters: ") + cudaGetErrorString(e4));
         return -1;
@@ -799,21 +817,24 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   // Short products are bound by the epilogue, which then runs with two groups of warps per CTA; long
   // ones (r = 1024 lists) are bound by the tensor pipe and keep one.
   const bool two_groups = rmax <= 512;
-#define FIRA_LAUNCH_K1(PSI, FUSE)                                                     \
-  k_tc_project<EPI_ADAM, PSI, FUSE><<<k1_grid, K1_THREADS, K1_SMEM_BYTES, st>>>(      \
-      pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev)
-  if (hp.mode & HYPER_PSI_RMSPROP) FIRA_LAUNCH_K1(PSI_RMSPROP, 0);
-  else if (hp.mode & HYPER_PSI_ADAGRAD) FIRA_LAUNCH_K1(PSI_ADAGRAD, 0);
-  else if (two_groups) {
-    if (fused)
-      k_tc_project<EPI_ADAM, PSI_ADAM, 1, 2><<<k1_grid, k1_threads(2), k1_smem_bytes(2), st>>>(
-          pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev);
-    else
-      k_tc_project<EPI_ADAM, PSI_ADAM, 0, 2><<<k1_grid, k1_threads(2), k1_smem_bytes(2), st>>>(
-          pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev);
+  bool keep_r = fused;
+  for (int q = qa; q < qb; ++q) {
+    const MatDev& mq = c->mats[c->tc_list[q]];
+    if (fuse_x_matrix(mq.d, mq.r) && mq.d < FUSE_KEEP_R_MIN_D) keep_r = false;
   }
-  else if (fused) FIRA_LAUNCH_K1(PSI_ADAM, 1);
-  else FIRA_LAUNCH_K1(PSI_ADAM, 0);
+#define FIRA_LAUNCH_K1(PSI, FUSE, EG)                                                                       \
+  k_tc_project<EPI_ADAM, PSI, FUSE, EG><<<k1_grid, k1_threads(EG), k1_smem_bytes(EG), st>>>(                 \
+      pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev)
+  if (hp.mode & HYPER_PSI_RMSPROP) FIRA_LAUNCH_K1(PSI_RMSPROP, 0, 1);
+  else if (hp.mode & HYPER_PSI_ADAGRAD) FIRA_LAUNCH_K1(PSI_ADAGRAD, 0, 1);
+  else if (two_groups) {
+    if (keep_r) FIRA_LAUNCH_K1(PSI_ADAM, 2, 2);
+    else if (fused) FIRA_LAUNCH_K1(PSI_ADAM, 1, 2);
+    else FIRA_LAUNCH_K1(PSI_ADAM, 0, 2);
+  }
+  else if (keep_r) FIRA_LAUNCH_K1(PSI_ADAM, 2, 1);
+  else if (fused) FIRA_LAUNCH_K1(PSI_ADAM, 1, 1);
+  else FIRA_LAUNCH_K1(PSI_ADAM, 0, 1);
 #undef FIRA_LAUNCH_K1
   tm->mark(st);
   k_tc_colfactors<<<csn, 256, 0, st>>>(mats, pl->list, pl->nlist, pl->col_start, csa, hp);
@@ -838,7 +859,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   if (any_plain)
     k_tc_form_x<<<(rsb - rsa + 7) / 8, 256, 0, st>>>(mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
                                                      hp.a_low, hp.a_res, pl->fast_dev, fused ? 1 : 0);
-  if (any_fused) k_tc_fix_x<<<dim3(16, nq), 256, 0, st>>>(mats, pl->list, qa, hp.a_low, hp.eps, pl->fast_dev);
+  if (any_fused) k_tc_fix_x<<<dim3(32, nq), 256, 0, st>>>(mats, pl->list, qa, hp.a_low, hp.a_res, hp.eps, keep_r ? 1 : 0, pl->fast_dev);
   tm->mark(st);
   // long products keep five operand stages; short ones trade one for more epilogue boxes in flight
   if (rmax >= 1024)

@@ -57,9 +57,12 @@
 // follows, on its pair, a tile far below it, so the waits cannot form a cycle as long as every block
 // of the grid is resident, which the launch ensures), the thread adds the partial sums in the fixed
 // order that k_tc_colfactors uses, and sweep 2 reads the pairs back and writes X (through the map of
-// the X buffer).  Nothing else leaves the kernel: where the limiter acts, k_tc_fix_x rebuilds N from
-// the stored moments, X_lambda = lambda X + (1 - lambda) a_low N.  (Adam only: with RMSProp or Adagrad
-// N cannot be rebuilt from V alone, and those steps keep the separate pass.)
+// the X buffer).  Where the limiter acts, k_tc_fix_x puts X right afterwards.  FUSE_X = 2 (lists of long products, see
+// FUSE_KEEP_R_MIN_D) leaves R for it, written in sweep 1, and it makes X_lambda = X + (1 - lambda) a_res k_l R,
+// 6 bytes per element; after FUSE_X = 1 it rebuilds N from the stored moments, X_lambda = lambda X + (1 - lambda) a_low N,
+// 12 bytes per element.
+// (Adam only: with RMSProp or Adagrad N cannot be rebuilt from V alone, and those steps keep the
+// separate pass.)
 constexpr int K1_STAGES = 4;
 constexpr int K1_STAGE_BYTES = 2 * A_STAGE_BYTES;       // A: 128 l x 64 d, B half: 128 r x 64 d
 constexpr int K1_ECOLS = 32;                            // columns per epilogue box
@@ -109,6 +112,11 @@ constexpr int PROJ_OUT_BF16 = 1 << 28, PROJ_OUT_REMAINDER = 1 << 27;
 // not been measured and keep the separate pass.
 constexpr int FUSE_X_MIN_D = 2048;
 __host__ __device__ inline bool fuse_x_matrix(int d, int r) { return d >= FUSE_X_MIN_D || r <= 256; }
+// R's boxes cost the epilogue a store, a wait and 2 bytes per element on every step, its absence 6 bytes per element of
+// the matrices whose limiter acts: half of them and more, since the remembered norm is the limited one.  Under a long
+// product the epilogue has the time.  Measured on the step, limiter acting: 1B list (d = 2048) -4 %, 7B list (d = 4096)
+// -4 %; 350M list (d = 1024), whose epilogue is its critical path, +3 %.
+constexpr int FUSE_KEEP_R_MIN_D = 2048;
 
 // EPI_PLAIN products may run over up to three k-segments that accumulate into the same tile: segment
 // s multiplies A taken through the map g1a (bit s of asel clear) or g2a (set) with B taken through
@@ -439,7 +447,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
         const TcMaps* mp = &maps[d.slot];
         const int bn = d.bn_left & 0xffff;
         const int l0 = d.l0 + BM * (int)rank;
-        const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X);
+        const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_r = FUSE_X == 2 && fuse;
         for (int b = 0; b < 2 * (bn / K1_ECOLS); ++b) {
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->eready[mv]), mvphase, abort_flag)) { ok = false; break; }
           const int nr = b & 1;
@@ -449,7 +457,9 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
             if (EPI == EPI_ADAM) {
               ptx::tma_store_2d(&mp->em, src, j, row);
               ptx::tma_store_2d(&mp->ev, src + K1_FBOX_BYTES, j, row);
-              if (!fuse) {
+              if (keep_r) {
+                ptx::tma_store_2d(&mp->er, srn + ((b >> 1) & 1) * K1_HBOX_BYTES, j, row);
+              } else if (!fuse) {
                 ptx::tma_store_2d(&mp->en, srn, j, row);
                 ptx::tma_store_2d(&mp->er, srn + K1_HBOX_BYTES, j, row);
               }
@@ -463,7 +473,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
             ptx::bulk_wait_group_read<0>();              // the boxes have been read: the buffers are free
           }
           ptx::mbar_arrive(ptx::smem_u32(&ctl->eempty[mv]));
-          if (!fuse) ptx::mbar_arrive(ptx::smem_u32(&ctl->nrempty[nr]));
+          if (keep_r || !fuse) ptx::mbar_arrive(ptx::smem_u32(keep_r ? &ctl->xempty[nr][(b >> 1) & 1] : &ctl->nrempty[nr]));
           if (++mv == K1_MVBUFS) { mv = 0; mvphase ^= 1u; }
         }
         if (fuse && ok) {
@@ -527,7 +537,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
       const uint32_t tcol = tmem + ((uint32_t)(quarter * 32) << 16) + buf * BN_MAX;
       const uint32_t te = buf ? tmem_empty1 : tmem_empty0;
       const int nch = bn / K1_ECOLS;
-      const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X);
+      const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_r = FUSE_X == 2 && fuse;
       float nn = 0.f, rn = 0.f, rw = 0.f;
       for (int c = 0; c < nch; ++c) {
         uint32_t rr[GC];
@@ -543,7 +553,12 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
           if (lane == 0) ptx::mbar_arrive_cluster(te);
         }
         if (EPI == EPI_ADAM && !ptx::mbar_wait(ptx::smem_u32(&ctl->efull[mv][half]), mvphase, abort_flag)) { ok = false; break; }
-        if (!fuse && !ptx::mbar_wait(nrempty, nrphase ^ 1u, abort_flag)) { ok = false; break; }
+        const int xs = c & 1;                            // fuse: R boxes, then X boxes alternate between the two parts of the buffer
+        if (keep_r) {
+          if (!ptx::mbar_wait(ptx::smem_u32(&ctl->xempty[half][xs]), ((xeph >> xs) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          xeph ^= 1u << xs;
+        }
+        if ((!fuse || c == 0) && !ptx::mbar_wait(nrempty, nrphase ^ 1u, abort_flag)) { ok = false; break; }   // N, R of an earlier tile
         if (FUSE_X && !fuse && c == 0) {                 // the X boxes of an earlier tile have left the buffer too
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->xempty[half][0]), (xeph & 1u) ^ 1u, abort_flag) ||
               !ptx::mbar_wait(ptx::smem_u32(&ctl->xempty[half][1]), ((xeph >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
@@ -616,6 +631,9 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
               const __nv_bfloat162 pr = __floats2bfloat162_rn(nv[e], rv[e]);
               rr[8 * qq + e] = *reinterpret_cast<const uint32_t*>(&pr);
             }
+            const uint32_t* w = &rr[8 * qq];             // R's halves
+            if (keep_r) *reinterpret_cast<uint4*>(nb + xs * K1_HBOX_BYTES + hrow + (((uint32_t)q ^ hsw) << 4)) =
+                make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632), __byte_perm(w[4], w[5], 0x7632), __byte_perm(w[6], w[7], 0x7632));
           } else {
             const uint32_t h = hrow + (((uint32_t)q ^ hsw) << 4);
             *reinterpret_cast<uint4*>(nb + h) = pack8_bf16(nv);
@@ -708,9 +726,8 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_cluster(te);
           }
-          const int xs = c & 1;                          // X boxes alternate between the two parts of the buffer
+          const int xs = c & 1;
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->xempty[half][xs]), ((xeph >> xs) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
-          if (c == 0 && !ptx::mbar_wait(nrempty, nrphase ^ 1u, abort_flag)) { ok = false; break; }   // N, R of an earlier tile
           unsigned char* xb = nb + xs * K1_HBOX_BYTES;
 #pragma unroll
           for (int qq = 0; qq < QN; ++qq) {

@@ -1,0 +1,83 @@
+"""GPU checks of the fp32-precision tensor-core paths at the sizes where their tilings can go wrong: long lists
+(kernels of their own), tile remainders, ranks around the tile widths, the factorisation's blocks."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import fira_oracle as fo
+from paper_2410_01623_b200 import binding as fb
+from paper_2410_01623_b200 import workloads as wk
+from tests.parity_util import to_np64
+from tests.test_gpu_step import _random_case
+
+pytestmark = pytest.mark.gpu
+
+# remainders of every extent, both orientations, ranks that are no multiple of 4 or 8, above one tile (128) and above
+# the width up to which accumulators are double-buffered (256); 3 x 90 tiles of 128 x 128
+BASE = [(150, 333), (333, 150), (130, 130), (64, 200), (257, 129), (129, 257), (300, 1000), (1000, 300), (512, 700), (7, 9),
+        (640, 512), (512, 256)]
+RANKS = [36, 37, 64, 16, 100, 128, 200, 255, 130, 3, 300, 128]
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("flags,ranks", [(0, RANKS), (0, [r // 4 * 4 or 4 for r in RANKS]), (fb.FLAG_MATRIX_SCALING, RANKS),
+                                         (fb.FLAG_NO_RESIDUAL, RANKS), (fb.FLAG_PSI_ADAGRAD, RANKS), (fb.FLAG_ONLY_SCALING, RANKS)])
+def test_long_list_of_ragged_matrices(dtype, flags, ranks):
+    """A list of many tiles takes kernels of its own in fp32 precision; with ranks all multiples of 4 (no rank that TMA
+    cannot address) the projection's too."""
+    tr = _random_case(BASE * 3, ranks * 3, dtype, steps=3, seed=71, spike=(3,), flags=flags | fb.FLAG_FORCE_SIMT)
+    tr.assert_ok()
+    assert all(tr.f.diagnostics(i)["engine"] == 0 for i in range(len(BASE)))
+    assert tr.f.last_step_launches() > 4 or flags & fb.FLAG_ONLY_SCALING
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_long_list_with_pitches_and_in_chunks(dtype):
+    """The same list with padded rows, whole and as the host path's chunks: the same weights as without padding, bit for
+    bit (the order of every sum is the same), and the padding untouched."""
+    shapes, ranks = BASE * 3, [r // 4 * 4 or 4 for r in RANKS] * 3
+    g = torch.Generator().manual_seed(5)
+    hp = fb.make_hparams(lr=1e-2, alpha=0.25, gamma=1.01, flags=fb.FLAG_FORCE_SIMT)
+    lds = [n + (3, 8, 0)[i % 3] for i, (m, n) in enumerate(shapes)]
+    fs = [fb.Fira(shapes, ranks, dtype, hp), fb.Fira(shapes, ranks, dtype, hp, lds=lds), fb.Fira(shapes, ranks, dtype, hp)]
+    W0 = [(torch.randn(m, n, generator=g) * 0.02).to(dtype) for m, n in shapes]
+    for i, (m, n) in enumerate(shapes):
+        P = torch.linalg.qr(torch.randn(min(m, n), ranks[i], generator=g, dtype=torch.float64))[0].to(dtype).cuda()
+        for f in fs:
+            f.set_projection(i, P)
+    Wa = [w.cuda() for w in W0]
+    Wb = [torch.full((m, ld), 7.0, dtype=dtype, device="cuda") for (m, n), ld in zip(shapes, lds)]
+    Gb = [torch.full((m, ld), float("nan"), dtype=dtype, device="cuda") for (m, n), ld in zip(shapes, lds)]
+    for w, b, (m, n) in zip(W0, Wb, shapes):
+        b[:, :n] = w.cuda()
+    Wh = [w.clone().pin_memory() for w in W0]
+    staging = torch.empty(fs[2].staging_bytes(), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        G = [torch.randn(m, n, generator=g).to(dtype) for m, n in shapes]
+        for x, b, (m, n) in zip(G, Gb, shapes):
+            b[:, :n] = x.cuda()
+        fs[0].step(Wa, [x.cuda() for x in G])
+        fs[1].step(Wb, Gb)
+        fs[2].step_host(Wh, [x.pin_memory() for x in G], staging)
+        torch.cuda.synchronize()
+    assert [f.poll() for f in fs] == [0, 0, 0]
+    for i, (m, n) in enumerate(shapes):
+        assert torch.equal(Wa[i], Wb[i][:, :n]), (i, shapes[i])
+        assert torch.equal(Wa[i].cpu(), Wh[i]), (i, shapes[i])
+        assert (Wb[i][:, n:] == 7.0).all()
+
+
+@pytest.mark.parametrize("shape,r", [((300, 420), 1), ((300, 420), 127), ((420, 300), 128), ((300, 420), 129),
+                                     ((700, 515), 257), ((384, 1024), 384)])
+def test_refresh_at_the_edges_of_its_blocks(shape, r):
+    """Bases whose Gram factor has one row, one block less one, whole blocks, one row in its last block, and full rank:
+    orthonormal to fp32 and the SVD's subspace."""
+    m, n = shape
+    G = wk.planted_gradient(m, n, r, seed=r, gap=4.0).cuda() if r < min(m, n) else torch.randn(m, n, generator=torch.Generator().manual_seed(3)).cuda()
+    f = fb.Fira([shape], r, torch.float32, fb.make_hparams())
+    f.refresh_projection([G], seed=12, iters=6)
+    assert f.poll() == 0
+    P = to_np64(f.get_projection(0))
+    assert np.abs(P.T @ P - np.eye(r)).max() < 1e-5
+    if r < min(m, n):
+        assert fo.principal_angles(P, fo.refresh_projection(to_np64(G), r)).max() <= 1e-3
