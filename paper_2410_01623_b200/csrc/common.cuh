@@ -118,6 +118,24 @@ __device__ __forceinline__ int find_matrix(const int* __restrict__ start, int co
 
 void set_error(const std::string& msg);
 
+// Launches a kernel in clusters of `cluster` blocks (1: none).  chained: the kernel calls ptx::grid_wait, and its
+// blocks may start while the kernel in front of it in the stream is still running.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, bool chained, int cluster, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  if (chained) { at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[n].val.programmaticStreamSerializationAllowed = 1; ++n; }
+  if (cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  cfg.attrs = at; cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Optional per-kernel timing of a step: marks are CUDA events recorded between the
 // launches.  slot = the step's row of the event ring, next = the next mark.
 struct PhaseTimer {

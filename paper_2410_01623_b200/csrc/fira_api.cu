@@ -316,6 +316,7 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
     c->simt.mats = c->mats_dev;
     c->simt.list = c->ints_dev + o_list; c->simt.nlist = (int)lst.size();
     c->simt.proj_tile_start = c->ints_dev + o_pt; c->simt.proj_tiles = pt.back();
+    for (int i : c->simt_list) c->simt.max_d = std::max(c->simt.max_d, c->mats[i].d);
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
     c->simt.npart = c->ints_dev + o_np; c->simt.npart_tiles = c->ints_dev + o_npt;
     c->simt.row_start = c->ints_dev + o_rs; c->simt.h_row_start = rs;

@@ -251,6 +251,7 @@ __device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, int n, 
   constexpr uint64_t along_x = ptx::smem_desc_constant(ptx::LAYOUT_PLAIN, 128, X_SBO);
   constexpr uint64_t along_k = ptx::smem_desc_constant(ptx::LAYOUT_PLAIN, K_LBO, 128);
   constexpr int a_step = (A_X ? 256 : 2 * K_LBO) / 16, b_step = (B_X ? 256 : 2 * K_LBO) / 16;
+  slab &= 0x3ffff;                              // (in a cluster the address carries the block's rank above the descriptor's field)
   uint64_t a = (A_X ? along_x : along_k) + (slab >> 4), b = (B_X ? along_x : along_k) + ((slab + OPERAND_BYTES) >> 4);
   uint32_t acc_main = !fresh_main, acc = !first;
   for (int k = 0; k < steps; ++k, a += a_step, b += b_step) {

@@ -15,7 +15,9 @@
 // epilogue takes the finished tile from shared memory, one warp per row, so that all traffic with
 // global memory runs along rows.
 //
-// Measured (56 fp32 matrices of 8 layers 512 / 1376, r = 128; one 512 x 1376 matrix): see each kernel.
+// Short lists are bound by latency, so all of their kernels are chained (launch_chained): one's set-up (tables, barriers,
+// tensor memory) runs while the one before it ends.  Step of one 512 x 1376 matrix: 74 us without that and without the
+// split projection, 35 us with both.
 #include <algorithm>
 #include <atomic>
 
@@ -116,29 +118,61 @@ constexpr int ROWS_AT_ONCE = 4;                 // rows of a warp whose loads ar
 constexpr int WARP_ROWS = SIMT_TILE / (split::THREADS / 32);
 
 // ---------------------------------------------------------------- phase 1
-// Rows of the finished tile R: Adam (Eq. 2-4), N and R to scratch, row sums.
-template <int PSI, bool VEC>
+constexpr int MAX_SPLIT = 8;                    // blocks of a cluster (a portable size)
+
+// Four entries of row `row` of the tile that the blocks of the cluster hold parts of (in the order of their ranks).
+template <bool VEC>
+__device__ __forceinline__ void add_row_parts(uint32_t row, int blocks, int lane, int n, float (&v)[4]) {
+  float u[MAX_SPLIT][4];
+#pragma unroll
+  for (int b = 0; b < MAX_SPLIT; ++b) {
+    const uint32_t p = ptx::map_to_cta(row, min(b, blocks - 1));
+    if (VEC) {
+      const float4 w = ptx::ld_cluster_f4(p + 16 * lane);
+      u[b][0] = w.x; u[b][1] = w.y; u[b][2] = w.z; u[b][3] = w.w;
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) u[b][c] = ptx::ld_cluster_f1(p + 4 * (lane + 32 * c));
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    v[c] = u[0][c];
+#pragma unroll
+    for (int b = 1; b < MAX_SPLIT; ++b) if (b < blocks) v[c] += u[b][c];
+    if (lane_col<VEC>(lane, c) >= n) v[c] = 0.f;
+  }
+}
+
+// Rows of the finished tile R: Adam (Eq. 2-4), N and R to scratch, row sums.  SPLIT: the blocks of the cluster share the
+// rows; between cluster_arrive, which the caller has done, and the first look at the tile, M and V are fetched.
+template <int PSI, bool VEC, bool SPLIT>
 __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, const float* C, const Hyper& hp, float bias) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = min(SIMT_TILE, mt.r - j0);
   const int nrt = simt_tiles_dev(mt.r), q = j0 / SIMT_TILE;
+  const int blocks = SPLIT ? (int)ptx::cluster_nctarank() : 1, rows = WARP_ROWS / blocks;
+  const int row0 = SPLIT ? ((int)ptx::cluster_ctarank() * (split::THREADS / 32) + warp) * rows : warp * rows;
   constexpr bool momentum = PSI == PSI_ADAM;
-  for (int x = 0; x < WARP_ROWS; x += ROWS_AT_ONCE) {
+  for (int x = 0; x < rows; x += ROWS_AT_ONCE) {
     float m[ROWS_AT_ONCE][4], v[ROWS_AT_ONCE][4];
 #pragma unroll
     for (int y = 0; y < ROWS_AT_ONCE; ++y) {
-      const int l = l0 + warp * WARP_ROWS + x + y;
+      const int l = l0 + row0 + x + y;
+      const bool there = l < mt.l && (!SPLIT || x + y < rows);
       const long long at = (long long)l * mt.r + j0;
-      load_row<VEC>(mt.V + at, lane, l < mt.l ? n : 0, v[y]);
-      load_row<VEC>(mt.M + at, lane, l < mt.l && momentum ? n : 0, m[y]);
+      load_row<VEC>(mt.V + at, lane, there ? n : 0, v[y]);
+      load_row<VEC>(mt.M + at, lane, there && momentum ? n : 0, m[y]);
     }
+    if (SPLIT && x == 0) ptx::cluster_wait();
 #pragma unroll
     for (int y = 0; y < ROWS_AT_ONCE; ++y) {
-      const int row = warp * WARP_ROWS + x + y, l = l0 + row;
-      if (l >= mt.l) continue;
+      const int row = row0 + x + y, l = l0 + row;
+      if (l >= mt.l || (SPLIT && x + y >= rows)) continue;
       const long long at = (long long)l * mt.r + j0;
       float rv[4], nv[4], nn = 0.f, rn = 0.f;
-      load_row<VEC>(C + row * split::C_LD, lane, n, rv);
+      if (SPLIT) add_row_parts<VEC>(ptx::smem_u32(C + row * split::C_LD), blocks, lane, n, rv);
+      else load_row<VEC>(C + row * split::C_LD, lane, n, rv);
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         nv[c] = adam_direction<PSI>(hp, bias, rv[c], m[y][c], v[y][c]);
@@ -167,32 +201,49 @@ __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, cons
   }
 }
 
-template <typename T>
-__device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, unsigned char* smem, split::Ctl* ctl) {
+// The part of the tile's product that k in [k0, k1) makes.
+template <typename T, bool LONG_K>
+__device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, int k0, int k1, unsigned char* smem, split::Ctl* ctl) {
   // A(i = l, k = d): G[d][l] when left, G[l][d] when right.
-  split::Operand<T> a(static_cast<const T*>(mt.G), mt.left ? 1 : mt.ld, mt.left ? mt.ld : 1, mt.l, mt.d, l0);
-  split::Operand<T> b(static_cast<const T*>(mt.P), 1, mt.r, mt.r, mt.d, j0);
-  return split::tile_product<true>(a, b, mt.d, mt.r - j0, smem, ctl);
+  split::Operand<T> a(static_cast<const T*>(mt.G) + (mt.left ? k0 * mt.ld : (long long)k0), mt.left ? 1 : mt.ld, mt.left ? mt.ld : 1, mt.l, k1 - k0, l0);
+  split::Operand<T> b(static_cast<const T*>(mt.P) + (long long)k0 * mt.r, 1, mt.r, mt.r, k1 - k0, j0);
+  return split::tile_product<LONG_K>(a, b, k1 - k0, mt.r - j0, smem, ctl);
 }
 
-template <int PSI>
+// SPLIT: the blocks of a cluster share the tile's product by k, each leaves its part in its shared memory, and they add the
+// parts while they share the rows of the epilogue.  A list of few tiles leaves most SMs idle otherwise, and its time
+// is the latency of one block's slabs, about 2 us each.  LONG_K: a block's part is longer than split::PROMOTE.
+// Measured (one 512 x 1376 matrix, r = 128): 46 us as 11 blocks of 16 slabs, 15 us as 11 clusters of 8 blocks.
+template <int PSI, bool SPLIT, bool LONG_K>
 __global__ void __launch_bounds__(split::THREADS, 2)
 k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
           const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem[];
   split::Ctl* ctl = reinterpret_cast<split::Ctl*>(smem + split::STAGES * split::STAGE_BYTES);
-  const int gt = blockIdx.x + first;
+  const int blocks = SPLIT ? (int)ptx::cluster_nctarank() : 1, block = SPLIT ? (int)ptx::cluster_ctarank() : 0;
+  const int gt = blockIdx.x / blocks + first;
   const int p = find_matrix(tile_start, nlist, gt);
   const MatDev mt = mats[list[p]];
   const int tile = gt - tile_start[p], rt = simt_tiles_dev(mt.r);
   const int l0 = (tile / rt) * SIMT_TILE, j0 = (tile % rt) * SIMT_TILE;
   split::begin(ctl);
-  const bool ok = mt.bf16 ? project_tile<__nv_bfloat16>(mt, l0, j0, smem, ctl) : project_tile<float>(mt, l0, j0, smem, ctl);
-  if (ok) {
-    const float bias = mt.sc->pad;
-    if (mt.r % 4 == 0) adam_rows<PSI, true>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
-    else adam_rows<PSI, false>(mt, l0, j0, reinterpret_cast<const float*>(smem), hp, bias);
+  ptx::grid_launch_next();
+  const int slabs = (mt.d + split::BK - 1) / split::BK;
+  const int k0 = slabs * block / blocks * split::BK, k1 = min(mt.d, slabs * (block + 1) / blocks * split::BK);
+  const float* C = reinterpret_cast<const float*>(smem);
+  bool ok = true;
+  if (k1 > k0) {
+    ok = mt.bf16 ? project_tile<__nv_bfloat16, LONG_K>(mt, l0, j0, k0, k1, smem, ctl) : project_tile<float, LONG_K>(mt, l0, j0, k0, k1, smem, ctl);
+  } else {                                      // fewer slabs than blocks
+    for (int i = threadIdx.x; i < SIMT_TILE * split::C_LD; i += split::THREADS) reinterpret_cast<float*>(smem)[i] = 0.f;
   }
+  if (SPLIT) ptx::cluster_arrive();
+  if (SPLIT || ok) {                            // (a block whose wait ran out still meets the others)
+    const float bias = mt.sc->pad;
+    if (mt.r % 4 == 0) adam_rows<PSI, true, SPLIT>(mt, l0, j0, C, hp, bias);
+    else adam_rows<PSI, false, SPLIT>(mt, l0, j0, C, hp, bias);
+  }
+  if (SPLIT) ptx::cluster_sync_all();           // nobody leaves while others read its part
   split::end(ctl, status);
 }
 
@@ -300,6 +351,8 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
   const int tile = gt - tile_start[p], ct = simt_tiles_dev(mt.n);
   const int i0 = (tile / ct) * SIMT_TILE, j0 = (tile % ct) * SIMT_TILE;
   split::begin(ctl);
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   float ss = mt.bf16 ? back_tile<__nv_bfloat16, MODE>(mt, i0, j0, hp, smem, ctl, ks)
                      : back_tile<float, MODE>(mt, i0, j0, hp, smem, ctl, ks);
   if (MODE == MODE_NORM) {
@@ -475,11 +528,13 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   __shared__ float smin[256], smax[256];
   const MatDev mt = mats[list[blockIdx.x]];
   const int npart = npart_of[blockIdx.x];
-  // the bias factor sqrt(1 - b2^s) / (1 - b1^s) of the NEXT step, in double, while the others add up
+  // the bias factor sqrt(1 - b2^s) / (1 - b1^s) of the NEXT step, in double, while the others wait and add up
   if (threadIdx.x == 255) {
     if (mt.step_bias) *mt.step_bias = mt.sc->pad;
     mt.sc->pad = bias_factor(hp.beta1, hp.beta2, mt.sc->t + 2);
   }
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   double acc = 0.0;
   for (int i = threadIdx.x; i < npart; i += 256) acc += (double)mt.part[i];
   // Matrix-level factor (Eq. 9): the phases before ran with k = 1, so `part` holds ||G - P R||^2;
@@ -569,13 +624,35 @@ static bool allow_smem() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && !done[dev].load()) {
-    const void* kernels[5] = {(const void*)k_project<PSI_ADAM>, (const void*)k_project<PSI_RMSPROP>, (const void*)k_project<PSI_ADAGRAD>, (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
+    const void* kernels[11] = {(const void*)k_project<PSI_ADAM, false, true>, (const void*)k_project<PSI_RMSPROP, false, true>,
+                               (const void*)k_project<PSI_ADAGRAD, false, true>, (const void*)k_project<PSI_ADAM, true, true>,
+                               (const void*)k_project<PSI_RMSPROP, true, true>, (const void*)k_project<PSI_ADAGRAD, true, true>,
+                               (const void*)k_project<PSI_ADAM, true, false>, (const void*)k_project<PSI_RMSPROP, true, false>,
+                               (const void*)k_project<PSI_ADAGRAD, true, false>,
+                               (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
     for (const void* k : kernels)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
     if (e == cudaSuccess) done[dev].store(true);
   }
   if (e != cudaSuccess) set_error(std::string("step kernels, shared memory: ") + cudaGetErrorString(e));
   return e == cudaSuccess;
+}
+
+// Blocks that share a tile of the projection: of a short list as many as keep the grid within one block per SM (but no
+// part below two slabs).  Counted over the whole list, whatever range of it is stepped: the sums have the same order then.
+static int split_of(const SimtPlan& pl) {
+  constexpr int SMS = 148;
+  int split = 1;
+  while (split < MAX_SPLIT && 2 * split * pl.proj_tiles <= SMS && 4 * split * split::BK <= pl.max_d) split *= 2;
+  return split;
+}
+
+template <int PSI>
+static cudaError_t launch_project(const SimtPlan& pl, int first, int tiles, const Hyper& hp, unsigned* status_dev, cudaStream_t st) {
+  const int split = split_of(pl);
+  const bool long_k = (pl.max_d + split::BK - 1) / split::BK > split * (split::PROMOTE / split::BK);
+  auto k = split == 1 ? k_project<PSI, false, true> : long_k ? k_project<PSI, true, true> : k_project<PSI, true, false>;
+  return launch_chained(k, tiles * split, split::THREADS, split::SMEM_BYTES, st, false, split, pl.mats, pl.list, pl.nlist, pl.proj_tile_start, first, hp, status_dev);
 }
 
 int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, cudaStream_t st,
@@ -594,6 +671,8 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     qa = 0;
   }
   constexpr int TH = split::THREADS, SM = split::SMEM_BYTES;
+  cudaError_t error = cudaSuccess;
+  auto launch_error = [&](cudaError_t e) { if (error == cudaSuccess) error = e; };
   const bool only_scaling = hp.mode & HYPER_ONLY_SCALING;     // W <- W - lr phi(R) G: no back-projection
   const bool parts = pl.parts.table && !only_scaling;          // (a long list's only-scaling step has no back-projection)
   const int psi = psi_of(hp);
@@ -604,19 +683,20 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 0, st);
   if (pl.parts.proj_table) {           // (also before only-scaling, which needs the row sums)
     if (part_project_run(pl.parts, pl.mats, qa, qe, hp, status_dev, st) != FIRA_OK) return -1;
-  } else
-    (psi == PSI_ADAM ? k_project<PSI_ADAM> : psi == PSI_RMSPROP ? k_project<PSI_RMSPROP> : k_project<PSI_ADAGRAD>)
-        <<<pt1 - pt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.proj_tile_start, pt0, hp, status_dev);
+  } else {
+    launch_error((psi == PSI_ADAM ? launch_project<PSI_ADAM> : psi == PSI_RMSPROP ? launch_project<PSI_RMSPROP> : launch_project<PSI_ADAGRAD>)(
+        pl, pt0, pt1 - pt0, hp, status_dev, st));
+  }
   tm->mark(st);
   if (only_scaling)
     launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 0, hp, st);
   else if (parts) {
     if (part_step_run(pl.parts, pl.mats, qa, qe, 0, hp, status_dev, st) != FIRA_OK) return -1;
   } else
-    k_back_project<MODE_NORM><<<wt1 - wt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev);
+    launch_error(launch_chained(k_back_project<MODE_NORM>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   // (only-scaling leaves one partial sum per 128 x 128 tile whatever the list)
-  k_finalize<<<nq, 256, 0, st>>>(pl.mats, pl.list + qa, nq, (only_scaling ? pl.npart_tiles : pl.npart) + qa, hp, status_dev);
+  launch_error(launch_chained(k_finalize, nq, 256, 0, st, true, 1, pl.mats, pl.list + qa, nq, (only_scaling ? pl.npart_tiles : pl.npart) + qa, hp, status_dev));
   tm->mark(st);
   if (parts) {
     const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
@@ -629,8 +709,9 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     if (part_step_run(pl.parts, pl.mats, qa, qe, 1, hp, status_dev, st) != FIRA_OK) return -1;
     launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 1, st);
   } else
-    k_back_project<MODE_UPDATE><<<wt1 - wt0, TH, SM, st>>>(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev);
+    launch_error(launch_chained(k_back_project<MODE_UPDATE>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
+  if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
   return 4 + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
 }
 

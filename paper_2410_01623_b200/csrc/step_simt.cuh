@@ -43,6 +43,7 @@ struct SimtPlan {
   int nlist = 0;
   const int* proj_tile_start = nullptr;  // 128 x 128 tiles of R (l x r)
   int proj_tiles = 0;
+  int max_d = 0;                         // largest d of the list
   const int* w_tile_start = nullptr;     // 128 x 128 tiles of W (m x n)
   int w_tiles = 0;
   const int* npart = nullptr;            // partial sums of ||S||^2 per matrix
