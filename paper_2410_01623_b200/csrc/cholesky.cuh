@@ -2,7 +2,7 @@
 // Included by refresh.cu inside its namespace.
 //
 // Blocked over columns of NB = 128, three launches per block column J, each over every matrix:
-//   k_factor_block   one block per matrix: factors C[J, J] and inverts the factor in shared memory; U[J, J]
+//   k_factor_block   one block per matrix: factors C[J, J] and inverts the factor in registers; U[J, J]
 //   k_factor_tiles   phase 0: the panel, L[I, J] = C[I, J] U[J, J] for the rows I below (in place), and the
 //                    first half of U's block column, U[a, J] = sum_k U[a, k] L[J, k]^T over k < J
 //                    phase 1: the trailing matrix, C[I, K] -= L[I, J] L[K, J]^T, and the second half of
@@ -11,133 +11,80 @@
 // tile that is written in place reads nothing else than itself of what it writes.  Factor and inverse
 // grow together, so the inverse costs no launches of its own.
 //
-// C is used up (its lower triangle becomes L off the diagonal blocks).  U's blocks below the diagonal are not
-// written: they have to be zero where a product reads them.
+// C is used up (its lower triangle becomes L off the diagonal blocks).  What of U is below the diagonal is not
+// written: it has to be zero where a product reads it.  Finished entries of U are also left in the form that the
+// application's products read (InverseOut).
 // A non-positive or non-finite pivot is replaced and flagged.  Matrices whose r does not reach the
 // block column do nothing.
 //
 // Measured on 75 matrices with r = 1024: see k_factor_block and k_factor_tiles.
 constexpr int NB = split::TILE;
-constexpr int SB = 32;                          // sub-blocks of k_factor_block
-constexpr int FP = NB + 4;                      // pitch: 16-byte rows, eight neighbouring rows in different banks
-constexpr int FACTOR_THREADS = 256;
-constexpr int FACTOR_SMEM = 2 * NB * FP * 4;
+constexpr int PANEL = 8;                        // columns that k_factor_block eliminates at a time
+constexpr int PP = PANEL + 4;                   // pitch of a panel's rows in shared memory
+constexpr int FI = 8, FJ = 4;                   // tile (rows and columns) of a thread
+// Row i of a panel in shared memory: rows i, i + 4, ... are neighbours, which the threads of a row of tiles read
+// together; with the pitch above eight of them hit different banks.
+__device__ __forceinline__ int panel_row(int i) { return (i % FJ * (NB / FJ) + i / FJ) * PP; }
+constexpr int FACTOR_TILES = (NB / FI) * (NB / FI + 1);         // that reach into a lower triangle
+constexpr int FACTOR_THREADS = (FACTOR_TILES + 31) / 32 * 32;
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-// Eight steps of factor_subblock on rows whose last W entries are still to be done.  a: lane i's row i, moved left by
-// one entry per step, so that the loop body is the same for every step (unrolled over all 32 steps one warp waits for
-// its instructions: 20 us per sub-block instead of 4); t: lane j's column j of the identity on its way to the inverse,
-// moved the same way.  Both take the entries of the factor's column below the pivot from `column` (the first of them,
-// on which the next pivot waits, by a shuffle).
-template <int W>
-__device__ __forceinline__ void factor_steps(float (&a)[SB], float (&t)[SB], int k0, float* S, float* X, float* column,
-                                             int n, float floor_pivot, bool& bad) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll 1
-  for (int k = k0; k < k0 + 8; ++k) {
-    float pv = __shfl_sync(0xffffffffu, a[0], k);
-    if (k < n && !(pv > floor_pivot && pv < INFINITY)) { bad = true; pv = floor_pivot; }
-    float s = rsqrtf(pv);
-    s = s * (1.5f - 0.5f * pv * s * s);         // one Newton step: to working precision
-    const float l = lane == k ? pv * s : a[0] * s, x = t[0] * s;
-    float* c = column + (k & 1) * SB;           // (two in turn: nobody is more than a step behind)
-    if (lane > k) c[lane - k - 1] = l;
-    S[lane * FP + k] = lane >= k ? l : 0.f;
-    X[k * FP + lane] = x;
-    const float next = __shfl_sync(0xffffffffu, l, k + 1);
-    a[0] = a[1] - l * next;
-    t[0] = t[1] - next * x;
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < W; j += 4) {            // (entries past the row's end never come to the front)
-      const float4 v = ld4(c + j);
-      const float w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (j + q > 0 && j + q < W - 1) {
-          a[j + q] = a[j + q + 1] - l * w[q];
-          t[j + q] = t[j + q + 1] - w[q] * x;
-        }
-    }
+// U = L^-T in every form that products read: fp32, and as parts or (on the tensor-core path) as bf16 with its remainder.
+struct InverseOut {
+  float* u;
+  __nv_bfloat16* hi;                            // the second form lies `second` behind it, the third as far behind that
+  long long second, pitch;
+  int r, third;
+  __device__ __forceinline__ explicit InverseOut(const RefreshMat& m) {
+    u = m.U; r = m.r; third = !m.tc;
+    hi = m.tc ? m.Ub[0] : m.Up.base;
+    pitch = m.tc ? m.r : m.Up.pitch;
+    second = m.tc ? m.Ub[1] - m.Ub[0] : m.Up.part_stride;
   }
-}
-
-// One warp: Cholesky factor of the SB x SB block at S (pitch FP) in place and its inverse at X.
-// n of its rows are the matrix's, the others the identity's.
-__device__ __forceinline__ void factor_subblock(float* S, float* X, float* column, int n, float floor_pivot, bool& bad) {
-  const int lane = threadIdx.x & 31;
-  float a[SB], t[SB];
-#pragma unroll
-  for (int j = 0; j < SB; j += 4) {
-    const float4 v = ld4(S + lane * FP + j);
-    a[j] = v.x; a[j + 1] = v.y; a[j + 2] = v.z; a[j + 3] = v.w;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) t[j + q] = j + q == lane ? 1.f : 0.f;
-  }
-  __syncwarp();
-  factor_steps<32>(a, t, 0, S, X, column, n, floor_pivot, bad);
-  factor_steps<24>(a, t, 8, S, X, column, n, floor_pivot, bad);
-  factor_steps<16>(a, t, 16, S, X, column, n, floor_pivot, bad);
-  factor_steps<8>(a, t, 24, S, X, column, n, floor_pivot, bad);
-}
-
-// Products in shared memory (pitch FP), NX blocks of 32 x 32, four neighbours of a row of every block per thread.
-//   by_rows:  acc[x][y] = sum_k P[row + 32 x][k] Q[col + 8 y][k]      (col = lane % 8)
-//   otherwise acc[x][y] = sum_k P[row][k] Q[k][32 x + 4 col + y]
-// Four of k at a time, all loads 16 bytes and free of bank conflicts: for three blocks 7 or 13 of them for 48
-// multiply-adds.
-template <int NX, bool BY_ROWS>
-__device__ __forceinline__ void small_product(float (&acc)[3][4], const float* P, const float* Q, int depth) {
-  const int col = threadIdx.x & 7, row = threadIdx.x >> 3;
-#pragma unroll
-  for (int x = 0; x < NX; ++x)
-#pragma unroll
-    for (int y = 0; y < 4; ++y) acc[x][y] = 0.f;
-#pragma unroll 2
-  for (int k = 0; k < depth; k += 4) {
-    if (BY_ROWS) {
-      float4 p[NX], q[4];
-#pragma unroll
-      for (int x = 0; x < NX; ++x) p[x] = ld4(P + (row + 32 * x) * FP + k);
-#pragma unroll
-      for (int y = 0; y < 4; ++y) q[y] = ld4(Q + (col + 8 * y) * FP + k);
-#pragma unroll
-      for (int x = 0; x < NX; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y)
-          acc[x][y] = fmaf(p[x].w, q[y].w, fmaf(p[x].z, q[y].z, fmaf(p[x].y, q[y].y, fmaf(p[x].x, q[y].x, acc[x][y]))));
+  // n (<= 4) neighbours of row i from column j; vec: all four, from an aligned place.
+  __device__ __forceinline__ void put(int i, int j, const float (&v)[4], int n, bool vec) const {
+    float* f = u + (long long)i * r + j;
+    __nv_bfloat16 *a = hi + i * pitch + j, *b = a + second, *c = b + second;
+    uint32_t h[2], m[2], l[2];
+    split::split3(v[0], v[1], h[0], m[0], l[0]);
+    split::split3(v[2], v[3], h[1], m[1], l[1]);
+    if (vec) {
+      *reinterpret_cast<float4*>(f) = make_float4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<uint2*>(a) = make_uint2(h[0], h[1]);
+      *reinterpret_cast<uint2*>(b) = make_uint2(m[0], m[1]);
+      if (third) *reinterpret_cast<uint2*>(c) = make_uint2(l[0], l[1]);
     } else {
-      const float4 p = ld4(P + row * FP + k);
-      const float pk[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
-      for (int x = 0; x < NX; ++x)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float4 q = ld4(Q + (k + u) * FP + 32 * x + 4 * col);
-          acc[x][0] = fmaf(pk[u], q.x, acc[x][0]);
-          acc[x][1] = fmaf(pk[u], q.y, acc[x][1]);
-          acc[x][2] = fmaf(pk[u], q.z, acc[x][2]);
-          acc[x][3] = fmaf(pk[u], q.w, acc[x][3]);
+      for (int e = 0; e < 4; ++e)
+        if (e < n) {
+          f[e] = v[e];
+          reinterpret_cast<unsigned short*>(a)[e] = (unsigned short)(h[e / 2] >> (16 * (e & 1)));
+          reinterpret_cast<unsigned short*>(b)[e] = (unsigned short)(m[e / 2] >> (16 * (e & 1)));
+          if (third) reinterpret_cast<unsigned short*>(c)[e] = (unsigned short)(l[e / 2] >> (16 * (e & 1)));
         }
     }
   }
-}
-template <bool BY_ROWS>
-__device__ __forceinline__ void small_product(int nx, float (&acc)[3][4], const float* P, const float* Q, int depth) {
-  if (nx == 3) small_product<3, BY_ROWS>(acc, P, Q, depth);
-  else if (nx == 2) small_product<2, BY_ROWS>(acc, P, Q, depth);
-  else if (nx == 1) small_product<1, BY_ROWS>(acc, P, Q, depth);
-}
+};
 
-// Diagonal block J0 / NB of every matrix.  Bound by the chain of 128 pivots, which one warp runs through.
+// Diagonal block J0 / NB of every matrix: U = L^-T of the block C = L L^T.
+//
+// The lower triangle lives in registers, 8 x 4 entries per thread, eliminated in panels of 8 columns.  Where a column has
+// been eliminated, its place takes the inverse's (T, the identity under the same row operations): one triangle
+// holds both, and one update serves both, a(i, j) -= sum_k Q[i][k] Q[j][k] with
+//   Q[i] = row i of L in the panel's columns            for rows below the panel,
+//   Q[j] = column j of the inverse in the panel's rows  for columns up to the panel's end,
+// both of which come out of the same forward substitution with the panel's diagonal 8 x 8 block.  That block's own
+// factorisation is a chain of 8 pivots (root, reciprocal, product, difference); each of the 128 threads that
+// substitute a row or column works it out for itself, which costs no exchange.
+//
+// Bound by the chain of 128 pivots, about 60 cycles each, and two block barriers per panel.  Measured (56 to 109
+// matrices): 33 us; a blocked factorisation in shared memory with the chain in one warp (285 cycles per pivot)
+// took 51.
 __global__ void __launch_bounds__(FACTOR_THREADS)
 k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsigned* __restrict__ status) {
-  extern __shared__ __align__(16) float fsm[];
+  __shared__ __align__(16) float in[NB * PP], Q[NB * PP], diag[PANEL * PANEL];
   __shared__ float red[FACTOR_THREADS / 32];
-  __shared__ __align__(16) float column[2 * SB];
-  float* S = fsm;                               // the block, later its factor
-  float* X = fsm + NB * FP;                     // the factor's inverse
   const RefreshMat& m = rm[blockIdx.x];
   const int r = m.r, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (J0 >= r) return;
@@ -159,85 +106,120 @@ k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsig
     mean_diag = m.info[0];
   }
   const float shift = shift_rel * mean_diag, floor_pivot = fmaxf(1e-30f, 1e-12f * mean_diag);
-  // eight groups of four entries per thread at a time, their loads before their stores to shared memory
   const bool vec = r % 4 == 0;
-#pragma unroll 1
-  for (int h = 0; h < NB * NB / 4; h += 8 * FACTOR_THREADS) {
-    float v[8][4];
+  const InverseOut out(m);
+  // this thread's tile: row of tiles ti, column tj <= 2 ti + 1, numbered row by row
+  int ti = 0;
+  while ((ti + 1) * (ti + 2) <= tid) ++ti;
+  const int tj = tid - ti * (ti + 1);
+  const bool mine = tid < FACTOR_TILES;
+  const int i0 = FI * ti, j0 = FJ * tj;
+  float a[FI][FJ];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int e = h + q * FACTOR_THREADS + tid, i = e / (NB / 4), j = e % (NB / 4) * 4;
-      if (vec && i < nb && j < nb) {
-        const float4 u = __ldcg(reinterpret_cast<const float4*>(C + (long long)i * r + j));
-        v[q][0] = u.x; v[q][1] = u.y; v[q][2] = u.z; v[q][3] = u.w;
-      } else {
+  for (int x = 0; x < FI; ++x) {
+    const int i = i0 + x;
+    if (mine && vec && i < nb && j0 + 4 <= nb) {
+      const float4 u = __ldcg(reinterpret_cast<const float4*>(C + (long long)i * r + j0));
+      a[x][0] = u.x; a[x][1] = u.y; a[x][2] = u.z; a[x][3] = u.w;
+    } else {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) v[q][c] = i < nb && j + c < nb ? __ldcg(C + (long long)i * r + j + c) : (i == j + c ? 1.f : 0.f);
-      }
+      for (int y = 0; y < FJ; ++y) a[x][y] = mine && i < nb && j0 + y < nb ? __ldcg(C + (long long)i * r + j0 + y) : 0.f;
     }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int e = h + q * FACTOR_THREADS + tid, i = e / (NB / 4), j = e % (NB / 4) * 4;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {             // the lower triangle, shifted
-        if (j + c > i) v[q][c] = 0.f;
-        else if (j + c == i && i < nb) v[q][c] += shift;
-      }
-      *reinterpret_cast<float4*>(S + i * FP + j) = make_float4(v[q][0], v[q][1], v[q][2], v[q][3]);
-      *reinterpret_cast<float4*>(X + i * FP + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int y = 0; y < FJ; ++y) {              // the lower triangle, shifted; past the matrix the identity's
+      if (j0 + y > i) a[x][y] = 0.f;
+      else if (j0 + y == i) a[x][y] = i < nb ? a[x][y] + shift : 1.f;
     }
   }
-  __syncthreads();
   bool bad = false;
-  const int col = tid & 7, row = tid >> 3;
-  for (int b = 0; b < NB; b += SB) {
-    if (warp == 0) factor_subblock(S + b * FP + b, X + b * FP + b, column, nb - b, floor_pivot, bad);
-    __syncthreads();
-    const int lo = b + SB, below = (NB - lo) / SB;
-    float acc[3][4];
-    // rows below: S[i][b + j] <- sum_k S[i][b + k] X[b + j][b + k]
-    small_product<true>(below, acc, S + lo * FP + b, X + b * FP + b, SB);
-    __syncthreads();
+#pragma unroll 1
+  for (int c0 = 0; c0 < NB; c0 += PANEL) {
+    const int q = c0 / FI, k0 = j0 - c0;        // the panel: row of tiles q, tile columns 2 q and 2 q + 1
+    if (mine && ti == q) {
+      if (k0 >= 0) {
 #pragma unroll
-    for (int x = 0; x < 3; ++x)
+        for (int x = 0; x < FI; ++x) *reinterpret_cast<float4*>(diag + x * PANEL + k0) = make_float4(a[x][0], a[x][1], a[x][2], a[x][3]);
+      } else {                                  // the panel's rows of T
 #pragma unroll
-      for (int y = 0; y < 4; ++y)
-        if (x < below) S[(lo + row + 32 * x) * FP + b + col + 8 * y] = acc[x][y];
-    // X[b + j][i] = -sum_k X[b + j][b + k] T[k][i] with T[j][i] = sum_k S[b + j][k] X[k][i], over the columns
-    // i < b; T takes the place of the row block of S that it is made of
-    small_product<false>(b / SB, acc, S + b * FP, X, b);
-    __syncthreads();
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      if (c * SB < b) *reinterpret_cast<float4*>(S + (b + row) * FP + c * SB + 4 * col) = make_float4(acc[c][0], acc[c][1], acc[c][2], acc[c][3]);
-    // the rest of the block: S[i][j] -= sum_k S[i][b + k] S[j][b + k], 32 columns at a time
-    for (int c = 0; c < below; ++c) {
-      small_product<true>(below, acc, S + lo * FP + b, S + (lo + SB * c) * FP + b, SB);
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) {
-          const int i = lo + row + 32 * x, j = lo + SB * c + col + 8 * y;
-          if (x < below && j <= i) S[i * FP + j] -= acc[x][y];
+        for (int y = 0; y < FJ; ++y) {
+          float* p = in + panel_row(j0 + y);
+          *reinterpret_cast<float4*>(p) = make_float4(a[0][y], a[1][y], a[2][y], a[3][y]);
+          *reinterpret_cast<float4*>(p + 4) = make_float4(a[4][y], a[5][y], a[6][y], a[7][y]);
         }
+      }
+    } else if (mine && ti > q && (k0 == 0 || k0 == FJ)) {        // rows below: the panel's columns of C
+#pragma unroll
+      for (int x = 0; x < FI; ++x) {
+        *reinterpret_cast<float4*>(in + panel_row(i0 + x) + k0) = make_float4(a[x][0], a[x][1], a[x][2], a[x][3]);
+#pragma unroll
+        for (int y = 0; y < FJ; ++y) a[x][y] = 0.f;              // from here on T's
+      }
     }
     __syncthreads();
-    small_product<false>(b / SB, acc, X + b * FP + b, S + b * FP, SB);
+    float v[PANEL];
+    const int own = tid - c0;                   // a column of the panel itself starts as the identity's
+    if (tid < NB) {
+      float d[PANEL][PANEL];
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-      if (c * SB < b) *reinterpret_cast<float4*>(X + (b + row) * FP + c * SB + 4 * col) = make_float4(-acc[c][0], -acc[c][1], -acc[c][2], -acc[c][3]);
+      for (int i = 0; i < PANEL; ++i)
+#pragma unroll
+        for (int k = 0; k < PANEL; k += 4) {
+          if (k > i) continue;
+          const float4 u = ld4(diag + i * PANEL + k);
+          d[i][k] = u.x; d[i][k + 1] = u.y; d[i][k + 2] = u.z; d[i][k + 3] = u.w;
+        }
+#pragma unroll
+      for (int k = 0; k < PANEL; k += 4) {
+        const float4 u = ld4(in + panel_row(tid) + k);
+        v[k] = u.x; v[k + 1] = u.y; v[k + 2] = u.z; v[k + 3] = u.w;
+      }
+      if (own >= 0 && own < PANEL) {
+#pragma unroll
+        for (int k = 0; k < PANEL; ++k) v[k] = k == own ? 1.f : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < PANEL; ++k) {
+        float pv = d[k][k];
+        if (c0 + k < nb && !(pv > floor_pivot && pv < INFINITY)) { bad = true; pv = floor_pivot; }
+        float s = rsqrtf(pv);
+        s = s * (1.5f - 0.5f * pv * s * s);     // one Newton step: to working precision
+        v[k] *= s;
+#pragma unroll
+        for (int i = k + 1; i < PANEL; ++i) {
+          d[i][k] *= s;
+          v[i] = fmaf(-d[i][k], v[k], v[i]);
+#pragma unroll
+          for (int j = k + 1; j <= i; ++j) d[i][j] = fmaf(-d[i][k], d[j][k], d[i][j]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < PANEL; k += 4) *reinterpret_cast<float4*>(Q + panel_row(tid) + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+    }
     __syncthreads();
-  }
-  if (bad && lane == 0) atomicOr(status, DEV_STATUS_NONFINITE);
-  float* out = m.U + (long long)J0 * r + J0;    // U = X^T: a lane is a row of X
-  for (int e = warp; e < (NB / 32) * (NB / 4); e += FACTOR_THREADS / 32) {
-    const int j = (e % (NB / 32)) * 32 + lane, k = (e / (NB / 32)) * 4;
-    const float4 v = ld4(X + j * FP + k);
-    const float w[4] = {v.x, v.y, v.z, v.w};
+    if (tid < NB && own < PANEL && tid < nb) {  // rows c0 ... of the inverse are final: U's row `tid`
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (j < nb && k + q < nb) out[(long long)(k + q) * r + j] = w[q];
+      for (int k = 0; k < PANEL; k += 4) {
+        const float w[4] = {v[k], v[k + 1], v[k + 2], v[k + 3]};
+        out.put(J0 + tid, J0 + c0 + k, w, nb - c0 - k, vec && c0 + k + 4 <= nb);
+      }
+    }
+    if (mine && ti > q) {
+#pragma unroll
+      for (int k = 0; k < PANEL; k += 4) {
+        float4 x[FI], y[FJ];
+#pragma unroll
+        for (int e = 0; e < FI; ++e) x[e] = ld4(Q + panel_row(i0 + e) + k);
+#pragma unroll
+        for (int f = 0; f < FJ; ++f) y[f] = ld4(Q + panel_row(j0 + f) + k);
+#pragma unroll
+        for (int e = 0; e < FI; ++e)
+#pragma unroll
+          for (int f = 0; f < FJ; ++f)
+            a[e][f] = fmaf(-x[e].w, y[f].w, fmaf(-x[e].z, y[f].z, fmaf(-x[e].y, y[f].y, fmaf(-x[e].x, y[f].x, a[e][f]))));
+      }
+    }
   }
+  if (bad) atomicOr(status, DEV_STATUS_NONFINITE);
 }
 
 // dst[i][j] (+)= sign * the finished tile, rows x cols of it, pitch r.
@@ -299,7 +281,17 @@ k_factor_tiles(const RefreshMat* __restrict__ rm, int J, int phase, int tiles_pe
       if (split::tile_product<true>(a, b, J0 - A0, nj, smem, ctl)) write_tile<false>(u, r, NB, nj, Cs, 1.f);
     } else {
       split::Operand<float> a(u, ld, 1, NB, nj, 0), b(ujj, 1, ld, nj, nj, 0);
-      if (split::tile_product<false>(a, b, nj, nj, smem, ctl)) write_tile<false>(u, r, NB, nj, Cs, -1.f);
+      if (split::tile_product<false>(a, b, nj, nj, smem, ctl)) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n = min(4, nj - 4 * lane);
+        const InverseOut out(m);
+#pragma unroll 4
+        for (int i = warp; i < NB; i += split::THREADS / 32)
+          if (n > 0) {
+            const float4 v = *reinterpret_cast<const float4*>(Cs + i * split::C_LD + 4 * lane);
+            const float w[4] = {-v.x, -v.y, -v.z, -v.w};
+            out.put(A0 + i, J0 + 4 * lane, w, n, r % 4 == 0 && n == 4);
+          }
+      }
     }
   }
   split::end(ctl, status);
@@ -312,14 +304,13 @@ cudaError_t factor_and_invert(const RefreshMat* rm_dev, int nm, int rmax, float 
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && !ready[dev].load()) {
-    e = cudaFuncSetAttribute(k_factor_block, cudaFuncAttributeMaxDynamicSharedMemorySize, FACTOR_SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_factor_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
+    e = cudaFuncSetAttribute(k_factor_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
     if (e == cudaSuccess) ready[dev].store(true);
   }
   if (e != cudaSuccess) return e;
   const int blocks = (rmax + NB - 1) / NB;
   for (int J = 0; J < blocks; ++J) {
-    k_factor_block<<<nm, FACTOR_THREADS, FACTOR_SMEM, st>>>(rm_dev, J * NB, shift_rel, status_dev);
+    k_factor_block<<<nm, FACTOR_THREADS, 0, st>>>(rm_dev, J * NB, shift_rel, status_dev);
     for (int phase = 0; phase < 2; ++phase) {
       const int below = blocks - 1 - J, tiles = (phase == 0 ? below : below * (below + 1) / 2) + J;
       if (tiles) k_factor_tiles<<<nm * tiles, split::THREADS, split::SMEM_BYTES, st>>>(rm_dev, J, phase, tiles, status_dev);

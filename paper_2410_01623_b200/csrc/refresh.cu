@@ -120,8 +120,7 @@ k_gauss(const RefreshMat* __restrict__ rm) {
 }
 
 // ------------------------------------------------------------------ parts
-// What is kept as parts: G (which = 0, once) and L^-T (which = 1).  Eight neighbours per thread; the columns
-// between a matrix's width and its pitch become zeros.
+// G as parts, once.  Eight neighbours per thread; the columns between its width and its pitch become zeros.
 template <typename T>
 __device__ __forceinline__ void to_parts(const T* src, long long ld, const PartMatrix& p) {
   const bool vec = ld * (long long)sizeof(T) % 16 == 0 && reinterpret_cast<unsigned long long>(src) % 16 == 0;
@@ -134,11 +133,10 @@ __device__ __forceinline__ void to_parts(const T* src, long long ld, const PartM
   }
 }
 __global__ void __launch_bounds__(256)
-k_to_parts(const RefreshMat* __restrict__ rm, int which) {
+k_to_parts(const RefreshMat* __restrict__ rm) {
   const RefreshMat& m = rm[blockIdx.y];
   if (m.tc) return;
-  if (which == 1) to_parts(m.U, m.r, m.Up);
-  else if (m.bf16) to_parts((const __nv_bfloat16*)m.G, m.ld, m.Gp);
+  if (m.bf16) to_parts((const __nv_bfloat16*)m.G, m.ld, m.Gp);
   else to_parts((const float*)m.G, m.ld, m.Gp);
 }
 
@@ -163,39 +161,15 @@ k_store_projection(const RefreshMat* __restrict__ rm) {
   }
 }
 
-// bf16 operands of the products with U = L^-T: hi = bf16(x) and, if asked for, lo = bf16(x - hi).
-__global__ void __launch_bounds__(256)
-k_split_inverse(const RefreshMat* __restrict__ rm, int with_lo) {
-  const RefreshMat& m = rm[blockIdx.y];
-  if (!m.tc) return;
-  const float* src = m.U;
-  __nv_bfloat16 *hi = m.Ub[0], *lo = m.Ub[1];
-  const long long quads = (long long)m.r * m.r / 4;      // r is a multiple of 128
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < quads;
-       q += (long long)gridDim.x * blockDim.x) {
-    const float4 v = reinterpret_cast<const float4*>(src)[q];
-    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-    uint2 u;
-    u.x = *reinterpret_cast<const unsigned*>(&a); u.y = *reinterpret_cast<const unsigned*>(&b);
-    reinterpret_cast<uint2*>(hi)[q] = u;
-    if (with_lo) {
-      const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
-      const __nv_bfloat162 c = __floats2bfloat162_rn(v.x - fa.x, v.y - fa.y), e = __floats2bfloat162_rn(v.z - fb.x, v.w - fb.y);
-      uint2 w;
-      w.x = *reinterpret_cast<const unsigned*>(&c); w.y = *reinterpret_cast<const unsigned*>(&e);
-      reinterpret_cast<uint2*>(lo)[q] = w;
-    }
-  }
-}
-
-// U <- 0, once: its blocks below the diagonal are never written.
+// U <- 0 in all its forms, once: what is below the diagonal is never written.
 __global__ void __launch_bounds__(256)
 k_clear_inverse(const RefreshMat* __restrict__ rm) {
   const RefreshMat& m = rm[blockIdx.y];
-  const long long total = (long long)m.r * m.r;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x)
-    m.U[i] = 0.f;
+  const long long total = (long long)m.r * m.r, first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < total; i += step) m.U[i] = 0.f;
+  uint4* p = reinterpret_cast<uint4*>(m.tc ? m.Ub[0] : m.Up.base);      // (two or three forms, one behind the other)
+  const long long units = (m.tc ? 2 * total : 3 * m.Up.part_stride) / 8;
+  for (long long i = first; i < units; i += step) p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // descriptor tables of a chunk: per-matrix entries plus alignment slack
@@ -457,12 +431,10 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
       return ntc ? tc_gemm_run(c, tab[tc_kind], ntc, jtiles[tc_kind], st) : FIRA_OK;
     };
     // CholeskyQR of an iterate: Gram product, U = L^-T, application.
-    auto orth = [&](int tc_gram, int part_gram, bool split, float shift, int tc_apply, int part_apply) -> fira_status {
+    auto orth = [&](int tc_gram, int part_gram, float shift, int tc_apply, int part_apply) -> fira_status {
       fira_status s = run(tc_gram, part_gram);
       if (s != FIRA_OK) return s;
       RF_CUDA(factor_and_invert(rm_dev, nm, rmax, shift, c->status_dev, st));
-      if (nparts) k_to_parts<<<ew_grid(umax, 8), 256, 0, st>>>(rm_dev, 1);
-      if (ntc) k_split_inverse<<<ew_grid(umax, 4), 256, 0, st>>>(rm_dev, split ? 1 : 0);
       return run(tc_apply, part_apply);
     };
     // split: the iterate enters the products with its bf16 remainder and the orthonormalisation has split operands; the
@@ -472,17 +444,17 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
     auto round_y = [&](bool split, bool split_follows) -> fira_status {
       fira_status s = run(split ? JOB_AZ_SPLIT : JOB_AZ, PART_AZ);
       if (s == FIRA_OK)
-        s = orth(split ? JOB_GRAM_Y_SPLIT : JOB_GRAM_Y, PART_GRAM_Y, split, 1e-6f,
+        s = orth(split ? JOB_GRAM_Y_SPLIT : JOB_GRAM_Y, PART_GRAM_Y, 1e-6f,
                  split ? JOB_APPLY_Y_SPLIT : split_follows ? JOB_APPLY_Y_LO : JOB_APPLY_Y, PART_APPLY_Y);
-      if (s == FIRA_OK && split) s = orth(JOB_GRAM_Y2_SPLIT, PART_GRAM_Y2, true, 0.f, JOB_APPLY_Y2_SPLIT, PART_APPLY_Y2);
+      if (s == FIRA_OK && split) s = orth(JOB_GRAM_Y2_SPLIT, PART_GRAM_Y2, 0.f, JOB_APPLY_Y2_SPLIT, PART_APPLY_Y2);
       return s;
     };
     auto round_z = [&](bool split) -> fira_status {
       const fira_status s = run(split ? JOB_ATY_SPLIT : JOB_ATY, PART_ATY);
       if (s != FIRA_OK) return s;
-      return orth(split ? JOB_GRAM_Z_SPLIT : JOB_GRAM_Z, PART_GRAM_Z, split, 1e-6f, split ? JOB_APPLY_Z_SPLIT : JOB_APPLY_Z, PART_APPLY_Z);
+      return orth(split ? JOB_GRAM_Z_SPLIT : JOB_GRAM_Z, PART_GRAM_Z, 1e-6f, split ? JOB_APPLY_Z_SPLIT : JOB_APPLY_Z, PART_APPLY_Z);
     };
-    if (nparts) k_to_parts<<<ew_grid(gmax, 8), 256, 0, st>>>(rm_dev, 0);
+    if (nparts) k_to_parts<<<ew_grid(gmax, 8), 256, 0, st>>>(rm_dev);
     k_clear_inverse<<<ew_grid(umax, 4), 256, 0, st>>>(rm_dev);
     k_gauss<<<ew_grid(zmax, 4), 256, 0, st>>>(rm_dev);
     fira_status prs = round_y(iters == 0, iters == 1);
