@@ -87,6 +87,8 @@ k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsig
   __shared__ float red[FACTOR_THREADS / 32];
   const RefreshMat& m = rm[blockIdx.x];
   const int r = m.r, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   if (J0 >= r) return;
   const int nb = min(NB, r - J0);
   const float* C = m.C + (long long)J0 * r + J0;
@@ -179,9 +181,11 @@ k_factor_block(const RefreshMat* __restrict__ rm, int J0, float shift_rel, unsig
       }
 #pragma unroll
       for (int k = 0; k < PANEL; ++k) {
-        float pv = d[k][k];
-        if (c0 + k < nb && !(pv > floor_pivot && pv < INFINITY)) { bad = true; pv = floor_pivot; }
-        float s = rsqrtf(pv);
+        // (a pivot that is not a positive finite number becomes the bound it misses; padding's are 1)
+        const float pv = fminf(fmaxf(d[k][k], c0 + k < nb ? floor_pivot : 0.f), 3.4e38f);
+        bad |= pv != d[k][k];
+        float s;
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(pv));
         s = s * (1.5f - 0.5f * pv * s * s);     // one Newton step: to working precision
         v[k] *= s;
 #pragma unroll
@@ -251,6 +255,8 @@ k_factor_tiles(const RefreshMat* __restrict__ rm, int J, int phase, int tiles_pe
   const RefreshMat& m = rm[blockIdx.x / tiles_per_matrix];
   int t = blockIdx.x % tiles_per_matrix;
   const int r = m.r, blocks = (r + NB - 1) / NB, below = blocks - 1 - J, J0 = J * NB;
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   if (J >= blocks) return;
   const int nj = min(NB, r - J0);
   const int ours = phase == 0 ? below : below * (below + 1) / 2;    // tiles of the factor; then J tiles of the inverse
@@ -310,11 +316,12 @@ cudaError_t factor_and_invert(const RefreshMat* rm_dev, int nm, int rmax, float 
   if (e != cudaSuccess) return e;
   const int blocks = (rmax + NB - 1) / NB;
   for (int J = 0; J < blocks; ++J) {
-    k_factor_block<<<nm, FACTOR_THREADS, 0, st>>>(rm_dev, J * NB, shift_rel, status_dev);
+    if (e == cudaSuccess) e = launch_chained(k_factor_block, nm, FACTOR_THREADS, 0, st, true, 1, rm_dev, J * NB, shift_rel, status_dev);
     for (int phase = 0; phase < 2; ++phase) {
       const int below = blocks - 1 - J, tiles = (phase == 0 ? below : below * (below + 1) / 2) + J;
-      if (tiles) k_factor_tiles<<<nm * tiles, split::THREADS, split::SMEM_BYTES, st>>>(rm_dev, J, phase, tiles, status_dev);
+      if (tiles && e == cudaSuccess)
+        e = launch_chained(k_factor_tiles, nm * tiles, split::THREADS, split::SMEM_BYTES, st, true, 1, rm_dev, J, phase, tiles, status_dev);
     }
   }
-  return cudaSuccess;
+  return e;
 }

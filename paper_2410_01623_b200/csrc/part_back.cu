@@ -141,6 +141,8 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
   __syncthreads();
   ptx::cluster_sync_all();
   ptx::tc_fence_after();
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   volatile int* abort_flag = &ctl->abort_flag;
   const uint32_t slabs = ptx::smem_u32(smem), boxes_u32 = ptx::smem_u32(boxes);
   const uint32_t sets = deep ? 1u : 2u;         // accumulator sets in use
@@ -461,8 +463,9 @@ fira_status part_step_run(const PartStepPlan& plan, const MatDev* mats_dev, int 
   const BackJob* jobs = reinterpret_cast<const BackJob*>(plan.table) + (update ? plan.njobs : 0);
   const TileDev* tiles = reinterpret_cast<const TileDev*>(plan.table + align_up(plan.jobs.size())) + first;
   const int grid = 2 * std::min(count, sms / 2);
-  if (update) k_part_back<MODE_UPDATE><<<grid, THREADS, smem_bytes(MODE_UPDATE), st>>>(jobs, tiles, count, plan.deep, mats_dev, hp, status_dev);
-  else k_part_back<MODE_NORM><<<grid, THREADS, smem_bytes(MODE_NORM), st>>>(jobs, tiles, count, plan.deep, mats_dev, hp, status_dev);
+  const cudaError_t e = launch_chained(update ? k_part_back<MODE_UPDATE> : k_part_back<MODE_NORM>, grid, THREADS,
+                                       smem_bytes(update ? MODE_UPDATE : MODE_NORM), st, true, 1, jobs, tiles, count, plan.deep, mats_dev, hp, status_dev);
+  if (e != cudaSuccess) { set_error(std::string("step back-projection: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }
 

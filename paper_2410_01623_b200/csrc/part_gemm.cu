@@ -132,6 +132,8 @@ k_part_gemm(const JobDev* __restrict__ jobs, const int* __restrict__ starts, con
   __syncthreads();
   ptx::cluster_sync_all();
   ptx::tc_fence_after();
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   volatile int* abort_flag = &ctl->abort_flag;
   const uint32_t slabs = ptx::smem_u32(smem);
 
@@ -333,10 +335,11 @@ fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, int a_pa
   if (ntiles == 0) return FIRA_OK;
   const int a_bytes = a_parts * A_PART, stage_bytes = a_bytes + b_parts * B_PART;
   const char* starts = table_dev + align_up(sizeof(JobDev) * (size_t)njobs);
-  k_part_gemm<<<2 * std::min(ntiles, sms / 2), PG_THREADS, PG_SMEM_BYTES, st>>>(
-      reinterpret_cast<const JobDev*>(table_dev), reinterpret_cast<const int*>(starts),
+  const cudaError_t e = launch_chained(
+      k_part_gemm, 2 * std::min(ntiles, sms / 2), PG_THREADS, PG_SMEM_BYTES, st, true, 1, reinterpret_cast<const JobDev*>(table_dev), reinterpret_cast<const int*>(starts),
       reinterpret_cast<const TileDev*>(starts + starts_bytes()), std::min(PG_MAX_STAGES, PG_SLAB_BYTES / stage_bytes), a_bytes,
       stage_bytes, status_dev);
+  if (e != cudaSuccess) { set_error(std::string("part product: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }
 

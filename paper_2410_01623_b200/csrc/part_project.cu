@@ -159,6 +159,8 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
   __syncthreads();
   ptx::cluster_sync_all();
   ptx::tc_fence_after();
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   volatile int* abort_flag = &ctl->abort_flag;
   const uint32_t slabs = ptx::smem_u32(smem);
 
@@ -537,7 +539,9 @@ fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, i
   const ProjJob* jobs = reinterpret_cast<const ProjJob*>(plan.proj_table);
   const TileDev* tiles = reinterpret_cast<const TileDev*>(plan.proj_table + align_up(sizeof(ProjJob) * (size_t)plan.njobs)) + first;
   const int psi = psi_of(hp);
-  (psi == PSI_ADAM ? k_part_project<PSI_ADAM> : psi == PSI_RMSPROP ? k_part_project<PSI_RMSPROP> : k_part_project<PSI_ADAGRAD>)<<<2 * std::min(count, sms / 2), THREADS, SMEM_BYTES, st>>>(jobs, tiles, count, mats_dev, hp, status_dev);
+  const cudaError_t e = launch_chained(psi == PSI_ADAM ? k_part_project<PSI_ADAM> : psi == PSI_RMSPROP ? k_part_project<PSI_RMSPROP> : k_part_project<PSI_ADAGRAD>,
+                                       2 * std::min(count, sms / 2), THREADS, SMEM_BYTES, st, false, 1, jobs, tiles, count, mats_dev, hp, status_dev);
+  if (e != cudaSuccess) { set_error(std::string("step projection: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }
 

@@ -393,6 +393,8 @@ __global__ void __launch_bounds__(256)
 k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist, const int* __restrict__ row_start, int first_row,
          int rows_end, Hyper hp) {
   int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * FORM_X_ROWS;
+  ptx::grid_wait();
+  ptx::grid_launch_next();
   if (row >= rows_end) return;
   int p = find_matrix(row_start, nlist, row);
   const int end = min(row + FORM_X_ROWS, rows_end);
@@ -700,7 +702,8 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   tm->mark(st);
   if (parts) {
     const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
-    (psi == PSI_ADAM ? k_form_x<PSI_ADAM> : psi == PSI_RMSPROP ? k_form_x<PSI_RMSPROP> : k_form_x<PSI_ADAGRAD>)<<<(r1 - r0 + 8 * FORM_X_ROWS - 1) / (8 * FORM_X_ROWS), 256, 0, st>>>(pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp);
+    launch_error(launch_chained(psi == PSI_ADAM ? k_form_x<PSI_ADAM> : psi == PSI_RMSPROP ? k_form_x<PSI_RMSPROP> : k_form_x<PSI_ADAGRAD>,
+                                (r1 - r0 + 8 * FORM_X_ROWS - 1) / (8 * FORM_X_ROWS), 256, 0, st, true, 1, pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp));
   }
   tm->mark(st);
   if (only_scaling)
