@@ -806,6 +806,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   PhaseTimer* tm = &c->timer;
   const MatDev* mats = c->mats_dev;
   cudaError_t error = cudaSuccess;
+  // (not chained: these kernels are long, and chaining them cost the 1B list 2 %, 350M unchanged)
   auto chain = [&](cudaError_t e) { if (error == cudaSuccess) error = e; };
   if (c->proj_weights_dirty) {        // the stored projection has changed since the weights were taken
     k_tc_proj_weights<<<pl->wq_blocks, 256, 0, st>>>(mats, pl->list, pl->wq_off, pl->wq_blk, pl->nlist, pl->wq_dev);
@@ -832,7 +833,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     if (fuse_x_matrix(mq.d, mq.r) && mq.d < FUSE_KEEP_R_MIN_D) keep_r = false;
   }
 #define FIRA_LAUNCH_K1(PSI, FUSE, EG)                                                                       \
-  chain(launch_chained(k_tc_project<EPI_ADAM, PSI, FUSE, EG>, k1_grid, k1_threads(EG), k1_smem_bytes(EG), st, true, 1,  \
+  chain(launch_chained(k_tc_project<EPI_ADAM, PSI, FUSE, EG>, k1_grid, k1_threads(EG), k1_smem_bytes(EG), st, false, 1,  \
       pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev))
   if (hp.mode & HYPER_PSI_RMSPROP) FIRA_LAUNCH_K1(PSI_RMSPROP, 0, 1);
   else if (hp.mode & HYPER_PSI_ADAGRAD) FIRA_LAUNCH_K1(PSI_ADAGRAD, 0, 1);
@@ -846,9 +847,9 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   else FIRA_LAUNCH_K1(PSI_ADAM, 0, 1);
 #undef FIRA_LAUNCH_K1
   tm->mark(st);
-  chain(launch_chained(k_tc_colfactors, csn, 256, 0, st, true, 1, mats, pl->list, pl->nlist, pl->col_start, csa, hp));
+  chain(launch_chained(k_tc_colfactors, csn, 256, 0, st, false, 1, mats, pl->list, pl->nlist, pl->col_start, csa, hp));
   tm->mark(st);
-  chain(launch_chained(k_finalize, nq, 256, 0, st, true, 1, mats, pl->list + qa, nq, pl->npart + qa, hp, c->status_dev));
+  chain(launch_chained(k_finalize, nq, 256, 0, st, false, 1, mats, pl->list + qa, nq, pl->npart + qa, hp, c->status_dev));
   tm->mark(st);
   if (hp.mode & HYPER_ONLY_SCALING) {
     // W <- W - lr phi(R) G: no back-projection; the element-wise update works on the caller's W and
@@ -866,17 +867,17 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     if (fused && fuse_x_matrix(mq.d, mq.r)) any_fused = true; else any_plain = true;
   }
   if (any_plain)
-    chain(launch_chained(k_tc_form_x, (rsb - rsa + 7) / 8, 256, 0, st, true, 1, mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
+    chain(launch_chained(k_tc_form_x, (rsb - rsa + 7) / 8, 256, 0, st, false, 1, mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
                          hp.a_low, hp.a_res, pl->fast_dev, fused ? 1 : 0));
   if (any_fused)
-    chain(launch_chained(k_tc_fix_x, dim3(32, nq), 256, 0, st, true, 1, mats, pl->list, qa, hp.a_low, hp.a_res, hp.eps, keep_r ? 1 : 0, pl->fast_dev));
+    chain(launch_chained(k_tc_fix_x, dim3(32, nq), 256, 0, st, false, 1, mats, pl->list, qa, hp.a_low, hp.a_res, hp.eps, keep_r ? 1 : 0, pl->fast_dev));
   tm->mark(st);
   // long products keep five operand stages; short ones trade one for more epilogue boxes in flight
   if (rmax >= 1024)
-    chain(launch_chained(k_tc_back_project<5, 2>, 2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(5, 2), st, true, 1,
+    chain(launch_chained(k_tc_back_project<5, 2>, 2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(5, 2), st, false, 1,
                          pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev));
   else
-    chain(launch_chained(k_tc_back_project<4, 3>, 2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(4, 3), st, true, 1,
+    chain(launch_chained(k_tc_back_project<4, 3>, 2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(4, 3), st, false, 1,
                          pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev));
   tm->mark(st);
   launch_stage(mats, pl->stage_list, pl->nstage, pl->stage_start, sra, srn, 1, st);
