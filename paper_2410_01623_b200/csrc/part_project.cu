@@ -3,14 +3,14 @@
 //
 //   R[l][j] = sum_d G(d,l) Pi[d][j];  M, V, N (Eq. 2-4);  row sums ||N_l||^2, ||R_l||^2;  R as parts for the norm
 //
-// CTA pairs, one CTA per SM, persistent; 256 l x 128 j tiles.  Four converter warps per CTA read a slab of G (32 deep, 128 of
+// CTA pairs, one CTA per SM, persistent; 256 l x 128 j tiles.  Eight converter warps per CTA read a slab of G (32 deep, 128 of
 // its l) with ordinary loads, two slabs ahead, whatever its alignment, and write its parts in the operand's swizzled layout:
 // no copy of G in another form is made in memory.  The projection's slabs come by TMA (part_slab.cuh).  Tensor memory as in
 // part_gemm.cu: the main product alternates between two accumulators every PROMOTE of k and is summed in fp32 registers.
 //
-// Epilogue: two groups of four warps, one thread per row and half of the tile's columns.  M and V come and go as TMA boxes of
-// 128 rows x 16 columns (64-byte swizzle), updated in place, the parts of R and X leave as boxes of three parts; each group has
-// its own buffers, one thread stores them.  (Rows read and written by their threads with ordinary 32-byte accesses
+// Epilogue: two groups, each on half of the tile's columns, of two teams of four warps: a thread has one row and half of the
+// columns of its group's boxes.  M and V come and go as TMA boxes of 128 rows x 16 columns (64-byte swizzle), updated
+// in place, the parts of R and X leave as boxes of three parts; each group has its own buffers, one thread stores them.  (Rows read and written by their threads with ordinary 32-byte accesses
 // took five times as long: every access touches 32 lines.)  In the plain step (column factors, Adam) of a matrix with r <= 128, whose row sums are complete in one tile, the operand X = a_low N -
 // a_res k_l R of the update is formed here for limiter factor 1: N waits in tensor memory (the tile's small products have
 // been read) while the two halves of a row exchange their sums.  k_form_x does the rest: matrices whose limiter acted, larger
@@ -19,7 +19,7 @@
 // What bounds it: G, M and V at the copy bandwidth, closely followed by the MMAs (12 per slab).
 //
 // Warp roles: 0 producer of the projection's slabs, 1 MMA issuer (even CTA) and owner of the tensor memory, 2 M and V box loader,
-// 3-10 epilogue, 11 box storer, 12-15 converters.
+// 3-18 epilogue, 19 box storer, 20-27 converters.
 #include <string.h>
 
 #include <algorithm>
@@ -37,8 +37,8 @@ namespace {
 constexpr int STAGES = 3;
 constexpr int PROMOTE_SLABS = split::PROMOTE / PK;
 constexpr int SLAB_BYTES = 3 * (A_PART + B_PART);
-constexpr int EPI_WARPS = 8, CONV_WARPS = 4, CONV_THREADS = 32 * CONV_WARPS;
-constexpr int GROUPS = 2, GROUP_THREADS = 128;
+constexpr int EPI_WARPS = 16, CONV_WARPS = 8, CONV_THREADS = 32 * CONV_WARPS;
+constexpr int GROUPS = 2, TEAMS = 2, GROUP_THREADS = 128 * TEAMS;
 constexpr int FIRST_CONV = 4 + EPI_WARPS;                 // warp
 constexpr int THREADS = 32 * (FIRST_CONV + CONV_WARPS);
 constexpr int COLS = 16;                        // of a box
@@ -47,6 +47,7 @@ constexpr int MV_BOX = PM / 2 * COLS * 4, MV_BUF = 2 * MV_BOX;              // 8
 constexpr int OUT_PART = PM / 2 * COLS * 2, OUT_BUF = 3 * OUT_PART;         // 4 KiB; three parts
 constexpr int GROUP_BYTES = MV_BUFS * MV_BUF + OUT_BUFS * OUT_BUF;
 constexpr int BOXES = PN / 2 / COLS;            // of a group per tile
+constexpr int TCOLS = COLS / TEAMS;             // columns of a box per thread
 constexpr int UNITS = PM / 2 * PK / 8 / CONV_THREADS;      // units of eight neighbours of a slab per converter thread
 
 struct alignas(64) ProjJob {
@@ -65,10 +66,10 @@ struct ProjCtl {
   uint64_t small_empty[2];                      // the small products of a tile have been read (and N, which took their place)
   uint64_t efull[GROUPS][MV_BUFS], eready[GROUPS][MV_BUFS], eempty[GROUPS][MV_BUFS];   // M and V landed / updated / stored
   uint64_t oready[GROUPS][OUT_BUFS], oempty[GROUPS][OUT_BUFS];                         // parts written / stored
-  uint64_t sums;                                // the row sums of a tile are in place
+  uint64_t sums, sums_read;                     // the row sums of a tile are in place / have been read
   uint32_t tmem_base;
   int abort_flag;
-  float2 row_sums[2][2][PM / 2];                // [tile parity][half][row]: ||N||^2, ||R||^2
+  float2 row_sums[GROUPS * TEAMS][PM / 2];      // [group and team][row]: ||N||^2, ||R||^2
 };
 constexpr size_t SMEM_BYTES = (size_t)STAGES * SLAB_BYTES + GROUPS * GROUP_BYTES + sizeof(ProjCtl);
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
@@ -148,6 +149,7 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
       }
     }
     ptx::mbar_init(ptx::smem_u32(&ctl->sums), 32 * EPI_WARPS);
+    ptx::mbar_init(ptx::smem_u32(&ctl->sums_read), 32 * EPI_WARPS);
     ctl->abort_flag = smem_ok ? 0 : 1;
     ptx::fence_barrier_init();
   }
@@ -239,6 +241,13 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
     // ------------------------------------------------------------ box storer
     if (lane == 0 && smem_ok) {
       int mv[GROUPS] = {0, 0}, out[GROUPS] = {0, 0}; uint32_t mphase[GROUPS] = {0, 0}, ophase[GROUPS] = {0, 0}; bool ok = true;
+      // A box's buffers are handed back when the next box is on its way: its own are others (two per group), so nobody
+      // waits for what is held back, and the reading of one box overlaps the issue of the next.
+      uint32_t held_mv = 0, held_out = 0;               // barriers to arrive on (0: none)
+      auto release = [&]() {
+        if (held_mv) ptx::mbar_arrive(held_mv);
+        if (held_out) ptx::mbar_arrive(held_out);
+      };
       for (int t = pair; t < count && ok; t += npairs) {
         const TileDev d = load_tile(tiles + t);
         const ProjJob* jb = jobs + d.job;
@@ -261,17 +270,21 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
                   ptx::tma_store_2d(&jb->v, base + mv[g] * MV_BUF + MV_BOX, j, l0);
                 }
                 ptx::tma_store_3d(pass == 0 ? &jb->ro : &jb->xo, base + MV_BUFS * MV_BUF + out[g] * OUT_BUF, j, l0, 0);
-                ptx::bulk_commit_group();
-                ptx::bulk_wait_group_read<0>();          // the boxes have been read: the buffers are free
               }
+              ptx::bulk_commit_group();                  // (empty where the rows are past the matrix)
+              ptx::bulk_wait_group_read<1>();            // the box before this one has been read
+              release();
+              held_mv = 0;
               if (pass == 0) {
-                ptx::mbar_arrive(ptx::smem_u32(&ctl->eempty[g][mv[g]]));
+                held_mv = ptx::smem_u32(&ctl->eempty[g][mv[g]]);
                 if (++mv[g] == MV_BUFS) { mv[g] = 0; mphase[g] ^= 1u; }
               }
-              ptx::mbar_arrive(ptx::smem_u32(&ctl->oempty[g][out[g]]));
+              held_out = ptx::smem_u32(&ctl->oempty[g][out[g]]);
               if (++out[g] == OUT_BUFS) { out[g] = 0; ophase[g] ^= 1u; }
             }
       }
+      ptx::bulk_wait_group_read<0>();
+      release();
       ptx::bulk_wait_group_all();
     }
   } else if (warp >= FIRST_CONV) {
@@ -322,14 +335,14 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
     }
   } else if (smem_ok) {
     // ------------------------------------------------------------ epilogue
-    const int g = (warp - 3) >> 2;                      // group: half of the tile's columns
+    const int ew = (warp - 3) >> 2, g = ew & 1, h = ew >> 1;      // group: half of the tile's columns; team: half of a box's
     const int quarter = warp & 3, c0 = g * (PN / 2);    // TMEM lanes 32 * quarter .. + 31
     const int row = 32 * quarter + lane;
     const uint32_t sw = (uint32_t)(row >> 1) & 3u;      // 64-byte swizzle: slot ^= (row / 2) % 4
     unsigned char* gbase = boxes + g * GROUP_BYTES;
     int mv = 0, out = 0;
     uint32_t mphase = 0, ophase = 0;
-    const uint32_t tmem = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + c0;
+    const uint32_t tmem = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + c0 + TCOLS * h;
     const uint32_t me[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->main_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->main_empty[1]), 0)};
     const uint32_t se[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[1]), 0)};
     int piece = 0, tile = 0;
@@ -341,61 +354,70 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
       const MatDev& mt = mats[jb.mat];
       const int npieces = (d.nk + PROMOTE_SLABS - 1) / PROMOTE_SLABS;
       const uint32_t small = tmem + 2 * PN + (tile & 1) * PN;
-      float r[64];
+      float r[BOXES * TCOLS];                           // this thread's columns of every box
 #pragma unroll
-      for (int e = 0; e < 64; ++e) r[e] = 0.f;
+      for (int e = 0; e < BOXES * TCOLS; ++e) r[e] = 0.f;
+      auto add = [&](uint32_t taddr) {
+        uint32_t v[BOXES][TCOLS];
+        __syncwarp();
+#pragma unroll
+        for (int b = 0; b < BOXES; ++b) ptx::tmem_ld_32x32b_x8(taddr + COLS * b, v[b]);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int b = 0; b < BOXES; ++b)
+#pragma unroll
+          for (int e = 0; e < TCOLS; ++e) r[TCOLS * b + e] += __uint_as_float(v[b][e]);
+      };
       for (int p = 0; p < npieces; ++p, ++piece) {
         const int mb = piece & 1;
         if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->main_full[mb]), (piece >> 1) & 1, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
-        add_columns(r, tmem + mb * PN);
+        add(tmem + mb * PN);
         if (lane == 0) ptx::mbar_arrive_cluster(me[mb]);
       }
       if (!ok) break;
-      if ((jb.shape & 15) != 5) add_columns(r, small);          // G and the projection have more than one part
+      if ((jb.shape & 15) != 5) add(small);          // G and the projection have more than one part
       const int l = d.l0 + PM / 2 * (int)rank + row, j0 = d.j0 + c0, R = mt.r;
       const bool in = l < mt.l;
       const float bias = mt.sc->pad;
       const bool fused = part_forms_x(R, hp);
       float nn = 0.f, rn = 0.f;
-      // 16 values of this thread's row as parts into the next out buffer
+      // this thread's values of a box as parts into the next out buffer
       auto put_parts = [&](const float* x) {
-        unsigned char* o = gbase + MV_BUFS * MV_BUF + out * OUT_BUF + row * (COLS * 2);
+        unsigned char* o = gbase + MV_BUFS * MV_BUF + out * OUT_BUF + row * (COLS * 2) + 16 * h;
+        uint32_t hi[4], mid[4], lo[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t hi[4], mid[4], lo[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) split::split3(x[8 * h + 2 * i], x[8 * h + 2 * i + 1], hi[i], mid[i], lo[i]);
-          *reinterpret_cast<uint4*>(o + 16 * h) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          *reinterpret_cast<uint4*>(o + OUT_PART + 16 * h) = make_uint4(mid[0], mid[1], mid[2], mid[3]);
-          *reinterpret_cast<uint4*>(o + 2 * OUT_PART + 16 * h) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-        }
+        for (int i = 0; i < 4; ++i) split::split3(x[2 * i], x[2 * i + 1], hi[i], mid[i], lo[i]);
+        *reinterpret_cast<uint4*>(o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4*>(o + OUT_PART) = make_uint4(mid[0], mid[1], mid[2], mid[3]);
+        *reinterpret_cast<uint4*>(o + 2 * OUT_PART) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         ptx::fence_proxy_async_smem();
         ptx::mbar_arrive(ptx::smem_u32(&ctl->oready[g][out]));
         if (++out == OUT_BUFS) { out = 0; ophase ^= 1u; }
       };
       // The boxes of a tile are a loop (unrolled, its divisions and roots are more instructions than the caches hold:
-      // half of the time went into waiting for them), so the registers move instead of the index: four times around
-      // and r is as it was.
+      // half of the time went into waiting for them), so the registers move instead of the index: once around and r
+      // is as it was.
       auto rotate = [&]() {
-        float first[COLS];
+        float first[TCOLS];
 #pragma unroll
-        for (int e = 0; e < COLS; ++e) first[e] = r[e];
+        for (int e = 0; e < TCOLS; ++e) first[e] = r[e];
 #pragma unroll
-        for (int e = 0; e < 64 - COLS; ++e) r[e] = r[e + COLS];
+        for (int e = 0; e < (BOXES - 1) * TCOLS; ++e) r[e] = r[e + TCOLS];
 #pragma unroll
-        for (int e = 0; e < COLS; ++e) r[64 - COLS + e] = first[e];
+        for (int e = 0; e < TCOLS; ++e) r[(BOXES - 1) * TCOLS + e] = first[e];
       };
 #pragma unroll 1
       for (int q = 0; q < PN / 2; q += COLS) {
         if (j0 + q >= R) { rotate(); continue; }
         if (!ptx::mbar_wait(ptx::smem_u32(&ctl->efull[g][mv]), mphase, abort_flag)) { ok = false; break; }
         unsigned char* mb = gbase + mv * MV_BUF + row * (COLS * 4);
-        uint32_t nw[16];
+        uint32_t nw[TCOLS];
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          float4* mp = reinterpret_cast<float4*>(mb + (((uint32_t)w ^ sw) << 4));
-          float4* vp = reinterpret_cast<float4*>(mb + MV_BOX + (((uint32_t)w ^ sw) << 4));
+        for (int w = 0; w < TCOLS / 4; ++w) {
+          const uint32_t slot = ((uint32_t)(TCOLS / 4 * h + w) ^ sw) << 4;
+          float4* mp = reinterpret_cast<float4*>(mb + slot);
+          float4* vp = reinterpret_cast<float4*>(mb + MV_BOX + slot);
           const float4 m4 = *mp, v4 = *vp;
           float m[4] = {m4.x, m4.y, m4.z, m4.w}, v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
@@ -414,42 +436,44 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
         if (++mv == MV_BUFS) { mv = 0; mphase ^= 1u; }
         if (fused) {
           __syncwarp();
-          ptx::tmem_st_32x32b_x16(small + q, nw);
+          ptx::tmem_st_32x32b_x8(small + q, nw);
         }
         if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oempty[g][out]), ophase ^ 1u, abort_flag)) { ok = false; break; }
         put_parts(r);
         rotate();
       }
       if (!ok) break;
+      float2(*xs)[PM / 2] = ctl->row_sums;
+      if (!ptx::mbar_wait(ptx::smem_u32(&ctl->sums_read), yphase ^ 1u, abort_flag)) break;      // the tile before
+      xs[2 * g + h][row] = make_float2(nn, rn);
+      if (fused) ptx::tmem_st_wait();
+      ptx::mbar_arrive(ptx::smem_u32(&ctl->sums));
+      if (!ptx::mbar_wait(ptx::smem_u32(&ctl->sums), yphase, abort_flag)) break;
+      yphase ^= 1u;
+      const float2 a = xs[2 * g][row], b = xs[2 * g + 1][row], oa = xs[2 * (g ^ 1)][row], ob = xs[2 * (g ^ 1) + 1][row];
+      ptx::mbar_arrive(ptx::smem_u32(&ctl->sums_read));
       if (hp.mode & HYPER_NO_SCALING) {
-        if (in && g == 0 && d.j0 == 0) mt.kvec[l] = 1.f;
+        if (in && ew == 0 && d.j0 == 0) mt.kvec[l] = 1.f;
       } else if (!fused) {
-        if (in && j0 < R) {
+        if (in && h == 0 && j0 < R) {
           const int slot = j0 / 64;
-          mt.aux[(long long)slot * mt.l + l] = nn;
-          mt.aux[(long long)(mt.aux_slots + slot) * mt.l + l] = rn;
+          mt.aux[(long long)slot * mt.l + l] = a.x + b.x;
+          mt.aux[(long long)(mt.aux_slots + slot) * mt.l + l] = a.y + b.y;
         }
       }
       if (fused) {
-        float2(*xs)[PM / 2] = ctl->row_sums[tile & 1];
-        xs[g][row] = make_float2(nn, rn);
-        ptx::tmem_st_wait();
-        ptx::mbar_arrive(ptx::smem_u32(&ctl->sums));
-        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->sums), yphase, abort_flag)) break;
-        yphase ^= 1u;
-        const float2 a = xs[0][row], b = xs[1][row];
-        const float k = sqrtf(a.x + b.x) / (sqrtf(a.y + b.y) + hp.eps);
-        if (in && g == 0) mt.kvec[l] = k;
+        const float k = sqrtf((a.x + b.x) + (oa.x + ob.x)) / (sqrtf((a.y + b.y) + (oa.y + ob.y)) + hp.eps);
+        if (in && ew == 0) mt.kvec[l] = k;
         const float c = hp.a_res * k;
 #pragma unroll 1
         for (int q = 0; q < PN / 2 && j0 + q < R; q += COLS) {
-          uint32_t nw[16];
-          float x[16];
+          uint32_t nw[TCOLS];
+          float x[TCOLS];
           __syncwarp();
-          ptx::tmem_ld_32x32b_x16(small + q, nw);
+          ptx::tmem_ld_32x32b_x8(small + q, nw);
           ptx::tmem_ld_wait();
 #pragma unroll
-          for (int e = 0; e < 16; ++e) x[e] = hp.a_low * __uint_as_float(nw[e]) - c * r[e];
+          for (int e = 0; e < TCOLS; ++e) x[e] = hp.a_low * __uint_as_float(nw[e]) - c * r[e];
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oempty[g][out]), ophase ^ 1u, abort_flag)) { ok = false; break; }
           put_parts(x);
           rotate();
