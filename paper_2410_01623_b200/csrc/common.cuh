@@ -43,10 +43,9 @@ struct MatDev {
   float* step_bias;   //   "      this step's bias factor (k_finalize puts the next one into MatScalars)
   int rp_pitch, pp_pitch;
   int aux_slots;      // row sums per l in aux
-  int tma_proj;       // long lists: the projection is part_project.cu's (slots of 64 columns), otherwise k_project's (of 128)
   float* kvec;        // scratch: l factors
   float* part;        // scratch: partial sums of ||S||^2
-  float* aux;         // scratch: row sums [aux_slots][l] of ||N_l||^2, then of ||R_l||^2 (engine 0: one slot per tile of r)
+  float* aux;         // scratch: row sums [aux_slots][l] of ||N_l||^2, then of ||R_l||^2 (engine 0, short lists: one slot per tile of r)
   __nv_bfloat16* Nb;  // scratch of the tensor-core path: l x r bf16 N
   __nv_bfloat16* Rb;  //   "      l x r bf16 R
   __nv_bfloat16* Xb;  //   "      l x r bf16 X

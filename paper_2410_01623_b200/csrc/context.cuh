@@ -60,7 +60,6 @@ struct Layout {
   std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux, offRp, offXp, offPp, offBias;
   std::vector<int> engine;
   bool parts = false;       // the fp32-precision engine's list is long
-  bool tma_proj = false;    // and its projection runs on part_project.cu
   size_t off_parts = 0, off_proj_parts = 0;
   size_t step_work_bytes = 0, refresh_min_bytes = 0;
   size_t scratch_bytes = 0;

@@ -66,7 +66,7 @@ static long long part_staging_pitch(const fira_matrix_desc& d, uint32_t flags) {
 }
 
 // Row sums per l: one per tile of R, whose width depends on the kernels.
-static int aux_slots(const Layout& L, int i, int r) { return L.engine[i] == 1 ? 1 : L.tma_proj ? (r + 63) / 64 : simt_tiles(r); }
+static int aux_slots(const Layout& L, int i, int r) { return L.engine[i] == 1 || L.parts ? 1 : simt_tiles(r); }
 
 constexpr size_t REFRESH_SMALL_LIST_BYTES = (size_t)512 << 20;
 
@@ -102,12 +102,10 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
         ptiles += part_project_tiles(std::max(descs[i].m, descs[i].n), descs[i].r);
       }
     L.parts = !own.empty() && simt_long_list(own);
-    L.tma_proj = L.parts;             // M and V move as TMA boxes: rows on 16-byte boundaries
-    for (const fira_matrix_desc& d : own) L.tma_proj = L.tma_proj && d.r % 4 == 0;
     L.off_parts = wo;
     if (L.parts) wo += part_step_table_bytes((int)own.size(), tiles);
     L.off_proj_parts = wo;
-    if (L.tma_proj) wo += part_project_table_bytes((int)own.size(), ptiles);
+    if (L.parts) wo += part_project_table_bytes((int)own.size(), ptiles);
   }
   L.off_work = wo;
   size_t w = 0;
@@ -260,7 +258,6 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
     mt.aux = (float*)(c->work_base + L.offAux[i]);
     mt.part = (float*)(c->work_base + L.offPart[i]);
     mt.aux_slots = aux_slots(L, i, d.r);
-    mt.tma_proj = L.tma_proj && mt.engine == 0;
     if (mt.engine == 0) {
       if (L.parts) {
         mt.Rp = (__nv_bfloat16*)(c->work_base + L.offRp[i]);
@@ -316,7 +313,10 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
     c->simt.mats = c->mats_dev;
     c->simt.list = c->ints_dev + o_list; c->simt.nlist = (int)lst.size();
     c->simt.proj_tile_start = c->ints_dev + o_pt; c->simt.proj_tiles = pt.back();
-    for (int i : c->simt_list) c->simt.max_d = std::max(c->simt.max_d, c->mats[i].d);
+    for (int i : c->simt_list) {
+      c->simt.max_d = std::max(c->simt.max_d, c->mats[i].d);
+      c->simt.max_r = std::max(c->simt.max_r, c->mats[i].r);
+    }
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
     c->simt.npart = c->ints_dev + o_np; c->simt.npart_tiles = c->ints_dev + o_npt;
     c->simt.row_start = c->ints_dev + o_rs; c->simt.h_row_start = rs;
@@ -326,7 +326,7 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
   }
   fira_status ts = FIRA_OK;
   if (L.parts) ts = part_step_prepare(c->mats, c->simt_list, c->scratch_base + L.off_parts, &c->simt.parts, c->stream);
-  if (L.tma_proj && ts == FIRA_OK) ts = part_project_prepare(c->mats, c->simt_list, c->scratch_base + L.off_proj_parts, &c->simt.parts, c->stream);
+  if (L.parts && ts == FIRA_OK) ts = part_project_prepare(c->mats, c->simt_list, c->scratch_base + L.off_proj_parts, &c->simt.parts, c->stream);
   if (ts == FIRA_OK) ts = tc_build_plan(c, ints);
   if (ts != FIRA_OK) { tc_destroy_plan(c); delete c; return ts; }
   if (ints.size() > c->ints_count) { set_error("internal: schedule arrays overflow"); tc_destroy_plan(c); delete c; return FIRA_ERR_INVALID_ARG; }

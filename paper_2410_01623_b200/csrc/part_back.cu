@@ -68,16 +68,10 @@ __device__ __forceinline__ TileDev load_tile(const TileDev* t) {
   return TileDev{v.x, v.y, v.z, v.w};
 }
 
-// The factor k_l.  The norm comes first: it makes the factor from the row sums (unless the projection's epilogue has) and (keep)
-// leaves it in the k table.
+// The factor k_l; the norm of a matrix with one factor is scaled in the end.
 template <int MODE>
-__device__ __forceinline__ float step_factor(const MatDev& mt, int l, const Hyper& hp, bool keep) {
-  if (MODE == MODE_UPDATE) return mt.kvec[l];
-  if (hp.mode & (HYPER_NO_SCALING | HYPER_MATRIX_SCALING)) return 1.f;
-  if (factors_ready(mt, hp)) return mt.kvec[l];
-  const float k = row_factor(mt, l, hp);
-  if (keep) mt.kvec[l] = k;
-  return k;
+__device__ __forceinline__ float step_factor(const MatDev& mt, int l, const Hyper& hp) {
+  return MODE == MODE_NORM && (hp.mode & HYPER_MATRIX_SCALING) ? 1.f : mt.kvec[l];
 }
 
 __device__ __forceinline__ void unpack(const uint4& u, float (&v)[4]) {
@@ -263,10 +257,10 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
       if (left) {
         if (tid_g < KS) {                                // column x of the group's boxes, one box after the other
           const int j = d.j0 + (GROUPS * (tid_g / cols) + g) * cols + tid_g % cols;
-          ks[tid_g] = j < n ? step_factor<MODE>(mt, j, hp, i0 == 0) : 0.f;
+          ks[tid_g] = j < n ? step_factor<MODE>(mt, j, hp) : 0.f;
         }
       } else if (i0 + row < m) {
-        krow = step_factor<MODE>(mt, i0 + row, hp, d.j0 == 0 && g == 0);
+        krow = step_factor<MODE>(mt, i0 + row, hp);
       }
       ptx::mbar_arrive(esync);                           // the group's factors are in place
       if (!ptx::mbar_wait(esync, yphase, abort_flag)) break;

@@ -43,7 +43,7 @@ fira_status part_gemm_prepare(const PartGemm* jobs, int njobs, char* table_dev, 
 // One grouped launch over the prepared jobs.  a_parts, b_parts: the most parts that an operand of theirs has.
 fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, int a_parts, int b_parts, unsigned* status_dev, cudaStream_t st);
 
-// ---- the three products of the fp32-precision step, with their epilogues, for long lists: the projection (part_project.cu),
+// ---- the three products of the fp32-precision step for long lists: the projection (part_project.cu),
 // D = Pi R and D = Pi X (part_back.cu); R, X and Pi are kept as parts.
 struct PartStepPlan {
   const char* table = nullptr;      // device; null: the list is short, its products split their operands themselves
@@ -59,12 +59,11 @@ constexpr int PART_SUMS_PER_TILE = 16;   // partial sums of ||S||^2 that a tile 
 inline int part_rank_pitch(int r) { return (r + 7) / 8 * 8; }
 inline int part_step_tiles(int m, int n) { return ((m + 255) / 256) * ((n + 127) / 128); }
 inline int part_project_tiles(int l, int r) { return ((l + 255) / 256) * ((r + 127) / 128); }
-// Whether the projection's epilogue forms X (for limiter factor 1): the plain step of a matrix whose row sums are complete
-// in one tile.
-__host__ __device__ inline bool part_forms_x(int r, const Hyper& hp) { return r <= 128 && hp.mode == 0; }
+// Whether k_moments forms X (for limiter factor 1): its factors are known row by row.
+__host__ __device__ inline bool part_forms_x(const Hyper& hp) { return !(hp.mode & (HYPER_MATRIX_SCALING | HYPER_ONLY_SCALING)); }
 size_t part_project_table_bytes(int njobs, int ntiles);
 fira_status part_project_prepare(const std::vector<MatDev>& mats, const std::vector<int>& list, char* table_dev, PartStepPlan* plan, cudaStream_t st);
-fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, const Hyper& hp, unsigned* status_dev, cudaStream_t st);
+fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, unsigned* status_dev, cudaStream_t st);
 size_t part_step_table_bytes(int njobs, int ntiles);
 // mats: the host copies of the problem table, list: the indices of this engine's matrices in it.
 fira_status part_step_prepare(const std::vector<MatDev>& mats, const std::vector<int>& list, char* table_dev, PartStepPlan* plan, cudaStream_t st);

@@ -1,25 +1,22 @@
-// The step's projection R = G^T Pi (or G Pi) with Adam in its epilogue, in fp32 precision, for long lists (part_gemm.cuh:
-// PartStepPlan).  G is split into bf16 parts on its way into shared memory, the projection is kept as parts.
+// The step's projection R = G^T Pi (or G Pi) in fp32 precision, for long lists (part_gemm.cuh: PartStepPlan).  G is split
+// into bf16 parts on its way into shared memory, the projection is kept as parts, R is left as parts.
 //
-//   R[l][j] = sum_d G(d,l) Pi[d][j];  M, V, N (Eq. 2-4);  row sums ||N_l||^2, ||R_l||^2;  R as parts for the norm
+//   R[l][j] = sum_d G(d,l) Pi[d][j]
 //
 // CTA pairs, one CTA per SM, persistent; 256 l x 128 j tiles.  Eight converter warps per CTA read a slab of G (32 deep, 128 of
 // its l) with ordinary loads, two slabs ahead, whatever its alignment, and write its parts in the operand's swizzled layout:
 // no copy of G in another form is made in memory.  The projection's slabs come by TMA (part_slab.cuh).  Tensor memory as in
 // part_gemm.cu: the main product alternates between two accumulators every PROMOTE of k and is summed in fp32 registers.
 //
-// Epilogue: two groups, each on half of the tile's columns, of two teams of four warps: a thread has one row and half of the
-// columns of its group's boxes.  M and V come and go as TMA boxes of 128 rows x 16 columns (64-byte swizzle), updated
-// in place, the parts of R and X leave as boxes of three parts; each group has its own buffers, one thread stores them.  (Rows read and written by their threads with ordinary 32-byte accesses
-// took five times as long: every access touches 32 lines.)  In the plain step (column factors, Adam) of a matrix with r <= 128, whose row sums are complete in one tile, the operand X = a_low N -
-// a_res k_l R of the update is formed here for limiter factor 1: N waits in tensor memory (the tile's small products have
-// been read) while the two halves of a row exchange their sums.  k_form_x does the rest: matrices whose limiter acted, larger
-// ranks, the variants.
+// Epilogue: two groups of four warps, each on half of the tile's columns, one row per thread; R's parts leave as TMA boxes of
+// 128 rows x 16 columns x three parts.  The moments are a pass of their own (k_moments).  With Adam in this epilogue, M and V as
+// boxes, the epilogue took 30000 cycles per tile and the product, whose main accumulators wait for the same warps
+// every PROMOTE of k, stood still for half of them: MEASURE.
 //
-// What bounds it: G, M and V at the copy bandwidth, closely followed by the MMAs (12 per slab).
+// What bounds it: the MMAs (12 per slab), G at the copy bandwidth close behind.
 //
-// Warp roles: 0 producer of the projection's slabs, 1 MMA issuer (even CTA) and owner of the tensor memory, 2 M and V box loader,
-// 3-18 epilogue, 19 box storer, 20-27 converters.
+// Warp roles: 0 producer of the projection's slabs, 1 MMA issuer (even CTA) and owner of the tensor memory, 2-9 epilogue,
+// 10 box storer, 11-18 converters.
 #include <string.h>
 
 #include <algorithm>
@@ -34,26 +31,23 @@ namespace fira {
 
 namespace {
 
-constexpr int STAGES = 3;
+constexpr int STAGES = 4;
 constexpr int PROMOTE_SLABS = split::PROMOTE / PK;
 constexpr int SLAB_BYTES = 3 * (A_PART + B_PART);
-constexpr int EPI_WARPS = 16, CONV_WARPS = 8, CONV_THREADS = 32 * CONV_WARPS;
-constexpr int GROUPS = 2, TEAMS = 2, GROUP_THREADS = 128 * TEAMS;
-constexpr int FIRST_CONV = 4 + EPI_WARPS;                 // warp
+constexpr int EPI_WARPS = 8, CONV_WARPS = 8, CONV_THREADS = 32 * CONV_WARPS;
+constexpr int GROUPS = 2, GROUP_THREADS = 128;
+constexpr int FIRST_CONV = 3 + EPI_WARPS;                 // warp
 constexpr int THREADS = 32 * (FIRST_CONV + CONV_WARPS);
 constexpr int COLS = 16;                        // of a box
-constexpr int MV_BUFS = 2, OUT_BUFS = 2;        // per group
-constexpr int MV_BOX = PM / 2 * COLS * 4, MV_BUF = 2 * MV_BOX;              // 8 KiB; M and V
+constexpr int OUT_BUFS = 2;                     // per group
 constexpr int OUT_PART = PM / 2 * COLS * 2, OUT_BUF = 3 * OUT_PART;         // 4 KiB; three parts
-constexpr int GROUP_BYTES = MV_BUFS * MV_BUF + OUT_BUFS * OUT_BUF;
+constexpr int GROUP_BYTES = OUT_BUFS * OUT_BUF;
 constexpr int BOXES = PN / 2 / COLS;            // of a group per tile
-constexpr int TCOLS = COLS / TEAMS;             // columns of a box per thread
 constexpr int UNITS = PM / 2 * PK / 8 / CONV_THREADS;      // units of eight neighbours of a slab per converter thread
 
 struct alignas(64) ProjJob {
   CUtensorMap b;                                // the projection's parts, [d][r]
-  CUtensorMap m, v;                             // [l][r] fp32
-  CUtensorMap ro, xo;                           // parts of R and X, [3][l][r]
+  CUtensorMap ro;                               // parts of R, [3][l][r]
   int mat;                                      // index into the problem table
   int shape;                                    // see issue_parts
 };
@@ -63,13 +57,10 @@ struct TileDev { int job, l0, j0, nk; };
 struct ProjCtl {
   uint64_t full[STAGES], empty[STAGES];
   uint64_t main_full[2], main_empty[2];         // a piece of the main product is complete / has been read
-  uint64_t small_empty[2];                      // the small products of a tile have been read (and N, which took their place)
-  uint64_t efull[GROUPS][MV_BUFS], eready[GROUPS][MV_BUFS], eempty[GROUPS][MV_BUFS];   // M and V landed / updated / stored
-  uint64_t oready[GROUPS][OUT_BUFS], oempty[GROUPS][OUT_BUFS];                         // parts written / stored
-  uint64_t sums, sums_read;                     // the row sums of a tile are in place / have been read
+  uint64_t small_empty[2];                      // the small products of a tile have been read
+  uint64_t oready[GROUPS][OUT_BUFS], oempty[GROUPS][OUT_BUFS];   // R's parts written / stored
   uint32_t tmem_base;
   int abort_flag;
-  float2 row_sums[GROUPS * TEAMS][PM / 2];      // [group and team][row]: ||N||^2, ||R||^2
 };
 constexpr size_t SMEM_BYTES = (size_t)STAGES * SLAB_BYTES + GROUPS * GROUP_BYTES + sizeof(ProjCtl);
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
@@ -116,10 +107,9 @@ struct Slab {
   }
 };
 
-template <int PSI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ tiles, int count, const MatDev* __restrict__ mats,
-               Hyper hp, unsigned* __restrict__ status) {
+               unsigned* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* boxes = smem + STAGES * SLAB_BYTES;
   ProjCtl* ctl = reinterpret_cast<ProjCtl*>(boxes + GROUPS * GROUP_BYTES);
@@ -137,19 +127,11 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
       ptx::mbar_init(ptx::smem_u32(&ctl->main_empty[b]), 2 * EPI_WARPS);
       ptx::mbar_init(ptx::smem_u32(&ctl->small_empty[b]), 2 * EPI_WARPS);
     }
-    for (int g = 0; g < GROUPS; ++g) {
-      for (int b = 0; b < MV_BUFS; ++b) {
-        ptx::mbar_init(ptx::smem_u32(&ctl->efull[g][b]), 1);
-        ptx::mbar_init(ptx::smem_u32(&ctl->eready[g][b]), GROUP_THREADS);
-        ptx::mbar_init(ptx::smem_u32(&ctl->eempty[g][b]), 1);
-      }
+    for (int g = 0; g < GROUPS; ++g)
       for (int b = 0; b < OUT_BUFS; ++b) {
         ptx::mbar_init(ptx::smem_u32(&ctl->oready[g][b]), GROUP_THREADS);
         ptx::mbar_init(ptx::smem_u32(&ctl->oempty[g][b]), 1);
       }
-    }
-    ptx::mbar_init(ptx::smem_u32(&ctl->sums), 32 * EPI_WARPS);
-    ptx::mbar_init(ptx::smem_u32(&ctl->sums_read), 32 * EPI_WARPS);
     ctl->abort_flag = smem_ok ? 0 : 1;
     ptx::fence_barrier_init();
   }
@@ -214,77 +196,35 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
         ++tile;
       }
     }
-  } else if (warp == 2) {
-    // ------------------------------------------------------------ M and V box loader
-    if (lane == 0 && smem_ok) {
-      int buf[GROUPS] = {0, 0}; uint32_t phase[GROUPS] = {0, 0}; bool ok = true;
-      for (int t = pair; t < count && ok; t += npairs) {
-        const TileDev d = load_tile(tiles + t);
-        const ProjJob* jb = jobs + d.job;
-        const int l0 = d.l0 + PM / 2 * (int)rank, R = mats[jb->mat].r;
-        for (int b = 0; b < BOXES && ok; ++b)
-#pragma unroll
-          for (int g = 0; g < GROUPS; ++g) {
-            const int j = d.j0 + g * (PN / 2) + b * COLS;
-            if (j >= R) continue;
-            if (!ptx::mbar_wait(ptx::smem_u32(&ctl->eempty[g][buf[g]]), phase[g] ^ 1u, abort_flag)) { ok = false; break; }
-            const uint32_t fb = ptx::smem_u32(&ctl->efull[g][buf[g]]);
-            const uint32_t dst = slabs + STAGES * SLAB_BYTES + g * GROUP_BYTES + buf[g] * MV_BUF;
-            ptx::mbar_expect_tx(fb, MV_BUF);
-            ptx::tma_load_2d(dst, &jb->m, fb, j, l0);
-            ptx::tma_load_2d(dst + MV_BOX, &jb->v, fb, j, l0);
-            if (++buf[g] == MV_BUFS) { buf[g] = 0; phase[g] ^= 1u; }
-          }
-      }
-    }
-  } else if (warp == 3 + EPI_WARPS) {
+  } else if (warp == 2 + EPI_WARPS) {
     // ------------------------------------------------------------ box storer
     if (lane == 0 && smem_ok) {
-      int mv[GROUPS] = {0, 0}, out[GROUPS] = {0, 0}; uint32_t mphase[GROUPS] = {0, 0}, ophase[GROUPS] = {0, 0}; bool ok = true;
-      // A box's buffers are handed back when the next box is on its way: its own are others (two per group), so nobody
+      int out[GROUPS] = {0, 0}; uint32_t ophase[GROUPS] = {0, 0}; bool ok = true;
+      // A box's buffer is handed back when the next box is on its way: that one has another (two per group), so nobody
       // waits for what is held back, and the reading of one box overlaps the issue of the next.
-      uint32_t held_mv = 0, held_out = 0;               // barriers to arrive on (0: none)
-      auto release = [&]() {
-        if (held_mv) ptx::mbar_arrive(held_mv);
-        if (held_out) ptx::mbar_arrive(held_out);
-      };
+      uint32_t held = 0;                                // barrier to arrive on (0: none)
       for (int t = pair; t < count && ok; t += npairs) {
         const TileDev d = load_tile(tiles + t);
         const ProjJob* jb = jobs + d.job;
         const MatDev& mt = mats[jb->mat];
         const int l0 = d.l0 + PM / 2 * (int)rank, R = mt.r;
         const bool rows = l0 < mt.l;
-        const int passes = part_forms_x(R, hp) ? 2 : 1;          // R, M and V; then X
-        for (int pass = 0; pass < passes && ok; ++pass)
-          for (int b = 0; b < BOXES && ok; ++b)
+        for (int b = 0; b < BOXES && ok; ++b)
 #pragma unroll
-            for (int g = 0; g < GROUPS; ++g) {
-              const int j = d.j0 + g * (PN / 2) + b * COLS;
-              if (j >= R) continue;
-              if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oready[g][out[g]]), ophase[g], abort_flag)) { ok = false; break; }
-              if (pass == 0 && !ptx::mbar_wait(ptx::smem_u32(&ctl->eready[g][mv[g]]), mphase[g], abort_flag)) { ok = false; break; }
-              const uint32_t base = slabs + STAGES * SLAB_BYTES + g * GROUP_BYTES;
-              if (rows) {
-                if (pass == 0) {
-                  if (PSI == PSI_ADAM) ptx::tma_store_2d(&jb->m, base + mv[g] * MV_BUF, j, l0);
-                  ptx::tma_store_2d(&jb->v, base + mv[g] * MV_BUF + MV_BOX, j, l0);
-                }
-                ptx::tma_store_3d(pass == 0 ? &jb->ro : &jb->xo, base + MV_BUFS * MV_BUF + out[g] * OUT_BUF, j, l0, 0);
-              }
-              ptx::bulk_commit_group();                  // (empty where the rows are past the matrix)
-              ptx::bulk_wait_group_read<1>();            // the box before this one has been read
-              release();
-              held_mv = 0;
-              if (pass == 0) {
-                held_mv = ptx::smem_u32(&ctl->eempty[g][mv[g]]);
-                if (++mv[g] == MV_BUFS) { mv[g] = 0; mphase[g] ^= 1u; }
-              }
-              held_out = ptx::smem_u32(&ctl->oempty[g][out[g]]);
-              if (++out[g] == OUT_BUFS) { out[g] = 0; ophase[g] ^= 1u; }
-            }
+          for (int g = 0; g < GROUPS; ++g) {
+            const int j = d.j0 + g * (PN / 2) + b * COLS;
+            if (j >= R) continue;
+            if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oready[g][out[g]]), ophase[g], abort_flag)) { ok = false; break; }
+            if (rows) ptx::tma_store_3d(&jb->ro, slabs + STAGES * SLAB_BYTES + g * GROUP_BYTES + out[g] * OUT_BUF, j, l0, 0);
+            ptx::bulk_commit_group();                  // (empty where the rows are past the matrix)
+            ptx::bulk_wait_group_read<1>();            // the box before this one has been read
+            if (held) ptx::mbar_arrive(held);
+            held = ptx::smem_u32(&ctl->oempty[g][out[g]]);
+            if (++out[g] == OUT_BUFS) { out[g] = 0; ophase[g] ^= 1u; }
+          }
       }
       ptx::bulk_wait_group_read<0>();
-      release();
+      if (held) ptx::mbar_arrive(held);
       ptx::bulk_wait_group_all();
     }
   } else if (warp >= FIRST_CONV) {
@@ -335,154 +275,55 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
     }
   } else if (smem_ok) {
     // ------------------------------------------------------------ epilogue
-    const int ew = (warp - 3) >> 2, g = ew & 1, h = ew >> 1;      // group: half of the tile's columns; team: half of a box's
+    const int g = (warp - 2) >> 2;                      // group: half of the tile's columns
     const int quarter = warp & 3, c0 = g * (PN / 2);    // TMEM lanes 32 * quarter .. + 31
     const int row = 32 * quarter + lane;
-    const uint32_t sw = (uint32_t)(row >> 1) & 3u;      // 64-byte swizzle: slot ^= (row / 2) % 4
-    unsigned char* gbase = boxes + g * GROUP_BYTES;
-    int mv = 0, out = 0;
-    uint32_t mphase = 0, ophase = 0;
-    const uint32_t tmem = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + c0 + TCOLS * h;
+    int out = 0;
+    uint32_t ophase = 0;
+    const uint32_t tmem = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16) + c0;
     const uint32_t me[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->main_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->main_empty[1]), 0)};
     const uint32_t se[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[1]), 0)};
     int piece = 0, tile = 0;
-    uint32_t yphase = 0;
     bool ok = true;
     for (int t = pair; t < count && ok; t += npairs, ++tile) {
       const TileDev d = load_tile(tiles + t);
       const ProjJob& jb = jobs[d.job];
-      const MatDev& mt = mats[jb.mat];
-      const int npieces = (d.nk + PROMOTE_SLABS - 1) / PROMOTE_SLABS;
-      const uint32_t small = tmem + 2 * PN + (tile & 1) * PN;
-      float r[BOXES * TCOLS];                           // this thread's columns of every box
+      const int npieces = (d.nk + PROMOTE_SLABS - 1) / PROMOTE_SLABS, R = mats[jb.mat].r;
+      float r[PN / 2];
 #pragma unroll
-      for (int e = 0; e < BOXES * TCOLS; ++e) r[e] = 0.f;
-      auto add = [&](uint32_t taddr) {
-        uint32_t v[BOXES][TCOLS];
-        __syncwarp();
-#pragma unroll
-        for (int b = 0; b < BOXES; ++b) ptx::tmem_ld_32x32b_x8(taddr + COLS * b, v[b]);
-        ptx::tmem_ld_wait();
-#pragma unroll
-        for (int b = 0; b < BOXES; ++b)
-#pragma unroll
-          for (int e = 0; e < TCOLS; ++e) r[TCOLS * b + e] += __uint_as_float(v[b][e]);
-      };
+      for (int e = 0; e < PN / 2; ++e) r[e] = 0.f;
       for (int p = 0; p < npieces; ++p, ++piece) {
         const int mb = piece & 1;
         if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->main_full[mb]), (piece >> 1) & 1, abort_flag)) { ok = false; break; }
         ptx::tc_fence_after();
-        add(tmem + mb * PN);
+        add_columns(r, tmem + mb * PN);
+        ptx::tc_fence_before();
+        __syncwarp();
         if (lane == 0) ptx::mbar_arrive_cluster(me[mb]);
       }
       if (!ok) break;
-      if ((jb.shape & 15) != 5) add(small);          // G and the projection have more than one part
-      const int l = d.l0 + PM / 2 * (int)rank + row, j0 = d.j0 + c0, R = mt.r;
-      const bool in = l < mt.l;
-      const float bias = mt.sc->pad;
-      const bool fused = part_forms_x(R, hp);
-      float nn = 0.f, rn = 0.f;
-      // this thread's values of a box as parts into the next out buffer
-      auto put_parts = [&](const float* x) {
-        unsigned char* o = gbase + MV_BUFS * MV_BUF + out * OUT_BUF + row * (COLS * 2) + 16 * h;
-        uint32_t hi[4], mid[4], lo[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) split::split3(x[2 * i], x[2 * i + 1], hi[i], mid[i], lo[i]);
-        *reinterpret_cast<uint4*>(o) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(o + OUT_PART) = make_uint4(mid[0], mid[1], mid[2], mid[3]);
-        *reinterpret_cast<uint4*>(o + 2 * OUT_PART) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-        ptx::fence_proxy_async_smem();
-        ptx::mbar_arrive(ptx::smem_u32(&ctl->oready[g][out]));
-        if (++out == OUT_BUFS) { out = 0; ophase ^= 1u; }
-      };
-      // The boxes of a tile are a loop (unrolled, its divisions and roots are more instructions than the caches hold:
-      // half of the time went into waiting for them), so the registers move instead of the index: once around and r
-      // is as it was.
-      auto rotate = [&]() {
-        float first[TCOLS];
-#pragma unroll
-        for (int e = 0; e < TCOLS; ++e) first[e] = r[e];
-#pragma unroll
-        for (int e = 0; e < (BOXES - 1) * TCOLS; ++e) r[e] = r[e + TCOLS];
-#pragma unroll
-        for (int e = 0; e < TCOLS; ++e) r[(BOXES - 1) * TCOLS + e] = first[e];
-      };
-#pragma unroll 1
-      for (int q = 0; q < PN / 2; q += COLS) {
-        if (j0 + q >= R) { rotate(); continue; }
-        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->efull[g][mv]), mphase, abort_flag)) { ok = false; break; }
-        unsigned char* mb = gbase + mv * MV_BUF + row * (COLS * 4);
-        uint32_t nw[TCOLS];
-#pragma unroll
-        for (int w = 0; w < TCOLS / 4; ++w) {
-          const uint32_t slot = ((uint32_t)(TCOLS / 4 * h + w) ^ sw) << 4;
-          float4* mp = reinterpret_cast<float4*>(mb + slot);
-          float4* vp = reinterpret_cast<float4*>(mb + MV_BOX + slot);
-          const float4 m4 = *mp, v4 = *vp;
-          float m[4] = {m4.x, m4.y, m4.z, m4.w}, v[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            // (past the row's end R, M and V are zeros: the projection has no such columns)
-            const float rv = r[4 * w + e], nv = adam_direction<PSI>(hp, bias, rv, m[e], v[e]);
-            nn = fmaf(nv, nv, nn);
-            rn = fmaf(rv, rv, rn);
-            nw[4 * w + e] = __float_as_uint(nv);
-          }
-          *mp = make_float4(m[0], m[1], m[2], m[3]);
-          *vp = make_float4(v[0], v[1], v[2], v[3]);
-        }
-        ptx::fence_proxy_async_smem();
-        ptx::mbar_arrive(ptx::smem_u32(&ctl->eready[g][mv]));
-        if (++mv == MV_BUFS) { mv = 0; mphase ^= 1u; }
-        if (fused) {
-          __syncwarp();
-          ptx::tmem_st_32x32b_x8(small + q, nw);
-        }
-        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oempty[g][out]), ophase ^ 1u, abort_flag)) { ok = false; break; }
-        put_parts(r);
-        rotate();
-      }
-      if (!ok) break;
-      float2(*xs)[PM / 2] = ctl->row_sums;
-      if (!ptx::mbar_wait(ptx::smem_u32(&ctl->sums_read), yphase ^ 1u, abort_flag)) break;      // the tile before
-      xs[2 * g + h][row] = make_float2(nn, rn);
-      if (fused) ptx::tmem_st_wait();
-      ptx::mbar_arrive(ptx::smem_u32(&ctl->sums));
-      if (!ptx::mbar_wait(ptx::smem_u32(&ctl->sums), yphase, abort_flag)) break;
-      yphase ^= 1u;
-      const float2 a = xs[2 * g][row], b = xs[2 * g + 1][row], oa = xs[2 * (g ^ 1)][row], ob = xs[2 * (g ^ 1) + 1][row];
-      ptx::mbar_arrive(ptx::smem_u32(&ctl->sums_read));
-      if (hp.mode & HYPER_NO_SCALING) {
-        if (in && ew == 0 && d.j0 == 0) mt.kvec[l] = 1.f;
-      } else if (!fused) {
-        if (in && h == 0 && j0 < R) {
-          const int slot = j0 / 64;
-          mt.aux[(long long)slot * mt.l + l] = a.x + b.x;
-          mt.aux[(long long)(mt.aux_slots + slot) * mt.l + l] = a.y + b.y;
-        }
-      }
-      if (fused) {
-        const float k = sqrtf((a.x + b.x) + (oa.x + ob.x)) / (sqrtf((a.y + b.y) + (oa.y + ob.y)) + hp.eps);
-        if (in && ew == 0) mt.kvec[l] = k;
-        const float c = hp.a_res * k;
-#pragma unroll 1
-        for (int q = 0; q < PN / 2 && j0 + q < R; q += COLS) {
-          uint32_t nw[TCOLS];
-          float x[TCOLS];
-          __syncwarp();
-          ptx::tmem_ld_32x32b_x8(small + q, nw);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < TCOLS; ++e) x[e] = hp.a_low * __uint_as_float(nw[e]) - c * r[e];
-          if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oempty[g][out]), ophase ^ 1u, abort_flag)) { ok = false; break; }
-          put_parts(x);
-          rotate();
-        }
-        if (!ok) break;
-      }
+      if ((jb.shape & 15) != 5) add_columns(r, tmem + 2 * PN + (tile & 1) * PN);      // G and the projection have more than one part
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive_cluster(se[tile & 1]);
+#pragma unroll
+      for (int b = 0; b < BOXES; ++b) {
+        if (d.j0 + c0 + COLS * b >= R) break;
+        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->oempty[g][out]), ophase ^ 1u, abort_flag)) { ok = false; break; }
+        unsigned char* o = boxes + g * GROUP_BYTES + out * OUT_BUF + row * (COLS * 2);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t hi[4], mid[4], lo[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) split::split3(r[COLS * b + 8 * h + 2 * i], r[COLS * b + 8 * h + 2 * i + 1], hi[i], mid[i], lo[i]);
+          *reinterpret_cast<uint4*>(o + 16 * h) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<uint4*>(o + OUT_PART + 16 * h) = make_uint4(mid[0], mid[1], mid[2], mid[3]);
+          *reinterpret_cast<uint4*>(o + 2 * OUT_PART + 16 * h) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+        ptx::fence_proxy_async_smem();
+        ptx::mbar_arrive(ptx::smem_u32(&ctl->oready[g][out]));
+        if (++out == OUT_BUFS) { out = 0; ophase ^= 1u; }
+      }
     }
   }
   // neither CTA may leave while its partner can still reach into its shared memory
@@ -503,9 +344,7 @@ int prepared_sms() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && (sms = sms_of_device[dev].load()) == 0) {
-    const void* kernels[3] = {(const void*)k_part_project<PSI_ADAM>, (const void*)k_part_project<PSI_RMSPROP>, (const void*)k_part_project<PSI_ADAGRAD>};
-    for (const void* k : kernels)
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+    e = cudaFuncSetAttribute(k_part_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) sms_of_device[dev].store(sms);
   }
@@ -531,11 +370,10 @@ fira_status part_project_prepare(const std::vector<MatDev>& mats, const std::vec
     memset(&j, 0, sizeof(j));
     if (!encode_operand(&j.b, pi, true, PN / 2)) return FIRA_ERR_CUDA;
     {
-      const unsigned long long extent[3] = {(unsigned long long)mt.r, (unsigned long long)mt.l, 3}, mstride[1] = {4ull * mt.r};
+      const unsigned long long extent[3] = {(unsigned long long)mt.r, (unsigned long long)mt.l, 3};
       const unsigned long long pstride[2] = {2ull * mt.rp_pitch, 2ull * mt.l * mt.rp_pitch};
       const unsigned box[3] = {COLS, PM / 2, 3};
-      if (!encode_tiled(&j.m, mt.M, true, 2, extent, mstride, box, 64) || !encode_tiled(&j.v, mt.V, true, 2, extent, mstride, box, 64) ||
-          !encode_tiled(&j.ro, mt.Rp, false, 3, extent, pstride, box, 0) || !encode_tiled(&j.xo, mt.Xp, false, 3, extent, pstride, box, 0))
+      if (!encode_tiled(&j.ro, mt.Rp, false, 3, extent, pstride, box, 0))
         return FIRA_ERR_CUDA;
     }
     j.mat = list[q];
@@ -555,16 +393,14 @@ fira_status part_project_prepare(const std::vector<MatDev>& mats, const std::vec
   return FIRA_OK;
 }
 
-fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, const Hyper& hp, unsigned* status_dev, cudaStream_t st) {
+fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, unsigned* status_dev, cudaStream_t st) {
   const int sms = prepared_sms();
   if (!sms) return FIRA_ERR_CUDA;
   const int first = plan.proj_start[qa], count = plan.proj_start[qb] - first;
   if (count == 0) return FIRA_OK;
   const ProjJob* jobs = reinterpret_cast<const ProjJob*>(plan.proj_table);
   const TileDev* tiles = reinterpret_cast<const TileDev*>(plan.proj_table + align_up(sizeof(ProjJob) * (size_t)plan.njobs)) + first;
-  const int psi = psi_of(hp);
-  const cudaError_t e = launch_chained(psi == PSI_ADAM ? k_part_project<PSI_ADAM> : psi == PSI_RMSPROP ? k_part_project<PSI_RMSPROP> : k_part_project<PSI_ADAGRAD>,
-                                       2 * std::min(count, sms / 2), THREADS, SMEM_BYTES, st, false, 1, jobs, tiles, count, mats_dev, hp, status_dev);
+  const cudaError_t e = launch_chained(k_part_project, 2 * std::min(count, sms / 2), THREADS, SMEM_BYTES, st, false, 1, jobs, tiles, count, mats_dev, status_dev);
   if (e != cudaSuccess) { set_error(std::string("step projection: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }

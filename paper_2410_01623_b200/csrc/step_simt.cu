@@ -181,12 +181,8 @@ __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, cons
       }
       if (momentum) store_row<VEC>(mt.M + at, lane, n, m[y]);
       store_row<VEC>(mt.V + at, lane, n, v[y]);
-      if (!mt.Rp) {
-        store_row<VEC>(mt.Xt + at, lane, n, nv);
-        store_row<VEC>(mt.Rt + at, lane, n, rv);
-      } else {                                  // a long list whose ranks TMA cannot address
-        store_row_parts<VEC>(mt.Rp + (long long)l * mt.rp_pitch + j0, (long long)mt.l * mt.rp_pitch, lane, n, rv);
-      }
+      store_row<VEC>(mt.Xt + at, lane, n, nv);
+      store_row<VEC>(mt.Rt + at, lane, n, rv);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         nn += __shfl_xor_sync(0xffffffffu, nn, o);
@@ -370,6 +366,88 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
 }
 
 // ---------------------------------------------------------------- long lists
+// Adam (Eq. 2-4) on rows of R that the projection left as parts, the rows' factors k_l, and X for limiter factor 1: one warp
+// per row, R whole in registers (CHUNKS of 128 columns), ROWS rows with their loads in flight together.
+template <int PSI, bool VEC, int CHUNKS, int ROWS>
+__device__ __forceinline__ void moment_rows(const MatDev& mt, int l0, int count, const Hyper& hp, float bias) {
+  const int lane = threadIdx.x & 31;
+  const long long stride = (long long)mt.l * mt.rp_pitch;
+  float m[ROWS][CHUNKS][4], v[ROWS][CHUNKS][4], rv[ROWS][CHUNKS][4];
+#pragma unroll
+  for (int y = 0; y < ROWS; ++y)
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) {
+      const int l = l0 + y, j = 128 * c, n = y < count ? min(128, mt.r - j) : 0;
+      load_row<VEC>(mt.V + (long long)l * mt.r + j, lane, n, v[y][c]);
+      load_row<VEC>(mt.M + (long long)l * mt.r + j, lane, PSI == PSI_ADAM ? n : 0, m[y][c]);
+      load_row_parts<VEC>(mt.Rp + (long long)l * mt.rp_pitch + j, stride, lane, n, rv[y][c]);
+    }
+#pragma unroll
+  for (int y = 0; y < ROWS; ++y) {
+    if (y >= count) break;
+    const int l = l0 + y;
+    float nv[CHUNKS][4], nn = 0.f, rn = 0.f;
+#pragma unroll
+    for (int c = 0; c < CHUNKS; ++c) {
+      const int j = 128 * c, n = min(128, mt.r - j);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        nv[c][q] = adam_direction<PSI>(hp, bias, rv[y][c][q], m[y][c][q], v[y][c][q]);
+        nn = fmaf(nv[c][q], nv[c][q], nn);      // (entries past the row's end are zeros throughout)
+        rn = fmaf(rv[y][c][q], rv[y][c][q], rn);
+      }
+      if (PSI == PSI_ADAM) store_row<VEC>(mt.M + (long long)l * mt.r + j, lane, n, m[y][c]);
+      store_row<VEC>(mt.V + (long long)l * mt.r + j, lane, n, v[y][c]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      nn += __shfl_xor_sync(0xffffffffu, nn, o);
+      rn += __shfl_xor_sync(0xffffffffu, rn, o);
+    }
+    const float k = hp.mode & HYPER_NO_SCALING ? 1.f : sqrtf(nn) / (sqrtf(rn) + hp.eps);
+    if (lane == 0) {
+      if (hp.mode & HYPER_MATRIX_SCALING) { mt.aux[l] = nn; mt.aux[mt.l + l] = rn; }
+      else mt.kvec[l] = k;
+    }
+    if (part_forms_x(hp)) {
+      const float ck = hp.a_res * k;
+#pragma unroll
+      for (int c = 0; c < CHUNKS; ++c) {
+        float x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = hp.a_low * nv[c][q] - ck * rv[y][c][q];
+        store_row_parts<VEC>(mt.Xp + (long long)l * mt.rp_pitch + 128 * c, stride, lane, min(128, mt.r - 128 * c), x);
+      }
+    }
+  }
+}
+constexpr int MOMENT_ROWS = 4;                  // per warp: what it costs to find the matrix is shared
+// Bound by memory: 28 bytes per entry.  As an epilogue of the projection the same work held up its product (part_project.cu).
+// CHUNKS: for ranks up to 128 CHUNKS.  (One kernel for all ranks has the registers of the largest: 45 us instead of MEASURE2.)
+template <int PSI, int CHUNKS>
+__global__ void __launch_bounds__(256, CHUNKS == 1 ? 4 : CHUNKS == 2 ? 3 : 2)
+k_moments(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist, const int* __restrict__ row_start, int first_row,
+          int rows_end, Hyper hp) {
+  int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * MOMENT_ROWS;
+  int p = row < rows_end ? find_matrix(row_start, nlist, row) : 0;
+  ptx::grid_wait();
+  ptx::grid_launch_next();
+  const int end = min(row + MOMENT_ROWS, rows_end);
+  while (row < end) {
+    const MatDev& mt = mats[list[p]];
+    const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
+    const float bias = mt.sc->pad;
+    constexpr int ROWS = CHUNKS == 1 ? 2 : 1;
+    if (mt.r % 4 == 0) {
+      for (int l = l0; l < l1; l += ROWS) moment_rows<PSI, true, CHUNKS, ROWS>(mt, l, min(ROWS, l1 - l), hp, bias);
+    } else {
+      for (int l = l0; l < l1; l += ROWS) moment_rows<PSI, false, CHUNKS, ROWS>(mt, l, min(ROWS, l1 - l), hp, bias);
+    }
+    row += l1 - l0;
+    ++p;
+  }
+}
+
 // X = a_low N - a_res lambda k_l R as parts, one warp per row l; N from the updated moments, by the arithmetic that the
 // projection's epilogue used.  (r % 4 != 0: scalar accesses.)
 template <int PSI, bool VEC>
@@ -402,8 +480,8 @@ k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlis
     const MatDev& mt = mats[list[p]];
     const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
     const float lambda = mt.sc->lambda, c = hp.a_res * lambda, bias = *mt.step_bias;
-    if (mt.tma_proj && part_forms_x(mt.r, hp) && lambda == 1.f) {
-      // the projection's epilogue has formed it
+    if (part_forms_x(hp) && lambda == 1.f) {
+      // k_moments has formed it
     } else if (mt.r % 4 == 0) {
 #pragma unroll 2
       for (int l = l0; l < l1; ++l) form_x_row<PSI, true>(mt, l, hp, bias, c * mt.kvec[l]);
@@ -599,7 +677,7 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   }
 }
 
-const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"};
+const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_moments", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"};
 
 // Measured below.
 constexpr long long LONG_LIST_TILES = 256;
@@ -657,6 +735,12 @@ static cudaError_t launch_project(const SimtPlan& pl, int first, int tiles, cons
   return launch_chained(k, tiles * split, split::THREADS, split::SMEM_BYTES, st, false, split, pl.mats, pl.list, pl.nlist, pl.proj_tile_start, first, hp, status_dev);
 }
 
+template <int PSI>
+static cudaError_t launch_moments(const SimtPlan& pl, int r0, int r1, const Hyper& hp, cudaStream_t st) {
+  auto k = pl.max_r <= 128 ? k_moments<PSI, 1> : pl.max_r <= 256 ? k_moments<PSI, 2> : k_moments<PSI, PART_STEP_MAX_RANK / 128>;
+  return launch_chained(k, (r1 - r0 + 8 * MOMENT_ROWS - 1) / (8 * MOMENT_ROWS), 256, 0, st, true, 1, pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp);
+}
+
 int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, cudaStream_t st,
                      PhaseTimer* tm, int qa, int qb) {
   if (pl.nlist == 0) return 0;
@@ -683,11 +767,15 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   const int staged = pl.parts.table ? pl.h_stage_start[pl.h_stage_pos[qe]] - s0 : 0, nstage = pl.parts.table ? pl.h_stage_pos.back() : 0;
   tm->mark(st);
   launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 0, st);
-  if (pl.parts.proj_table) {           // (also before only-scaling, which needs the row sums)
-    if (part_project_run(pl.parts, pl.mats, qa, qe, hp, status_dev, st) != FIRA_OK) return -1;
+  if (pl.parts.table) {                // (also before only-scaling, which needs the factors)
+    if (part_project_run(pl.parts, pl.mats, qa, qe, status_dev, st) != FIRA_OK) return -1;
+    tm->mark(st);
+    const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
+    launch_error((psi == PSI_ADAM ? launch_moments<PSI_ADAM> : psi == PSI_RMSPROP ? launch_moments<PSI_RMSPROP> : launch_moments<PSI_ADAGRAD>)(pl, r0, r1, hp, st));
   } else {
     launch_error((psi == PSI_ADAM ? launch_project<PSI_ADAM> : psi == PSI_RMSPROP ? launch_project<PSI_RMSPROP> : launch_project<PSI_ADAGRAD>)(
         pl, pt0, pt1 - pt0, hp, status_dev, st));
+    tm->mark(st);
   }
   tm->mark(st);
   if (only_scaling)
@@ -715,7 +803,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     launch_error(launch_chained(k_back_project<MODE_UPDATE>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
-  return 4 + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
+  return 4 + (pl.parts.table ? 1 : 0) + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
 }
 
 }  // namespace fira

@@ -7,7 +7,7 @@ namespace fira {
 
 constexpr int SIMT_TILE = 128;              // tiles of R (l x r) and of W (m x n)
 inline int simt_tiles(long long extent) { return (int)((extent + SIMT_TILE - 1) / SIMT_TILE); }
-constexpr int SIMT_PHASES = 5;
+constexpr int SIMT_PHASES = 6;
 
 // The factor k_l from the row sums.
 __device__ __forceinline__ float row_factor(const MatDev& mt, int l, const Hyper& hp) {
@@ -18,7 +18,7 @@ __device__ __forceinline__ float row_factor(const MatDev& mt, int l, const Hyper
 
 // Whether the projection's epilogue has made the factors k_l itself: the row sums were complete in one tile.
 __device__ __forceinline__ bool factors_ready(const MatDev& mt, const Hyper& hp) {
-  return mt.tma_proj ? part_forms_x(mt.r, hp) : mt.r <= SIMT_TILE;
+  return mt.Rp || mt.r <= SIMT_TILE;             // (Rp: k_moments has)
 }
 
 inline int psi_of(const Hyper& hp) { return hp.mode & HYPER_PSI_RMSPROP ? PSI_RMSPROP : hp.mode & HYPER_PSI_ADAGRAD ? PSI_ADAGRAD : PSI_ADAM; }
@@ -43,7 +43,7 @@ struct SimtPlan {
   int nlist = 0;
   const int* proj_tile_start = nullptr;  // 128 x 128 tiles of R (l x r)
   int proj_tiles = 0;
-  int max_d = 0;                         // largest d of the list
+  int max_d = 0, max_r = 0;              // largest d and r of the list
   const int* w_tile_start = nullptr;     // 128 x 128 tiles of W (m x n)
   int w_tiles = 0;
   const int* npart = nullptr;            // partial sums of ||S||^2 per matrix
