@@ -20,6 +20,7 @@
 
 #include "context.cuh"
 #include "step_simt.cuh"
+#include "tc_ptx.cuh"
 
 namespace fira {
 
@@ -91,6 +92,7 @@ struct NoAllocInts { int v[6]; };
 // MatScalars block that the step kernels use.
 __global__ void k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, int* ints_out,
                                 const float* norm_prev, const long long* t, float beta1, float beta2) {
+  ptx::grid_launch_next();
   *mats_out = mt;
   for (int i = 0; i < 6; ++i) ints_out[i] = ints.v[i];
   MatScalars* sc = mt.sc;
@@ -100,6 +102,7 @@ __global__ void k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, i
   sc->t = *t;
 }
 __global__ void k_noalloc_store_scalars(const MatScalars* sc, float* norm_prev, long long* t) {
+  ptx::grid_wait();
   *norm_prev = sc->prev_norm;
   *t = sc->t;
 }
@@ -169,7 +172,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
                                    norm_prev_dev, reinterpret_cast<const long long*>(t_dev), hp->beta1, hp->beta2);
   SimtPlan pl;
   pl.mats = reinterpret_cast<const MatDev*>(base + cv.off_mats);
-  pl.list = ints_dev; pl.nlist = 1;
+  pl.list = ints_dev; pl.nlist = 1; pl.chained = true;
   pl.proj_tile_start = ints_dev + 1; pl.proj_tiles = ptiles; pl.max_d = mt.d;
   pl.w_tile_start = ints_dev + 3; pl.w_tiles = wtiles;
   pl.npart = ints_dev + 5;
@@ -182,8 +185,8 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   h.gamma = hp->gamma;
   PhaseTimer no_timer;
   if (launch_simt_step(pl, h, status_dev, st, &no_timer) < 0) return FIRA_ERR_CUDA;
-  k_noalloc_store_scalars<<<1, 1, 0, st>>>(mt.sc, norm_prev_dev, reinterpret_cast<long long*>(t_dev));
-  const cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_chained(k_noalloc_store_scalars, 1, 1, 0, st, true, 1, mt.sc, norm_prev_dev, reinterpret_cast<long long*>(t_dev));
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error(std::string("fira_step_single_noalloc: ") + cudaGetErrorString(e));
     return FIRA_ERR_CUDA;

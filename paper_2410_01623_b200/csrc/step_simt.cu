@@ -216,6 +216,7 @@ k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
           const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem[];
   split::Ctl* ctl = reinterpret_cast<split::Ctl*>(smem + split::STAGES * split::STAGE_BYTES);
+  ptx::grid_wait();                             // (the single-matrix entry point writes its tables just before)
   const int blocks = SPLIT ? (int)ptx::cluster_nctarank() : 1, block = SPLIT ? (int)ptx::cluster_ctarank() : 0;
   const int gt = blockIdx.x / blocks + first;
   const int p = find_matrix(tile_start, nlist, gt);
@@ -421,18 +422,19 @@ __device__ __forceinline__ void moment_rows(const MatDev& mt, int l0, int count,
     }
   }
 }
-constexpr int MOMENT_ROWS = 4;                  // per warp: what it costs to find the matrix is shared
+// Row passes: so many rows per warp that the grid is resident at once (rows_per_warp): what it costs a warp to find its
+// matrix, five dependent loads and more, is paid once.
 // Bound by memory: 28 bytes per entry.  As an epilogue of the projection the same work held up its product (part_project.cu).
 // CHUNKS: for ranks up to 128 CHUNKS.  (One kernel for all ranks has the registers of the largest: 45 us instead of MEASURE2.)
 template <int PSI, int CHUNKS>
 __global__ void __launch_bounds__(256, CHUNKS == 1 ? 4 : CHUNKS == 2 ? 3 : 2)
 k_moments(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist, const int* __restrict__ row_start, int first_row,
-          int rows_end, Hyper hp) {
-  int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * MOMENT_ROWS;
+          int rows_end, int per_warp, Hyper hp) {
+  int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * per_warp;
   int p = row < rows_end ? find_matrix(row_start, nlist, row) : 0;
   ptx::grid_wait();
   ptx::grid_launch_next();
-  const int end = min(row + MOMENT_ROWS, rows_end);
+  const int end = min(row + per_warp, rows_end);
   while (row < end) {
     const MatDev& mt = mats[list[p]];
     const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
@@ -448,34 +450,45 @@ k_moments(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
   }
 }
 
-// X = a_low N - a_res lambda k_l R as parts, one warp per row l; N from the updated moments, by the arithmetic that the
-// projection's epilogue used.  (r % 4 != 0: scalar accesses.)
+// X = a_low N - a_res lambda k_l R as parts, one warp per row l; N from the updated moments, by the arithmetic that
+// k_moments used.  (r % 4 != 0: scalar accesses.)  Two rows with their loads in flight together.
 template <int PSI, bool VEC>
-__device__ __forceinline__ void form_x_row(const MatDev& mt, int l, const Hyper& hp, float bias, float c) {
+__device__ __forceinline__ void form_x_rows(const MatDev& mt, int l0, int count, const Hyper& hp, float bias, float c) {
+  constexpr int ROWS = 2;
   const int lane = threadIdx.x & 31;
-  const long long stride = (long long)mt.l * mt.rp_pitch, at = (long long)l * mt.rp_pitch;
-  for (int j = 0; j < mt.r; j += 128) {
-    const int n = min(128, mt.r - j);
-    float m[4], v[4], rv[4], x[4];
-    load_row<VEC>(mt.M + (long long)l * mt.r + j, lane, n, m);
-    load_row<VEC>(mt.V + (long long)l * mt.r + j, lane, n, v);
-    load_row_parts<VEC>(mt.Rp + at + j, stride, lane, n, rv);
+  const long long stride = (long long)mt.l * mt.rp_pitch;
+  float ck[ROWS];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) x[q] = hp.a_low * direction<PSI>(hp, bias, rv[q], m[q], v[q]) - c * rv[q];
-    store_row_parts<VEC>(mt.Xp + at + j, stride, lane, n, x);
+  for (int y = 0; y < ROWS; ++y) ck[y] = y < count ? c * mt.kvec[l0 + y] : 0.f;
+  for (int j = 0; j < mt.r; j += 128) {
+    float m[ROWS][4], v[ROWS][4], rv[ROWS][4];
+#pragma unroll
+    for (int y = 0; y < ROWS; ++y) {
+      const int n = y < count ? min(128, mt.r - j) : 0;
+      load_row<VEC>(mt.M + (long long)(l0 + y) * mt.r + j, lane, PSI == PSI_ADAM ? n : 0, m[y]);
+      load_row<VEC>(mt.V + (long long)(l0 + y) * mt.r + j, lane, n, v[y]);
+      load_row_parts<VEC>(mt.Rp + (long long)(l0 + y) * mt.rp_pitch + j, stride, lane, n, rv[y]);
+    }
+#pragma unroll
+    for (int y = 0; y < ROWS; ++y) {
+      float x[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = hp.a_low * direction<PSI>(hp, bias, rv[y][q], m[y][q], v[y][q]) - ck[y] * rv[y][q];
+      store_row_parts<VEC>(mt.Xp + (long long)(l0 + y) * mt.rp_pitch + j, stride, lane, y < count ? min(128, mt.r - j) : 0, x);
+    }
   }
 }
-constexpr int FORM_X_ROWS = 4;                  // per warp: what it costs to find the matrix is shared
+constexpr int FORM_X_BLOCKS = 3;                // resident per SM
 template <int PSI>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, FORM_X_BLOCKS)
 k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist, const int* __restrict__ row_start, int first_row,
-         int rows_end, Hyper hp) {
-  int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * FORM_X_ROWS;
+         int rows_end, int per_warp, Hyper hp) {
+  int row = first_row + (blockIdx.x * 8 + (threadIdx.x >> 5)) * per_warp;
   ptx::grid_wait();
   ptx::grid_launch_next();
   if (row >= rows_end) return;
   int p = find_matrix(row_start, nlist, row);
-  const int end = min(row + FORM_X_ROWS, rows_end);
+  const int end = min(row + per_warp, rows_end);
   while (row < end) {
     const MatDev& mt = mats[list[p]];
     const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
@@ -483,10 +496,9 @@ k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlis
     if (part_forms_x(hp) && lambda == 1.f) {
       // k_moments has formed it
     } else if (mt.r % 4 == 0) {
-#pragma unroll 2
-      for (int l = l0; l < l1; ++l) form_x_row<PSI, true>(mt, l, hp, bias, c * mt.kvec[l]);
+      for (int l = l0; l < l1; l += 2) form_x_rows<PSI, true>(mt, l, min(2, l1 - l), hp, bias, c);
     } else {
-      for (int l = l0; l < l1; ++l) form_x_row<PSI, false>(mt, l, hp, bias, c * mt.kvec[l]);
+      for (int l = l0; l < l1; l += 2) form_x_rows<PSI, false>(mt, l, min(2, l1 - l), hp, bias, c);
     }
     row += l1 - l0;
     ++p;
@@ -679,15 +691,17 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
 
 const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_moments", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"};
 
-// Measured below.
-constexpr long long LONG_LIST_TILES = 256;
+// Measured (fp32 / bf16 storage, times of a step in us, short against long): 6 matrices 512 x 1376, r = 128, 63 / 51 against 71 / 62,
+// 8 of them 102 / 72 against 82 / 69; 4 of 1024 x 1024, r = 256, 92 / 65 against 94 / 71, 6 of them 151 / 98 against 113 / 82; 24 of
+// 300 x 417, r = 64, whose rows are copied to an aligned pitch first, 78 / 77 against 114 / 110.
+constexpr long long LONG_LIST_ELEMENTS = 5 << 20;
 bool simt_long_list(const std::vector<fira_matrix_desc>& list) {
-  long long tiles = 0;
+  long long elements = 0;
   for (const fira_matrix_desc& d : list) {
     if (d.r > PART_STEP_MAX_RANK) return false;
-    tiles += (long long)simt_tiles(d.m) * simt_tiles(d.n);
+    elements += (long long)d.m * d.n;
   }
-  return tiles >= LONG_LIST_TILES;
+  return elements >= LONG_LIST_ELEMENTS;
 }
 
 void launch_split_projections(const SimtPlan& pl, const std::vector<MatDev>& mats, const std::vector<int>& list, cudaStream_t st) {
@@ -732,13 +746,18 @@ static cudaError_t launch_project(const SimtPlan& pl, int first, int tiles, cons
   const int split = split_of(pl);
   const bool long_k = (pl.max_d + split::BK - 1) / split::BK > split * (split::PROMOTE / split::BK);
   auto k = split == 1 ? k_project<PSI, false, true> : long_k ? k_project<PSI, true, true> : k_project<PSI, true, false>;
-  return launch_chained(k, tiles * split, split::THREADS, split::SMEM_BYTES, st, false, split, pl.mats, pl.list, pl.nlist, pl.proj_tile_start, first, hp, status_dev);
+  return launch_chained(k, tiles * split, split::THREADS, split::SMEM_BYTES, st, pl.chained, split, pl.mats, pl.list, pl.nlist, pl.proj_tile_start, first, hp, status_dev);
 }
 
+static int rows_per_warp(int rows, int blocks_per_sm) {
+  const int warps = 148 * blocks_per_sm * 8;
+  return std::max(2, (rows + warps - 1) / warps);
+}
 template <int PSI>
 static cudaError_t launch_moments(const SimtPlan& pl, int r0, int r1, const Hyper& hp, cudaStream_t st) {
   auto k = pl.max_r <= 128 ? k_moments<PSI, 1> : pl.max_r <= 256 ? k_moments<PSI, 2> : k_moments<PSI, PART_STEP_MAX_RANK / 128>;
-  return launch_chained(k, (r1 - r0 + 8 * MOMENT_ROWS - 1) / (8 * MOMENT_ROWS), 256, 0, st, true, 1, pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp);
+  const int per = rows_per_warp(r1 - r0, pl.max_r <= 128 ? 4 : pl.max_r <= 256 ? 3 : 2);
+  return launch_chained(k, (r1 - r0 + 8 * per - 1) / (8 * per), 256, 0, st, true, 1, pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, per, hp);
 }
 
 int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, cudaStream_t st,
@@ -790,8 +809,9 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   tm->mark(st);
   if (parts) {
     const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
+    const int per = rows_per_warp(r1 - r0, FORM_X_BLOCKS);
     launch_error(launch_chained(psi == PSI_ADAM ? k_form_x<PSI_ADAM> : psi == PSI_RMSPROP ? k_form_x<PSI_RMSPROP> : k_form_x<PSI_ADAGRAD>,
-                                (r1 - r0 + 8 * FORM_X_ROWS - 1) / (8 * FORM_X_ROWS), 256, 0, st, true, 1, pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, hp));
+                                (r1 - r0 + 8 * per - 1) / (8 * per), 256, 0, st, true, 1, pl.mats, pl.list, pl.nlist, pl.row_start, r0, r1, per, hp));
   }
   tm->mark(st);
   if (only_scaling)

@@ -41,6 +41,7 @@ struct SimtPlan {
   const MatDev* mats = nullptr;
   const int* list = nullptr;
   int nlist = 0;
+  bool chained = false;                  // the kernel in front of the step lets its first kernel in early (short lists)
   const int* proj_tile_start = nullptr;  // 128 x 128 tiles of R (l x r)
   int proj_tiles = 0;
   int max_d = 0, max_r = 0;              // largest d and r of the list

@@ -7,13 +7,12 @@ import torch
 from oracle import fira_oracle as fo
 from paper_2410_01623_b200 import binding as fb
 from paper_2410_01623_b200 import workloads as wk
-from tests.parity_util import to_np64
-from tests.test_gpu_step import _random_case
+from tests.parity_util import Trajectory, residual_jump, to_np64
 
 pytestmark = pytest.mark.gpu
 
 # remainders of every extent, both orientations, ranks that are no multiple of 4 or 8, above one tile (128) and above
-# the width up to which accumulators are double-buffered (256); 3 x 90 tiles of 128 x 128
+# the width up to which accumulators are double-buffered (256)
 BASE = [(150, 333), (333, 150), (130, 130), (64, 200), (257, 129), (129, 257), (300, 1000), (1000, 300), (512, 700), (7, 9),
         (640, 512), (512, 256)]
 RANKS = [36, 37, 64, 16, 100, 128, 200, 255, 130, 3, 300, 128]
@@ -21,21 +20,39 @@ RANKS = [36, 37, 64, 16, 100, 128, 200, 255, 130, 3, 300, 128]
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("flags,ranks", [(0, RANKS), (0, [r // 4 * 4 or 4 for r in RANKS]), (fb.FLAG_MATRIX_SCALING, RANKS),
-                                         (fb.FLAG_NO_RESIDUAL, RANKS), (fb.FLAG_PSI_ADAGRAD, RANKS), (fb.FLAG_ONLY_SCALING, RANKS)])
+                                         (fb.FLAG_NO_RESIDUAL, RANKS), (fb.FLAG_ONLY_SCALING, RANKS),
+                                         (fb.FLAG_PSI_RMSPROP, RANKS), (fb.FLAG_PSI_ADAGRAD, RANKS)])
 def test_long_list_of_ragged_matrices(dtype, flags, ranks):
-    """A list of many tiles takes kernels of its own in fp32 precision; with ranks all multiples of 4 (no rank that TMA
-    cannot address) the projection's too."""
-    tr = _random_case(BASE * 3, ranks * 3, dtype, steps=3, seed=71, spike=(3,), flags=flags | fb.FLAG_FORCE_SIMT)
+    """A list of many elements takes kernels of its own in fp32 precision (step variants, row lengths that are and are not
+    multiples of four).  From moments of ordinary size: on a first step N = R / (|R| + eps) is the sign of R, and among
+    some 10^6 entries of R a few lie within fp32's error of zero, where that sign, and with it a column of the update, is
+    not determined."""
+    g = torch.Generator().manual_seed(11)
+    hp = fb.make_hparams(lr=1e-2, alpha=0.25, gamma=1.01, flags=flags | fb.FLAG_FORCE_SIMT)
+    W0 = [(torch.randn(m, n, generator=g) * 0.02).to(dtype) for m, n in BASE * 4]
+    tr = Trajectory(BASE * 4, ranks * 4, dtype, hp, W0)
+    Ps = []
+    for i, (m, n) in enumerate(tr.shapes):
+        q, _ = torch.linalg.qr(torch.randn(min(m, n), tr.f.ranks[i], generator=g, dtype=torch.float64))
+        Ps.append(q.to(dtype))
+        tr.f.set_projection(i, Ps[i].cuda())
+        V = torch.rand(max(m, n), tr.f.ranks[i], generator=g) + 0.5
+        tr.f.set_state(i, torch.zeros_like(V).cuda(), V.cuda(), 1e6, 3)
+        tr.st[i].V, tr.st[i].prev_norm, tr.st[i].t = to_np64(V.T if m <= n else V).copy(), 1e6, 3
+    for step in range(3):
+        G = [torch.randn(m, n, generator=g).to(dtype) for m, n in tr.shapes]
+        tr.step([residual_jump(x, p) for x, p in zip(G, Ps)] if step == 2 else G)
     tr.assert_ok()
     assert all(tr.f.diagnostics(i)["engine"] == 0 for i in range(len(BASE)))
-    assert tr.f.last_step_launches() > 4 or flags & fb.FLAG_ONLY_SCALING
+    assert flags & fb.FLAG_NO_RESIDUAL or any(l < 1.0 for l in tr.lams[-1])
+    assert tr.f.last_step_launches() > 4
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_long_list_with_pitches_and_in_chunks(dtype):
     """The same list with padded rows, whole and as the host path's chunks: the same weights as without padding, bit for
     bit (the order of every sum is the same), and the padding untouched."""
-    shapes, ranks = BASE * 3, [r // 4 * 4 or 4 for r in RANKS] * 3
+    shapes, ranks = BASE * 4, [r // 4 * 4 or 4 for r in RANKS] * 4
     g = torch.Generator().manual_seed(5)
     hp = fb.make_hparams(lr=1e-2, alpha=0.25, gamma=1.01, flags=fb.FLAG_FORCE_SIMT)
     lds = [n + (3, 8, 0)[i % 3] for i, (m, n) in enumerate(shapes)]
