@@ -264,51 +264,43 @@ __device__ __forceinline__ void tile_factors(const MatDev& mt, int i0, int j0, i
   }
 }
 
-// G and (MODE_UPDATE) W of ROWS rows of the tile.
-template <typename T, int MODE, bool VEC, int ROWS> struct TileRows {
-  float g[ROWS][4], w[MODE == MODE_UPDATE ? ROWS : 1][4];
-  __device__ __forceinline__ void load(const MatDev& mt, int i, int j0) {
-    const int lane = threadIdx.x & 31, n = min(SIMT_TILE, mt.n - j0);
-#pragma unroll
-    for (int y = 0; y < ROWS; ++y) {
-      const long long at = (long long)(i + y) * mt.ld + j0;
-      load_row<VEC>(static_cast<const T*>(mt.G) + at, lane, i + y < mt.m ? n : 0, g[y]);
-      if (MODE == MODE_UPDATE) load_row<VEC>(static_cast<const T*>(mt.W) + at, lane, i + y < mt.m ? n : 0, w[MODE == MODE_UPDATE ? y : 0]);
-    }
-  }
-};
-
-// Rows of the finished tile D.  ks[]: the factors of the tile's columns (left) or rows (right).  WHOLE: t holds all rows of
-// the warp already.
-template <typename T, int MODE, bool VEC, int ROWS, bool WHOLE>
-__device__ __forceinline__ float back_rows(const MatDev& mt, int i0, int j0, const float* C, const float* ks, float lr, float cres,
-                                           TileRows<T, MODE, VEC, ROWS>& t) {
+// Rows of the finished tile D.  ks[]: the factors of the tile's columns (left) or rows (right).
+template <typename T, int MODE, bool VEC>
+__device__ __forceinline__ float back_rows(const MatDev& mt, int i0, int j0, const float* C, const float* ks, float lr, float cres) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = min(SIMT_TILE, mt.n - j0);
+  const T* G = static_cast<const T*>(mt.G);
+  T* W = static_cast<T*>(mt.W);
   float kc[4], ss = 0.f;
 #pragma unroll
   for (int c = 0; c < 4; ++c) kc[c] = mt.left ? ks[lane_col<VEC>(lane, c)] : 0.f;
-  for (int x = 0; x < WARP_ROWS; x += ROWS) {
-    if (!WHOLE) t.load(mt, i0 + warp * WARP_ROWS + x, j0);
+  for (int x = 0; x < WARP_ROWS; x += ROWS_AT_ONCE) {
+    float g[ROWS_AT_ONCE][4], w[ROWS_AT_ONCE][4];
 #pragma unroll
-    for (int y = 0; y < ROWS; ++y) {
+    for (int y = 0; y < ROWS_AT_ONCE; ++y) {
+      const int i = i0 + warp * WARP_ROWS + x + y;
+      const long long at = (long long)i * mt.ld + j0;
+      load_row<VEC>(G + at, lane, i < mt.m ? n : 0, g[y]);
+      if (MODE == MODE_UPDATE) load_row<VEC>(W + at, lane, i < mt.m ? n : 0, w[y]);
+    }
+#pragma unroll
+    for (int y = 0; y < ROWS_AT_ONCE; ++y) {
       const int row = warp * WARP_ROWS + x + y, i = i0 + row;
       if (i >= mt.m) continue;
       float dv[4];
       load_row<VEC>(C + row * split::C_LD, lane, n, dv);
       const float kr = mt.left ? 0.f : ks[row];
-      float* w = t.w[MODE == MODE_UPDATE ? y : 0];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const float kf = mt.left ? kc[c] : kr;
         if (MODE == MODE_NORM) {
-          const float sv = kf * (t.g[y][c] - dv[c]);        // (zero past the row's end)
+          const float sv = kf * (g[y][c] - dv[c]);          // (zero past the row's end)
           ss = fmaf(sv, sv, ss);
         } else {
-          w[c] = w[c] - lr * (dv[c] + cres * kf * t.g[y][c]);
+          w[y][c] = w[y][c] - lr * (dv[c] + cres * kf * g[y][c]);
         }
       }
-      if (MODE == MODE_UPDATE) store_row<VEC>(static_cast<T*>(mt.W) + (long long)i * mt.ld + j0, lane, n, *reinterpret_cast<const float(*)[4]>(w));
+      if (MODE == MODE_UPDATE) store_row<VEC>(W + (long long)i * mt.ld + j0, lane, n, w[y]);
     }
   }
   return ss;
@@ -332,31 +324,19 @@ __device__ __forceinline__ bool back_product(const MatDev& mt, int i0, int j0, f
   }
 }
 
-template <typename T, int MODE, bool WHOLE, bool VEC>
+template <typename T, int MODE>
 __device__ __forceinline__ float back_tile(const MatDev& mt, int i0, int j0, const Hyper& hp, unsigned char* smem,
                                            split::Ctl* ctl, float* ks) {
-  constexpr int ROWS = WHOLE ? WARP_ROWS : ROWS_AT_ONCE;
-  TileRows<T, MODE, VEC, ROWS> t;
-  if (WHOLE) t.load(mt, i0 + (threadIdx.x >> 5) * WARP_ROWS, j0);
-  ptx::grid_wait();
-  ptx::grid_launch_next();
   const float cres = MODE == MODE_UPDATE ? hp.a_res * mt.sc->lambda : 0.f;
   tile_factors<MODE>(mt, i0, j0, SIMT_TILE, hp, ks);
   if (!back_product<T, MODE>(mt, i0, j0, hp.a_low, cres, smem, ctl)) return 0.f;
-  return back_rows<T, MODE, VEC, ROWS, WHOLE>(mt, i0, j0, reinterpret_cast<const float*>(smem), ks, hp.lr, cres, t);
-}
-template <typename T, int MODE, bool WHOLE>
-__device__ __forceinline__ float back_tile(const MatDev& mt, int i0, int j0, const Hyper& hp, unsigned char* smem,
-                                           split::Ctl* ctl, float* ks) {
+  const float* C = reinterpret_cast<const float*>(smem);
   const bool vec = rows_vec(static_cast<const T*>(mt.G), mt.ld, mt.n) && rows_vec(static_cast<const T*>(mt.W), mt.ld, mt.n);
-  return vec ? back_tile<T, MODE, WHOLE, true>(mt, i0, j0, hp, smem, ctl, ks) : back_tile<T, MODE, WHOLE, false>(mt, i0, j0, hp, smem, ctl, ks);
+  return vec ? back_rows<T, MODE, true>(mt, i0, j0, C, ks, hp.lr, cres) : back_rows<T, MODE, false>(mt, i0, j0, C, ks, hp.lr, cres);
 }
 
-// WHOLE: a block has an SM to itself, and the registers to fetch its tile of G and W before the product, even before the
-// kernel in front has ended (neither of the two writes them): four load latencies less at the end of the tile.
-// Measured (one 512 x 1376 matrix, r = 128): MEASURE.
-template <int MODE, bool WHOLE>
-__global__ void __launch_bounds__(split::THREADS, WHOLE ? 1 : 2)
+template <int MODE>
+__global__ void __launch_bounds__(split::THREADS, 2)
 k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
                const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -368,8 +348,10 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
   const int tile = gt - tile_start[p], ct = simt_tiles_dev(mt.n);
   const int i0 = (tile / ct) * SIMT_TILE, j0 = (tile % ct) * SIMT_TILE;
   split::begin(ctl);
-  float ss = mt.bf16 ? back_tile<__nv_bfloat16, MODE, WHOLE>(mt, i0, j0, hp, smem, ctl, ks)
-                     : back_tile<float, MODE, WHOLE>(mt, i0, j0, hp, smem, ctl, ks);
+  ptx::grid_wait();
+  ptx::grid_launch_next();
+  float ss = mt.bf16 ? back_tile<__nv_bfloat16, MODE>(mt, i0, j0, hp, smem, ctl, ks)
+                     : back_tile<float, MODE>(mt, i0, j0, hp, smem, ctl, ks);
   if (MODE == MODE_NORM) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -736,13 +718,12 @@ static bool allow_smem() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && !done[dev].load()) {
-    const void* kernels[13] = {(const void*)k_project<PSI_ADAM, false, true>, (const void*)k_project<PSI_RMSPROP, false, true>,
+    const void* kernels[11] = {(const void*)k_project<PSI_ADAM, false, true>, (const void*)k_project<PSI_RMSPROP, false, true>,
                                (const void*)k_project<PSI_ADAGRAD, false, true>, (const void*)k_project<PSI_ADAM, true, true>,
                                (const void*)k_project<PSI_RMSPROP, true, true>, (const void*)k_project<PSI_ADAGRAD, true, true>,
                                (const void*)k_project<PSI_ADAM, true, false>, (const void*)k_project<PSI_RMSPROP, true, false>,
                                (const void*)k_project<PSI_ADAGRAD, true, false>,
-                               (const void*)k_back_project<MODE_NORM, false>, (const void*)k_back_project<MODE_UPDATE, false>,
-                               (const void*)k_back_project<MODE_NORM, true>, (const void*)k_back_project<MODE_UPDATE, true>};
+                               (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
     for (const void* k : kernels)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
     if (e == cudaSuccess) done[dev].store(true);
@@ -800,7 +781,6 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   const bool only_scaling = hp.mode & HYPER_ONLY_SCALING;     // W <- W - lr phi(R) G: no back-projection
   const bool parts = pl.parts.table && !only_scaling;          // (a long list's only-scaling step has no back-projection)
   const int psi = psi_of(hp);
-  const bool whole = wt1 - wt0 <= 148;                         // a block per SM
   const int qe = qb >= 0 ? qb : pl.nlist;
   const int s0 = pl.parts.table ? pl.h_stage_start[pl.h_stage_pos[qa]] : 0;
   const int staged = pl.parts.table ? pl.h_stage_start[pl.h_stage_pos[qe]] - s0 : 0, nstage = pl.parts.table ? pl.h_stage_pos.back() : 0;
@@ -822,7 +802,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   else if (parts) {
     if (part_step_run(pl.parts, pl.mats, qa, qe, 0, hp, status_dev, st) != FIRA_OK) return -1;
   } else
-    launch_error(launch_chained(whole ? k_back_project<MODE_NORM, true> : k_back_project<MODE_NORM, false>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
+    launch_error(launch_chained(k_back_project<MODE_NORM>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   // (only-scaling leaves one partial sum per 128 x 128 tile whatever the list)
   launch_error(launch_chained(k_finalize, nq, 256, 0, st, true, 1, pl.mats, pl.list + qa, nq, (only_scaling ? pl.npart_tiles : pl.npart) + qa, hp, status_dev));
@@ -840,7 +820,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     if (part_step_run(pl.parts, pl.mats, qa, qe, 1, hp, status_dev, st) != FIRA_OK) return -1;
     launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 1, st);
   } else
-    launch_error(launch_chained(whole ? k_back_project<MODE_UPDATE, true> : k_back_project<MODE_UPDATE, false>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
+    launch_error(launch_chained(k_back_project<MODE_UPDATE>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
   return 4 + (pl.parts.table ? 1 : 0) + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
