@@ -67,8 +67,13 @@ def measured_peaks():
     return dict(hbm_gbs=6650.0, bf16_tflops=1590.0, bf16_tflops_sustained=1400.0, source="fallback")
 
 
-# fp32 CUDA-core peak: 148 SMs x 128 FMA lanes x 2 flop x 1.965 GHz (maximum SM clock)
-ALU_FP32_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
+# A product in fp32 precision is six bf16 products of the operands' parts on the tensor cores.
+PART_PRODUCTS = 6
+
+
+def tensor_peak(peaks, dtype, sustained):
+    return peaks["bf16_tflops_sustained" if sustained else "bf16_tflops"] / (1 if dtype == "bf16" else PART_PRODUCTS)
+
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch, from an ncu capture of 2 layers of
 # the llama-7b list (every layer has the same shapes, so the traffic of a full launch is this times
@@ -77,7 +82,7 @@ NCU_DRAM_BYTES_2_LAYERS = {"k_tc_project": 1.855e9 + 0.971e9, "k_tc_back_project
 
 # kernel name -> (pipe that does its arithmetic, share of the step's 4 m n r flops)
 KERNEL_PIPE = {
-    "k_project": ("alu", 0.5), "k_back_project<norm>": ("alu", 0.5), "k_back_project<update>": ("alu", 0.5),
+    "k_project": ("tensor", 0.5), "k_back_project<norm>": ("tensor", 0.5), "k_back_project<update>": ("tensor", 0.5),
     "k_tc_project": ("tensor", 0.5), "k_tc_back_project": ("tensor", 0.5),
 }
 
@@ -93,6 +98,10 @@ def kernel_min_bytes(name, wl):
         l, d = max(m, n), min(m, n)
         if "back_project" in name:
             by += 2 * e * m * n
+        elif name == "k_project":          # fp32 precision: the moments are counted at k_moments
+            by += e * m * n + e * wl.r * d
+        elif name == "k_moments":
+            by += 16 * wl.r * l
         elif "project" in name:
             by += e * m * n + e * wl.r * d + 16 * wl.r * l
     return by
@@ -407,17 +416,16 @@ def main():
     # the copy bandwidth; the sustained tensor figure applies to a kernel timed inside a long step,
     # the burst figure is given beside it
     t_hbm = by / (peaks["hbm_gbs"] * 1e9)
-    pipe_peak = peaks["bf16_tflops_sustained"] if wl.dtype == "bf16" else ALU_FP32_TFLOPS
+    pipe_peak = tensor_peak(peaks, wl.dtype, True)
     roof_ms = max(fl / (pipe_peak * 1e12), t_hbm) * 1e3
-    roof_ms_burst = max(fl / ((peaks["bf16_tflops"] if wl.dtype == "bf16" else ALU_FP32_TFLOPS) * 1e12), t_hbm) * 1e3
+    roof_ms_burst = max(fl / (tensor_peak(peaks, wl.dtype, False) * 1e12), t_hbm) * 1e3
     top = max(phases, key=lambda p: p[1]) if phases else ("", 0.0)
     pipe, share = KERNEL_PIPE.get(top[0], ("hbm", None))
     kbytes = kernel_min_bytes(top[0], wl)
     kflops = fl * share if share else 0.0
     if pipe == "tensor":
-        ppeak, peak_kind = peaks["bf16_tflops_sustained"], f"cuBLAS bf16 sustained, {peaks['source']}"
-    elif pipe == "alu":
-        ppeak, peak_kind = ALU_FP32_TFLOPS, "fp32 FMA: 148 SMs x 128 lanes x 2 x 1.965 GHz (derived)"
+        ppeak = tensor_peak(peaks, wl.dtype, True)
+        peak_kind = f"cuBLAS bf16 sustained, {peaks['source']}" + ("" if wl.dtype == "bf16" else f", / {PART_PRODUCTS} part products")
     else:
         ppeak, peak_kind = None, None
     # which roof bounds THIS kernel on THIS workload: its flop time against its byte time
@@ -443,7 +451,7 @@ def main():
         # Eq. 7 by subspace iteration: 2 q + 1 big products of 2 m n r flops each (q rounds)
         q = refresh["rounds"]
         rfl = (2 * q + 1) * fl / 2
-        rpeak = peaks["bf16_tflops_sustained"] if wl.dtype == "bf16" else ALU_FP32_TFLOPS
+        rpeak = tensor_peak(peaks, wl.dtype, True)
         refresh["achieved_tflops"] = rfl / (refresh["ms"] * 1e-3) / 1e12
         refresh["frac"] = refresh["achieved_tflops"] / rpeak
         refresh["peak_tflops"] = rpeak

@@ -75,7 +75,7 @@ typedef enum { FIRA_F32 = 0, FIRA_BF16 = 1 } fira_dtype;
 /* fira_hparams.flags */
 #define FIRA_FLAG_ALPHA_LOWRANK_ONLY 1u /* G~ = alpha P N + S instead of alpha (P N + S) */
 #define FIRA_FLAG_AUTO_REFRESH 2u       /* fira_step() refreshes a matrix's projection when t mod T == 0 */
-#define FIRA_FLAG_FORCE_SIMT 4u         /* bf16 matrices also use the fp32 CUDA-core kernels */
+#define FIRA_FLAG_FORCE_SIMT 4u         /* bf16 matrices also use the kernels of fp32 precision */
 /* Ablation variants of Section 5.4 ("Ablation Study"); epilogue switches of the same kernels.  The
  * first two exclude each other. */
 #define FIRA_FLAG_MATRIX_SCALING 8u     /* Fira-matrix: one factor ||N||_F / (||R||_F + eps) per matrix (Eq. 9-10) */
@@ -128,7 +128,7 @@ typedef struct {
   float norm_prev;    /* ||S_prev|| now stored (norm after limiting); < 0 = unset */
   float k_min, k_max; /* range of the factors k */
   int64_t t;          /* steps taken */
-  int32_t engine;     /* 0 = fp32 CUDA-core kernels, 1 = bf16 tensor-core kernels */
+  int32_t engine;     /* 0 = fp32 precision (any size and type), 1 = bf16 tensor-core kernels */
 } fira_diag;
 
 typedef struct fira_ctx fira_ctx;
@@ -279,10 +279,10 @@ FIRA_API const char* fira_phase_name(const fira_ctx* ctx, int32_t phase);
  * stay out of the driver's allocator, a process whose memory was budgeted at start
  * -- and therefore cannot provide the state and scratch buffers of fira_init().  The
  * intermediates live in a fixed array inside the library image instead:
- * fira_noalloc_max_scratch_bytes() bytes (8 MiB), held on every GPU that loads the
- * library until the process exits.  The call allocates nothing.
+ * fira_noalloc_max_scratch_bytes() bytes (8 MiB) and 144 KiB of row sums, held on every GPU
+ * that loads the library until the process exits.  The call allocates nothing.
  *
- * desc: the matrix (fp32 or bf16; it always runs on the fp32 CUDA-core kernels).  Its
+ * desc: the matrix (fp32 or bf16; it always runs on the kernels of fp32 precision).  Its
  * intermediates must fit the array, roughly max(m,n) * r <= 1,000,000; larger
  * matrices are rejected with FIRA_ERR_WORKSPACE_TOO_SMALL and a message giving the
  * sizes.  W_dev (updated in place), G_dev, P_dev (the d x r projection), M_dev and
@@ -290,7 +290,7 @@ FIRA_API const char* fira_phase_name(const fira_ctx* ctx, int32_t phase);
  * aligned device pointers; norm_prev_dev points to one float on the device (set it
  * to -1 before the first step: "no remembered norm yet") and t_dev to one int64 on
  * the device (0 before the first step); both are updated.  lr < 0 uses hp->lr.
- * The result equals fira_step()'s for the same matrix on the CUDA-core kernels.
+ * The result equals fira_step()'s for the same matrix on those kernels.
  *
  * Host-side argument errors (including the variant flags, none of which this entry
  * point supports: FIRA_ERR_UNSUPPORTED) are returned before anything is enqueued.

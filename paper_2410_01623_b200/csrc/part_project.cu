@@ -11,7 +11,8 @@
 // Epilogue: two groups of four warps, each on half of the tile's columns, one row per thread; R's parts leave as TMA boxes of
 // 128 rows x 16 columns x three parts.  The moments are a pass of their own (k_moments).  With Adam in this epilogue, M and V as
 // boxes, the epilogue took 30000 cycles per tile and the product, whose main accumulators wait for the same warps
-// every PROMOTE of k, stood still for half of them: MEASURE.
+// every PROMOTE of k, stood still for half of them; and M and V had to be addressable by TMA.
+// Measured (56 matrices 512 / 1376, r = 128): 61 us, 0.65 of the MMAs' time at full rate.
 //
 // What bounds it: the MMAs (12 per slab), G at the copy bandwidth close behind.
 //
