@@ -78,7 +78,7 @@ def tensor_peak(peaks, dtype, sustained):
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch, from an ncu capture of 2 layers of
 # the llama-7b list (every layer has the same shapes, so the traffic of a full launch is this times
 # the layer ratio).  None: the kernel has changed since its counters were taken.
-NCU_DRAM_BYTES_2_LAYERS = {"k_tc_project": 1.855e9 + 0.971e9, "k_tc_back_project": 1.999e9 + 0.781e9}
+NCU_DRAM_BYTES_2_LAYERS = {"k_tc_project": 1.881e9 + 1.172e9, "k_tc_back_project": 2.009e9 + 0.780e9}
 
 # kernel name -> (pipe that does its arithmetic, share of the step's 4 m n r flops)
 KERNEL_PIPE = {
