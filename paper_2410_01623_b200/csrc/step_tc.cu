@@ -13,7 +13,7 @@
 //   k_tc_form_x        X = a_low N - a_res lambda k_l R  (bf16).  In the plain step the projection
 //                      epilogue has written X for lambda = 1 already (see tc_project.cuh) and this
 //                      kernel only touches the matrices whose limiter acted (k_tc_fix_x):
-//                      X <- X + (1 - lambda) a_res k_l R, or the same with N from the stored moments
+//                      X <- lambda X + (1 - lambda) a_low N, N as the projection kept it or rebuilt from the stored moments
 //   k_tc_back_project  D = Pi X on the tensor cores; epilogue: W -= lr (D + a_res lambda k_l G)
 //
 // ||S_l||^2 = ||G_l - Pi R_l||^2 = ||G_l||^2 - 2 ||R_l||^2 + R_l^T (Pi^T Pi) R_l.  For orthonormal
@@ -292,13 +292,20 @@ k_tc_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int n
 }
 
 // The matrices whose X the projection epilogue has formed for lambda = 1 (FUSE_X): where the limiter
-// acted, X_lambda = a_low N - a_res lambda k_l R is X + (1 - lambda) a_res k_l R if the projection kept R (FUSE_X = 2), otherwise
-// lambda X + (1 - lambda) a_low N with N rebuilt from the moments that the epilogue stored, by the epilogue's
-// own arithmetic and rounded to bf16 as it was there; the other matrices are left as they are.
+// acted, X_lambda = a_low N - a_res lambda k_l R = lambda X + (1 - lambda) a_low N, with N as the projection kept it
+// (FUSE_X = 2), otherwise rebuilt from the moments that the epilogue stored, by the epilogue's own arithmetic and
+// rounded to bf16 as it was there; the other matrices are left as they are.
 // blockIdx.y = matrix of the range, the blocks of a matrix stride over its rows, one warp per row.  Bound by
 // memory.
+__device__ __forceinline__ uint4 limited_x(const uint4& x, const float (&n)[8], float lambda, float cn) {
+  float v[8];
+  unpack8_bf16(x, v);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = fmaf(cn, n[e], lambda * v[e]);
+  return pack8_bf16(v);
+}
 __global__ void __launch_bounds__(256)
-k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int first, float a_low, float a_res, float eps, int kept,
+k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int first, float a_low, float eps, int kept,
            float* __restrict__ fast) {
   const int p = first + blockIdx.y;
   const MatDev& mt = mats[list[p]];
@@ -310,21 +317,17 @@ k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int fi
   if (lambda == 1.f) return;
   const int lane = threadIdx.x & 31;
   const float bias = fast[2 * p];                      // this step's bias factor (k_tc_prep)
-  const float cn = (1.f - lambda) * a_low, cr = (1.f - lambda) * a_res;
+  const float cn = (1.f - lambda) * a_low;
   for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < mt.l; l += gridDim.x * 8) {
     const long long base = (long long)l * mt.r;
     if (kept) {
-      const float c = cr * mt.kvec[l];
 #pragma unroll 2
       for (int j = lane * 8; j < mt.r; j += 256) {
         const uint4 xu = *reinterpret_cast<const uint4*>(mt.Xb + base + j);
-        const uint4 ru = *reinterpret_cast<const uint4*>(mt.Rb + base + j);
-        float xv[8], rv[8];
-        unpack8_bf16(xu, xv);
-        unpack8_bf16(ru, rv);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) xv[e] = fmaf(c, rv[e], xv[e]);
-        *reinterpret_cast<uint4*>(mt.Xb + base + j) = pack8_bf16(xv);
+        const uint4 nu = *reinterpret_cast<const uint4*>(mt.Nb + base + j);
+        float nv[8];
+        unpack8_bf16(nu, nv);
+        *reinterpret_cast<uint4*>(mt.Xb + base + j) = limited_x(xu, nv, lambda, cn);
       }
       continue;
     }
@@ -334,14 +337,10 @@ k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int fi
       const float4 v0 = *reinterpret_cast<const float4*>(mt.V + base + j), v1 = *reinterpret_cast<const float4*>(mt.V + base + j + 4);
       const float mo[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
       const float vo[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-      float xv[8], x[8];
-      unpack8_bf16(xu, xv);
+      float nv[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float nv = __bfloat162float(__float2bfloat16_rn(__fdividef(bias * mo[e], fast_sqrt(vo[e]) + eps)));
-        x[e] = lambda * xv[e] + cn * nv;
-      }
-      *reinterpret_cast<uint4*>(mt.Xb + base + j) = pack8_bf16(x);
+      for (int e = 0; e < 8; ++e) nv[e] = __bfloat162float(__float2bfloat16_rn(__fdividef(bias * mo[e], fast_sqrt(vo[e]) + eps)));
+      *reinterpret_cast<uint4*>(mt.Xb + base + j) = limited_x(xu, nv, lambda, cn);
     }
   }
 }
@@ -827,10 +826,10 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   // Short products are bound by the epilogue, which then runs with two groups of warps per CTA; long
   // ones (r = 1024 lists) are bound by the tensor pipe and keep one.
   const bool two_groups = rmax <= 512;
-  bool keep_r = fused;
+  bool keep_n = fused;
   for (int q = qa; q < qb; ++q) {
     const MatDev& mq = c->mats[c->tc_list[q]];
-    if (fuse_x_matrix(mq.d, mq.r) && mq.d < FUSE_KEEP_R_MIN_D) keep_r = false;
+    if (fuse_x_matrix(mq.d, mq.r) && mq.d < FUSE_KEEP_N_MIN_D) keep_n = false;
   }
 #define FIRA_LAUNCH_K1(PSI, FUSE, EG)                                                                       \
   chain(launch_chained(k_tc_project<EPI_ADAM, PSI, FUSE, EG>, k1_grid, k1_threads(EG), k1_smem_bytes(EG), st, false, 1,  \
@@ -838,11 +837,11 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   if (hp.mode & HYPER_PSI_RMSPROP) FIRA_LAUNCH_K1(PSI_RMSPROP, 0, 1);
   else if (hp.mode & HYPER_PSI_ADAGRAD) FIRA_LAUNCH_K1(PSI_ADAGRAD, 0, 1);
   else if (two_groups) {
-    if (keep_r) FIRA_LAUNCH_K1(PSI_ADAM, 2, 2);
+    if (keep_n) FIRA_LAUNCH_K1(PSI_ADAM, 2, 2);
     else if (fused) FIRA_LAUNCH_K1(PSI_ADAM, 1, 2);
     else FIRA_LAUNCH_K1(PSI_ADAM, 0, 2);
   }
-  else if (keep_r) FIRA_LAUNCH_K1(PSI_ADAM, 2, 1);
+  else if (keep_n) FIRA_LAUNCH_K1(PSI_ADAM, 2, 1);
   else if (fused) FIRA_LAUNCH_K1(PSI_ADAM, 1, 1);
   else FIRA_LAUNCH_K1(PSI_ADAM, 0, 1);
 #undef FIRA_LAUNCH_K1
@@ -870,7 +869,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     chain(launch_chained(k_tc_form_x, (rsb - rsa + 7) / 8, 256, 0, st, false, 1, mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
                          hp.a_low, hp.a_res, pl->fast_dev, fused ? 1 : 0));
   if (any_fused)
-    chain(launch_chained(k_tc_fix_x, dim3(32, nq), 256, 0, st, false, 1, mats, pl->list, qa, hp.a_low, hp.a_res, hp.eps, keep_r ? 1 : 0, pl->fast_dev));
+    chain(launch_chained(k_tc_fix_x, dim3(32, nq), 256, 0, st, false, 1, mats, pl->list, qa, hp.a_low, hp.eps, keep_n ? 1 : 0, pl->fast_dev));
   tm->mark(st);
   // long products keep five operand stages; short ones trade one for more epilogue boxes in flight
   if (rmax >= 1024)

@@ -57,10 +57,11 @@
 // follows, on its pair, a tile far below it, so the waits cannot form a cycle as long as every block
 // of the grid is resident, which the launch ensures), the thread adds the partial sums in the fixed
 // order that k_tc_colfactors uses, and sweep 2 reads the pairs back and writes X (through the map of
-// the X buffer).  Where the limiter acts, k_tc_fix_x puts X right afterwards.  FUSE_X = 2 (lists of long products, see
-// FUSE_KEEP_R_MIN_D) leaves R for it, written in sweep 1, and it makes X_lambda = X + (1 - lambda) a_res k_l R,
-// 6 bytes per element; after FUSE_X = 1 it rebuilds N from the stored moments, X_lambda = lambda X + (1 - lambda) a_low N,
-// 12 bytes per element.
+// the X buffer).  Where the limiter acts, k_tc_fix_x puts X right afterwards, X_lambda = lambda X + (1 - lambda) a_low N.
+// FUSE_X = 2 (lists of long products, see FUSE_KEEP_N_MIN_D) leaves N for it, written in sweep 1: 6 bytes per element;
+// after FUSE_X = 1 it rebuilds the same N from the stored moments: 12 bytes per element.  (X + (1 - lambda) a_res k_l R from a
+// kept R costs the same and is less precise: X and R have each been rounded to bf16 before most of them cancels, which
+// leaves about 2.4 times the error.)
 // (Adam only: with RMSProp or Adagrad N cannot be rebuilt from V alone, and those steps keep the
 // separate pass.)
 constexpr int K1_STAGES = 4;
@@ -112,11 +113,11 @@ constexpr int PROJ_OUT_BF16 = 1 << 28, PROJ_OUT_REMAINDER = 1 << 27;
 // not been measured and keep the separate pass.
 constexpr int FUSE_X_MIN_D = 2048;
 __host__ __device__ inline bool fuse_x_matrix(int d, int r) { return d >= FUSE_X_MIN_D || r <= 256; }
-// R's boxes cost the epilogue a store, a wait and 2 bytes per element on every step, its absence 6 bytes per element of
+// N's boxes cost the epilogue a store, a wait and 2 bytes per element on every step, their absence 6 bytes per element of
 // the matrices whose limiter acts: half of them and more, since the remembered norm is the limited one.  Under a long
 // product the epilogue has the time.  Measured on the step, limiter acting: 1B list (d = 2048) -4 %, 7B list (d = 4096)
-// -4 %; 350M list (d = 1024), whose epilogue is its critical path, +3 %.
-constexpr int FUSE_KEEP_R_MIN_D = 2048;
+// -4 %; 350M list (d = 1024), whose epilogue is its critical path, +3 %.  X is the same bit for bit either way.
+constexpr int FUSE_KEEP_N_MIN_D = 2048;
 
 // EPI_PLAIN products may run over up to three k-segments that accumulate into the same tile: segment
 // s multiplies A taken through the map g1a (bit s of asel clear) or g2a (set) with B taken through
@@ -449,7 +450,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
         const TcMaps* mp = &maps[d.slot];
         const int bn = d.bn_left & 0xffff;
         const int l0 = d.l0 + BM * (int)rank;
-        const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_r = FUSE_X == 2 && fuse;
+        const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_n = FUSE_X == 2 && fuse;
         for (int b = 0; b < 2 * (bn / K1_ECOLS); ++b) {
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->eready[mv]), mvphase, abort_flag)) { ok = false; break; }
           const int nr = b & 1;
@@ -459,8 +460,8 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
             if (EPI == EPI_ADAM) {
               ptx::tma_store_2d(&mp->em, src, j, row);
               ptx::tma_store_2d(&mp->ev, src + K1_FBOX_BYTES, j, row);
-              if (keep_r) {
-                ptx::tma_store_2d(&mp->er, srn + ((b >> 1) & 1) * K1_HBOX_BYTES, j, row);
+              if (keep_n) {
+                ptx::tma_store_2d(&mp->en, srn + ((b >> 1) & 1) * K1_HBOX_BYTES, j, row);
               } else if (!fuse) {
                 ptx::tma_store_2d(&mp->en, srn, j, row);
                 ptx::tma_store_2d(&mp->er, srn + K1_HBOX_BYTES, j, row);
@@ -475,7 +476,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
             ptx::bulk_wait_group_read<0>();              // the boxes have been read: the buffers are free
           }
           ptx::mbar_arrive(ptx::smem_u32(&ctl->eempty[mv]));
-          if (keep_r || !fuse) ptx::mbar_arrive(ptx::smem_u32(keep_r ? &ctl->xempty[nr][(b >> 1) & 1] : &ctl->nrempty[nr]));
+          if (keep_n || !fuse) ptx::mbar_arrive(ptx::smem_u32(keep_n ? &ctl->xempty[nr][(b >> 1) & 1] : &ctl->nrempty[nr]));
           if (++mv == K1_MVBUFS) { mv = 0; mvphase ^= 1u; }
         }
         if (fuse && ok) {
@@ -539,7 +540,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
       const uint32_t tcol = tmem + ((uint32_t)(quarter * 32) << 16) + buf * BN_MAX;
       const uint32_t te = buf ? tmem_empty1 : tmem_empty0;
       const int nch = bn / K1_ECOLS;
-      const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_r = FUSE_X == 2 && fuse;
+      const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_n = FUSE_X == 2 && fuse;
       float nn = 0.f, rn = 0.f, rw = 0.f;
       for (int c = 0; c < nch; ++c) {
         uint32_t rr[GC];
@@ -555,8 +556,8 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
           if (lane == 0) ptx::mbar_arrive_cluster(te);
         }
         if (EPI == EPI_ADAM && !ptx::mbar_wait(ptx::smem_u32(&ctl->efull[mv][half]), mvphase, abort_flag)) { ok = false; break; }
-        const int xs = c & 1;                            // fuse: R boxes, then X boxes alternate between the two parts of the buffer
-        if (keep_r) {
+        const int xs = c & 1;                            // fuse: N boxes, then X boxes alternate between the two parts of the buffer
+        if (keep_n) {
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->xempty[half][xs]), ((xeph >> xs) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
           xeph ^= 1u << xs;
         }
@@ -633,9 +634,9 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
               const __nv_bfloat162 pr = __floats2bfloat162_rn(nv[e], rv[e]);
               rr[8 * qq + e] = *reinterpret_cast<const uint32_t*>(&pr);
             }
-            const uint32_t* w = &rr[8 * qq];             // R's halves
-            if (keep_r) *reinterpret_cast<uint4*>(nb + xs * K1_HBOX_BYTES + hrow + (((uint32_t)q ^ hsw) << 4)) =
-                make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632), __byte_perm(w[4], w[5], 0x7632), __byte_perm(w[6], w[7], 0x7632));
+            const uint32_t* w = &rr[8 * qq];             // N's halves
+            if (keep_n) *reinterpret_cast<uint4*>(nb + xs * K1_HBOX_BYTES + hrow + (((uint32_t)q ^ hsw) << 4)) =
+                make_uint4(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410), __byte_perm(w[4], w[5], 0x5410), __byte_perm(w[6], w[7], 0x5410));
           } else {
             const uint32_t h = hrow + (((uint32_t)q ^ hsw) << 4);
             *reinterpret_cast<uint4*>(nb + h) = pack8_bf16(nv);

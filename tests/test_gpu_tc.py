@@ -199,3 +199,46 @@ def test_run_twice_is_bitwise_deterministic_on_tensor_cores():
     b = _case([(512, 1376), (1376, 512)], 128, steps=3, seed=37, spike=(2,))
     for x, y in zip(a.W, b.W):
         assert torch.equal(x, y)
+
+
+def test_limited_x_does_not_depend_on_what_else_is_stepped():
+    """Where the limiter acts, X is corrected from the N that the projection left (lists of long products only) or from N
+    rebuilt from the moments: the same numbers, so W is bit for bit the same whether a long matrix is stepped with others
+    like it, in one list with a short one, or in a chunk of its own by fira_step_host."""
+    long_, r = [(2048, 2304), (2300, 2048)], 256
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda")                                    # noqa: E731
+    W0, G, P, M, V = [], [], [], [], []
+    for m, n in long_ + [(512, 768)]:
+        d, l = min(m, n), max(m, n)
+        W0.append((rand(m, n) * 0.02).to(torch.bfloat16))
+        G.append(rand(m, n).to(torch.bfloat16))
+        P.append(torch.linalg.qr(rand(d, r))[0].to(torch.bfloat16).contiguous())
+        M.append(rand(l, r) * 0.25)
+        V.append(rand(l, r).square() * 0.1 + 0.05)
+
+    def context(count):
+        f = fb.Fira((long_ + [(512, 768)])[:count], r, torch.bfloat16, fb.make_hparams())
+        for i in range(count):
+            f.set_projection(i, P[i])
+            f.set_state(i, M[i], V[i], 10.0, 100)
+        return f
+
+    alone, mixed, host = context(2), context(3), context(3)
+    Wa, Wm = [w.clone() for w in W0[:2]], [w.clone() for w in W0]
+    alone.step(Wa, G[:2])
+    mixed.step(Wm, G)
+    Wh = [w.cpu().pin_memory() for w in W0]
+    host.step_host(Wh, [x.cpu().pin_memory() for x in G], torch.empty(host.staging_bytes(), dtype=torch.uint8, device="cuda"))
+    torch.cuda.synchronize()
+    for i in range(2):
+        assert alone.diagnostics(i)["lam"] < 0.2
+        assert torch.equal(Wa[i], Wm[i])
+        assert torch.equal(Wh[i], Wm[i].cpu())
+
+
+def test_limiter_acts_on_a_list_of_long_products_with_ragged_rows():
+    """Every matrix has d >= 2048: the projection keeps N for the limiter's correction, with one and with two r-tiles."""
+    tr = _case([(2048, 2300), (2309, 2048)], [512, 256], steps=3, seed=78, spike=(3,))
+    tr.assert_ok()
+    assert all(l < 0.5 for l in tr.lams[2])
