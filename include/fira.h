@@ -34,7 +34,10 @@
  * (each l x r, row major, float: row i belongs to column i of G when m <= n and to
  * row i of G when m > n, i.e. the transpose of the paper's r x n layout in the
  * first case), ||S_prev|| (float) and t (int64): the d r + 2 l r + 1 numbers of the
- * paper's comparison table plus the step count.  The scratch buffer holds
+ * paper's comparison table plus the step count.  A caller may save these bytes and
+ * write them back between calls; matrices of the bf16 tensor-core engine then keep the
+ * column norms (1 to about 2^-8) of the projection that was last set or refreshed
+ * through a call, which enter ||S|| only.  The scratch buffer holds
  * intermediates and is overwritten by every call.
  *
  * Streams and errors.  All device work is enqueued on the stream given to

@@ -21,10 +21,19 @@ struct MatScalars {
   float lambda;       // limiter factor of the latest step
   float norm_scaled;  // ||S|| before the limiter
   float k_min, k_max;
-  float pad;          // bias factor sqrt(1-b2^s)/(1-b1^s) of the next step, s = t + 1
+  float bias;         // bias factor sqrt(1-b2^s)/(1-b1^s) of the latest step (bf16 engine; nothing reads it)
   long long t;        // steps taken
 };
 static_assert(sizeof(MatScalars) == 32, "MatScalars layout");
+
+// The bias factor that k_finalize works out ahead for the step after, while it waits (in double it costs a microsecond), and
+// the step it is for: whoever takes it compares that with the step count in the state buffer, whose bytes the caller may
+// have changed since, and makes his own if they differ.
+struct BiasSlot {
+  long long step;
+  float next;         // the factor of `step`
+  float now;          // long lists of fp32 precision: the factor of the running step
+};
 
 // One entry of the device-resident problem table.  l = max(m,n) indexes the
 // unprojected extent, d = min(m,n) the projected one.
@@ -35,12 +44,12 @@ struct MatDev {
   float* M;           // l x r
   float* V;           // l x r
   MatScalars* sc;
+  BiasSlot* bias;     // scratch, outside the area that the refresh uses
   float* Rt;          // scratch: l x r fp32 low-rank gradient (transposed layout)
   float* Xt;          // scratch: l x r fp32 N
   __nv_bfloat16* Rp;  //   "      long lists (PartStepPlan): R and X as three bf16 parts [3][l][rp_pitch]
   __nv_bfloat16* Xp;
   __nv_bfloat16* Pp;  //   "      the projection as parts [3 or 1][d][pp_pitch]
-  float* step_bias;   //   "      this step's bias factor (k_finalize puts the next one into MatScalars)
   int rp_pitch, pp_pitch;
   int aux_slots;      // row sums per l in aux
   float* kvec;        // scratch: l factors
@@ -75,8 +84,12 @@ enum HyperMode : unsigned {
 };
 
 // sqrt(1 - b2^s) / (1 - b1^s) (Eq. 4), in double.
-__host__ __device__ inline float bias_factor(float beta1, float beta2, long long s) {
+__device__ __noinline__ inline float bias_factor(float beta1, float beta2, long long s) {
   return (float)(sqrt(1.0 - pow((double)beta2, (double)s)) / (1.0 - pow((double)beta1, (double)s)));
+}
+// The factor of step s.
+__device__ __forceinline__ float step_bias(const BiasSlot& slot, long long s, const Hyper& hp) {
+  return slot.step == s ? slot.next : bias_factor(hp.beta1, hp.beta2, s);
 }
 
 enum DeviceStatusBits : unsigned {

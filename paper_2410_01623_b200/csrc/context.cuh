@@ -43,7 +43,6 @@ struct fira_ctx {
   fira::HostPipe pipe;
   bool table_dirty = true;
   bool proj_weights_dirty = true;        // tensor-core path: column norms of the stored projections to be retaken
-  bool proj_parts_dirty = true;          // long lists of the fp32-precision engine: the stored projections to be split again
   int last_launches = 0;
 };
 
@@ -54,10 +53,10 @@ struct Layout {
   std::vector<size_t> offP, offM, offV, offS;
   size_t state_bytes = 0;
   // byte offsets inside the scratch buffer
-  size_t off_mats = 0, off_status = 0, off_ints = 0, off_tcmaps = 0, off_work = 0;
+  size_t off_mats = 0, off_status = 0, off_bias = 0, off_ints = 0, off_tcmaps = 0, off_work = 0;
   size_t ints_count = 0;
   // byte offsets per matrix inside the work area
-  std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux, offRp, offXp, offPp, offBias;
+  std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux, offRp, offXp, offPp;
   std::vector<int> engine;
   bool parts = false;       // the fp32-precision engine's list is long
   size_t off_parts = 0, off_proj_parts = 0;

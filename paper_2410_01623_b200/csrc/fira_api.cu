@@ -88,6 +88,7 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
   size_t wo = 0;
   L.off_mats = wo; wo += align_up(sizeof(MatDev) * count);
   L.off_status = wo; wo += 256;
+  L.off_bias = wo; wo += align_up(sizeof(BiasSlot) * count);
   L.ints_count = 20 * (size_t)(count + 1);
   L.off_ints = wo; wo += align_up(L.ints_count * sizeof(int));
   L.off_tcmaps = wo; wo += tc_tables_bytes(hp, descs, count);
@@ -113,7 +114,7 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
   L.offRt.assign(count, 0); L.offXt.assign(count, 0); L.offK.assign(count, 0); L.offPart.assign(count, 0);
   L.offNb.assign(count, 0); L.offRb.assign(count, 0); L.offXb.assign(count, 0);
   L.offColpart.assign(count, 0); L.offGs.assign(count, 0); L.offWs.assign(count, 0); L.offAux.assign(count, 0); L.offRp.assign(count, 0); L.offPp.assign(count, 0);
-  L.offXp.assign(count, 0); L.offBias.assign(count, 0);
+  L.offXp.assign(count, 0);
   for (int i = 0; i < count; ++i) {
     fira_matrix_desc d = descs[i];
     if (d.ld == 0) d.ld = d.n;
@@ -127,7 +128,6 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
         L.offRp[i] = w; w += align_up(3 * ll * pitch * 2);
         L.offXp[i] = w; w += align_up(3 * ll * pitch * 2);
         L.offPp[i] = w; w += align_up((d.dtype == FIRA_BF16 ? 1 : 3) * dd * part_pitch(d.r) * 2);
-        L.offBias[i] = w; w += 256;
         const size_t bytes = (size_t)d.m * part_staging_pitch(d, hp.flags) * (d.dtype == FIRA_BF16 ? 2 : 4);
         L.offGs[i] = w; w += align_up(bytes);
         L.offWs[i] = w; w += align_up(bytes);
@@ -254,6 +254,7 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
     mt.M = (float*)(c->state_base + L.offM[i]);
     mt.V = (float*)(c->state_base + L.offV[i]);
     mt.sc = (MatScalars*)(c->state_base + L.offS[i]);
+    mt.bias = L.engine[i] == 0 ? (BiasSlot*)(c->scratch_base + L.off_bias) + i : nullptr;    // (the bf16 engine has k_tc_prep)
     mt.kvec = (float*)(c->work_base + L.offK[i]);
     mt.aux = (float*)(c->work_base + L.offAux[i]);
     mt.part = (float*)(c->work_base + L.offPart[i]);
@@ -263,7 +264,6 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
         mt.Rp = (__nv_bfloat16*)(c->work_base + L.offRp[i]);
         mt.Pp = (__nv_bfloat16*)(c->work_base + L.offPp[i]);
         mt.Xp = (__nv_bfloat16*)(c->work_base + L.offXp[i]);
-        mt.step_bias = (float*)(c->work_base + L.offBias[i]);
         mt.rp_pitch = part_rank_pitch(d.r);
         mt.pp_pitch = (int)part_pitch(d.r);
         mt.lds = part_staging_pitch(c->descs[i], c->hp.flags);
@@ -316,6 +316,7 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
     for (int i : c->simt_list) {
       c->simt.max_d = std::max(c->simt.max_d, c->mats[i].d);
       c->simt.max_r = std::max(c->simt.max_r, c->mats[i].r);
+      c->simt.max_proj_units = std::max(c->simt.max_proj_units, (long long)c->mats[i].d * c->mats[i].pp_pitch / 8);
     }
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
     c->simt.npart = c->ints_dev + o_np; c->simt.npart_tiles = c->ints_dev + o_npt;
@@ -335,10 +336,11 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
   if (!ints.empty()) ce = cudaMemcpyAsync(c->ints_dev, ints.data(), ints.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(c->state_base, 0, L.state_bytes, c->stream);
   if (ce == cudaSuccess) ce = cudaMemsetAsync(c->status_dev, 0, 256, c->stream);
+  if (ce == cudaSuccess) ce = cudaMemsetAsync(c->scratch_base + L.off_bias, 0, sizeof(BiasSlot) * count, c->stream);   // (no step is the 0th)
   // ||S_prev|| = -1 marks "unset"
   MatScalars init;
   memset(&init, 0, sizeof(init));
-  init.prev_norm = -1.f; init.lambda = 1.f; init.pad = bias_factor(hp->beta1, hp->beta2, 1);
+  init.prev_norm = -1.f; init.lambda = 1.f;
   for (int i = 0; i < count && ce == cudaSuccess; ++i)
     ce = cudaMemcpyAsync(c->mats[i].sc, &init, sizeof(MatScalars), cudaMemcpyHostToDevice, c->stream);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(c->mats_dev, c->mats.data(), sizeof(MatDev) * count, cudaMemcpyHostToDevice, c->stream);
@@ -372,10 +374,6 @@ static fira_status set_pointers(fira_ctx* c, void* const* W_dev, const void* con
 // Enqueues the step of the matrices [i0, i1) (both engines' lists are ascending, so the range maps
 // to one sub-range of each); returns the number of launches or -1.
 static int launch_range(fira_ctx* c, const Hyper& h, int i0, int i1, bool whole) {
-  if (c->proj_parts_dirty) {          // the stored projections have changed since they were split
-    launch_split_projections(c->simt, c->mats, c->simt_list, c->stream);
-    c->proj_parts_dirty = false;
-  }
   if (whole) {
     const int launches = launch_simt_step(c->simt, h, c->status_dev, c->stream, &c->timer);
     if (launches < 0) return -1;
@@ -612,7 +610,7 @@ fira_status fira_set_projection(fira_ctx* c, int32_t idx, const void* P_dev) {
   const MatDev& mt = c->mats[idx];
   const size_t bytes = (size_t)mt.d * mt.r * (mt.bf16 ? 2 : 4);
   FIRA_CUDA(cudaMemcpyAsync(mt.P, P_dev, bytes, cudaMemcpyDeviceToDevice, c->stream));
-  c->proj_weights_dirty = c->proj_parts_dirty = true;
+  c->proj_weights_dirty = true;
   return FIRA_OK;
 }
 
@@ -652,7 +650,6 @@ fira_status fira_set_state(fira_ctx* c, int32_t idx, const float* M_dev, const f
   memset(&sc, 0, sizeof(sc));
   sc.prev_norm = norm_prev < 0.f ? -1.f : norm_prev;
   sc.lambda = 1.f;
-  sc.pad = bias_factor(c->hp.beta1, c->hp.beta2, t + 1);
   sc.t = t;
   FIRA_CUDA(cudaMemcpyAsync(mt.sc, &sc, sizeof(sc), cudaMemcpyHostToDevice, c->stream));
   FIRA_CUDA(cudaStreamSynchronize(c->stream));

@@ -62,7 +62,7 @@ unsigned char* scratch_base() {
 }
 
 struct Carve {
-  size_t off_mats, off_status, off_ints, off_sc, off_rt, off_xt, off_k, off_part, total;
+  size_t off_mats, off_status, off_ints, off_sc, off_bias, off_rt, off_xt, off_k, off_part, total;
 };
 
 Carve carve(int m, int n, int r) {
@@ -73,7 +73,7 @@ Carve carve(int m, int n, int r) {
   c.off_mats = o; o += align_up(sizeof(MatDev));
   c.off_status = o; o += 256;
   c.off_ints = o; o += 256;
-  c.off_sc = o; o += align_up(sizeof(MatScalars));
+  c.off_sc = o; c.off_bias = o + sizeof(MatScalars); o += align_up(sizeof(MatScalars) + sizeof(BiasSlot));
   c.off_rt = o; o += align_up(l * r * 4);
   c.off_xt = o; o += align_up(l * r * 4);
   c.off_k = o; o += align_up(l * 4);
@@ -97,9 +97,10 @@ __global__ void k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, i
   for (int i = 0; i < 6; ++i) ints_out[i] = ints.v[i];
   MatScalars* sc = mt.sc;
   sc->prev_norm = (*norm_prev < 0.f) ? -1.f : *norm_prev;
-  sc->lambda = 1.f; sc->norm_scaled = 0.f; sc->k_min = 0.f; sc->k_max = 0.f;
-  sc->pad = bias_factor(beta1, beta2, *t + 1);
+  sc->lambda = 1.f; sc->norm_scaled = 0.f; sc->k_min = 0.f; sc->k_max = 0.f; sc->bias = 0.f;
   sc->t = *t;
+  mt.bias->step = *t + 1;
+  mt.bias->next = bias_factor(beta1, beta2, *t + 1);
 }
 __global__ void k_noalloc_store_scalars(const MatScalars* sc, float* norm_prev, long long* t) {
   ptx::grid_wait();
@@ -148,6 +149,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   memset(&mt, 0, sizeof(mt));
   mt.W = W_dev; mt.G = G_dev; mt.P = const_cast<void*>(P_dev); mt.M = M_dev; mt.V = V_dev;
   mt.sc = reinterpret_cast<MatScalars*>(base + cv.off_sc);
+  mt.bias = reinterpret_cast<BiasSlot*>(base + cv.off_bias);
   mt.Rt = reinterpret_cast<float*>(base + cv.off_rt);
   mt.Xt = reinterpret_cast<float*>(base + cv.off_xt);
   mt.kvec = reinterpret_cast<float*>(base + cv.off_k);

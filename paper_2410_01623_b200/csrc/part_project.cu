@@ -401,7 +401,8 @@ fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, i
   if (count == 0) return FIRA_OK;
   const ProjJob* jobs = reinterpret_cast<const ProjJob*>(plan.proj_table);
   const TileDev* tiles = reinterpret_cast<const TileDev*>(plan.proj_table + align_up(sizeof(ProjJob) * (size_t)plan.njobs)) + first;
-  const cudaError_t e = launch_chained(k_part_project, 2 * std::min(count, sms / 2), THREADS, SMEM_BYTES, st, false, 1, jobs, tiles, count, mats_dev, status_dev);
+  // (chained: behind k_split_projection)
+  const cudaError_t e = launch_chained(k_part_project, 2 * std::min(count, sms / 2), THREADS, SMEM_BYTES, st, true, 1, jobs, tiles, count, mats_dev, status_dev);
   if (e != cudaSuccess) { set_error(std::string("step projection: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }

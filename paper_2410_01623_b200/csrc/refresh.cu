@@ -323,7 +323,7 @@ fira_status refresh_impl(fira_ctx* c, const void* const* G_dev, const std::vecto
   RefreshTarget own;
   own.work_base = c->work_base; own.work_bytes = c->work_bytes; own.stream = c->stream;
   const RefreshTarget& tg = target ? *target : own;
-  if (!tg.P_out) c->proj_weights_dirty = c->proj_parts_dirty = true;
+  if (!tg.P_out) c->proj_weights_dirty = true;
   cudaStream_t st = tg.stream;
   size_t pos = 0;
   while (pos < which.size()) {

@@ -51,6 +51,7 @@ struct Ctl {
   uint32_t tmem_base;
   int abort_flag;
   float red[THREADS / 32];
+  float bias;                                   // (k_project)
 };
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + (int)sizeof(Ctl);
 static_assert(2 * (SMEM_BYTES + 1024) <= 228 * 1024, "two blocks per SM");
@@ -279,8 +280,8 @@ __device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, bool a_
 }
 
 // The slabs of tile_product: loads one slab ahead, splits, issues; sum: pieces of the main product.
-template <bool LONG_K, bool REGULAR, class A, class B>
-__device__ __forceinline__ void product_slabs(A& a, B& b, int K, int n, unsigned char* slabs, Ctl* ctl, float (&sum)[LONG_K ? TILE / 2 : 1]) {
+template <bool LONG_K, bool REGULAR, class A, class B, class F>
+__device__ __forceinline__ void product_slabs(A& a, B& b, int K, int n, unsigned char* slabs, Ctl* ctl, float (&sum)[LONG_K ? TILE / 2 : 1], const F& meanwhile) {
   const int ns = (K + BK - 1) / BK;
   const int warp = threadIdx.x >> 5, c0 = (warp >> 2) * (TILE / 2);
   const uint32_t tmem = ctl->tmem_base;
@@ -288,6 +289,7 @@ __device__ __forceinline__ void product_slabs(A& a, B& b, int K, int n, unsigned
   bool fresh = true;
   a.template load<REGULAR>(0);
   b.template load<REGULAR>(0);
+  meanwhile();
   for (int s = 0; s < ns; ++s) {
     unsigned char* slab = slabs + (s % STAGES) * STAGE_BYTES;
     const uint32_t done = ptx::smem_u32(&ctl->done[s % STAGES]);
@@ -328,8 +330,10 @@ __device__ __forceinline__ void product_slabs(A& a, B& b, int K, int n, unsigned
 // The tile A B over k < K into shared memory, row x of A at C[x * C_LD]; ends with a block barrier.
 // cols: columns of the tile that are wanted (the others hold garbage).  C overlays the slabs.
 // Returns false if a wait ran out (bounded as in tc_ptx.cuh); all threads take the same path even then.
-template <bool LONG_K, class A, class B>
-__device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsigned char* slabs, Ctl* ctl) {
+// meanwhile: called by every thread while its first loads are on their way.
+struct Nothing { __device__ __forceinline__ void operator()() const {} };
+template <bool LONG_K, class A, class B, class F = Nothing>
+__device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsigned char* slabs, Ctl* ctl, const F& meanwhile = F()) {
   constexpr bool SMALL = A::PARTS > 1 || B::PARTS > 1;
   const int n = (min(cols, TILE) + 15) / 16 * 16;
   const int ns = (K + BK - 1) / BK;
@@ -341,8 +345,8 @@ __device__ __forceinline__ bool tile_product(A& a, B& b, int K, int cols, unsign
 #pragma unroll
     for (int i = 0; i < TILE / 2; ++i) sum[LONG_K ? i : 0] = 0.f;
   }
-  if (a.regular() && b.regular()) product_slabs<LONG_K, true>(a, b, K, n, slabs, ctl, sum);
-  else product_slabs<LONG_K, false>(a, b, K, n, slabs, ctl, sum);
+  if (a.regular() && b.regular()) product_slabs<LONG_K, true>(a, b, K, n, slabs, ctl, sum, meanwhile);
+  else product_slabs<LONG_K, false>(a, b, K, n, slabs, ctl, sum, meanwhile);
   // all MMAs: the last commit covers the earlier ones; nobody overwrites the slabs before everybody has seen it
   const int last = ns - 1;
   const bool ok = ptx::mbar_wait(ptx::smem_u32(&ctl->done[last % STAGES]), (last / STAGES) & 1, &ctl->abort_flag);

@@ -198,12 +198,12 @@ __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, cons
 }
 
 // The part of the tile's product that k in [k0, k1) makes.
-template <typename T, bool LONG_K>
-__device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, int k0, int k1, unsigned char* smem, split::Ctl* ctl) {
+template <typename T, bool LONG_K, class F>
+__device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, int k0, int k1, unsigned char* smem, split::Ctl* ctl, const F& meanwhile) {
   // A(i = l, k = d): G[d][l] when left, G[l][d] when right.
   split::Operand<T> a(static_cast<const T*>(mt.G) + (mt.left ? k0 * mt.ld : (long long)k0), mt.left ? 1 : mt.ld, mt.left ? mt.ld : 1, mt.l, k1 - k0, l0);
   split::Operand<T> b(static_cast<const T*>(mt.P) + (long long)k0 * mt.r, 1, mt.r, mt.r, k1 - k0, j0);
-  return split::tile_product<LONG_K>(a, b, k1 - k0, mt.r - j0, smem, ctl);
+  return split::tile_product<LONG_K>(a, b, k1 - k0, mt.r - j0, smem, ctl, meanwhile);
 }
 
 // SPLIT: the blocks of a cluster share the tile's product by k, each leaves its part in its shared memory, and they add the
@@ -228,17 +228,25 @@ k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
   const int slabs = (mt.d + split::BK - 1) / split::BK;
   const int k0 = slabs * block / blocks * split::BK, k1 = min(mt.d, slabs * (block + 1) / blocks * split::BK);
   const float* C = reinterpret_cast<const float*>(smem);
+  // The bias factor, by one thread: while its first loads are on their way, or before them (not SPLIT: registers).
+  const long long step = mt.sc->t + 1;
+  const BiasSlot slot = *mt.bias;
+  auto put_bias = [&] { if (PSI == PSI_ADAM && threadIdx.x == split::THREADS - 1) ctl->bias = step_bias(slot, step, hp); };
+  if (!SPLIT) put_bias();
+  auto bias_factor_of_step = [&] { if (SPLIT) put_bias(); };
   bool ok = true;
   if (k1 > k0) {
-    ok = mt.bf16 ? project_tile<__nv_bfloat16, LONG_K>(mt, l0, j0, k0, k1, smem, ctl) : project_tile<float, LONG_K>(mt, l0, j0, k0, k1, smem, ctl);
+    ok = mt.bf16 ? project_tile<__nv_bfloat16, LONG_K>(mt, l0, j0, k0, k1, smem, ctl, bias_factor_of_step)
+                 : project_tile<float, LONG_K>(mt, l0, j0, k0, k1, smem, ctl, bias_factor_of_step);
   } else {                                      // fewer slabs than blocks
+    bias_factor_of_step();
+    __syncthreads();
     for (int i = threadIdx.x; i < SIMT_TILE * split::C_LD; i += split::THREADS) reinterpret_cast<float*>(smem)[i] = 0.f;
   }
   if (SPLIT) ptx::cluster_arrive();
   if (SPLIT || ok) {                            // (a block whose wait ran out still meets the others)
-    const float bias = mt.sc->pad;
-    if (mt.r % 4 == 0) adam_rows<PSI, true, SPLIT>(mt, l0, j0, C, hp, bias);
-    else adam_rows<PSI, false, SPLIT>(mt, l0, j0, C, hp, bias);
+    if (mt.r % 4 == 0) adam_rows<PSI, true, SPLIT>(mt, l0, j0, C, hp, ctl->bias);
+    else adam_rows<PSI, false, SPLIT>(mt, l0, j0, C, hp, ctl->bias);
   }
   if (SPLIT) ptx::cluster_sync_all();           // nobody leaves while others read its part
   split::end(ctl, status);
@@ -439,7 +447,7 @@ k_moments(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
   while (row < end) {
     const MatDev& mt = mats[list[p]];
     const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
-    const float bias = mt.sc->pad;
+    const float bias = mt.bias->now;
     constexpr int ROWS = CHUNKS == 1 ? 2 : 1;
     if (mt.r % 4 == 0) {
       for (int l = l0; l < l1; l += ROWS) moment_rows<PSI, true, CHUNKS, ROWS>(mt, l, min(ROWS, l1 - l), hp, bias);
@@ -493,7 +501,7 @@ k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlis
   while (row < end) {
     const MatDev& mt = mats[list[p]];
     const int l0 = row - row_start[p], l1 = min(l0 + end - row, mt.l);
-    const float lambda = mt.sc->lambda, c = hp.a_res * lambda, bias = *mt.step_bias;
+    const float lambda = mt.sc->lambda, c = hp.a_res * lambda, bias = mt.bias->now;
     if (part_forms_x(hp) && lambda == 1.f) {
       // k_moments has formed it
     } else if (mt.r % 4 == 0) {
@@ -506,25 +514,30 @@ k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlis
   }
 }
 
-// The projection's parts, eight neighbours per thread (blockIdx.y = matrix of the list).
-__global__ void __launch_bounds__(256)
-k_split_projection(const MatDev* __restrict__ mats, const int* __restrict__ list) {
-  const MatDev& mt = mats[list[blockIdx.y]];
-  const long long per_row = mt.pp_pitch / 8, units = mt.d * per_row, stride = 2ll * mt.d * mt.pp_pitch;
+// The projection's parts, eight neighbours per thread and pass, `per` blocks per matrix, and the step's bias factor.  In
+// every step: projection and step count are in the caller's state buffer, whose bytes may have changed since the last one.
+// (56 matrices 512 / 1376, r = 128: 37 MB, 5.5 of the step's 242 us; k_part_project's set-up, which is chained to it, runs
+// meanwhile.)
+template <typename T>
+__device__ __forceinline__ void split_units(const MatDev& mt, int block, int blocks) {
+  const unsigned per_row = mt.pp_pitch / 8, units = mt.d * per_row, step = 256 * blocks;        // (r <= PART_STEP_MAX_RANK)
+  const long long stride = 2ll * mt.d * mt.pp_pitch;
   const bool vec = mt.r % 8 == 0;
-  for (long long u = blockIdx.x * 256ll + threadIdx.x; u < units; u += gridDim.x * 256ll) {
-    const long long i = u / per_row, j = u % per_row * 8;
-    unsigned char* out = reinterpret_cast<unsigned char*>(mt.Pp + i * mt.pp_pitch + j);
-    if (mt.bf16) {
-      split::Frag<__nv_bfloat16> f;
-      split::load_frag(static_cast<const __nv_bfloat16*>(mt.P) + i * mt.r + j, (int)(mt.r - j), vec, f);
-      split::store_parts(out, f);
-    } else {
-      split::Frag<float> f;
-      split::load_frag(static_cast<const float*>(mt.P) + i * mt.r + j, (int)(mt.r - j), vec, f);
-      split::store_parts(out, f, stride);
-    }
+  for (unsigned u = 256 * block + threadIdx.x; u < units; u += step) {
+    const unsigned i = u / per_row, j = u % per_row * 8;
+    split::Frag<T> f;
+    split::load_frag(static_cast<const T*>(mt.P) + (long long)i * mt.r + j, mt.r - (int)j, vec, f);
+    split::store_parts(reinterpret_cast<unsigned char*>(mt.Pp + (long long)i * mt.pp_pitch + j), f, stride);
   }
+}
+__global__ void __launch_bounds__(256)
+k_split_projection(const MatDev* __restrict__ mats, const int* __restrict__ list, int per, Hyper hp) {
+  ptx::grid_launch_next();
+  const MatDev& mt = mats[list[blockIdx.x / per]];
+  const int block = blockIdx.x % per;
+  if (block == 0 && threadIdx.x == 0) mt.bias->now = step_bias(*mt.bias, mt.sc->t + 1, hp);
+  if (mt.bf16) split_units<__nv_bfloat16>(mt, block, per);
+  else split_units<float>(mt, block, per);
 }
 
 // ---------------------------------------------------------------- Fira-only-scaling
@@ -621,10 +634,10 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   __shared__ float smin[256], smax[256];
   const MatDev mt = mats[list[blockIdx.x]];
   const int npart = npart_of[blockIdx.x];
-  // the bias factor sqrt(1 - b2^s) / (1 - b1^s) of the NEXT step, in double, while the others wait and add up
-  if (threadIdx.x == 255) {
-    if (mt.step_bias) *mt.step_bias = mt.sc->pad;
-    mt.sc->pad = bias_factor(hp.beta1, hp.beta2, mt.sc->t + 2);
+  if (threadIdx.x == 255 && mt.bias && !(hp.mode & (HYPER_PSI_RMSPROP | HYPER_PSI_ADAGRAD))) {    // the next step's bias factor
+    const long long next = mt.sc->t + 2;
+    mt.bias->next = bias_factor(hp.beta1, hp.beta2, next);
+    mt.bias->step = next;
   }
   ptx::grid_wait();
   ptx::grid_launch_next();
@@ -705,11 +718,9 @@ bool simt_long_list(const std::vector<fira_matrix_desc>& list) {
   return elements >= LONG_LIST_ELEMENTS;
 }
 
-void launch_split_projections(const SimtPlan& pl, const std::vector<MatDev>& mats, const std::vector<int>& list, cudaStream_t st) {
-  if (!pl.parts.table) return;
-  long long units = 1;
-  for (int i : list) units = std::max(units, (long long)mats[i].d * mats[i].pp_pitch / 8);
-  k_split_projection<<<dim3((unsigned)std::min<long long>(64, (units + 255) / 256), (unsigned)list.size()), 256, 0, st>>>(pl.mats, pl.list);
+static void split_projections(const SimtPlan& pl, int qa, int qb, const Hyper& hp, cudaStream_t st) {
+  const int per = (int)std::min<long long>(64, (pl.max_proj_units + 255) / 256);
+  k_split_projection<<<(unsigned)((qb - qa) * per), 256, 0, st>>>(pl.mats, pl.list + qa, per, hp);
 }
 
 // The products' shared memory is above the default limit: a per-device, per-kernel setting.
@@ -788,6 +799,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   tm->mark(st);
   launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 0, st);
   if (pl.parts.table) {                // (also before only-scaling, which needs the factors)
+    split_projections(pl, qa, qe, hp, st);
     if (part_project_run(pl.parts, pl.mats, qa, qe, status_dev, st) != FIRA_OK) return -1;
     tm->mark(st);
     const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
@@ -824,7 +836,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     launch_error(launch_chained(k_back_project<MODE_UPDATE>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
-  return 4 + (pl.parts.table ? 1 : 0) + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
+  return 4 + (pl.parts.table ? 2 : 0) + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);
 }
 
 }  // namespace fira

@@ -45,6 +45,7 @@ struct SimtPlan {
   const int* proj_tile_start = nullptr;  // 128 x 128 tiles of R (l x r)
   int proj_tiles = 0;
   int max_d = 0, max_r = 0;              // largest d and r of the list
+  long long max_proj_units = 0;          // long lists: largest projection, in units of eight entries of its parts
   const int* w_tile_start = nullptr;     // 128 x 128 tiles of W (m x n)
   int w_tiles = 0;
   const int* npart = nullptr;            // partial sums of ||S||^2 per matrix
@@ -65,11 +66,8 @@ struct SimtPlan {
 bool simt_long_list(const std::vector<fira_matrix_desc>& list);
 // Copies rows of staged matrices (MatDev Gs, Ws): dir 0 G and W in, 1 W out (step_tc.cu).
 void launch_stage(const MatDev* mats, const int* list, int nlist, const int* row_start, int first_row, int rows, int dir, cudaStream_t st);
-// Splits the stored projections into parts; to be called after they have changed.
-void launch_split_projections(const SimtPlan& pl, const std::vector<MatDev>& mats, const std::vector<int>& list, cudaStream_t st);
 // Enqueues the phases for the matrices [qa, qb) of the list (qb < 0: the whole list); returns
-// the number of launches (negative: error, message set).  MatScalars::pad has to hold the bias factor of
-// the step (bias_factor).
+// the number of launches (negative: error, message set).
 int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, cudaStream_t st,
                      PhaseTimer* tm, int qa = 0, int qb = -1);
 extern const char* const kSimtPhaseNames[SIMT_PHASES];
@@ -77,7 +75,7 @@ extern const char* const kSimtPhaseNames[SIMT_PHASES];
 // One block of 256 threads per matrix of the list: sums the matrix's partial sums
 // of ||S||^2 (npart_of[i] floats at mt.part) in a fixed order, applies the limiter
 // rule (Eq. 12 in Algorithm 1's form), stores lambda and the new ||S_prev||,
-// records the range of k, advances t and leaves the next step's bias factor.
+// records the range of k and advances t.
 __global__ void k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
                            const int* __restrict__ npart_of, Hyper hp, unsigned* __restrict__ status);
 

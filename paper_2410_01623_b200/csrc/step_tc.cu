@@ -120,7 +120,7 @@ k_tc_prep(const MatDev* __restrict__ mats, const int* __restrict__ list, int fir
   if (threadIdx.x == 0) {
     const double s = (double)(mt.sc->t + 1);
     const float bias = (float)(sqrt(1.0 - pow((double)hp.beta2, s)) / (1.0 - pow((double)hp.beta1, s)));
-    mt.sc->pad = bias;
+    mt.sc->bias = bias;
     fast[2 * p] = bias;          // read by the projection epilogue
   }
   // the counters through which the projection epilogues of a row of tiles tell one another that
