@@ -175,7 +175,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   SimtPlan pl;
   pl.mats = reinterpret_cast<const MatDev*>(base + cv.off_mats);
   pl.list = ints_dev; pl.nlist = 1; pl.chained = true;
-  pl.proj_tile_start = ints_dev + 1; pl.proj_tiles = ptiles; pl.max_d = mt.d;
+  pl.proj_tile_start = ints_dev + 1; pl.proj_tiles = ptiles; pl.max_d = mt.d; pl.max_r = mt.r;
   pl.w_tile_start = ints_dev + 3; pl.w_tiles = wtiles;
   pl.npart = ints_dev + 5;
   Hyper h;

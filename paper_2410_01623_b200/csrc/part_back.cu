@@ -9,9 +9,13 @@
 // and W along rows with ordinary loads needed 10 us per tile where this needs 4: four times the instructions, and two
 // load latencies per tile that nothing covered.)
 //
-// Tensor memory: main and small products (split_gemm.cuh) of a tile take 2 x 128 columns, two such sets alternate.
-// No sums in registers: a rank up to 256 is 16 truncated additions of the main product, as many as PROMOTE allows twice
-// over; ranks up to 512 (`deep`) put the second half into a second main accumulator and use one set only.
+// Tensor memory: main and small products (split_gemm.cuh) of a tile take 2 x 128 columns, two such sets alternate.  That is
+// for lists of ranks up to PROMOTE.  With a longer one among them (DEEP) the main product alternates between two accumulators
+// every PROMOTE of k and the small products between two others from tile to tile, as in part_project.cu; all pieces but the
+// last are added to fp32 sums in registers.  (256 of k in one accumulator and 512 in two saved the sums, but MMAs add by
+// truncation: D was biased towards zero by 2.8e-7 at r = 256, positive operands, where pieces of 128 leave 1.2e-7.  Norm and
+// update of 14 matrices 1024 / 2736, r = 256: 77 and 90 us then, 89 and 95 now; with the sums
+// kept in tensor memory 100 and 112.)
 //
 // What bounds it: G (and W in and out) at the copy bandwidth.
 //
@@ -21,8 +25,10 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "part_slab.cuh"
+#include "split_gemm.cuh"
 #include "step_simt.cuh"
 
 namespace fira {
@@ -37,6 +43,7 @@ constexpr int BOX_BYTES = PM / 2 * 64;          // 8 KiB: 128 rows of 16 fp32 or
 constexpr int GROUP_THREADS = 128;
 constexpr int THREADS = 32 * 3 + GROUPS * GROUP_THREADS + 32 * GROUPS;
 constexpr int KS = PN / GROUPS;                 // factors that a group needs per tile (its boxes' columns)
+constexpr int PROMOTE_SLABS = split::PROMOTE / PK;
 constexpr int stages_of(int mode) { return mode == MODE_NORM ? 4 : 3; }
 constexpr int bufs_of(int mode) { return mode == MODE_NORM ? 4 : 3; }            // box buffers per group
 constexpr int buf_bytes(int mode) { return (mode == MODE_NORM ? 1 : 2) * BOX_BYTES; }
@@ -51,7 +58,8 @@ struct TileDev { int job, i0, j0, nk; };
 
 struct BackCtl {
   uint64_t full[4], empty[4];
-  uint64_t tmem_full[2], tmem_empty[2];
+  uint64_t tmem_full[2], tmem_empty[2];         // a set, or (DEEP) a main accumulator
+  uint64_t small_empty[2];                      // (DEEP) the small products of a tile have been read
   uint64_t efull[GROUPS][4], eready[GROUPS][4], eempty[GROUPS][4];
   uint64_t esync[GROUPS];
   uint32_t tmem_base;
@@ -95,10 +103,10 @@ __device__ __forceinline__ uint4 pack(const float (&v)[8]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-template <int MODE>
+template <int MODE, bool DEEP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
-k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles, int count, int deep, const MatDev* __restrict__ mats,
-            Hyper hp, unsigned* __restrict__ status) {
+k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles, int count, const MatDev* __restrict__ mats, Hyper hp,
+            unsigned* __restrict__ status) {
   constexpr int STAGES = stages_of(MODE), BUFS = bufs_of(MODE), BUF_BYTES = buf_bytes(MODE);
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* boxes = smem + STAGES * SLAB_BYTES;
@@ -115,6 +123,7 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(ptx::smem_u32(&ctl->tmem_full[b]), 1);
       ptx::mbar_init(ptx::smem_u32(&ctl->tmem_empty[b]), 2 * GROUPS * 4);        // every epilogue warp of the pair
+      ptx::mbar_init(ptx::smem_u32(&ctl->small_empty[b]), 2 * GROUPS * 4);
     }
     for (int g = 0; g < GROUPS; ++g) {
       for (int b = 0; b < BUFS; ++b) {
@@ -139,7 +148,6 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
   ptx::grid_launch_next();
   volatile int* abort_flag = &ctl->abort_flag;
   const uint32_t slabs = ptx::smem_u32(smem), boxes_u32 = ptx::smem_u32(boxes);
-  const uint32_t sets = deep ? 1u : 2u;         // accumulator sets in use
 
   if (warp == 0) {
     if (lane == 0 && smem_ok) {
@@ -168,25 +176,33 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
   } else if (warp == 1) {
     if (lane == 0 && smem_ok && rank == 0) {
       int stage = 0; uint32_t phase = 0; bool ok = true;
-      uint32_t set = 0, sphase = 0;
-      for (int t = pair; t < count && ok; t += npairs) {
+      uint32_t set = 0, sphase = 0;                     // of a tile, or (DEEP) main accumulator of a piece
+      uint32_t tile = 0;
+      for (int t = pair; t < count && ok; t += npairs, ++tile) {
         const TileDev d = load_tile(tiles + t);
         const int shape = jobs[d.job].shape;
-        if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_empty[set]), sphase ^ 1u, abort_flag)) break;
-        const uint32_t base = ctl->tmem_base + set * 2 * PN;     // main | small, or (deep) main, main | small
-        const uint32_t small = base + (deep ? 2 : 1) * PN;
+        if (DEEP && !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->small_empty[tile & 1]), ((tile >> 1) & 1) ^ 1u, abort_flag)) break;
+        if (!DEEP && !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_empty[set]), sphase ^ 1u, abort_flag)) break;
         for (int k = 0; k < d.nk; ++k) {
+          const bool first = DEEP ? k % PROMOTE_SLABS == 0 : k == 0;
+          if (DEEP && first && !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_empty[set]), sphase ^ 1u, abort_flag)) { ok = false; break; }
           if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->full[stage]), phase, abort_flag)) { ok = false; break; }
           ptx::tc_fence_after();
-          const bool second = deep && k >= PART_STEP_RANK / PK;
-          issue_parts(shape, base + (second ? PN : 0), small, slabs + stage * SLAB_BYTES, 3 * A_PART,
-                      k == 0 || (deep && k == PART_STEP_RANK / PK), k == 0);
+          // main, small | main, small; DEEP: main, main | small, small
+          const uint32_t main = ctl->tmem_base + set * (DEEP ? 1 : 2) * PN, small = DEEP ? ctl->tmem_base + (2 + (tile & 1)) * PN : main + PN;
+          issue_parts(shape, main, small, slabs + stage * SLAB_BYTES, 3 * A_PART, first, k == 0);
           ptx::umma_commit_pair(ptx::smem_u32(&ctl->empty[stage]), 3);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          if (DEEP && ((k + 1) % PROMOTE_SLABS == 0 || k + 1 == d.nk)) {
+            ptx::umma_commit_pair(ptx::smem_u32(&ctl->tmem_full[set]), 3);
+            if (++set == 2) { set = 0; sphase ^= 1u; }
+          }
         }
         if (!ok) break;
-        ptx::umma_commit_pair(ptx::smem_u32(&ctl->tmem_full[set]), 3);
-        if (++set == sets) { set = 0; sphase ^= 1u; }
+        if (!DEEP) {
+          ptx::umma_commit_pair(ptx::smem_u32(&ctl->tmem_full[set]), 3);
+          if (++set == 2) { set = 0; sphase ^= 1u; }
+        }
       }
     }
   } else if (warp == 2) {
@@ -242,8 +258,9 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
     const uint32_t rowoff = (uint32_t)row * 64, sw = (uint32_t)(row >> 1) & 3u;    // 64-byte swizzle: slot ^= (row / 2) % 4
     const uint32_t esync = ptx::smem_u32(&ctl->esync[g]);
     const uint32_t te[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->tmem_empty[1]), 0)};
+    const uint32_t se[2] = {ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[0]), 0), ptx::map_to_cta(ptx::smem_u32(&ctl->small_empty[1]), 0)};
     const uint32_t tmem = ctl->tmem_base + ((uint32_t)(quarter * 32) << 16);
-    uint32_t yphase = 0, set = 0, sphase = 0, ephase = 0;
+    uint32_t yphase = 0, set = 0, sphase = 0, ephase = 0, tile = 0;
     int eb = 0, parity = 0;
     bool ok = true;
     for (int t = pair; t < count && ok; t += npairs) {
@@ -265,32 +282,51 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
       ptx::mbar_arrive(esync);                           // the group's factors are in place
       if (!ptx::mbar_wait(esync, yphase, abort_flag)) break;
       yphase ^= 1u;
-      if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_full[set]), sphase, abort_flag)) break;
+      float dv[DEEP ? PN / GROUPS : 32];                 // D: DEEP: in the columns of all of the group's boxes; else of one
+      if (DEEP) {
+#pragma unroll
+        for (int e = 0; e < PN / GROUPS; ++e) dv[DEEP ? e : 0] = 0.f;
+        for (int k = PROMOTE_SLABS; k < d.nk; k += PROMOTE_SLABS) {       // all pieces but the last
+          if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_full[set]), sphase, abort_flag)) { ok = false; break; }
+          ptx::tc_fence_after();
+#pragma unroll
+          for (int e = 0; e < PN / GROUPS; e += 16) {
+            uint32_t v[16];
+            __syncwarp();
+            ptx::tmem_ld_32x32b_x16(tmem + set * PN + (cols == 32 ? 32 * (GROUPS * (e / 32) + g) + e % 32 : GROUPS * e + 16 * g), v);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) dv[DEEP ? e + i : 0] += __uint_as_float(v[i]);
+          }
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive_cluster(te[set]);
+          if (++set == 2) { set = 0; sphase ^= 1u; }
+        }
+      }
+      if (!ok || !ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_full[set]), sphase, abort_flag)) break;
       ptx::tc_fence_after();
-      const uint32_t tbase = tmem + set * 2 * PN, tsmall = tbase + (deep ? 2 : 1) * PN;
-      const bool two_mains = deep && d.nk > PART_STEP_RANK / PK;
+      const uint32_t tbase = tmem + set * (DEEP ? 1 : 2) * PN, tsmall = DEEP ? tmem + (2 + (tile & 1)) * PN : tbase + PN;
       const int nch = min(PN / cols, (n - d.j0 + cols - 1) / cols);
       float ss = 0.f;
-      if (g >= nch) {                                    // this group has no box in this tile
+      auto accumulators_read = [&] {                     // this warp has read all it needs of them
         ptx::tc_fence_before();
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(te[set]);
-      }
-      // 16 columns of the accumulators, as D
-      auto product = [&](int col, float (&dv)[16]) {
+        if (lane == 0) {
+          ptx::mbar_arrive_cluster(te[set]);
+          if (DEEP) ptx::mbar_arrive_cluster(se[tile & 1]);
+        }
+      };
+      if (g >= nch) accumulators_read();                 // this group has no box in this tile
+      // 16 columns of the accumulators
+      auto product = [&](int col, float* out) {
         uint32_t v[16], w[16];
         __syncwarp();
         ptx::tmem_ld_32x32b_x16(tbase + col, v);
         ptx::tmem_ld_32x32b_x16(tsmall + col, w);
         ptx::tmem_ld_wait();
 #pragma unroll
-        for (int e = 0; e < 16; ++e) dv[e] = __uint_as_float(v[e]) + __uint_as_float(w[e]);
-        if (two_mains) {
-          ptx::tmem_ld_32x32b_x16(tbase + PN + col, v);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int e = 0; e < 16; ++e) dv[e] += __uint_as_float(v[e]);
-        }
+        for (int e = 0; e < 16; ++e) out[e] = (DEEP ? out[e] + __uint_as_float(v[e]) : __uint_as_float(v[e])) + __uint_as_float(w[e]);
       };
       // PER values of one 16-byte word of the row: per group of 16 product columns 16 / PER words
       auto word = [&](unsigned char* gb, int q, const float* dv, const float* kf, auto zero) {
@@ -313,38 +349,36 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
       };
       struct F4 { float v[4]; };
       struct F8 { float v[8]; };
-      for (int c = g; c < nch; c += GROUPS) {
+      // kind: F4 or F8 where the type of the matrix is known, int where it is not
+      auto box = [&](int c, float* dbox, auto kind) {
+        const bool wide = std::is_same<decltype(kind), int>::value ? cols == 32 : std::is_same<decltype(kind), F8>::value;
         unsigned char* gb = boxes + (g * BUFS + eb) * BUF_BYTES;
         const float* kf = ks + (c / GROUPS) * cols;
-        float dv[32];
-        {
-          float lo[16];
-          product(c * cols, lo);
+        product(c * cols, dbox);
+        if (wide) product(c * cols + 16, dbox + 16);
+        if (c + GROUPS >= nch) accumulators_read();
+        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->efull[g][eb]), ephase, abort_flag)) { ok = false; return; }
+        if (wide) {
 #pragma unroll
-          for (int e = 0; e < 16; ++e) dv[e] = lo[e];
-        }
-        if (cols == 32) {
-          float hi[16];
-          product(c * cols + 16, hi);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) dv[16 + e] = hi[e];
-        }
-        if (c + GROUPS >= nch) {                         // this warp has read all it needs of the accumulators
-          ptx::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive_cluster(te[set]);
-        }
-        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->efull[g][eb]), ephase, abort_flag)) { ok = false; break; }
-        if (cols == 32) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) word(gb, q, dv + 8 * q, kf + 8 * q, F8());
+          for (int q = 0; q < 4; ++q) word(gb, q, dbox + 8 * q, kf + 8 * q, F8());
         } else {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) word(gb, q, dv + 4 * q, kf + 4 * q, F4());
+          for (int q = 0; q < 4; ++q) word(gb, q, dbox + 4 * q, kf + 4 * q, F4());
         }
         if (MODE == MODE_UPDATE) ptx::fence_proxy_async_smem();
         ptx::mbar_arrive(ptx::smem_u32(&ctl->eready[g][eb]));
         if (++eb == BUFS) { eb = 0; ephase ^= 1u; }
+      };
+      if (!DEEP) {
+        for (int c = g; c < nch && ok; c += GROUPS) box(c, dv, 0);
+      } else if (cols == 32) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+          if (ok && GROUPS * b + g < nch) box(GROUPS * b + g, dv + (DEEP ? 32 * b : 0), F8());
+      } else {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          if (ok && GROUPS * b + g < nch) box(GROUPS * b + g, dv + (DEEP ? 16 * b : 0), F4());
       }
       if (!ok) break;
       if (MODE == MODE_NORM) {
@@ -354,7 +388,8 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
         if (lane == 0) mt.part[in_matrix * PART_SUMS_PER_TILE + (int)rank * 8 + ew] = ss;
       }
       parity ^= 1;
-      if (++set == sets) { set = 0; sphase ^= 1u; }
+      if (++set == 2) { set = 0; sphase ^= 1u; }
+      ++tile;
     }
   }
   // neither CTA may leave while its partner can still reach into its shared memory
@@ -369,6 +404,11 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
   if (threadIdx.x == 0 && ctl->abort_flag) atomicOr(status, DEV_STATUS_TIMEOUT);
 }
 
+auto kernel_of(int mode, int deep) {
+  return mode == MODE_NORM ? (deep ? k_part_back<MODE_NORM, true> : k_part_back<MODE_NORM, false>)
+                           : (deep ? k_part_back<MODE_UPDATE, true> : k_part_back<MODE_UPDATE, false>);
+}
+
 // SMs of the current device (0: error) once the kernels may use their shared memory there.
 int prepared_sms() {
   static std::atomic<int> sms_of_device[64];    // (the shared-memory limit is a per-device setting)
@@ -376,8 +416,9 @@ int prepared_sms() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && (sms = sms_of_device[dev].load()) == 0) {
-    e = cudaFuncSetAttribute(k_part_back<MODE_NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(MODE_NORM));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_part_back<MODE_UPDATE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(MODE_UPDATE));
+    for (int deep = 0; deep < 2; ++deep)
+      for (int mode : {MODE_NORM, MODE_UPDATE})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel_of(mode, deep), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(mode));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) sms_of_device[dev].store(sms);
   }
@@ -423,7 +464,7 @@ fira_status part_step_prepare(const std::vector<MatDev>& mats, const std::vector
     for (int i0 = 0; i0 < mt.m; i0 += PM)
       for (int j0 = 0; j0 < mt.n; j0 += PN) td.push_back(TileDev{(int)q, i0, j0, (mt.r + PK - 1) / PK});
     plan->tile_start.push_back((int)td.size());
-    if (mt.r > PART_STEP_RANK) plan->deep = 1;
+    if (mt.r > split::PROMOTE) plan->deep = 1;
   }
   plan->table = table_dev; plan->njobs = (int)list.size();
   cudaError_t e = cudaMemcpyAsync(table_dev + align_up(plan->jobs.size()), td.data(), sizeof(TileDev) * td.size(), cudaMemcpyHostToDevice, st);
@@ -457,8 +498,8 @@ fira_status part_step_run(const PartStepPlan& plan, const MatDev* mats_dev, int 
   const BackJob* jobs = reinterpret_cast<const BackJob*>(plan.table) + (update ? plan.njobs : 0);
   const TileDev* tiles = reinterpret_cast<const TileDev*>(plan.table + align_up(plan.jobs.size())) + first;
   const int grid = 2 * std::min(count, sms / 2);
-  const cudaError_t e = launch_chained(update ? k_part_back<MODE_UPDATE> : k_part_back<MODE_NORM>, grid, THREADS,
-                                       smem_bytes(update ? MODE_UPDATE : MODE_NORM), st, true, 1, jobs, tiles, count, plan.deep, mats_dev, hp, status_dev);
+  const cudaError_t e = launch_chained(kernel_of(update ? MODE_UPDATE : MODE_NORM, plan.deep), grid, THREADS,
+                                       smem_bytes(update ? MODE_UPDATE : MODE_NORM), st, true, 1, jobs, tiles, count, mats_dev, hp, status_dev);
   if (e != cudaSuccess) { set_error(std::string("step back-projection: ") + cudaGetErrorString(e)); return FIRA_ERR_CUDA; }
   return FIRA_OK;
 }

@@ -52,9 +52,9 @@ struct PartStepPlan {
   std::vector<int> proj_start;      // 256 x 128 tiles of R, prefix sums over the list
   std::vector<unsigned char> jobs;  // host image of the table's first part: the norm's jobs, then the update's
   std::vector<int> tile_start;      // 256 x 128 tiles of W, prefix sums over the list
-  int deep = 0;                     // some rank exceeds PART_STEP_RANK
+  int deep = 0;                     // some rank exceeds split::PROMOTE
 };
-constexpr int PART_STEP_RANK = 256, PART_STEP_MAX_RANK = 512;
+constexpr int PART_STEP_MAX_RANK = 512;    // (k_moments keeps a row of R in registers)
 constexpr int PART_SUMS_PER_TILE = 16;   // partial sums of ||S||^2 that a tile leaves
 inline int part_rank_pitch(int r) { return (r + 7) / 8 * 8; }
 inline int part_step_tiles(int m, int n) { return ((m + 255) / 256) * ((n + 127) / 128); }

@@ -314,7 +314,7 @@ __device__ __forceinline__ float back_rows(const MatDev& mt, int i0, int j0, con
   return ss;
 }
 
-template <typename T, int MODE>
+template <typename T, int MODE, bool LONG_K>
 __device__ __forceinline__ bool back_product(const MatDev& mt, int i0, int j0, float a_low, float cres,
                                              unsigned char* smem, split::Ctl* ctl) {
   // left: D[d][l] = sum_j Pi[d][j] X[l][j]; right: D[l][d] = sum_j X[l][j] Pi[d][j]
@@ -325,26 +325,30 @@ __device__ __forceinline__ bool back_product(const MatDev& mt, int i0, int j0, f
   if (MODE == MODE_NORM) {
     split::Operand<float> x(mt.Rt, mt.r, 1, mt.l, mt.r, x0);
     x.along_x = false; x.ld = mt.r;
-    return mt.left ? split::tile_product<false>(p, x, mt.r, cols, smem, ctl) : split::tile_product<false>(x, p, mt.r, cols, smem, ctl);
+    return mt.left ? split::tile_product<LONG_K>(p, x, mt.r, cols, smem, ctl) : split::tile_product<LONG_K>(x, p, mt.r, cols, smem, ctl);
   } else {
     split::CombinedOperand x(mt.Xt, mt.Rt, mt.r, mt.l, mt.r, x0, mt.kvec, a_low, cres);
-    return mt.left ? split::tile_product<false>(p, x, mt.r, cols, smem, ctl) : split::tile_product<false>(x, p, mt.r, cols, smem, ctl);
+    return mt.left ? split::tile_product<LONG_K>(p, x, mt.r, cols, smem, ctl) : split::tile_product<LONG_K>(x, p, mt.r, cols, smem, ctl);
   }
 }
 
-template <typename T, int MODE>
+template <typename T, int MODE, bool LONG_K>
 __device__ __forceinline__ float back_tile(const MatDev& mt, int i0, int j0, const Hyper& hp, unsigned char* smem,
                                            split::Ctl* ctl, float* ks) {
   const float cres = MODE == MODE_UPDATE ? hp.a_res * mt.sc->lambda : 0.f;
   tile_factors<MODE>(mt, i0, j0, SIMT_TILE, hp, ks);
-  if (!back_product<T, MODE>(mt, i0, j0, hp.a_low, cres, smem, ctl)) return 0.f;
+  if (!back_product<T, MODE, LONG_K>(mt, i0, j0, hp.a_low, cres, smem, ctl)) return 0.f;
   const float* C = reinterpret_cast<const float*>(smem);
   const bool vec = rows_vec(static_cast<const T*>(mt.G), mt.ld, mt.n) && rows_vec(static_cast<const T*>(mt.W), mt.ld, mt.n);
   return vec ? back_rows<T, MODE, true>(mt, i0, j0, C, ks, hp.lr, cres) : back_rows<T, MODE, false>(mt, i0, j0, C, ks, hp.lr, cres);
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(split::THREADS, 2)
+// LONG_K: some rank of the list is above split::PROMOTE, the main product is added up in registers.  With those, two blocks
+// per SM spill (the update 2 KiB per thread); a grid of no more tiles than SMs has one block per SM in any case (BLOCKS = 1).
+// Measured with BLOCKS 2 / 1: one 768 x 2048 matrix, r = 300 (96 tiles) 129 / 117 us; 7 of 512 / 1376, r = 200 (240 tiles)
+// 127 / 156; 7 of 2048 / 5461, r = 640 1851 / 1976.
+template <int MODE, bool LONG_K, int BLOCKS>
+__global__ void __launch_bounds__(split::THREADS, BLOCKS)
 k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
                const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -358,8 +362,8 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
   split::begin(ctl);
   ptx::grid_wait();
   ptx::grid_launch_next();
-  float ss = mt.bf16 ? back_tile<__nv_bfloat16, MODE>(mt, i0, j0, hp, smem, ctl, ks)
-                     : back_tile<float, MODE>(mt, i0, j0, hp, smem, ctl, ks);
+  float ss = mt.bf16 ? back_tile<__nv_bfloat16, MODE, LONG_K>(mt, i0, j0, hp, smem, ctl, ks)
+                     : back_tile<float, MODE, LONG_K>(mt, i0, j0, hp, smem, ctl, ks);
   if (MODE == MODE_NORM) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
@@ -730,12 +734,14 @@ static bool allow_smem() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && (dev < 0 || dev >= 64)) e = cudaErrorInvalidDevice;
   if (e == cudaSuccess && !done[dev].load()) {
-    const void* kernels[11] = {(const void*)k_project<PSI_ADAM, false, true>, (const void*)k_project<PSI_RMSPROP, false, true>,
+    const void* kernels[15] = {(const void*)k_project<PSI_ADAM, false, true>, (const void*)k_project<PSI_RMSPROP, false, true>,
                                (const void*)k_project<PSI_ADAGRAD, false, true>, (const void*)k_project<PSI_ADAM, true, true>,
                                (const void*)k_project<PSI_RMSPROP, true, true>, (const void*)k_project<PSI_ADAGRAD, true, true>,
                                (const void*)k_project<PSI_ADAM, true, false>, (const void*)k_project<PSI_RMSPROP, true, false>,
                                (const void*)k_project<PSI_ADAGRAD, true, false>,
-                               (const void*)k_back_project<MODE_NORM>, (const void*)k_back_project<MODE_UPDATE>};
+                               (const void*)k_back_project<MODE_NORM, false, 2>, (const void*)k_back_project<MODE_UPDATE, false, 2>,
+                               (const void*)k_back_project<MODE_NORM, true, 2>, (const void*)k_back_project<MODE_UPDATE, true, 2>,
+                               (const void*)k_back_project<MODE_NORM, true, 1>, (const void*)k_back_project<MODE_UPDATE, true, 1>};
     for (const void* k : kernels)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
     if (e == cudaSuccess) done[dev].store(true);
@@ -744,10 +750,15 @@ static bool allow_smem() {
   return e == cudaSuccess;
 }
 
+constexpr int SMS = 148;
+template <int MODE>
+static auto back_kernel(const SimtPlan& pl, int tiles) {
+  return pl.max_r <= split::PROMOTE ? k_back_project<MODE, false, 2> : tiles <= SMS ? k_back_project<MODE, true, 1> : k_back_project<MODE, true, 2>;
+}
+
 // Blocks that share a tile of the projection: of a short list as many as keep the grid within one block per SM (but no
 // part below two slabs).  Counted over the whole list, whatever range of it is stepped: the sums have the same order then.
 static int split_of(const SimtPlan& pl) {
-  constexpr int SMS = 148;
   int split = 1;
   while (split < MAX_SPLIT && 2 * split * pl.proj_tiles <= SMS && 4 * split * split::BK <= pl.max_d) split *= 2;
   return split;
@@ -762,7 +773,7 @@ static cudaError_t launch_project(const SimtPlan& pl, int first, int tiles, cons
 }
 
 static int rows_per_warp(int rows, int blocks_per_sm) {
-  const int warps = 148 * blocks_per_sm * 8;
+  const int warps = SMS * blocks_per_sm * 8;
   return std::max(2, (rows + warps - 1) / warps);
 }
 template <int PSI>
@@ -815,7 +826,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   else if (parts) {
     if (part_step_run(pl.parts, pl.mats, qa, qe, 0, hp, status_dev, st) != FIRA_OK) return -1;
   } else
-    launch_error(launch_chained(k_back_project<MODE_NORM>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
+    launch_error(launch_chained(back_kernel<MODE_NORM>(pl, wt1 - wt0), wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   // (only-scaling leaves one partial sum per 128 x 128 tile whatever the list)
   launch_error(launch_chained(k_finalize, nq, 256, 0, st, true, 1, pl.mats, pl.list + qa, nq, (only_scaling ? pl.npart_tiles : pl.npart) + qa, hp, status_dev));
@@ -833,7 +844,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     if (part_step_run(pl.parts, pl.mats, qa, qe, 1, hp, status_dev, st) != FIRA_OK) return -1;
     launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 1, st);
   } else
-    launch_error(launch_chained(k_back_project<MODE_UPDATE>, wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
+    launch_error(launch_chained(back_kernel<MODE_UPDATE>(pl, wt1 - wt0), wt1 - wt0, TH, SM, st, true, 1, pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, hp, status_dev));
   tm->mark(st);
   if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
   return 4 + (pl.parts.table ? 2 : 0) + (parts ? 1 : 0) + (staged ? (parts ? 2 : 1) : 0);

@@ -98,3 +98,68 @@ def test_refresh_at_the_edges_of_its_blocks(shape, r):
     assert np.abs(P.T @ P - np.eye(r)).max() < 1e-5
     if r < min(m, n):
         assert fo.principal_angles(P, fo.refresh_projection(to_np64(G), r)).max() <= 1e-3
+
+
+def _stepped_from_ordinary_moments(shapes, ranks, dtype, flags, steps=3, seed=11):
+    """See test_long_list_of_ragged_matrices; the last step's gradient jumps."""
+    g = torch.Generator().manual_seed(seed)
+    hp = fb.make_hparams(lr=1e-2, alpha=0.25, gamma=1.01, flags=flags | fb.FLAG_FORCE_SIMT)
+    tr = Trajectory(shapes, ranks, dtype, hp, [(torch.randn(m, n, generator=g) * 0.02).to(dtype) for m, n in shapes])
+    Ps = []
+    for i, (m, n) in enumerate(shapes):
+        q, _ = torch.linalg.qr(torch.randn(min(m, n), ranks[i], generator=g, dtype=torch.float64))
+        Ps.append(q.to(dtype))
+        tr.f.set_projection(i, Ps[i].cuda())
+        V = torch.rand(max(m, n), ranks[i], generator=g) + 0.5
+        tr.f.set_state(i, torch.zeros_like(V).cuda(), V.cuda(), 1e6, 3)
+        tr.st[i].V, tr.st[i].prev_norm, tr.st[i].t = to_np64(V.T if m <= n else V).copy(), 1e6, 3
+    for step in range(steps):
+        G = [torch.randn(m, n, generator=g).to(dtype) for m, n in shapes]
+        tr.step([residual_jump(x, p) for x, p in zip(G, Ps)] if step == steps - 1 else G)
+    return tr
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("flags", [0, fb.FLAG_MATRIX_SCALING, fb.FLAG_NO_SCALING, fb.FLAG_ONLY_SCALING])
+@pytest.mark.parametrize("shapes,ranks", [([(333, 517), (517, 333)], [129, 200]), ([(640, 900), (900, 640)], [300, 640]),
+                                          ([(1100, 1376)], [1000])])
+def test_short_list_of_ranks_above_one_tile(shapes, ranks, flags, dtype):
+    """Row sums over several tiles of R, factors made from them, products longer than one piece of the main accumulator;
+    grids of fewer and of more tiles than SMs, and a list that a rank above 512 keeps short."""
+    tr = _stepped_from_ordinary_moments(shapes, ranks, dtype, flags)
+    tr.assert_ok()
+    assert all(tr.f.diagnostics(i)["engine"] == 0 for i in range(len(shapes)))
+
+
+def test_more_tiles_than_sms_with_ranks_above_one_tile():
+    _stepped_from_ordinary_moments([(512, 1376)] * 4, [200] * 4, torch.float32, 0, steps=2).assert_ok()
+
+
+def test_projection_split_over_blocks_of_more_than_one_piece():
+    """44 tiles of R: two blocks per tile, 256 of k each."""
+    _stepped_from_ordinary_moments([(512, 1376), (1376, 512)] * 2, [128] * 4, torch.float32, 0).assert_ok()
+
+
+@pytest.mark.parametrize("shapes,r", [([(520, 1376)], 200), ([(520, 1376)], 512), ([(1100, 1376)], 1024),
+                                      ([(520, 1376), (1376, 520)] * 5, 256), ([(520, 1376), (1376, 520)] * 5, 512)])
+def test_long_products_do_not_drift(shapes, r):
+    """Products of positive numbers, W = -lr alpha Pi N alone.  An MMA adds to its accumulator by truncation, which loses half
+    a unit in the last place on average: 0.72 / 2 2^-23 = 4.3e-8 of the running sum.  Over the 8 additions of one piece
+    of 128 that is 4.5 / 8 of it each, 1.9e-7 in all, and the pieces are added to nearest; the whole of k in one
+    accumulator gives 3.7e-7 at 256 and twice that at 512.  A bound of 2e-7 lies between."""
+    f = fb.Fira(shapes, r, torch.float32, fb.make_hparams(lr=1.0, alpha=1.0, beta1=0.0, beta2=0.5, flags=fb.FLAG_NO_RESIDUAL))
+    g = torch.Generator(device="cuda").manual_seed(5)
+    W, G, P = [], [], []
+    for i, (m, n) in enumerate(shapes):
+        P.append(torch.randn(min(m, n), r, generator=g, device="cuda").abs())
+        G.append(torch.randn(m, n, generator=g, device="cuda").abs())
+        W.append(torch.zeros(m, n, device="cuda"))
+        V = torch.rand(max(m, n), r, generator=g, device="cuda") + 0.5
+        f.set_projection(i, P[i])
+        f.set_state(i, torch.zeros_like(V), V, None, 100)
+    f.step(W, G)
+    for i, (m, n) in enumerate(shapes):
+        M, V, _, _ = f.get_state(i)
+        N = (1 - 0.5 ** 101) ** 0.5 * M.double() / (V.double().sqrt() + 1e-8)
+        D = P[i].double() @ N.T if m <= n else N @ P[i].double().T
+        assert abs(float((-W[i].double() - D).sum() / D.sum())) < 2e-7

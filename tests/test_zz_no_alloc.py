@@ -144,3 +144,41 @@ def test_nonfinite_gradient_is_reported_by_the_poll():
                                           M.data_ptr(), V.data_ptr(), pn.data_ptr(), t.data_ptr(), -1.0, None))
     assert lib.fira_noalloc_poll(None) == 6                # FIRA_ERR_NONFINITE
     assert lib.fira_noalloc_poll(None) == 0                # cleared by the read
+
+
+@pytest.mark.parametrize("shape,r,dtype", [((768, 1000), 300, torch.float32), ((1000, 768), 200, torch.bfloat16),
+                                           ((160, 5000), 129, torch.float32)])
+def test_ranks_of_several_tiles(shape, r, dtype):
+    """Row sums of several tiles of R, in the area behind the array."""
+    _run_both(shape, r, dtype)
+
+
+def test_calls_of_different_matrices_behind_one_another():
+    """The calls share the array and each one's kernels start while the ones before them end: no call may see another's
+    tables.  Enqueued without waiting, they give what they give one at a time."""
+    lib, hp = fb.lib(), fb.make_hparams()
+    g = torch.Generator(device="cuda").manual_seed(6)
+    cases = [((512, 1376), 128), ((64, 96), 8), ((300, 200), 150), ((1000, 130), 40)]
+
+    def run(wait):
+        outs = []
+        for (m, n), r in cases:
+            g.manual_seed(m)
+            d, l = min(m, n), max(m, n)
+            t = [torch.randn(m, n, generator=g, device="cuda") * 0.02, torch.randn(m, n, generator=g, device="cuda"),
+                 torch.linalg.qr(torch.randn(d, r, generator=g, device="cuda"))[0].contiguous(),
+                 torch.zeros(l, r, device="cuda"), torch.ones(l, r, device="cuda"), torch.full((1,), -1.0, device="cuda"),
+                 torch.zeros(1, dtype=torch.int64, device="cuda")]
+            outs.append((t, fb.MatrixDesc(m, n, r, fb.FIRA_F32, 0)))
+        torch.cuda.synchronize()
+        for _ in range(10):
+            for t, desc in outs:
+                fb.check(lib.fira_step_single_noalloc(C.byref(hp), C.byref(desc), *[x.data_ptr() for x in t], -1.0,
+                                                      torch.cuda.current_stream().cuda_stream))
+                if wait:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return [t for t, _ in outs]
+
+    for a, b in zip(run(True), run(False)):
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
