@@ -145,15 +145,18 @@ __device__ __forceinline__ void add_row_parts(uint32_t row, int blocks, int lane
 }
 
 // Rows of the finished tile R: Adam (Eq. 2-4), N and R to scratch, row sums.  SPLIT: the blocks of the cluster share the
-// rows; between cluster_arrive, which the caller has done, and the first look at the tile, M and V are fetched.
+// rows; between cluster_arrive, which the caller has done, and the first look at the tile, M and V are fetched.  Where a
+// wait of any of them ran out the tile is garbage, and nothing is stored.
 template <int PSI, bool VEC, bool SPLIT>
-__device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, const float* C, const Hyper& hp, float bias) {
+__device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, const float* C, const Hyper& hp, const split::Ctl* ctl) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = min(SIMT_TILE, mt.r - j0);
   const int nrt = simt_tiles_dev(mt.r), q = j0 / SIMT_TILE;
   const int blocks = SPLIT ? (int)ptx::cluster_nctarank() : 1, rows = WARP_ROWS / blocks;
   const int row0 = SPLIT ? ((int)ptx::cluster_ctarank() * (split::THREADS / 32) + warp) * rows : warp * rows;
   constexpr bool momentum = PSI == PSI_ADAM;
+  const float bias = ctl->bias;
+  int aborted = 0;                              // (one block's flag per lane)
   for (int x = 0; x < rows; x += ROWS_AT_ONCE) {
     float m[ROWS_AT_ONCE][4], v[ROWS_AT_ONCE][4];
 #pragma unroll
@@ -164,7 +167,10 @@ __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, cons
       load_row<VEC>(mt.V + at, lane, there ? n : 0, v[y]);
       load_row<VEC>(mt.M + at, lane, there && momentum ? n : 0, m[y]);
     }
-    if (SPLIT && x == 0) ptx::cluster_wait();
+    if (SPLIT && x == 0) {
+      ptx::cluster_wait();
+      aborted = ptx::ld_cluster_s32(ptx::map_to_cta(ptx::smem_u32(&ctl->abort_flag), min(lane, blocks - 1)));
+    }
 #pragma unroll
     for (int y = 0; y < ROWS_AT_ONCE; ++y) {
       const int row = row0 + x + y, l = l0 + row;
@@ -173,6 +179,7 @@ __device__ __forceinline__ void adam_rows(const MatDev& mt, int l0, int j0, cons
       float rv[4], nv[4], nn = 0.f, rn = 0.f;
       if (SPLIT) add_row_parts<VEC>(ptx::smem_u32(C + row * split::C_LD), blocks, lane, n, rv);
       else load_row<VEC>(C + row * split::C_LD, lane, n, rv);
+      if (SPLIT && __any_sync(0xffffffffu, aborted)) return;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         nv[c] = adam_direction<PSI>(hp, bias, rv[c], m[y][c], v[y][c]);
@@ -245,8 +252,8 @@ k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nli
   }
   if (SPLIT) ptx::cluster_arrive();
   if (SPLIT || ok) {                            // (a block whose wait ran out still meets the others)
-    if (mt.r % 4 == 0) adam_rows<PSI, true, SPLIT>(mt, l0, j0, C, hp, ctl->bias);
-    else adam_rows<PSI, false, SPLIT>(mt, l0, j0, C, hp, ctl->bias);
+    if (mt.r % 4 == 0) adam_rows<PSI, true, SPLIT>(mt, l0, j0, C, hp, ctl);
+    else adam_rows<PSI, false, SPLIT>(mt, l0, j0, C, hp, ctl);
   }
   if (SPLIT) ptx::cluster_sync_all();           // nobody leaves while others read its part
   split::end(ctl, status);

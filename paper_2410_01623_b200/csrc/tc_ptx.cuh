@@ -282,6 +282,11 @@ __device__ __forceinline__ float ld_cluster_f1(uint32_t cluster_addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
   return v;
 }
+__device__ __forceinline__ int ld_cluster_s32(uint32_t cluster_addr) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr) : "memory");
+  return v;
+}
 // Kernels that are launched before the kernel in front of them has ended (launch_chained): what comes before grid_wait
 // may not touch anything that kernel writes.  grid_launch_next, after grid_wait, lets the next one in: what comes before
 // ITS wait may then rely on everything that came before this kernel.
