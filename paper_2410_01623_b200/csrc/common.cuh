@@ -84,12 +84,13 @@ enum HyperMode : unsigned {
 };
 
 // sqrt(1 - b2^s) / (1 - b1^s) (Eq. 4), in double.
-__device__ __noinline__ inline float bias_factor(float beta1, float beta2, long long s) {
+__device__ __forceinline__ float bias_factor(float beta1, float beta2, long long s) {
   return (float)(sqrt(1.0 - pow((double)beta2, (double)s)) / (1.0 - pow((double)beta1, (double)s)));
 }
-// The factor of step s.
+// The factor of step s.  (A call: the arithmetic inline cost the projection its registers.)
+__device__ __noinline__ inline float bias_factor_call(float beta1, float beta2, long long s) { return bias_factor(beta1, beta2, s); }
 __device__ __forceinline__ float step_bias(const BiasSlot& slot, long long s, const Hyper& hp) {
-  return slot.step == s ? slot.next : bias_factor(hp.beta1, hp.beta2, s);
+  return slot.step == s ? slot.next : bias_factor_call(hp.beta1, hp.beta2, s);
 }
 
 enum DeviceStatusBits : unsigned {

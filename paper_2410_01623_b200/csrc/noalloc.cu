@@ -93,14 +93,16 @@ struct NoAllocInts { int v[6]; };
 __global__ void k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, int* ints_out,
                                 const float* norm_prev, const long long* t, float beta1, float beta2) {
   ptx::grid_launch_next();
+  const long long steps = *t;
+  const float norm = *norm_prev;
   *mats_out = mt;
   for (int i = 0; i < 6; ++i) ints_out[i] = ints.v[i];
   MatScalars* sc = mt.sc;
-  sc->prev_norm = (*norm_prev < 0.f) ? -1.f : *norm_prev;
+  sc->prev_norm = (norm < 0.f) ? -1.f : norm;
   sc->lambda = 1.f; sc->norm_scaled = 0.f; sc->k_min = 0.f; sc->k_max = 0.f; sc->bias = 0.f;
-  sc->t = *t;
-  mt.bias->step = *t + 1;
-  mt.bias->next = bias_factor(beta1, beta2, *t + 1);
+  sc->t = steps;
+  mt.bias->step = steps + 1;
+  mt.bias->next = bias_factor(beta1, beta2, steps + 1);
 }
 __global__ void k_noalloc_store_scalars(const MatScalars* sc, float* norm_prev, long long* t) {
   ptx::grid_wait();

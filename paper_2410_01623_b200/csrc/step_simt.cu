@@ -219,11 +219,12 @@ __device__ __forceinline__ bool project_tile(const MatDev& mt, int l0, int j0, i
 // Measured (one 512 x 1376 matrix, r = 128): 46 us as 11 blocks of 16 slabs, 15 us as 11 clusters of 8 blocks.
 template <int PSI, bool SPLIT, bool LONG_K>
 __global__ void __launch_bounds__(split::THREADS, 2)
-k_project(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
-          const int* __restrict__ tile_start, int first, Hyper hp, unsigned* __restrict__ status) {
+k_project(const MatDev* mats, const int* list, int nlist, const int* tile_start, int first, Hyper hp, unsigned* status) {
+  // (The tables are not __restrict__: the single-matrix entry point writes them in the kernel that this one is chained to,
+  // so no load of them may come before grid_wait, and a compiler that takes them for constants may move it there.)
   extern __shared__ __align__(128) unsigned char smem[];
   split::Ctl* ctl = reinterpret_cast<split::Ctl*>(smem + split::STAGES * split::STAGE_BYTES);
-  ptx::grid_wait();                             // (the single-matrix entry point writes its tables just before)
+  ptx::grid_wait();
   const int blocks = SPLIT ? (int)ptx::cluster_nctarank() : 1, block = SPLIT ? (int)ptx::cluster_ctarank() : 0;
   const int gt = blockIdx.x / blocks + first;
   const int p = find_matrix(tile_start, nlist, gt);
