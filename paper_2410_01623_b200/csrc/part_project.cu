@@ -17,7 +17,14 @@
 // What bounds it: the MMAs (12 per slab), G at the copy bandwidth close behind.
 //
 // Warp roles: 0 producer of the projection's slabs, 1 MMA issuer (even CTA) and owner of the tensor memory, 2-9 epilogue,
-// 10 box storer, 11-18 converters.
+// 10 box storer, 11-18 converters, 19 and (odd CTA) 1 relays.
+//
+// The odd CTA's converted slabs are announced to the issuer, in the other CTA, by relays: the converters release their writes
+// to a barrier of their own CTA, a relay's thread acquires them there and releases them to the issuer's barrier at cluster
+// scope.  (Measured, 56 matrices 512 / 1376 fp32 / 28 of 640 / 1707 bf16: 72 / 62 us with two relays for the slabs in turn, 73 / 70
+// with one, 74 / 63 with three, 79 / 68 with a lane of one warp per stage, 100 / 88 where the converters release at cluster scope
+// themselves, which waits for their loads in flight.  70 / 60 with the barrier's default scope, the CTA: not enough by the
+// memory model.)
 #include <string.h>
 
 #include <algorithm>
@@ -38,7 +45,8 @@ constexpr int SLAB_BYTES = 3 * (A_PART + B_PART);
 constexpr int EPI_WARPS = 8, CONV_WARPS = 8, CONV_THREADS = 32 * CONV_WARPS;
 constexpr int GROUPS = 2, GROUP_THREADS = 128;
 constexpr int FIRST_CONV = 3 + EPI_WARPS;                 // warp
-constexpr int THREADS = 32 * (FIRST_CONV + CONV_WARPS);
+constexpr int RELAYS = 2, FIRST_RELAY = FIRST_CONV + CONV_WARPS;     // (the first relay is warp 1)
+constexpr int THREADS = 32 * (FIRST_RELAY + RELAYS - 1);
 constexpr int COLS = 16;                        // of a box
 constexpr int OUT_BUFS = 2;                     // per group
 constexpr int OUT_PART = PM / 2 * COLS * 2, OUT_BUF = 3 * OUT_PART;         // 4 KiB; three parts
@@ -57,6 +65,7 @@ struct TileDev { int job, l0, j0, nk; };
 
 struct ProjCtl {
   uint64_t full[STAGES], empty[STAGES];
+  uint64_t converted[STAGES];                   // (odd CTA) its converters have written the slab
   uint64_t main_full[2], main_empty[2];         // a piece of the main product is complete / has been read
   uint64_t small_empty[2];                      // the small products of a tile have been read
   uint64_t oready[GROUPS][OUT_BUFS], oempty[GROUPS][OUT_BUFS];   // R's parts written / stored
@@ -120,7 +129,8 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
   const bool smem_ok = (ptx::smem_u32(smem) & 1023u) == 0;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      ptx::mbar_init(ptx::smem_u32(&ctl->full[s]), 1 + 2 * CONV_WARPS);          // the producer and both CTAs' converters
+      ptx::mbar_init(ptx::smem_u32(&ctl->full[s]), 1 + CONV_WARPS + 1);          // the producer, this CTA's converters, a relay
+      ptx::mbar_init(ptx::smem_u32(&ctl->converted[s]), CONV_WARPS);
       ptx::mbar_init(ptx::smem_u32(&ctl->empty[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -149,6 +159,18 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
   volatile int* abort_flag = &ctl->abort_flag;
   const uint32_t slabs = ptx::smem_u32(smem);
 
+  // Every RELAYS-th slab of this pair's, from the `which`-th on.
+  auto relay = [&](int which) {
+    int slab = 0;                               // running number
+    for (int t = pair; t < count; t += npairs) {
+      const int end = slab + load_tile(tiles + t).nk;
+      for (int s = slab + (which + RELAYS - slab % RELAYS) % RELAYS; s < end; s += RELAYS) {
+        if (!ptx::mbar_wait(ptx::smem_u32(&ctl->converted[s % STAGES]), (s / STAGES) & 1, abort_flag)) return;
+        ptx::mbar_arrive_release_cluster(ptx::map_to_cta(ptx::smem_u32(&ctl->full[s % STAGES]), 0));
+      }
+      slab = end;
+    }
+  };
   if (warp == 0) {
     if (lane == 0 && smem_ok) {
       int stage = 0; uint32_t phase = 0; bool ok = true;
@@ -196,6 +218,8 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
         }
         ++tile;
       }
+    } else if (lane == 0 && smem_ok) {
+      relay(0);
     }
   } else if (warp == 2 + EPI_WARPS) {
     // ------------------------------------------------------------ box storer
@@ -228,6 +252,8 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
       if (held) ptx::mbar_arrive(held);
       ptx::bulk_wait_group_all();
     }
+  } else if (warp >= FIRST_RELAY) {
+    if (lane == 0 && smem_ok && rank == 1) relay(warp - FIRST_RELAY + 1);
   } else if (warp >= FIRST_CONV) {
     // ------------------------------------------------------------ converters
     if (smem_ok) {
@@ -252,9 +278,7 @@ k_part_project(const ProjJob* __restrict__ jobs, const TileDev* __restrict__ til
             s[h].store(smem + stage * SLAB_BYTES, left);
             ptx::fence_proxy_async_smem();
             __syncwarp();
-            // (default semantics: the proxy fence has put this warp's writes in place; a release at cluster scope would also
-            // wait for the loads in flight, which cost a load latency per slab)
-            if (lane == 0) ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_u32(&ctl->full[stage]), 0));
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(rank ? &ctl->converted[stage] : &ctl->full[stage]));
             s[h].template load<REGULAR>(mt, G, ld, L, l0, min(k + h + 2, nk - 1) * PK, left, vec);   // (at the end the last once more)
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
