@@ -138,7 +138,10 @@ typedef struct fira_ctx fira_ctx;
 
 /* Bytes needed for the state and scratch buffers of a matrix list (Algorithm 1's
  * "Input" line fixes what a matrix is; the state is the paper's comparison-table
- * count).  Both are rounded up to 256-byte multiples per section. */
+ * count).  Both are rounded up to 256-byte multiples per section.
+ * The scratch size follows the step's intermediates, 0.8 to 1.7 times the bytes of the weights;
+ * small lists also get room for the projection refresh to work on many matrices at a time, which
+ * brings them to 3 times the weights, 512 MiB in all at most. */
 FIRA_API fira_status fira_query_workspace(const fira_hparams* hp, const fira_matrix_desc* descs,
                                           int32_t count, size_t* state_bytes, size_t* scratch_bytes);
 

@@ -68,6 +68,13 @@ static long long part_staging_pitch(const fira_matrix_desc& d, uint32_t flags) {
 // Row sums per l: one per tile of R, whose width depends on the kernels.
 static int aux_slots(const Layout& L, int i, int r) { return L.engine[i] == 1 || L.parts ? 1 : simt_tiles(r); }
 
+// Room of the refresh beyond what the step needs, up to this bound.  The refresh takes as many matrices at a time as fit, each
+// pass has launches, uploads and a wait of its own, and a few small matrices do not fill the chip.  Measured (scratch, time of
+// a refresh, without the extra room / with it): 56 matrices 512 / 1376 fp32, 99 MB 3.4 ms / 288 MB 1.6 ms; 28 of 640 / 1707
+// bf16 79 MB 2.3 ms / 120 MB 1.3 ms; 14 of 1024 / 2736 fp32 98 MB 8.6 ms / 285 MB 2.7 ms; 14 of 2048 / 5461 bf16 335 MB 10.9 ms /
+// 517 MB 7.0 ms; 7 of 2048 / 5461 fp32, r = 640, 131 MB 24 ms / 537 MB 12 ms.  Where the step's own room is already
+// more than two thirds of the bound and the list does not fit as a whole it buys nothing (168 of 1024 / 2736 bf16: 466 MB
+// 8.83 ms, 538 MB 8.95 ms) and is not asked for.
 constexpr size_t REFRESH_SMALL_LIST_BYTES = (size_t)512 << 20;
 
 Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_t count) {
@@ -153,9 +160,10 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
     refresh_all += rb;
   }
   L.step_work_bytes = w;
-  // room for the largest matrix; small models get room for all of theirs, so that one pass takes the whole
-  // list (one matrix of theirs does not fill the chip)
-  L.refresh_min_bytes = std::max(refresh_max, std::min(refresh_all, REFRESH_SMALL_LIST_BYTES));
+  // room for the largest matrix; small models get more (REFRESH_SMALL_LIST_BYTES)
+  L.refresh_min_bytes = refresh_max;
+  if (refresh_all <= REFRESH_SMALL_LIST_BYTES || 3 * w <= 2 * REFRESH_SMALL_LIST_BYTES)
+    L.refresh_min_bytes = std::max(refresh_max, std::min(refresh_all, REFRESH_SMALL_LIST_BYTES));
   L.scratch_bytes = L.off_work + std::max(L.step_work_bytes, L.refresh_min_bytes);
   return L;
 }

@@ -8,6 +8,7 @@ import re
 import pytest
 
 from paper_2410_01623_b200 import binding as fb
+from paper_2410_01623_b200.workloads import llama_shapes
 from paper_2410_01623_b200 import build as fbuild
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -96,3 +97,15 @@ def test_init_rejects_null_and_small_buffers(lib):
     assert lib.fira_step(None, None, None, -1.0) == 1
     assert lib.fira_state_elements(None, 0) == -1
     lib.fira_destroy(None)
+
+
+@pytest.mark.parametrize("layers,hidden,mlp,r,dtype,most", [
+    (8, 512, 1376, 128, fb.FIRA_F32, 3.0), (4, 640, 1707, 100, fb.FIRA_BF16, 3.1), (8, 1024, 2736, 256, fb.FIRA_F32, 1.0),
+    (24, 1024, 2736, 256, fb.FIRA_BF16, 0.8), (32, 4096, 11008, 1024, fb.FIRA_BF16, 0.8)])
+def test_scratch_stays_in_proportion_to_the_weights(lib, layers, hidden, mlp, r, dtype, most):
+    """Small lists get room for the refresh of all their matrices at once; a list whose step needs most of that room
+    anyway gets no more than its step needs."""
+    descs = [fb.MatrixDesc(m, n, r, dtype, 0) for m, n in llama_shapes(layers, hidden, mlp)]
+    st, _, wb = _query(lib, fb.make_hparams(), descs)
+    assert st == 0
+    assert wb <= most * sum(d.m * d.n for d in descs) * (2 if dtype == fb.FIRA_BF16 else 4)
