@@ -225,8 +225,6 @@ __global__ void __launch_bounds__(256)
 k_tc_colfactors(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlist,
                 const int* __restrict__ start, int first, Hyper hp) {
   __shared__ float red[8];
-  ptx::grid_wait();
-  ptx::grid_launch_next();
   const int gb = blockIdx.x + first;
   const int p = find_matrix(start, nlist, gb);
   const MatDev& mt = mats[list[p]];
@@ -268,8 +266,6 @@ k_tc_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int n
             float* __restrict__ fast, int fused) {
   const int lane = threadIdx.x & 31;
   const int row = first_row + blockIdx.x * 8 + (threadIdx.x >> 5);
-  ptx::grid_wait();
-  ptx::grid_launch_next();
   if (row >= rows_total) return;
   const int p = find_matrix(row_start, nlist, row);
   const MatDev& mt = mats[list[p]];
@@ -309,8 +305,6 @@ k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int fi
            float* __restrict__ fast) {
   const int p = first + blockIdx.y;
   const MatDev& mt = mats[list[p]];
-  ptx::grid_wait();
-  ptx::grid_launch_next();
   if (!fuse_x_matrix(mt.d, mt.r)) return;              // k_tc_form_x's matrix
   const float lambda = mt.sc->lambda;
   if (blockIdx.x == 0 && threadIdx.x == 0) fast[2 * p + 1] = lambda;   // read by the back-projection epilogue
@@ -804,9 +798,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   const int sra = pl->nstage ? pl->h_ss[sa] : 0, srn = pl->nstage ? pl->h_ss[sb] - sra : 0;
   PhaseTimer* tm = &c->timer;
   const MatDev* mats = c->mats_dev;
-  cudaError_t error = cudaSuccess;
-  // (not chained: these kernels are long, and chaining them cost the 1B list 2 %, 350M unchanged)
-  auto chain = [&](cudaError_t e) { if (error == cudaSuccess) error = e; };
+  // (The kernels are not chained by programmatic dependent launch: they are long, and it cost the 1B list 2 %, 350M unchanged.)
   if (c->proj_weights_dirty) {        // the stored projection has changed since the weights were taken
     k_tc_proj_weights<<<pl->wq_blocks, 256, 0, st>>>(mats, pl->list, pl->wq_off, pl->wq_blk, pl->nlist, pl->wq_dev);
     c->proj_weights_dirty = false;
@@ -832,8 +824,8 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     if (fuse_x_matrix(mq.d, mq.r) && mq.d < FUSE_KEEP_N_MIN_D) keep_n = false;
   }
 #define FIRA_LAUNCH_K1(PSI, FUSE, EG)                                                                       \
-  chain(launch_chained(k_tc_project<EPI_ADAM, PSI, FUSE, EG>, k1_grid, k1_threads(EG), k1_smem_bytes(EG), st, false, 1,  \
-      pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev))
+  k_tc_project<EPI_ADAM, PSI, FUSE, EG><<<k1_grid, k1_threads(EG), k1_smem_bytes(EG), st>>>(                \
+      pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev)
   if (hp.mode & HYPER_PSI_RMSPROP) FIRA_LAUNCH_K1(PSI_RMSPROP, 0, 1);
   else if (hp.mode & HYPER_PSI_ADAGRAD) FIRA_LAUNCH_K1(PSI_ADAGRAD, 0, 1);
   else if (two_groups) {
@@ -846,9 +838,9 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   else FIRA_LAUNCH_K1(PSI_ADAM, 0, 1);
 #undef FIRA_LAUNCH_K1
   tm->mark(st);
-  chain(launch_chained(k_tc_colfactors, csn, 256, 0, st, false, 1, mats, pl->list, pl->nlist, pl->col_start, csa, hp));
+  k_tc_colfactors<<<csn, 256, 0, st>>>(mats, pl->list, pl->nlist, pl->col_start, csa, hp);
   tm->mark(st);
-  chain(launch_chained(k_finalize, nq, 256, 0, st, false, 1, mats, pl->list + qa, nq, pl->npart + qa, hp, c->status_dev));
+  k_finalize<<<nq, 256, 0, st>>>(mats, pl->list + qa, nq, pl->npart + qa, hp, c->status_dev);
   tm->mark(st);
   if (hp.mode & HYPER_ONLY_SCALING) {
     // W <- W - lr phi(R) G: no back-projection; the element-wise update works on the caller's W and
@@ -866,21 +858,22 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     if (fused && fuse_x_matrix(mq.d, mq.r)) any_fused = true; else any_plain = true;
   }
   if (any_plain)
-    chain(launch_chained(k_tc_form_x, (rsb - rsa + 7) / 8, 256, 0, st, false, 1, mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
-                         hp.a_low, hp.a_res, pl->fast_dev, fused ? 1 : 0));
+    k_tc_form_x<<<(rsb - rsa + 7) / 8, 256, 0, st>>>(mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
+                                                     hp.a_low, hp.a_res, pl->fast_dev, fused ? 1 : 0);
   if (any_fused)
-    chain(launch_chained(k_tc_fix_x, dim3(32, nq), 256, 0, st, false, 1, mats, pl->list, qa, hp.a_low, hp.eps, keep_n ? 1 : 0, pl->fast_dev));
+    k_tc_fix_x<<<dim3(32, nq), 256, 0, st>>>(mats, pl->list, qa, hp.a_low, hp.eps, keep_n ? 1 : 0, pl->fast_dev);
   tm->mark(st);
   // long products keep five operand stages; short ones trade one for more epilogue boxes in flight
   if (rmax >= 1024)
-    chain(launch_chained(k_tc_back_project<5, 2>, 2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(5, 2), st, false, 1,
-                         pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev));
+    k_tc_back_project<5, 2><<<2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(5, 2), st>>>(
+        pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev);
   else
-    chain(launch_chained(k_tc_back_project<4, 3>, 2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(4, 3), st, false, 1,
-                         pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev));
+    k_tc_back_project<4, 3><<<2 * std::min(k2n, pl->num_sms / 2), K2_THREADS, k2_smem_bytes(4, 3), st>>>(
+        pl->maps_dev, pl->td2_dev + k2a, k2n, pl->fast_dev, hp, c->status_dev);
   tm->mark(st);
   launch_stage(mats, pl->stage_list, pl->nstage, pl->stage_start, sra, srn, 1, st);
   tm->mark(st);
+  const cudaError_t error = cudaGetLastError();
   if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
   return (srn ? 7 : 5) + (any_plain ? 1 : 0) + (any_fused ? 1 : 0);
 }

@@ -124,8 +124,6 @@ k_tc_back_project(const TcMaps* __restrict__ maps, const BackTileDesc* __restric
   __syncthreads();
   ptx::cluster_sync_all();      // the partner's barriers exist before anything arrives on them
   ptx::tc_fence_after();
-  ptx::grid_wait();
-  ptx::grid_launch_next();
   volatile int* abort_flag = &ctl->abort_flag;
   const uint32_t tiles_u32 = ptx::smem_u32(tiles);
   const uint32_t ebuf_u32 = ptx::smem_u32(ebuf);
