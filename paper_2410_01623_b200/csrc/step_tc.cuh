@@ -9,7 +9,7 @@ struct fira_ctx;
 namespace fira {
 
 // Whether the tensor-core kernels can take this matrix (type, rank and size rules of the
-// tiles); otherwise it runs on the fp32 CUDA-core kernels.
+// tiles); otherwise it runs on the kernels of fp32 precision.
 bool tc_supported(const fira_matrix_desc& d);
 // Row pitch (elements) of the aligned copies of G and W that the tensor-core path makes when the
 // caller's rows are not 16-byte aligned (odd widths or pitches); 0 when TMA can read them in place.
