@@ -33,6 +33,7 @@ struct BiasSlot {
   long long step;
   float next;         // the factor of `step`
   float now;          // long lists of fp32 precision: the factor of the running step
+  float prev;         // norm and update in one kernel: the remembered norm before the step
 };
 
 // One entry of the device-resident problem table.  l = max(m,n) indexes the
@@ -80,6 +81,7 @@ enum HyperMode : unsigned {
   HYPER_NO_RESIDUAL = 4u,      // no residual term (Eq. 6)
   HYPER_PSI_RMSPROP = 8u,      // base optimizer: RMSProp instead of Adam
   HYPER_PSI_ADAGRAD = 16u,     // base optimizer: Adagrad instead of Adam
+  HYPER_X_IS_N = 64u,          // k_moments (with a_low = 1, a_res = 0): X = N, whatever the variant
   HYPER_ONLY_SCALING = 32u,    // Fira-only-scaling: W <- W - lr phi(R) G (no P N term, S = G diag k)
 };
 
@@ -134,12 +136,15 @@ void set_error(const std::string& msg);
 // Launches a kernel in clusters of `cluster` blocks (1: none, or the kernel's own).  chained: every block of the kernel
 // calls ptx::grid_wait, and its blocks may start while the kernel in front of it in the stream is still running: between
 // two short kernels that saves 3 to 5 us.
-template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool chained, int cluster, A... args) {
+// RESIDENT: blocks of the grid wait for one another: it starts when all of it fits on the device (a cooperative launch), whatever
+// else runs there.
+template <bool RESIDENT, typename... P, typename... A>
+inline cudaError_t launch_with(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool chained, int cluster, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[3];
   unsigned n = 0;
+  if (RESIDENT) { at[n].id = cudaLaunchAttributeCooperative; at[n].val.cooperative = 1; ++n; }
   if (chained) { at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization; at[n].val.programmaticStreamSerializationAllowed = 1; ++n; }
   if (cluster > 1) {
     at[n].id = cudaLaunchAttributeClusterDimension;
@@ -148,6 +153,14 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, 
   }
   cfg.attrs = at; cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool chained, int cluster, A... args) {
+  return launch_with<false>(kernel, grid, threads, smem, st, chained, cluster, args...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_resident(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, bool chained, int cluster, A... args) {
+  return launch_with<true>(kernel, grid, threads, smem, st, chained, cluster, args...);
 }
 
 // Optional per-kernel timing of a step: marks are CUDA events recorded between the

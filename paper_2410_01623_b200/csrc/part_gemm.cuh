@@ -48,19 +48,20 @@ fira_status part_gemm_run(const char* table_dev, int njobs, int ntiles, int a_pa
 struct PartStepPlan {
   const char* table = nullptr;      // device; null: the list is short, its products split their operands themselves
   const char* proj_table = nullptr;
-  int njobs = 0;
+  int njobs = 0, ntiles = 0;
   std::vector<int> proj_start;      // 256 x 128 tiles of R, prefix sums over the list
   std::vector<unsigned char> jobs;  // host image of the table's first part: the norm's jobs, then the update's
   std::vector<int> tile_start;      // 256 x 128 tiles of W, prefix sums over the list
   int deep = 0;                     // some rank exceeds split::PROMOTE
+  int one_kernel_pairs = 0;         // norm and update in one kernel, on so many CTA pairs (0: two kernels, some matrix has too many tiles)
 };
 constexpr int PART_STEP_MAX_RANK = 512;    // (k_moments keeps a row of R in registers)
 constexpr int PART_SUMS_PER_TILE = 16;   // partial sums of ||S||^2 that a tile leaves
 inline int part_rank_pitch(int r) { return (r + 7) / 8 * 8; }
-inline int part_step_tiles(int m, int n) { return ((m + 255) / 256) * ((n + 127) / 128); }
+__host__ __device__ inline int part_step_tiles(int m, int n) { return ((m + 255) / 256) * ((n + 127) / 128); }
 inline int part_project_tiles(int l, int r) { return ((l + 255) / 256) * ((r + 127) / 128); }
 // Whether k_moments forms X (for limiter factor 1): its factors are known row by row.
-__host__ __device__ inline bool part_forms_x(const Hyper& hp) { return !(hp.mode & (HYPER_MATRIX_SCALING | HYPER_ONLY_SCALING)); }
+__host__ __device__ inline bool part_forms_x(const Hyper& hp) { return (hp.mode & HYPER_X_IS_N) || !(hp.mode & (HYPER_MATRIX_SCALING | HYPER_ONLY_SCALING)); }
 size_t part_project_table_bytes(int njobs, int ntiles);
 fira_status part_project_prepare(const std::vector<MatDev>& mats, const std::vector<int>& list, char* table_dev, PartStepPlan* plan, cudaStream_t st);
 fira_status part_project_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, unsigned* status_dev, cudaStream_t st);
@@ -72,5 +73,7 @@ fira_status part_step_update_pointers(const std::vector<MatDev>& mats, const std
 // The norm (update = 0) or the update of the matrices [qa, qb) of the list.
 fira_status part_step_run(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, int update, const Hyper& hp,
                           unsigned* status_dev, cudaStream_t st);
+// Norm, limiter and update in one kernel (plan.one_kernel_pairs).
+fira_status part_step_run_one_kernel(const PartStepPlan& plan, const MatDev* mats_dev, int qa, int qb, const Hyper& hp, unsigned* status_dev, cudaStream_t st);
 
 }  // namespace fira

@@ -387,8 +387,8 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
 }
 
 // ---------------------------------------------------------------- long lists
-// Adam (Eq. 2-4) on rows of R that the projection left as parts, the rows' factors k_l, and X for limiter factor 1: one warp
-// per row, R whole in registers (CHUNKS of 128 columns), ROWS rows with their loads in flight together.
+// Adam (Eq. 2-4) on rows of R that the projection left as parts, the rows' factors k_l, and X for limiter factor 1 (or N: see
+// HYPER_X_IS_N) as parts: one warp per row, R whole in registers (CHUNKS of 128 columns), ROWS rows with their loads in flight together.
 template <int PSI, bool VEC, int CHUNKS, int ROWS>
 __device__ __forceinline__ void moment_rows(const MatDev& mt, int l0, int count, const Hyper& hp, float bias) {
   const int lane = threadIdx.x & 31;
@@ -526,7 +526,7 @@ k_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int nlis
   }
 }
 
-// The projection's parts, eight neighbours per thread and pass, `per` blocks per matrix, and the step's bias factor.  In
+// The projection's parts, eight neighbours per thread and pass, `per` blocks per matrix, and by one more the step's scalars.  In
 // every step: projection and step count are in the caller's state buffer, whose bytes may have changed since the last one.
 // (56 matrices 512 / 1376, r = 128: 37 MB, 5.5 of the step's 242 us; k_part_project's set-up, which is chained to it, runs
 // meanwhile.)
@@ -545,9 +545,16 @@ __device__ __forceinline__ void split_units(const MatDev& mt, int block, int blo
 __global__ void __launch_bounds__(256)
 k_split_projection(const MatDev* __restrict__ mats, const int* __restrict__ list, int per, Hyper hp) {
   ptx::grid_launch_next();
-  const MatDev& mt = mats[list[blockIdx.x / per]];
-  const int block = blockIdx.x % per;
-  if (block == 0 && threadIdx.x == 0) mt.bias->now = step_bias(*mt.bias, mt.sc->t + 1, hp);
+  const MatDev& mt = mats[list[blockIdx.x / (per + 1)]];
+  const int block = blockIdx.x % (per + 1);
+  if (block == per) {                           // the scalars
+    if (threadIdx.x == 0) {
+      mt.bias->prev = mt.sc->prev_norm;
+      mt.bias->now = step_bias(*mt.bias, mt.sc->t + 1, hp);
+    }
+    for (int i = threadIdx.x; i < part_step_tiles(mt.m, mt.n); i += 256) reinterpret_cast<unsigned long long*>(mt.part)[i] = 0ull;
+    return;
+  }
   if (mt.bf16) split_units<__nv_bfloat16>(mt, block, per);
   else split_units<float>(mt, block, per);
 }
@@ -732,7 +739,7 @@ bool simt_long_list(const std::vector<fira_matrix_desc>& list) {
 
 static void split_projections(const SimtPlan& pl, int qa, int qb, const Hyper& hp, cudaStream_t st) {
   const int per = (int)std::min<long long>(64, (pl.max_proj_units + 255) / 256);
-  k_split_projection<<<(unsigned)((qb - qa) * per), 256, 0, st>>>(pl.mats, pl.list + qa, per, hp);
+  k_split_projection<<<(unsigned)((qb - qa) * (per + 1)), 256, 0, st>>>(pl.mats, pl.list + qa, per, hp);
 }
 
 // The products' shared memory is above the default limit: a per-device, per-kernel setting.
@@ -811,6 +818,7 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   auto launch_error = [&](cudaError_t e) { if (error == cudaSuccess) error = e; };
   const bool only_scaling = hp.mode & HYPER_ONLY_SCALING;     // W <- W - lr phi(R) G: no back-projection
   const bool parts = pl.parts.table && !only_scaling;          // (a long list's only-scaling step has no back-projection)
+  const bool one_kernel = parts && pl.parts.one_kernel_pairs;  // norm, limiter and update
   const int psi = psi_of(hp);
   const int qe = qb >= 0 ? qb : pl.nlist;
   const int s0 = pl.parts.table ? pl.h_stage_start[pl.h_stage_pos[qa]] : 0;
@@ -822,13 +830,23 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     if (part_project_run(pl.parts, pl.mats, qa, qe, status_dev, st) != FIRA_OK) return -1;
     tm->mark(st);
     const int r0 = pl.h_row_start[qa], r1 = pl.h_row_start[qe];
-    launch_error((psi == PSI_ADAM ? launch_moments<PSI_ADAM> : psi == PSI_RMSPROP ? launch_moments<PSI_RMSPROP> : launch_moments<PSI_ADAGRAD>)(pl, r0, r1, hp, st));
+    Hyper hm = hp;
+    if (one_kernel) { hm.mode |= HYPER_X_IS_N; hm.a_low = 1.f; hm.a_res = 0.f; }
+    launch_error((psi == PSI_ADAM ? launch_moments<PSI_ADAM> : psi == PSI_RMSPROP ? launch_moments<PSI_RMSPROP> : launch_moments<PSI_ADAGRAD>)(pl, r0, r1, hm, st));
   } else {
     launch_error((psi == PSI_ADAM ? launch_project<PSI_ADAM> : psi == PSI_RMSPROP ? launch_project<PSI_RMSPROP> : launch_project<PSI_ADAGRAD>)(
         pl, pt0, pt1 - pt0, hp, status_dev, st));
     tm->mark(st);
   }
   tm->mark(st);
+  if (one_kernel) {
+    for (int i = 0; i < 3; ++i) tm->mark(st);    // (its time counts as the update's)
+    if (part_step_run_one_kernel(pl.parts, pl.mats, qa, qe, hp, status_dev, st) != FIRA_OK) return -1;
+    launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 1, st);
+    tm->mark(st);
+    if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
+    return 4 + (staged ? 2 : 0);
+  }
   if (only_scaling)
     launch_scaled_gradient(pl.mats, pl.list, pl.nlist, pl.w_tile_start, wt0, wt1 - wt0, SIMT_TILE, 0, hp, st);
   else if (parts) {

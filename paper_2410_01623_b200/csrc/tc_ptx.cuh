@@ -93,6 +93,7 @@ __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const void* tmap,
 
 // 2-D tiled store shared -> global, tracked by the issuing thread's bulk async-group.
 // Parts of the box outside the tensor are not written.
+__device__ __forceinline__ void prefetch_map(const void* tmap) { asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory"); }
 __device__ __forceinline__ void tma_store_2d(const void* tmap, uint32_t src, int c0, int c1) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
                ::"l"(tmap), "r"(src), "r"(c0), "r"(c1)
@@ -213,6 +214,17 @@ __device__ __forceinline__ bool wait_counter(const uint32_t* p, uint32_t target,
   return false;
 }
 
+// A float that others of the grid wait for, in one word with the mark that it is there: no order with other writes is needed.
+__device__ __forceinline__ void put_marked(unsigned long long* p, float v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"((1ull << 32) | __float_as_uint(v)) : "memory");
+}
+__device__ __forceinline__ bool get_marked(const unsigned long long* p, float* v) {
+  unsigned long long w;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  *v = __uint_as_float((uint32_t)w);
+  return w >> 32;
+}
+
 // ----------------------------------------------------------------------------- CTA pairs
 // Two CTAs of a cluster share one tcgen05.mma (cta_group::2): each holds half of the
 // rows of A and of B in its own shared memory and half of the accumulator rows in its
@@ -236,6 +248,11 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 // For ordinary writes that a thread of another CTA of the cluster, or the tensor core at its command, is to see.
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// A float into the shared memory of a CTA of the cluster; its four bytes count as transferred on a barrier there, whose waiters
+// then see it.
+__device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uint32_t cluster_bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(cluster_addr), "r"(__float_as_uint(v)), "r"(cluster_bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
   uint32_t ok;
