@@ -55,6 +55,7 @@ struct MatDev {
   int aux_slots;      // row sums per l in aux
   float* kvec;        // scratch: l factors
   float* part;        // scratch: partial sums of ||S||^2
+  unsigned long long* shares;   //   "      short lists that step in one kernel after the projection: marked words, two per tile of W
   float* aux;         // scratch: row sums [aux_slots][l] of ||N_l||^2, then of ||R_l||^2 (engine 0, short lists: one slot per tile of r)
   __nv_bfloat16* Nb;  // scratch of the tensor-core path: l x r bf16 N
   __nv_bfloat16* Rb;  //   "      l x r bf16 R

@@ -53,12 +53,13 @@ struct Layout {
   std::vector<size_t> offP, offM, offV, offS;
   size_t state_bytes = 0;
   // byte offsets inside the scratch buffer
-  size_t off_mats = 0, off_status = 0, off_bias = 0, off_ints = 0, off_tcmaps = 0, off_work = 0;
+  size_t off_mats = 0, off_status = 0, off_shares = 0, off_bias = 0, off_ints = 0, off_tcmaps = 0, off_work = 0;
   size_t ints_count = 0;
   // byte offsets per matrix inside the work area
   std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux, offRp, offXp, offPp;
   std::vector<int> engine;
   bool parts = false;       // the fp32-precision engine's list is long
+  bool one_kernel = false;  // it is short, and steps in one kernel after the projection
   size_t off_parts = 0, off_proj_parts = 0;
   size_t step_work_bytes = 0, refresh_min_bytes = 0;
   size_t scratch_bytes = 0;

@@ -110,6 +110,11 @@ Layout make_layout(const fira_hparams& hp, const fira_matrix_desc* descs, int32_
         ptiles += part_project_tiles(std::max(descs[i].m, descs[i].n), descs[i].r);
       }
     L.parts = !own.empty() && simt_long_list(own);
+    int w_tiles = 0, max_r = 0;
+    for (const fira_matrix_desc& d : own) { w_tiles += simt_tiles(d.m) * simt_tiles(d.n); max_r = std::max(max_r, d.r); }
+    L.one_kernel = !L.parts && short_one_kernel(w_tiles, (int)own.size(), max_r);
+    L.off_shares = wo;
+    if (L.one_kernel) wo += align_up(2 * sizeof(unsigned long long) * (size_t)w_tiles);
     L.off_parts = wo;
     if (L.parts) wo += part_step_table_bytes((int)own.size(), tiles);
     L.off_proj_parts = wo;
@@ -327,6 +332,9 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
       c->simt.max_proj_units = std::max(c->simt.max_proj_units, (long long)c->mats[i].d * c->mats[i].pp_pitch / 8);
     }
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
+    c->simt.one_kernel = L.one_kernel;
+    if (L.one_kernel)
+      for (size_t q = 0; q < lst.size(); ++q) c->mats[lst[q]].shares = reinterpret_cast<unsigned long long*>(c->scratch_base + L.off_shares) + 2 * wt[q];
     c->simt.npart = c->ints_dev + o_np; c->simt.npart_tiles = c->ints_dev + o_npt;
     c->simt.row_start = c->ints_dev + o_rs; c->simt.h_row_start = rs;
     c->simt.stage_list = c->ints_dev + o_sl; c->simt.stage_start = c->ints_dev + o_ss;

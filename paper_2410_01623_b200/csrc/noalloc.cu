@@ -30,7 +30,9 @@ constexpr size_t kNoAllocScratchBytes = 8u << 20;   // 8 MiB: what a caller's ma
 // The row sums of matrices whose rank spans several tiles come behind it.  Such a matrix has r > 128, so
 // l r <= 2^20 (N and R fill the 8 MiB) bounds them: 2 l ceil(r / 128) floats < 2 * 2^20 * (1 / 128 + 1 / 129).
 constexpr size_t kRowSumBytes = 144u << 10;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + kRowSumBytes];
+// Behind those the words of k_back_step, two per tile of W.
+constexpr size_t kShareBytes = 2 * 8 * SHORT_RESIDENT;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes + kRowSumBytes + kShareBytes];
 
 constexpr int kMaxDevices = 64;
 // Device addresses of g_noalloc_scratch, one per device, resolved on first use.  In
@@ -158,6 +160,8 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   mt.part = reinterpret_cast<float*>(base + cv.off_part);
   mt.aux = reinterpret_cast<float*>(base + kNoAllocScratchBytes);
   mt.aux_slots = simt_tiles(desc->r);
+  const bool one_kernel = short_one_kernel(simt_tiles(desc->m) * simt_tiles(desc->n), 1, desc->r);
+  if (one_kernel) mt.shares = reinterpret_cast<unsigned long long*>(base + kNoAllocScratchBytes + kRowSumBytes);
   mt.m = desc->m; mt.n = desc->n; mt.r = desc->r;
   mt.ld = desc->ld ? desc->ld : desc->n;
   mt.left = desc->m <= desc->n;
@@ -180,6 +184,8 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   pl.proj_tile_start = ints_dev + 1; pl.proj_tiles = ptiles; pl.max_d = mt.d; pl.max_r = mt.r;
   pl.w_tile_start = ints_dev + 3; pl.w_tiles = wtiles;
   pl.npart = ints_dev + 5;
+  pl.one_kernel = one_kernel;
+  if (one_kernel) { pl.norm_out = norm_prev_dev; pl.t_out = reinterpret_cast<long long*>(t_dev); }
   Hyper h;
   h.beta1 = hp->beta1; h.beta2 = hp->beta2; h.eps = hp->eps;
   h.lr = lr < 0.f ? hp->lr : lr;
@@ -189,7 +195,8 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   h.gamma = hp->gamma;
   PhaseTimer no_timer;
   if (launch_simt_step(pl, h, status_dev, st, &no_timer) < 0) return FIRA_ERR_CUDA;
-  cudaError_t e = launch_chained(k_noalloc_store_scalars, 1, 1, 0, st, true, 1, mt.sc, norm_prev_dev, reinterpret_cast<long long*>(t_dev));
+  cudaError_t e = cudaSuccess;
+  if (!one_kernel) e = launch_chained(k_noalloc_store_scalars, 1, 1, 0, st, true, 1, mt.sc, norm_prev_dev, reinterpret_cast<long long*>(t_dev));
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_error(std::string("fira_step_single_noalloc: ") + cudaGetErrorString(e));

@@ -27,6 +27,7 @@
 #include <atomic>
 #include <type_traits>
 
+#include "limit.cuh"
 #include "part_slab.cuh"
 #include "split_gemm.cuh"
 #include "step_simt.cuh"
@@ -509,93 +510,6 @@ __device__ __forceinline__ bool each_box(const TileDev& d, const F& f) {
   return true;
 }
 
-// What a matrix's tiles need to know of its norm: lambda, times the matrix's one factor if it has one.  By one warp of every pair
-// that has a tile of it, all of them with the same result: they wait for the shares themselves.  (Counting the tiles and having the last
-// one publish lambda took 8 us in place of 3: two trips through L2 and two fences more.)
-struct Limit { double sum; float kmat, norm, lambda; };
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ bool wait_limit(const TileNorm& tn, const MatDev* mats, const Hyper& hp, volatile int* abort_flag, Limit& out) {
-  const MatDev& mt = mats[tn.mat];
-  const int lane = threadIdx.x & 31;
-  const float prev = mt.bias->prev;
-  out.kmat = 1.f;
-  if (hp.mode & HYPER_MATRIX_SCALING) {          // Eq. 9: the tiles have worked with factor 1
-    double nn = 0.0, rn = 0.0;
-#pragma unroll 8
-    for (int i = lane; i < mt.l; i += 32) { nn += (double)__ldcg(mt.aux + i); rn += (double)__ldcg(mt.aux + mt.l + i); }
-    out.kmat = (float)(sqrt(warp_sum(nn)) / (sqrt(warp_sum(rn)) + (double)hp.eps));
-  }
-  for (uint32_t it = 0;; ++it) {
-    bool there = true;
-    double acc = 0.0;
-    for (int i = lane; i < tn.tiles; i += 32) {
-      float v;
-      there = ptx::get_marked(tn.shares + i, &v) && there;
-      acc += (double)v;
-    }
-    if (__all_sync(0xffffffffu, there)) { out.sum = warp_sum(acc); break; }
-    __nanosleep(it < 64 ? 32 : 256);
-    const bool stop = it == (1u << 21) || ((it & 63u) == 63u && *abort_flag);
-    if (__any_sync(0xffffffffu, stop)) { *abort_flag = 1; return false; }
-  }
-  const bool residual = !(hp.mode & HYPER_NO_RESIDUAL);
-  out.norm = residual ? out.kmat * (float)sqrt(out.sum > 0.0 ? out.sum : 0.0) : 0.f;
-  out.lambda = 1.f;
-  if (residual && prev >= 0.f && !isinf(hp.gamma)) {
-    const float ratio = out.norm / (prev + hp.eps);
-    out.lambda = hp.gamma / fmaxf(ratio, hp.gamma);
-  }
-  return true;
-}
-// The matrix's state and diagnostics (as k_finalize leaves them), by the pair that has its first tile.  (No more than that: who is
-// late with one tile is late with the next, so that microseconds add up over the matrices.  The next step's bias factor, in double,
-// made the kernel take 281 us where it took 166 without.)
-__device__ __forceinline__ void store_limit(const MatDev& mt, const Hyper& hp, const Limit& lim, unsigned* status) {
-  const int lane = threadIdx.x & 31;
-  float kmin = lim.kmat, kmax = lim.kmat;
-  if (!(hp.mode & HYPER_MATRIX_SCALING)) {
-    kmin = INFINITY; kmax = -INFINITY;
-    const int quads = mt.l / 4;                  // (the table is 256-byte aligned)
-    for (int q = lane; q < quads; q += 32 * 8) {
-      float4 v[8];                               // loads in flight together
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = __ldcg(reinterpret_cast<const float4*>(mt.kvec) + min(q + 32 * e, quads - 1));
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        kmin = fminf(kmin, fminf(fminf(v[e].x, v[e].y), fminf(v[e].z, v[e].w)));
-        kmax = fmaxf(kmax, fmaxf(fmaxf(v[e].x, v[e].y), fmaxf(v[e].z, v[e].w)));
-      }
-    }
-    if (4 * quads + lane < mt.l) {
-      const float k = __ldcg(mt.kvec + 4 * quads + lane);
-      kmin = fminf(kmin, k); kmax = fmaxf(kmax, k);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      kmin = fminf(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-      kmax = fmaxf(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    }
-  }
-  if (lane == 0) {
-    const bool residual = !(hp.mode & HYPER_NO_RESIDUAL);
-    MatScalars* sc = mt.sc;
-    sc->norm_scaled = lim.norm;
-    sc->lambda = lim.lambda;
-    if (residual) {
-      if (!isfinite((float)lim.sum) || !isfinite(kmax)) atomicOr(status, DEV_STATUS_NONFINITE);
-      sc->prev_norm = lim.lambda * lim.norm;
-    }
-    sc->k_min = residual ? kmin : 0.f;
-    sc->k_max = residual ? kmax : 0.f;
-    sc->t = sc->t + 1;
-  }
-}
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(RU_THREADS, 1)
 k_part_step(const BackJob* __restrict__ jobs, int njobs, const TileDev* __restrict__ tiles, const TileNorm* __restrict__ norms, int count,
             const MatDev* __restrict__ mats, Hyper hp, unsigned* __restrict__ status) {
@@ -708,10 +622,11 @@ k_part_step(const BackJob* __restrict__ jobs, int njobs, const TileDev* __restri
         }
         const int b = seconds++ & 1;
         Limit lim;
-        if (!wait_limit(tn, mats, hp, abort_flag, lim)) return false;
+        const MatDev& mt = mats[tn.mat];
+        if (!wait_limit(tn.shares, tn.tiles, mt, mt.bias->prev, hp, abort_flag, lim)) return false;
         if (lane < 2)
           ptx::st_async_f32(ptx::map_to_cta(ptx::smem_u32(&ctl->lambda[b]), lane), lim.lambda * lim.kmat, ptx::map_to_cta(ptx::smem_u32(&ctl->lambda_in[b]), lane));
-        if (tn.index == 0) store_limit(mats[tn.mat], hp, lim, status);
+        if (tn.index == 0) store_limit(mt, hp, lim, status);
         return true;
       });
     }

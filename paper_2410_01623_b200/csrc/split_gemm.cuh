@@ -247,16 +247,16 @@ __device__ __forceinline__ void end(Ctl* ctl, unsigned* status) {
   if (threadIdx.x == 0 && ctl->abort_flag) atomicOr(status, DEV_STATUS_TIMEOUT);
 }
 
-// MMAs of one slab, issued by one thread: `steps` of 16 along k, the main product into column 0 of the
+// MMAs of one slab (A's and B's place), issued by one thread: `steps` of 16 along k, the main product into column 0 of the
 // block's tensor memory, the small ones behind it.
 template <int PA, int PB, bool A_X, bool B_X>
-__device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, int n, int steps, bool first, bool fresh_main) {
+__device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab_a, uint32_t slab_b, int n, int steps, bool first, bool fresh_main) {
   const uint32_t idesc = ptx::make_idesc_bf16(TILE, n, A_X, B_X);
   constexpr uint64_t along_x = ptx::smem_desc_constant(ptx::LAYOUT_PLAIN, 128, X_SBO);
   constexpr uint64_t along_k = ptx::smem_desc_constant(ptx::LAYOUT_PLAIN, K_LBO, 128);
   constexpr int a_step = (A_X ? 256 : 2 * K_LBO) / 16, b_step = (B_X ? 256 : 2 * K_LBO) / 16;
-  slab &= 0x3ffff;                              // (in a cluster the address carries the block's rank above the descriptor's field)
-  uint64_t a = (A_X ? along_x : along_k) + (slab >> 4), b = (B_X ? along_x : along_k) + ((slab + OPERAND_BYTES) >> 4);
+  slab_a &= 0x3ffff; slab_b &= 0x3ffff;         // (in a cluster the address carries the block's rank above the descriptor's field)
+  uint64_t a = (A_X ? along_x : along_k) + (slab_a >> 4), b = (B_X ? along_x : along_k) + (slab_b >> 4);
   uint32_t acc_main = !fresh_main, acc = !first;
   for (int k = 0; k < steps; ++k, a += a_step, b += b_step) {
     ptx::umma_bf16(tmem, a, b, idesc, acc_main);
@@ -273,12 +273,13 @@ __device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, int n, 
 }
 template <int PA, int PB>
 __device__ __forceinline__ void issue_slab(uint32_t tmem, uint32_t slab, bool a_x, bool b_x, int n, int steps, bool first, bool fresh_main) {
+  const uint32_t slab_b = slab + OPERAND_BYTES;
   if (a_x) {
-    if (b_x) issue_slab<PA, PB, true, true>(tmem, slab, n, steps, first, fresh_main);
-    else issue_slab<PA, PB, true, false>(tmem, slab, n, steps, first, fresh_main);
+    if (b_x) issue_slab<PA, PB, true, true>(tmem, slab, slab_b, n, steps, first, fresh_main);
+    else issue_slab<PA, PB, true, false>(tmem, slab, slab_b, n, steps, first, fresh_main);
   } else {
-    if (b_x) issue_slab<PA, PB, false, true>(tmem, slab, n, steps, first, fresh_main);
-    else issue_slab<PA, PB, false, false>(tmem, slab, n, steps, first, fresh_main);
+    if (b_x) issue_slab<PA, PB, false, true>(tmem, slab, slab_b, n, steps, first, fresh_main);
+    else issue_slab<PA, PB, false, false>(tmem, slab, slab_b, n, steps, first, fresh_main);
   }
 }
 

@@ -17,11 +17,12 @@
 //
 // Short lists are bound by latency, so all of their kernels are chained (launch_chained): one's set-up (tables, barriers,
 // tensor memory) runs while the one before it ends.  Step of one 512 x 1376 matrix: 74 us without that and without the
-// split projection, 35 us with both.
+// split projection, 35 us with both, 26.7 us with phases 2 to 4 in one kernel (k_back_step).
 #include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
+#include "limit.cuh"
 #include "split_gemm.cuh"
 #include "step_simt.cuh"
 
@@ -32,21 +33,21 @@ namespace {
 __device__ __forceinline__ int simt_tiles_dev(int extent) { return (extent + SIMT_TILE - 1) / SIMT_TILE; }
 
 // Four entries of a row per lane: the neighbours 4 lane .. 4 lane + 3 where a row's groups of four are
-// aligned (VEC), lane, lane + 32, ... otherwise; either way a warp's access is contiguous.
-template <bool VEC>
-__device__ __forceinline__ int lane_col(int lane, int c) { return VEC ? 4 * lane + c : lane + 32 * c; }
+// aligned (VEC), lane, lane + LANES, ... otherwise; either way the access of the LANES lanes that share a row is contiguous.
+template <bool VEC, int LANES = 32>
+__device__ __forceinline__ int lane_col(int lane, int c) { return VEC ? 4 * lane + c : lane + LANES * c; }
 
-template <bool VEC>
+template <bool VEC, int LANES = 32>
 __device__ __forceinline__ void load_row(const float* p, int lane, int n, float (&v)[4]) {
   if (VEC) {
     const float4 u = 4 * lane < n ? *reinterpret_cast<const float4*>(p + 4 * lane) : make_float4(0.f, 0.f, 0.f, 0.f);
     v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
   } else {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = lane + 32 * c < n ? p[lane + 32 * c] : 0.f;
+    for (int c = 0; c < 4; ++c) v[c] = lane + LANES * c < n ? p[lane + LANES * c] : 0.f;
   }
 }
-template <bool VEC>
+template <bool VEC, int LANES = 32>
 __device__ __forceinline__ void load_row(const __nv_bfloat16* p, int lane, int n, float (&v)[4]) {
   if (VEC) {
     const uint2 u = 4 * lane < n ? *reinterpret_cast<const uint2*>(p + 4 * lane) : make_uint2(0u, 0u);
@@ -54,19 +55,19 @@ __device__ __forceinline__ void load_row(const __nv_bfloat16* p, int lane, int n
     v[2] = __uint_as_float(u.y << 16); v[3] = __uint_as_float(u.y & 0xffff0000u);
   } else {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) v[c] = lane + 32 * c < n ? __bfloat162float(p[lane + 32 * c]) : 0.f;
+    for (int c = 0; c < 4; ++c) v[c] = lane + LANES * c < n ? __bfloat162float(p[lane + LANES * c]) : 0.f;
   }
 }
-template <bool VEC>
+template <bool VEC, int LANES = 32>
 __device__ __forceinline__ void store_row(float* p, int lane, int n, const float (&v)[4]) {
   if (VEC) {
     if (4 * lane < n) *reinterpret_cast<float4*>(p + 4 * lane) = make_float4(v[0], v[1], v[2], v[3]);
   } else {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) if (lane + 32 * c < n) p[lane + 32 * c] = v[c];
+    for (int c = 0; c < 4; ++c) if (lane + LANES * c < n) p[lane + LANES * c] = v[c];
   }
 }
-template <bool VEC>
+template <bool VEC, int LANES = 32>
 __device__ __forceinline__ void store_row(__nv_bfloat16* p, int lane, int n, const float (&v)[4]) {
   if (VEC) {
     if (4 * lane < n) {
@@ -77,7 +78,7 @@ __device__ __forceinline__ void store_row(__nv_bfloat16* p, int lane, int n, con
     }
   } else {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) if (lane + 32 * c < n) p[lane + 32 * c] = __float2bfloat16_rn(v[c]);
+    for (int c = 0; c < 4; ++c) if (lane + LANES * c < n) p[lane + LANES * c] = __float2bfloat16_rn(v[c]);
   }
 }
 // The row's entries as three bf16 parts, `stride` elements apart.
@@ -233,6 +234,8 @@ k_project(const MatDev* mats, const int* list, int nlist, const int* tile_start,
   const int l0 = (tile / rt) * SIMT_TILE, j0 = (tile % rt) * SIMT_TILE;
   split::begin(ctl);
   ptx::grid_launch_next();
+  if (mt.shares && tile == 0 && block == 0)      // (k_back_step waits for them; the one of the step before is done)
+    for (int i = threadIdx.x; i < 2 * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n); i += split::THREADS) mt.shares[i] = 0ull;
   const int slabs = (mt.d + split::BK - 1) / split::BK;
   const int k0 = slabs * block / blocks * split::BK, k1 = min(mt.d, slabs * (block + 1) / blocks * split::BK);
   const float* C = reinterpret_cast<const float*>(smem);
@@ -383,6 +386,226 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
       mt.part[tile] = tot;
     }
   }
+  split::end(ctl, status);
+}
+
+// ---------------------------------------------------------------- phases 2 to 4 in one kernel
+// Short lists of no more tiles than SMs (ranks up to 128): a block per tile of W, or per half of one, 64 columns, where the SMs suffice
+// for that, keeps its residual S = k (G - Pi R) in registers while it
+// makes D = Pi N, waits for the shares of ||S||^2 of its matrix's other tiles, and updates W <- W - lr (a_low D + a_res lambda S).
+// G is read once; the blocks wait for one another (a cooperative launch).  One block more per matrix stores its state and works out
+// the next step's bias factor.
+// Bound by latency, that of fetching instructions included: the code runs once, from start to end.  So all of the projection's and
+// of R's slabs are loaded at once and each is multiplied as soon as it is stored, N and G are on their way meanwhile, the
+// projection's parts stay for the second product, N's take R's place; and 512 threads have half the code of 256.
+// Measured, one 512 x 1376 matrix, r = 128, the kernel's time: 22 us as two ordinary tile products in a row, 18.6 with all slabs loaded at
+// once, 15 with all of them stored before the first MMA is issued (of that 5.5 to the first product's end, 2 the second's, the rest rows
+// and conversions), 10.9 with half tiles (88 blocks).
+constexpr int STEP_THREADS = 512, STEP_ROWS = SIMT_TILE / (STEP_THREADS / 32);         // rows per warp
+constexpr int STEP_SLABS = 128 / split::BK;
+constexpr int STEP_X = STEP_SLABS * split::OPERAND_BYTES;       // the slabs of R, then N, behind those of the projection; the finished tile overlays them
+constexpr int STEP_SMEM = 2 * STEP_X + (int)sizeof(split::Ctl);
+static_assert(STEP_SMEM <= 227 * 1024 - 2048 && SIMT_TILE * split::C_LD * 4 <= STEP_X, "shared memory budget");
+static_assert(STEP_THREADS == SIMT_TILE * split::BK / 8, "a unit of eight per thread and slab");
+
+// This thread's units, one per slab, of rows [x0, x0 + rows) of Op(x, k) = base[x r + k], zero outside X x r.
+template <typename T>
+struct StepOperand {
+  static constexpr int PARTS = sizeof(T) == 4 ? 3 : 1;
+  split::Frag<T> f[STEP_SLABS];
+
+  // REGULAR: whole aligned units only; rows past the matrix read its last one again, for rows of the result that nobody looks
+  // at, and slabs past the rank the last one.
+  template <bool REGULAR>
+  __device__ __forceinline__ void load(const T* base, int r, int X, int x0, int ns) {
+    const int x = x0 + threadIdx.x / 4, k = threadIdx.x % 4 * 8;
+    const T* row = base + (long long)(REGULAR ? min(x, X - 1) : x) * r + k;
+#pragma unroll
+    for (int s = 0; s < STEP_SLABS; ++s) {
+      if (REGULAR) split::load_frag(row + min(s, ns - 1) * split::BK, f[s]);
+      else split::load_frag(row + s * split::BK, x < X ? max(0, r - k - s * split::BK) : 0, false, f[s]);
+    }
+  }
+  __device__ __forceinline__ void store(int s, int rows, unsigned char* place) const {
+    if ((int)threadIdx.x / 4 < rows) split::store_parts(place + (threadIdx.x % 4) * split::K_LBO + (threadIdx.x / 4) * 16, f[s]);
+  }
+};
+
+template <typename T, int COLS, bool VEC, bool REGULAR>
+__device__ __forceinline__ void step_tile(const MatDev& mt, int tile, int i0, int j0, const Hyper& hp, unsigned char* smem, split::Ctl* ctl, float* ks, float* coef) {
+  __shared__ float red[STEP_THREADS / 32];
+  constexpr int LANES = COLS / 4, AT_ONCE = 32 / LANES, PASSES = STEP_ROWS / AT_ONCE;    // lanes to a row, rows of a warp at a time
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row0 = warp * STEP_ROWS + lane / LANES, hl = lane % LANES;
+  const int rows_p = mt.left ? SIMT_TILE : COLS, rows_x = mt.left ? COLS : SIMT_TILE;
+  const int n = min(COLS, mt.n - j0), cols = (n + 15) / 16 * 16, ns = (mt.r + split::BK - 1) / split::BK;
+  unsigned char* xs = smem + STEP_X;
+  float* C = reinterpret_cast<float*>(xs);
+  const uint32_t tmem = ctl->tmem_base;
+  const T* G = static_cast<const T*>(mt.G);
+  T* W = static_cast<T*>(mt.W);
+  StepOperand<T> p;
+  StepOperand<float> x;
+  p.template load<REGULAR>(static_cast<const T*>(mt.P), mt.r, mt.d, mt.left ? i0 : j0, ns);
+  x.template load<REGULAR>(mt.Rt, mt.r, mt.l, mt.left ? j0 : i0, ns);
+  const float prev = mt.sc->prev_norm;           // (stored anew when every tile has left its share)
+  // All of the product's slabs at once: a thread that issues MMAs between its slabs' conversions holds up the other warps' next slab.
+  auto multiply = [&](bool with_p, uint64_t* done) {
+#pragma unroll
+    for (int s = 0; s < STEP_SLABS; ++s) {
+      if (s >= ns) break;
+      if (with_p) p.store(s, rows_p, smem + s * split::OPERAND_BYTES);
+      x.store(s, rows_x, xs + s * split::OPERAND_BYTES);
+    }
+    ptx::fence_proxy_async_smem();
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      ptx::tc_fence_after();
+      uint32_t pa = ptx::smem_u32(smem), xa = ptx::smem_u32(xs);
+#pragma unroll 1
+      for (int s = 0; s < ns; ++s, pa += split::OPERAND_BYTES, xa += split::OPERAND_BYTES) {
+        const int steps = min(split::BK, mt.r - s * split::BK + 15) / 16;
+        if (mt.left) split::issue_slab<StepOperand<T>::PARTS, 3, false, false>(tmem, pa, xa, cols, steps, s == 0, s == 0);
+        else split::issue_slab<3, StepOperand<T>::PARTS, false, false>(tmem, xa, pa, cols, steps, s == 0, s == 0);
+      }
+      ptx::umma_commit(ptx::smem_u32(done));
+    }
+  };
+  // The finished tile into shared memory, in the place of the X slabs.
+  auto read_back = [&](uint64_t* done) {
+    const bool ok = ptx::mbar_wait(ptx::smem_u32(done), 0, &ctl->abort_flag);
+    if (__syncthreads_or(!ok)) return false;
+    ptx::tc_fence_after();
+    const int c0 = (warp >> 2) * (COLS / 4);
+    if (c0 < cols) {
+      const uint32_t from = tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0;
+      float* to = C + (32 * (warp & 3) + lane) * split::C_LD + c0;
+#pragma unroll 1
+      for (int q = 0; q < COLS / 4; q += 16) {
+        uint32_t v[16], w[16];
+        __syncwarp();
+        ptx::tmem_ld_32x32b_x16(from + q, v);
+        ptx::tmem_ld_32x32b_x16(from + split::TILE + q, w);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 16; e += 4)
+          *reinterpret_cast<float4*>(to + q + e) = make_float4(__uint_as_float(v[e]) + __uint_as_float(w[e]), __uint_as_float(v[e + 1]) + __uint_as_float(w[e + 1]),
+                                                               __uint_as_float(v[e + 2]) + __uint_as_float(w[e + 2]), __uint_as_float(v[e + 3]) + __uint_as_float(w[e + 3]));
+      }
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    return true;
+  };
+  multiply(true, &ctl->done[0]);
+  float s[PASSES][4];                            // G, then the residual
+#pragma unroll
+  for (int y = 0; y < PASSES; ++y) load_row<VEC, LANES>(G + (long long)(i0 + row0 + AT_ONCE * y) * mt.ld + j0, hl, i0 + row0 + AT_ONCE * y < mt.m ? n : 0, s[y]);
+  x.template load<REGULAR>(mt.Xt, mt.r, mt.l, mt.left ? j0 : i0, ns);          // N
+  tile_factors<MODE_NORM>(mt, i0, j0, SIMT_TILE, hp, ks);
+  if (!read_back(&ctl->done[0])) return;
+  float kc[4], ss = 0.f;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) kc[c] = mt.left ? ks[lane_col<VEC, LANES>(hl, c)] : 0.f;
+#pragma unroll
+  for (int y = 0; y < PASSES; ++y) {
+    const int row = row0 + AT_ONCE * y;
+    float dv[4];
+    load_row<VEC, LANES>(C + row * split::C_LD, hl, n, dv);
+    const float kr = mt.left ? 0.f : ks[row];
+    const bool there = i0 + row < mt.m;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      s[y][c] = there ? (mt.left ? kc[c] : kr) * (s[y][c] - dv[c]) : 0.f;       // (zero past the row's end)
+      ss = fmaf(s[y][c], s[y][c], ss);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (lane == 0) red[warp] = ss;
+  __syncthreads();                               // (also: nobody reads the first product any more)
+  if (warp == 1) {
+    float tot = lane < STEP_THREADS / 32 ? red[lane] : 0.f;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    if (lane == 0) ptx::put_marked(mt.shares + tile, tot);
+  }
+  multiply(false, &ctl->done[1]);
+  float w[PASSES][4];
+#pragma unroll
+  for (int y = 0; y < PASSES; ++y) load_row<VEC, LANES>(W + (long long)(i0 + row0 + AT_ONCE * y) * mt.ld + j0, hl, i0 + row0 + AT_ONCE * y < mt.m ? n : 0, w[y]);
+  if (warp == STEP_THREADS / 32 - 1) {           // (while the product is made)
+    Limit lim;
+    const bool known = wait_limit(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, prev, hp, &ctl->abort_flag, lim);
+    if (lane == 0 && known) *coef = hp.a_res * lim.lambda * lim.kmat;
+  }
+  if (!read_back(&ctl->done[1]) || *(volatile int*)&ctl->abort_flag) return;
+  const float cres = *coef;
+#pragma unroll
+  for (int y = 0; y < PASSES; ++y) {
+    const int row = row0 + AT_ONCE * y;
+    if (i0 + row >= mt.m) continue;
+    float dv[4];
+    load_row<VEC, LANES>(C + row * split::C_LD, hl, n, dv);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w[y][c] = w[y][c] - hp.lr * (hp.a_low * dv[c] + cres * s[y][c]);
+    store_row<VEC, LANES>(W + (long long)(i0 + row) * mt.ld + j0, hl, n, w[y]);
+  }
+}
+template <typename T, int COLS>
+__device__ __forceinline__ void step_tile(const MatDev& mt, int tile, int i0, int j0, const Hyper& hp, unsigned char* smem, split::Ctl* ctl, float* ks, float* coef) {
+  if (j0 >= mt.n) {                              // the second half of a tile that has none
+    if (threadIdx.x == 0) ptx::put_marked(mt.shares + tile, 0.f);
+    return;
+  }
+  const bool vec = rows_vec(static_cast<const T*>(mt.G), mt.ld, mt.n) && rows_vec(static_cast<const T*>(mt.W), mt.ld, mt.n);
+  const bool regular = mt.r % split::BK == 0 && reinterpret_cast<unsigned long long>(mt.P) % 16 == 0;       // (R and N are aligned)
+  if (vec && regular) step_tile<T, COLS, true, true>(mt, tile, i0, j0, hp, smem, ctl, ks, coef);
+  else if (regular) step_tile<T, COLS, false, true>(mt, tile, i0, j0, hp, smem, ctl, ks, coef);
+  else step_tile<T, COLS, false, false>(mt, tile, i0, j0, hp, smem, ctl, ks, coef);
+}
+// norm_out, t_out: where the caller keeps the remembered norm and the step count (may be null).
+// tiles: blocks that have a tile (COLS = 128) or half of one (64).
+template <int COLS>
+__global__ void __launch_bounds__(STEP_THREADS, 1)
+k_back_step(const MatDev* mats, const int* list, int nlist, const int* tile_start, int first, int tiles, int first_matrix, Hyper hp, float* norm_out,
+            long long* t_out, unsigned* status) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ float ks[SIMT_TILE], coef;
+  __shared__ int waited;
+  split::Ctl* ctl = reinterpret_cast<split::Ctl*>(smem + 2 * STEP_X);
+  if ((int)blockIdx.x >= tiles) {                // a matrix's state
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) waited = 0;
+    __syncthreads();
+    ptx::grid_wait();
+    ptx::grid_launch_next();
+    const MatDev& mt = mats[list[first_matrix + blockIdx.x - tiles]];
+    const long long next = mt.sc->t + 2;
+    __syncthreads();                             // (t is read before it is stored)
+    if (threadIdx.x == 32 && !(hp.mode & (HYPER_PSI_RMSPROP | HYPER_PSI_ADAGRAD))) {
+      mt.bias->next = bias_factor_call(hp.beta1, hp.beta2, next);
+      mt.bias->step = next;
+    }
+    if (threadIdx.x < 32) {
+      Limit lim;
+      if (wait_limit(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, mt.sc->prev_norm, hp, &waited, lim)) store_limit(mt, hp, lim, status);
+      else if (lane == 0) atomicOr(status, DEV_STATUS_TIMEOUT);
+      if (lane == 0 && norm_out) { *norm_out = mt.sc->prev_norm; *t_out = mt.sc->t; }
+    }
+    return;
+  }
+  split::begin(ctl);
+  ptx::grid_wait();
+  ptx::grid_launch_next();
+  constexpr int PER = SIMT_TILE / COLS;
+  const int gt = blockIdx.x / PER + first, half = blockIdx.x % PER;
+  const int q = find_matrix(tile_start, nlist, gt);
+  const MatDev mt = mats[list[q]];
+  const int tile = gt - tile_start[q], ct = simt_tiles_dev(mt.n);
+  const int i0 = (tile / ct) * SIMT_TILE, j0 = (tile % ct) * SIMT_TILE + half * COLS;
+  if (mt.bf16) step_tile<__nv_bfloat16, COLS>(mt, PER * tile + half, i0, j0, hp, smem, ctl, ks, &coef);
+  else step_tile<float, COLS>(mt, PER * tile + half, i0, j0, hp, smem, ctl, ks, &coef);
   split::end(ctl, status);
 }
 
@@ -759,6 +982,8 @@ static bool allow_smem() {
                                (const void*)k_back_project<MODE_NORM, true, 1>, (const void*)k_back_project<MODE_UPDATE, true, 1>};
     for (const void* k : kernels)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, split::SMEM_BYTES);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_back_step<SIMT_TILE>, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_back_step<SIMT_TILE / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM);
     if (e == cudaSuccess) done[dev].store(true);
   }
   if (e != cudaSuccess) set_error(std::string("step kernels, shared memory: ") + cudaGetErrorString(e));
@@ -837,6 +1062,15 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     launch_error((psi == PSI_ADAM ? launch_project<PSI_ADAM> : psi == PSI_RMSPROP ? launch_project<PSI_RMSPROP> : launch_project<PSI_ADAGRAD>)(
         pl, pt0, pt1 - pt0, hp, status_dev, st));
     tm->mark(st);
+  }
+  if (pl.one_kernel && !only_scaling) {
+    for (int i = 0; i < 4; ++i) tm->mark(st);    // (its time counts as the update's)
+    const int per = short_one_kernel(2 * pl.w_tiles, pl.nlist, pl.max_r) ? 2 : 1, blocks = per * (wt1 - wt0);       // (of the whole list, whatever range is stepped)
+    launch_error(launch_resident(per == 2 ? k_back_step<SIMT_TILE / 2> : k_back_step<SIMT_TILE>, blocks + nq, STEP_THREADS, STEP_SMEM, st, true, 1, pl.mats, pl.list,
+                                 pl.nlist, pl.w_tile_start, wt0, blocks, qa, hp, pl.norm_out, pl.t_out, status_dev));
+    tm->mark(st);
+    if (error != cudaSuccess) { set_error(std::string("step kernels: ") + cudaGetErrorString(error)); return -1; }
+    return 2;
   }
   tm->mark(st);
   if (one_kernel) {

@@ -48,6 +48,9 @@ struct SimtPlan {
   long long max_proj_units = 0;          // long lists: largest projection, in units of eight entries of its parts
   const int* w_tile_start = nullptr;     // 128 x 128 tiles of W (m x n)
   int w_tiles = 0;
+  bool one_kernel = false;               // short lists: norm, limiter and update in one kernel (short_one_kernel; MatDev::shares are there)
+  float* norm_out = nullptr;             //   a single matrix's remembered norm and step count go there as well
+  long long* t_out = nullptr;
   const int* npart = nullptr;            // partial sums of ||S||^2 per matrix
   const int* row_start = nullptr;        // rows l (long lists)
   const int* npart_tiles = nullptr;      // the same where there is one per 128 x 128 tile of W
@@ -64,6 +67,10 @@ struct SimtPlan {
 // Whether a list of these matrices (the ones of this engine) is long: its products with the projection then run on
 // parts (part_gemm.cu), which R, X and the projection are kept as.
 bool simt_long_list(const std::vector<fira_matrix_desc>& list);
+// Whether a short list's norm, limiter and update are one kernel: w_tiles 128 x 128 tiles of W in nlist matrices, one block each and one
+// more per matrix, all resident at once.
+constexpr int SHORT_RESIDENT = 148;
+inline bool short_one_kernel(int w_tiles, int nlist, int max_r) { return nlist > 0 && w_tiles + nlist <= SHORT_RESIDENT && max_r <= 128; }
 // Copies rows of staged matrices (MatDev Gs, Ws): dir 0 G and W in, 1 W out (step_tc.cu).
 void launch_stage(const MatDev* mats, const int* list, int nlist, const int* row_start, int first_row, int rows, int dir, cudaStream_t st);
 // Enqueues the phases for the matrices [qa, qb) of the list (qb < 0: the whole list); returns

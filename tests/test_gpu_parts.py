@@ -163,3 +163,24 @@ def test_long_products_do_not_drift(shapes, r):
         N = (1 - 0.5 ** 101) ** 0.5 * M.double() / (V.double().sqrt() + 1e-8)
         D = P[i].double() @ N.T if m <= n else N @ P[i].double().T
         assert abs(float((-W[i].double() - D).sum() / D.sum())) < 2e-7
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("flags", [0, fb.FLAG_MATRIX_SCALING, fb.FLAG_NO_RESIDUAL, fb.FLAG_PSI_RMSPROP])
+@pytest.mark.parametrize("shapes,ranks", [([(130, 65), (65, 130), (64, 129), (129, 63), (200, 192)], [33, 32, 31, 5, 128]),
+                                          ([(512, 1376)], [128]), ([(384, 1030)] * 3, [100] * 3)])
+def test_short_list_that_steps_in_one_kernel(shapes, ranks, flags, dtype):
+    """Half tiles of W and their edges, ranks around the slabs' depth, a rank of whole slabs; whole tiles (81 of them)."""
+    tr = _stepped_from_ordinary_moments(shapes, ranks, dtype, flags)
+    tr.assert_ok()
+    assert tr.f.last_step_launches() == 2
+
+
+@pytest.mark.parametrize("shapes,ranks,launches", [([(1100, 2800), (512, 1376), (1376, 512)], [64, 200, 128], 4),
+                                                   ([(1200, 3840), (512, 1376)], [100, 128], 7)])
+def test_long_list_around_the_tiles_of_one_kernel(shapes, ranks, launches):
+    """fp32 matrices of more tiles than CTA pairs, whose pairs have two tiles of one matrix, and of more than twice as many, which
+    take two kernels."""
+    tr = _stepped_from_ordinary_moments(shapes, ranks, torch.float32, 0)
+    tr.assert_ok()
+    assert tr.f.last_step_launches() == launches
