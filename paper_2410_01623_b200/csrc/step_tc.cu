@@ -121,7 +121,8 @@ k_tc_prep(const MatDev* __restrict__ mats, const int* __restrict__ list, int fir
     const double s = (double)(mt.sc->t + 1);
     const float bias = (float)(sqrt(1.0 - pow((double)hp.beta2, s)) / (1.0 - pow((double)hp.beta1, s)));
     mt.sc->bias = bias;
-    fast[2 * p] = bias;          // read by the projection epilogue
+    fast[4 * p] = bias;          // read by the projection epilogue
+    fast[4 * p + 2] = mt.sc->lambda != 1.f ? 0.f : 1.f;     // whether it forms X (FUSE_X = 3)
   }
   // the counters through which the projection epilogues of a row of tiles tell one another that
   // their partial sums are in place (behind the partial sums; see tc_colpart_floats)
@@ -272,7 +273,7 @@ k_tc_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int n
   const int l = row - row_start[p];
   const float lambda = mt.sc->lambda;
   if (fused && fuse_x_matrix(mt.d, mt.r)) return;      // k_tc_fix_x's matrix
-  if (l == 0 && lane == 0) fast[2 * p + 1] = lambda;   // read by the back-projection epilogue
+  if (l == 0 && lane == 0) fast[4 * p + 1] = lambda;   // read by the back-projection epilogue
   const long long base = (long long)l * mt.r;
   const float c = a_res * lambda * mt.kvec[l];
   for (int j = lane * 8; j < mt.r; j += 256) {
@@ -291,6 +292,7 @@ k_tc_form_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int n
 // acted, X_lambda = a_low N - a_res lambda k_l R = lambda X + (1 - lambda) a_low N, with N as the projection kept it
 // (FUSE_X = 2), otherwise rebuilt from the moments that the epilogue stored, by the epilogue's own arithmetic and
 // rounded to bf16 as it was there; the other matrices are left as they are.
+// BY_LIMITER (after FUSE_X = 3): matrices that have left N and R: X for factor 1, rounded, and then as above.
 // blockIdx.y = matrix of the range, the blocks of a matrix stride over its rows, one warp per row.  Bound by
 // memory.
 __device__ __forceinline__ uint4 limited_x(const uint4& x, const float (&n)[8], float lambda, float cn) {
@@ -300,20 +302,39 @@ __device__ __forceinline__ uint4 limited_x(const uint4& x, const float (&n)[8], 
   for (int e = 0; e < 8; ++e) v[e] = fmaf(cn, n[e], lambda * v[e]);
   return pack8_bf16(v);
 }
+template <bool BY_LIMITER>
 __global__ void __launch_bounds__(256)
-k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int first, float a_low, float eps, int kept,
+k_tc_fix_x(const MatDev* __restrict__ mats, const int* __restrict__ list, int first, float a_low, float a_res, float eps, int kept,
            float* __restrict__ fast) {
   const int p = first + blockIdx.y;
   const MatDev& mt = mats[list[p]];
   if (!fuse_x_matrix(mt.d, mt.r)) return;              // k_tc_form_x's matrix
   const float lambda = mt.sc->lambda;
-  if (blockIdx.x == 0 && threadIdx.x == 0) fast[2 * p + 1] = lambda;   // read by the back-projection epilogue
-  if (lambda == 1.f) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) fast[4 * p + 1] = lambda;   // read by the back-projection epilogue
+  const bool formed = !BY_LIMITER || fast[4 * p + 2] != 0.f;
+  if (formed && lambda == 1.f) return;
   const int lane = threadIdx.x & 31;
-  const float bias = fast[2 * p];                      // this step's bias factor (k_tc_prep)
+  const float bias = fast[4 * p];                      // this step's bias factor (k_tc_prep)
   const float cn = (1.f - lambda) * a_low;
   for (int l = blockIdx.x * 8 + (threadIdx.x >> 5); l < mt.l; l += gridDim.x * 8) {
     const long long base = (long long)l * mt.r;
+    if (BY_LIMITER && !formed) {
+      const float ck = a_res * mt.kvec[l];
+#pragma unroll 2
+      for (int j = lane * 8; j < mt.r; j += 256) {
+        const uint4 nu = *reinterpret_cast<const uint4*>(mt.Nb + base + j);
+        const uint4 ru = *reinterpret_cast<const uint4*>(mt.Rb + base + j);
+        float nv[8], rv[8], x[8];
+        unpack8_bf16(nu, nv);
+        unpack8_bf16(ru, rv);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = unlimited_x(a_low, nv[e], ck, rv[e]);
+        uint4 xu = pack8_bf16(x);
+        if (lambda != 1.f) xu = limited_x(xu, nv, lambda, cn);
+        *reinterpret_cast<uint4*>(mt.Xb + base + j) = xu;
+      }
+      continue;
+    }
     if (kept) {
 #pragma unroll 2
       for (int j = lane * 8; j < mt.r; j += 256) {
@@ -432,7 +453,7 @@ struct TcPlan {
   const int* npart = nullptr;
   ProjTileDesc* td1_dev = nullptr;   // per-tile records of the projection
   BackTileDesc* td2_dev = nullptr;   // per-tile records of the back-projection
-  float* fast_dev = nullptr;         // per matrix of the list: {bias factor, lambda}
+  float* fast_dev = nullptr;         // per matrix of the list: {bias factor, lambda, whether the projection forms X, unused}
   float* wq_dev = nullptr;           // weights 2 - ||pi_j||^2 of all matrices of the list, r floats each
   const int* wq_off = nullptr;       // per matrix: its offset into wq_dev
   const int* wq_blk = nullptr;       // prefix sums of the blocks of k_tc_proj_weights
@@ -482,7 +503,7 @@ size_t tc_tables_bytes(const fira_hparams& hp, const fira_matrix_desc* descs, in
   size_t ntc = 0, tiles2 = 0, tiles1 = 0, rsum = 0;
   for (int i = 0; i < count; ++i)
     if (engine_for(hp, descs[i]) == 1) { ++ntc; tiles2 += back_tiles(descs[i]); tiles1 += proj_tiles(descs[i]); rsum += descs[i].r; }
-  return align_up(sizeof(TcMaps) * ntc) + align_up(2 * sizeof(float) * ntc) +
+  return align_up(sizeof(TcMaps) * ntc) + align_up(4 * sizeof(float) * ntc) +
          align_up(sizeof(BackTileDesc) * tiles2) + align_up(sizeof(ProjTileDesc) * tiles1) + align_up(sizeof(float) * rsum);
 }
 
@@ -553,7 +574,7 @@ fira_status tc_build_plan(fira_ctx* c, std::vector<int>& ints) {
   pl->maps.resize(lst.size());
   char* tab = c->tc_maps_dev;
   pl->maps_dev = reinterpret_cast<TcMaps*>(tab); tab += align_up(sizeof(TcMaps) * lst.size());
-  pl->fast_dev = reinterpret_cast<float*>(tab); tab += align_up(2 * sizeof(float) * lst.size());
+  pl->fast_dev = reinterpret_cast<float*>(tab); tab += align_up(4 * sizeof(float) * lst.size());
   pl->td2_dev = reinterpret_cast<BackTileDesc*>(tab); tab += align_up(sizeof(BackTileDesc) * (size_t)pl->k2_tiles);
   pl->td1_dev = reinterpret_cast<ProjTileDesc*>(tab); tab += align_up(sizeof(ProjTileDesc) * (size_t)pl->k1_tiles);
   pl->wq_dev = reinterpret_cast<float*>(tab);
@@ -740,12 +761,12 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     const void* k1s[5] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0>, (const void*)k_tc_project<EPI_ADAM, PSI_RMSPROP, 0>,
                           (const void*)k_tc_project<EPI_ADAM, PSI_ADAGRAD, 0>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1>,
                           (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 2>};
-    const void* k1g[3] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0, 2>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1, 2>,
+    const void* k1g[4] = {(const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 3, 2>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 0, 2>, (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 1, 2>,
                           (const void*)k_tc_project<EPI_ADAM, PSI_ADAM, 2, 2>};
     cudaError_t e1 = cudaSuccess;
     for (int i = 0; i < 5 && e1 == cudaSuccess; ++i)
       e1 = cudaFuncSetAttribute(k1s[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)K1_SMEM_BYTES);
-    for (int i = 0; i < 3 && e1 == cudaSuccess; ++i)
+    for (int i = 0; i < 4 && e1 == cudaSuccess; ++i)
       e1 = cudaFuncSetAttribute(k1g[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k1_smem_bytes(2));
     cudaError_t e2 = cudaFuncSetAttribute(k_tc_back_project<5, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k2_smem_bytes(5, 2));
     if (e2 == cudaSuccess)
@@ -771,7 +792,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
       }
       pl->max_pairs_fused = std::min(nclusters, pl->num_sms / 2);
       cfg.blockDim = dim3(k1_threads(2)); cfg.dynamicSmemBytes = k1_smem_bytes(2);
-      const cudaError_t e4 = cudaOccupancyMaxActiveClusters(&nclusters, k1g[2], &cfg);
+      const cudaError_t e4 = cudaOccupancyMaxActiveClusters(&nclusters, k1g[0], &cfg);
       if (e4 != cudaSuccess || nclusters <= 0) {
         set_error(std::string("cudaOccupancyMaxActiveClusters: ") + cudaGetErrorString(e4));
         return -1;
@@ -818,18 +839,21 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
   // Short products are bound by the epilogue, which then runs with two groups of warps per CTA; long
   // ones (r = 1024 lists) are bound by the tensor pipe and keep one.
   const bool two_groups = rmax <= 512;
-  bool keep_n = fused;
+  bool keep_n = fused, exchange = false;
   for (int q = qa; q < qb; ++q) {
     const MatDev& mq = c->mats[c->tc_list[q]];
     if (fuse_x_matrix(mq.d, mq.r) && mq.d < FUSE_KEEP_N_MIN_D) keep_n = false;
+    exchange = exchange || (fuse_x_matrix(mq.d, mq.r) && mq.r > host_tile_bn(mq.r));
   }
+  const bool by_limiter = two_groups && keep_n && exchange;
 #define FIRA_LAUNCH_K1(PSI, FUSE, EG)                                                                       \
   k_tc_project<EPI_ADAM, PSI, FUSE, EG><<<k1_grid, k1_threads(EG), k1_smem_bytes(EG), st>>>(                \
       pl->maps_dev, td1, k1n, pl->fast_dev, pl->wq_dev, pl->wq_off, hp, c->status_dev)
   if (hp.mode & HYPER_PSI_RMSPROP) FIRA_LAUNCH_K1(PSI_RMSPROP, 0, 1);
   else if (hp.mode & HYPER_PSI_ADAGRAD) FIRA_LAUNCH_K1(PSI_ADAGRAD, 0, 1);
   else if (two_groups) {
-    if (keep_n) FIRA_LAUNCH_K1(PSI_ADAM, 2, 2);
+    if (by_limiter) FIRA_LAUNCH_K1(PSI_ADAM, 3, 2);
+    else if (keep_n) FIRA_LAUNCH_K1(PSI_ADAM, 2, 2);
     else if (fused) FIRA_LAUNCH_K1(PSI_ADAM, 1, 2);
     else FIRA_LAUNCH_K1(PSI_ADAM, 0, 2);
   }
@@ -861,7 +885,7 @@ int launch_tc_step(fira_ctx* c, const Hyper& hp, int qa, int qb) {
     k_tc_form_x<<<(rsb - rsa + 7) / 8, 256, 0, st>>>(mats, pl->list, pl->nlist, pl->row_start, rsa, rsb,
                                                      hp.a_low, hp.a_res, pl->fast_dev, fused ? 1 : 0);
   if (any_fused)
-    k_tc_fix_x<<<dim3(32, nq), 256, 0, st>>>(mats, pl->list, qa, hp.a_low, hp.eps, keep_n ? 1 : 0, pl->fast_dev);
+    (by_limiter ? k_tc_fix_x<true> : k_tc_fix_x<false>)<<<dim3(32, nq), 256, 0, st>>>(mats, pl->list, qa, hp.a_low, hp.a_res, hp.eps, keep_n ? 1 : 0, pl->fast_dev);
   tm->mark(st);
   // long products keep five operand stages; short ones trade one for more epilogue boxes in flight
   if (rmax >= 1024)

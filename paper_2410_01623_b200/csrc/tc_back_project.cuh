@@ -263,7 +263,7 @@ k_tc_back_project(const TcMaps* __restrict__ maps, const BackTileDesc* __restric
       const int left = d.m_left < 0;
       const int m = d.m_left & 0x7fffffff;
       const int i0 = d.i0 + BM * (int)rank;
-      const float cres = hp.a_res * fast[2 * d.slot + 1];
+      const float cres = hp.a_res * fast[4 * d.slot + 1];
       float* ks = ksm + (g * 2 + tile_parity) * K2_KS_GROUP;   // box c of this group at ks + 32 (c / 2)
       float krow = 0.f;
       if (left) {

@@ -62,6 +62,12 @@
 // after FUSE_X = 1 it rebuilds the same N from the stored moments: 12 bytes per element.  (X + (1 - lambda) a_res k_l R from a
 // kept R costs the same and is less precise: X and R have each been rounded to bf16 before most of them cancels, which
 // leaves about 2.4 times the error.)
+// FUSE_X = 3: as 2, but the matrices that k_tc_prep has marked leave N and R instead, as without FUSE_X: those whose limiter acted on
+// the step before, and which are likely to be limited again; k_tc_fix_x makes the same X from them bit for bit.  For lists with two
+// groups of epilogue warps, where the second sweep and its exchange are on the critical path.  Measured, 1B list, limiter
+// acting on all: projection 1863 us forming X and correction 285 us; 1649 and 306 leaving N and R; step 5205 / 5065.  Not on the 350M list,
+// whose rows of tiles need no exchange (projection + 43, correction - 51, the check itself 1 % of the step), nor on the 7B list, one group
+// (projection + 2 %).
 // (Adam only: with RMSProp or Adagrad N cannot be rebuilt from V alone, and those steps keep the
 // separate pass.)
 constexpr int K1_STAGES = 4;
@@ -149,6 +155,9 @@ struct ProjCtl {
   int abort_flag;
 };
 static_assert(sizeof(ProjCtl) <= 512, "ProjCtl must fit its slot");
+
+// X for limiter factor 1, by the same arithmetic wherever it is formed.
+__device__ __forceinline__ float unlimited_x(float a_low, float n, float ck, float r) { return fmaf(a_low, n, -(ck * r)); }
 
 // sqrt.approx and the fast division are good to about 2 ulp each; N is rounded to bf16 next.
 __device__ __forceinline__ float fast_sqrt(float x) {
@@ -450,7 +459,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
         const TcMaps* mp = &maps[d.slot];
         const int bn = d.bn_left & 0xffff;
         const int l0 = d.l0 + BM * (int)rank;
-        const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_n = FUSE_X == 2 && fuse;
+        const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X) && (FUSE_X < 3 || fast[4 * d.slot + 2] != 0.f), keep_n = FUSE_X >= 2 && fuse;
         for (int b = 0; b < 2 * (bn / K1_ECOLS); ++b) {
           if (!ptx::mbar_wait(ptx::smem_u32(&ctl->eready[mv]), mvphase, abort_flag)) { ok = false; break; }
           const int nr = b & 1;
@@ -532,7 +541,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
       if (t + npairs < total_tiles) nd = load_desc(tdesc, t + npairs);
       const int bn = d.bn_left & 0xffff;
       const int l = d.l0 + BM * (int)rank + row;
-      const float bias = EPI == EPI_ADAM ? fast[2 * d.slot] : 0.f;
+      const float bias = EPI == EPI_ADAM ? fast[4 * d.slot] : 0.f;
       const float* wrow = EPI == EPI_ADAM ? wq_all + wq_off[d.slot] + d.r0 : nullptr;   // weights of this tile's rank range
       if (EPI == EPI_ADAM) asm volatile("prefetch.global.L1 [%0];" ::"l"(wrow));
       if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->tmem_full[buf]), bphase, abort_flag)) break;
@@ -540,7 +549,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
       const uint32_t tcol = tmem + ((uint32_t)(quarter * 32) << 16) + buf * BN_MAX;
       const uint32_t te = buf ? tmem_empty1 : tmem_empty0;
       const int nch = bn / K1_ECOLS;
-      const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X), keep_n = FUSE_X == 2 && fuse;
+      const bool fuse = FUSE_X && (d.bn_left & PROJ_FUSE_X) && (FUSE_X < 3 || fast[4 * d.slot + 2] != 0.f), keep_n = FUSE_X >= 2 && fuse;
       float nn = 0.f, rn = 0.f, rw = 0.f;
       for (int c = 0; c < nch; ++c) {
         uint32_t rr[GC];
@@ -717,7 +726,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
         xphase ^= 1u;
       }
       if (fuse && ok) {
-        const float ck = hp.a_res * 1.0f * kl;           // k_tc_form_x's coefficient at lambda = 1
+        const float ck = hp.a_res * kl;                  // k_tc_form_x's coefficient at lambda = 1
         // ---- sweep 2: X = a_low N - a_res k_l R as bf16 boxes
         for (int c = 0; c < nch; ++c) {
           uint32_t rr[GC];
@@ -739,7 +748,7 @@ k_tc_project(const TcMaps* __restrict__ maps, const ProjTileDesc* __restrict__ t
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
               const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&rr[8 * qq + e]));
-              xv[e] = hp.a_low * f.x - ck * f.y;
+              xv[e] = unlimited_x(hp.a_low, f.x, ck, f.y);
             }
             *reinterpret_cast<uint4*>(xb + hrow + (((uint32_t)q ^ hsw) << 4)) = pack8_bf16(xv);
           }
