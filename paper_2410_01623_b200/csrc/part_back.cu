@@ -452,7 +452,7 @@ k_part_back(const BackJob* __restrict__ jobs, const TileDev* __restrict__ tiles,
 // (12 warps in all: a thirteenth would leave 128 registers per thread), 11 box storer.
 constexpr int RU_STAGES = 4;
 constexpr int RU_BUFS = 5;
-constexpr int RU_RECORDS = 4;                   // (the box loader, who brings them, is three passes ahead at most)
+constexpr int RU_RECORDS = 4;                   // (the box loader, who brings them, may be as many passes ahead as there are buffers: it waits for a free place)
 constexpr int RU_GROUPS = 2;                    // of epilogue warps
 constexpr int RU_COLS = PN / RU_GROUPS;         // a group's columns: neighbours
 constexpr int RU_BOX_COLS = 32;
@@ -470,6 +470,7 @@ struct StepCtl {
   uint64_t shared_in[2];                        // (odd CTA; tiles in turn) the shares of the epilogue warps
   uint64_t lambda_in[2];
   uint64_t record_in[RU_RECORDS];               // the epilogue's copies of the tiles' records
+  uint64_t record_out[RU_RECORDS];              //   "  the epilogue warps have made the tile's second pass
   uint32_t tmem_base;
   int abort_flag;
   alignas(16) float ks[RU_GROUPS][2][RU_COLS];
@@ -538,7 +539,10 @@ k_part_step(const BackJob* __restrict__ jobs, int njobs, const TileDev* __restri
       ptx::mbar_init(ptx::smem_u32(&ctl->eempty[b]), 1);
     }
     for (int g = 0; g < RU_GROUPS; ++g) ptx::mbar_init(ptx::smem_u32(&ctl->esync[g]), GROUP_THREADS);
-    for (int b = 0; b < RU_RECORDS; ++b) ptx::mbar_init(ptx::smem_u32(&ctl->record_in[b]), 1);
+    for (int b = 0; b < RU_RECORDS; ++b) {
+      ptx::mbar_init(ptx::smem_u32(&ctl->record_in[b]), 1);
+      ptx::mbar_init(ptx::smem_u32(&ctl->record_out[b]), RU_WARPS);
+    }
     ctl->abort_flag = smem_ok ? 0 : 1;
     ptx::fence_barrier_init();
   }
@@ -637,8 +641,10 @@ k_part_step(const BackJob* __restrict__ jobs, int njobs, const TileDev* __restri
       passes(tiles, pair, count, npairs, [&](int pass, const TileDev& d, int) {
         const BackJob* jb = jobs + d.job;
         if (pass == 0) {
-          ctl->records[records % RU_RECORDS] = d;
-          ptx::mbar_arrive(ptx::smem_u32(&ctl->record_in[records % RU_RECORDS]));
+          const int place = records % RU_RECORDS;
+          if (!ptx::mbar_wait(ptx::smem_u32(&ctl->record_out[place]), ((records / RU_RECORDS) & 1) ^ 1u, abort_flag)) return false;
+          ctl->records[place] = d;
+          ptx::mbar_arrive(ptx::smem_u32(&ctl->record_in[place]));
           ++records;
         }
         const int i0 = d.i0 + PM / 2 * (int)rank;
@@ -806,7 +812,12 @@ k_part_step(const BackJob* __restrict__ jobs, int njobs, const TileDev* __restri
       const int r = firsts;
       if (t < count && (!ptx::mbar_wait(ptx::smem_u32(&ctl->record_in[r % RU_RECORDS]), (r / RU_RECORDS) & 1, abort_flag) ||
                         !first_pass(ctl->records[r % RU_RECORDS]))) break;
-      if (t > pair && !second_pass(ctl->records[seconds % RU_RECORDS])) break;
+      if (t > pair) {
+        const int q = seconds % RU_RECORDS;
+        if (!second_pass(ctl->records[q])) break;
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&ctl->record_out[q]));
+      }
       if (t >= count) break;
     }
   }

@@ -184,3 +184,29 @@ def test_long_list_around_the_tiles_of_one_kernel(shapes, ranks, launches):
     tr = _stepped_from_ordinary_moments(shapes, ranks, torch.float32, 0)
     tr.assert_ok()
     assert tr.f.last_step_launches() == launches
+
+
+@pytest.mark.parametrize("shapes,ranks", [(wk.llama_shapes(8, 288, 992), [64] * 56), (wk.llama_shapes(20, 160, 416), [40] * 140),
+                                          ([(1024, 32)] * 80 + [(1024, 1024)] * 5, [16] * 80 + [128] * 5)])
+def test_long_list_with_runs_of_narrow_tiles(shapes, ranks):
+    """Tiles whose last columns number 32 or fewer have one box of W where others have four: of the loader's buffers five such tiles
+    take no more than one wide one.  Pairs with four and more of them in a row and a wide tile, or one of another rank, behind."""
+    tr = _stepped_from_ordinary_moments(shapes, ranks, torch.float32, 0)
+    tr.assert_ok()
+    assert tr.f.last_step_launches() == 4
+    g = torch.Generator().manual_seed(3)
+    fs = [fb.Fira(shapes, ranks, torch.float32, fb.make_hparams(lr=1e-2, alpha=0.25, gamma=1.01)) for _ in range(2)]
+    for i, (m, n) in enumerate(shapes):
+        P = torch.linalg.qr(torch.randn(min(m, n), ranks[i], generator=g))[0].contiguous().cuda()
+        for f in fs:
+            f.set_projection(i, P)
+    Wh = [(torch.randn(s, generator=g) * 0.02).pin_memory() for s in shapes]
+    W = [w.cuda() for w in Wh]
+    staging = torch.empty(fs[1].staging_bytes(), dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        G = [torch.randn(s, generator=g).pin_memory() for s in shapes]
+        fs[0].step(W, [x.cuda() for x in G])
+        fs[1].step_host(Wh, G, staging)
+        torch.cuda.synchronize()
+    assert [f.poll() for f in fs] == [0, 0]
+    assert all(torch.equal(w.cpu(), h) for w, h in zip(W, Wh))
