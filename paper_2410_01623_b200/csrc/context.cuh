@@ -59,7 +59,7 @@ struct Layout {
   std::vector<size_t> offRt, offXt, offK, offPart, offNb, offRb, offXb, offColpart, offGs, offWs, offAux, offRp, offXp, offPp;
   std::vector<int> engine;
   bool parts = false;       // the fp32-precision engine's list is long
-  bool one_kernel = false;  // it is short, and steps in one kernel after the projection
+  bool one_kernel = false;  // it is short, and steps in one kernel after the projection (where enough SMs are there)
   size_t off_parts = 0, off_proj_parts = 0;
   size_t step_work_bytes = 0, refresh_min_bytes = 0;
   size_t scratch_bytes = 0;

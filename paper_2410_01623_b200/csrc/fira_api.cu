@@ -332,8 +332,9 @@ fira_status fira_init(fira_ctx** out, const fira_hparams* hp, const fira_matrix_
       c->simt.max_proj_units = std::max(c->simt.max_proj_units, (long long)c->mats[i].d * c->mats[i].pp_pitch / 8);
     }
     c->simt.w_tile_start = c->ints_dev + o_wt; c->simt.w_tiles = wt.back();
-    c->simt.one_kernel = L.one_kernel;
-    if (L.one_kernel)
+    const int resident = L.one_kernel ? short_resident(c->stream) : 0;
+    c->simt.resident = L.one_kernel && short_one_kernel(wt.back(), (int)lst.size(), c->simt.max_r, resident) ? resident : 0;
+    if (c->simt.resident)
       for (size_t q = 0; q < lst.size(); ++q) c->mats[lst[q]].shares = reinterpret_cast<unsigned long long*>(c->scratch_base + L.off_shares) + 2 * wt[q];
     c->simt.npart = c->ints_dev + o_np; c->simt.npart_tiles = c->ints_dev + o_npt;
     c->simt.row_start = c->ints_dev + o_rs; c->simt.h_row_start = rs;

@@ -165,7 +165,8 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   mt.part = reinterpret_cast<float*>(base + cv.off_part);
   mt.aux = reinterpret_cast<float*>(base + kNoAllocScratchBytes);
   mt.aux_slots = simt_tiles(desc->r);
-  const bool one_kernel = short_one_kernel(simt_tiles(desc->m) * simt_tiles(desc->n), 1, desc->r);
+  const int resident = short_resident(st);
+  const bool one_kernel = short_one_kernel(simt_tiles(desc->m) * simt_tiles(desc->n), 1, desc->r, resident);
   if (one_kernel) mt.shares = reinterpret_cast<unsigned long long*>(base + kNoAllocScratchBytes + kRowSumBytes);
   mt.m = desc->m; mt.n = desc->n; mt.r = desc->r;
   mt.ld = desc->ld ? desc->ld : desc->n;
@@ -189,8 +190,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   pl.proj_tile_start = ints_dev + 1; pl.proj_tiles = ptiles; pl.max_d = mt.d; pl.max_r = mt.r;
   pl.w_tile_start = ints_dev + 3; pl.w_tiles = wtiles;
   pl.npart = ints_dev + 5;
-  pl.one_kernel = one_kernel;
-  if (one_kernel) { pl.norm_out = norm_prev_dev; pl.t_out = reinterpret_cast<long long*>(t_dev); }
+  if (one_kernel) { pl.resident = resident; pl.norm_out = norm_prev_dev; pl.t_out = reinterpret_cast<long long*>(t_dev); }
   Hyper h;
   h.beta1 = hp->beta1; h.beta2 = hp->beta2; h.eps = hp->eps;
   h.lr = lr < 0.f ? hp->lr : lr;

@@ -893,8 +893,9 @@ fira_status part_step_prepare(const std::vector<MatDev>& mats, const std::vector
   plan->jobs.assign(2 * list.size() * sizeof(BackJob), 0);
   plan->tile_start.assign(1, 0);
   plan->deep = 0;
-  const int pairs = resident_pairs();
+  int pairs = resident_pairs();
   if (!pairs) return FIRA_ERR_CUDA;
+  pairs = std::min(pairs, stream_sms(st) / 2);
   // One kernel for norm and update: 56 matrices 512 / 1376 fp32, step 231 us against 246 with two (210 / 256 where the limiter acts on all and
   // a step finds its tables in L2).  bf16, where G is half of the traffic less: 28 of 640 / 1707, 189 / 185.
   plan->one_kernel_pairs = pairs;

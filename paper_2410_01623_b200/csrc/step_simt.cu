@@ -18,6 +18,8 @@
 // Short lists are bound by latency, so all of their kernels are chained (launch_chained): one's set-up (tables, barriers,
 // tensor memory) runs while the one before it ends.  Step of one 512 x 1376 matrix: 74 us without that and without the
 // split projection, 35 us with both, 26.7 us with phases 2 to 4 in one kernel (k_back_step).
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 
@@ -960,6 +962,37 @@ bool simt_long_list(const std::vector<fira_matrix_desc>& list) {
   return elements >= LONG_LIST_ELEMENTS;
 }
 
+int stream_sms(cudaStream_t st) {
+  struct Driver {
+    CUresult (*current)(CUcontext*) = nullptr;
+    CUresult (*of_context)(CUcontext, CUdevResource*, CUdevResourceType) = nullptr;
+    CUresult (*green)(CUstream, CUgreenCtx*) = nullptr;
+    CUresult (*of_green)(CUgreenCtx, CUdevResource*, CUdevResourceType) = nullptr;
+  };
+  static const Driver drv = [] {                 // (an older driver has none of them, and no such parts)
+    Driver d;
+    auto get = [](const char* name, void** f) {
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPoint(name, f, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) *f = nullptr;
+    };
+    get("cuCtxGetCurrent", (void**)&d.current);
+    get("cuCtxGetDevResource", (void**)&d.of_context);
+    get("cuStreamGetGreenCtx", (void**)&d.green);
+    get("cuGreenCtxGetDevResource", (void**)&d.of_green);
+    return d;
+  }();
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  CUdevResource part;
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  if (drv.current && drv.of_context && drv.current(&ctx) == CUDA_SUCCESS && ctx && drv.of_context(ctx, &part, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+    sms = std::min(sms, (int)part.sm.smCount);
+  if (drv.green && drv.of_green && drv.green((CUstream)st, &green) == CUDA_SUCCESS && green && drv.of_green(green, &part, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS)
+    sms = std::min(sms, (int)part.sm.smCount);
+  return sms;
+}
+
 static void split_projections(const SimtPlan& pl, int qa, int qb, const Hyper& hp, cudaStream_t st) {
   const int per = (int)std::min<long long>(64, (pl.max_proj_units + 255) / 256);
   k_split_projection<<<(unsigned)((qb - qa) * (per + 1)), 256, 0, st>>>(pl.mats, pl.list + qa, per, hp);
@@ -1063,9 +1096,9 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
         pl, pt0, pt1 - pt0, hp, status_dev, st));
     tm->mark(st);
   }
-  if (pl.one_kernel && !only_scaling) {
+  if (pl.resident && !only_scaling) {
     for (int i = 0; i < 4; ++i) tm->mark(st);    // (its time counts as the update's)
-    const int per = short_one_kernel(2 * pl.w_tiles, pl.nlist, pl.max_r) ? 2 : 1, blocks = per * (wt1 - wt0);       // (of the whole list, whatever range is stepped)
+    const int per = short_one_kernel(2 * pl.w_tiles, pl.nlist, pl.max_r, pl.resident) ? 2 : 1, blocks = per * (wt1 - wt0);       // (of the whole list, whatever range is stepped)
     launch_error(launch_resident(per == 2 ? k_back_step<SIMT_TILE / 2> : k_back_step<SIMT_TILE>, blocks + nq, STEP_THREADS, STEP_SMEM, st, true, 1, pl.mats, pl.list,
                                  pl.nlist, pl.w_tile_start, wt0, blocks, qa, hp, pl.norm_out, pl.t_out, status_dev));
     tm->mark(st);

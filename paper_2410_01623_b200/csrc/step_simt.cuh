@@ -48,7 +48,7 @@ struct SimtPlan {
   long long max_proj_units = 0;          // long lists: largest projection, in units of eight entries of its parts
   const int* w_tile_start = nullptr;     // 128 x 128 tiles of W (m x n)
   int w_tiles = 0;
-  bool one_kernel = false;               // short lists: norm, limiter and update in one kernel (short_one_kernel; MatDev::shares are there)
+  int resident = 0;                      // short lists: norm, limiter and update in one kernel, on so many blocks at most (short_one_kernel; MatDev::shares are there)
   float* norm_out = nullptr;             //   a single matrix's remembered norm and step count go there as well
   long long* t_out = nullptr;
   const int* npart = nullptr;            // partial sums of ||S||^2 per matrix
@@ -68,9 +68,12 @@ struct SimtPlan {
 // parts (part_gemm.cu), which R, X and the projection are kept as.
 bool simt_long_list(const std::vector<fira_matrix_desc>& list);
 // Whether a short list's norm, limiter and update are one kernel: w_tiles 128 x 128 tiles of W in nlist matrices, one block each and one
-// more per matrix, all resident at once.
+// more per matrix, all resident at once, one to an SM (resident: how many can be; there is room for the words of SHORT_RESIDENT).
 constexpr int SHORT_RESIDENT = 148;
-inline bool short_one_kernel(int w_tiles, int nlist, int max_r) { return nlist > 0 && w_tiles + nlist <= SHORT_RESIDENT && max_r <= 128; }
+inline bool short_one_kernel(int w_tiles, int nlist, int max_r, int resident = SHORT_RESIDENT) { return nlist > 0 && w_tiles + nlist <= resident && max_r <= 128; }
+// SMs that kernels of the stream may run on: the device's, or fewer in a context or on a stream that has a part of them.
+int stream_sms(cudaStream_t st);
+inline int short_resident(cudaStream_t st) { const int sms = stream_sms(st); return sms < SHORT_RESIDENT ? sms : SHORT_RESIDENT; }
 // Copies rows of staged matrices (MatDev Gs, Ws): dir 0 G and W in, 1 W out (step_tc.cu).
 void launch_stage(const MatDev* mats, const int* list, int nlist, const int* row_start, int first_row, int rows, int dir, cudaStream_t st);
 // Enqueues the phases for the matrices [qa, qb) of the list (qb < 0: the whole list); returns

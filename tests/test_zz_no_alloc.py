@@ -182,3 +182,36 @@ def test_calls_of_different_matrices_behind_one_another():
 
     for a, b in zip(run(True), run(False)):
         assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("shape,r", [((512, 1376), 128), ((300, 200), 150)])
+def test_captured_calls_replay(shape, r):
+    """A captured call, replayed, gives what the call gives."""
+    lib, hp = fb.lib(), fb.make_hparams()
+    (m, n), l = shape, max(shape)
+    desc = fb.MatrixDesc(m, n, r, fb.FIRA_F32, 0)
+
+    def inputs():
+        g = torch.Generator(device="cuda").manual_seed(m)
+        return [torch.randn(m, n, generator=g, device="cuda") * 0.02, torch.randn(m, n, generator=g, device="cuda"),
+                torch.linalg.qr(torch.randn(min(shape), r, generator=g, device="cuda"))[0].contiguous(),
+                torch.zeros(l, r, device="cuda"), torch.ones(l, r, device="cuda"), torch.full((1,), -1.0, device="cuda"),
+                torch.zeros(1, dtype=torch.int64, device="cuda")]
+
+    def call(t):
+        fb.check(lib.fira_step_single_noalloc(C.byref(hp), C.byref(desc), *[x.data_ptr() for x in t], -1.0,
+                                              torch.cuda.current_stream().cuda_stream))
+
+    a, b = inputs(), inputs()
+    for _ in range(3):
+        call(a)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(b)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert lib.fira_noalloc_poll(torch.cuda.current_stream().cuda_stream) == 0
+    assert int(b[-1].item()) == 3
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
