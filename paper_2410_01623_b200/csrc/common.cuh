@@ -33,7 +33,7 @@ struct BiasSlot {
   long long step;
   float next;         // the factor of `step`
   float now;          // long lists of fp32 precision: the factor of the running step
-  float prev;         // norm and update in one kernel: the remembered norm before the step
+  float prev;         // norm and update in one kernel: the remembered norm before the step, left by a kernel in front of it (the state's is stored anew by a block that others are not ordered before)
 };
 
 // One entry of the device-resident problem table.  l = max(m,n) indexes the

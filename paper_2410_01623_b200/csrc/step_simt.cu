@@ -236,14 +236,17 @@ k_project(const MatDev* mats, const int* list, int nlist, const int* tile_start,
   const int l0 = (tile / rt) * SIMT_TILE, j0 = (tile % rt) * SIMT_TILE;
   split::begin(ctl);
   ptx::grid_launch_next();
-  if (mt.shares && tile == 0 && block == 0)      // (k_back_step waits for them; the one of the step before is done)
+  if (mt.shares && tile == 0 && block == 0) {    // (k_back_step waits for them; the one of the step before is done)
     for (int i = threadIdx.x; i < 2 * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n); i += split::THREADS) mt.shares[i] = 0ull;
+    if (threadIdx.x == 0) mt.bias->prev = mt.sc->prev_norm;
+  }
   const int slabs = (mt.d + split::BK - 1) / split::BK;
   const int k0 = slabs * block / blocks * split::BK, k1 = min(mt.d, slabs * (block + 1) / blocks * split::BK);
   const float* C = reinterpret_cast<const float*>(smem);
   // The bias factor, by one thread: while its first loads are on their way, or before them (not SPLIT: registers).
   const long long step = mt.sc->t + 1;
-  const BiasSlot slot = *mt.bias;
+  BiasSlot slot;
+  slot.step = mt.bias->step; slot.next = mt.bias->next;
   auto put_bias = [&] { if (PSI == PSI_ADAM && threadIdx.x == split::THREADS - 1) ctl->bias = step_bias(slot, step, hp); };
   if (!SPLIT) put_bias();
   auto bias_factor_of_step = [&] { if (SPLIT) put_bias(); };
@@ -449,7 +452,7 @@ __device__ __forceinline__ void step_tile(const MatDev& mt, int tile, int i0, in
   StepOperand<float> x;
   p.template load<REGULAR>(static_cast<const T*>(mt.P), mt.r, mt.d, mt.left ? i0 : j0, ns);
   x.template load<REGULAR>(mt.Rt, mt.r, mt.l, mt.left ? j0 : i0, ns);
-  const float prev = mt.sc->prev_norm;           // (stored anew when every tile has left its share)
+  const float prev = mt.bias->prev;
   // All of the product's slabs at once: a thread that issues MMAs between its slabs' conversions holds up the other warps' next slab.
   auto multiply = [&](bool with_p, uint64_t* done) {
 #pragma unroll
@@ -591,7 +594,7 @@ k_back_step(const MatDev* mats, const int* list, int nlist, const int* tile_star
     }
     if (threadIdx.x < 32) {
       Limit lim;
-      if (wait_limit(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, mt.sc->prev_norm, hp, &waited, lim)) store_limit(mt, hp, lim, status);
+      if (wait_limit(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, mt.bias->prev, hp, &waited, lim)) store_limit(mt, hp, lim, status);
       else if (lane == 0) atomicOr(status, DEV_STATUS_TIMEOUT);
       if (lane == 0 && norm_out) { *norm_out = mt.sc->prev_norm; *t_out = mt.sc->t; }
     }
