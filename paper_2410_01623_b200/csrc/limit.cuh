@@ -6,8 +6,8 @@
 namespace fira {
 
 // What a matrix's tiles need to know of its norm: lambda, times the matrix's one factor if it has one.  By one warp of every block
-// (or pair) that has a tile of it, all of them with the same result: they wait for the shares themselves, one marked word per tile, which
-// a kernel before has zeroed.  (Counting the tiles and having the last
+// (or pair) that has a tile of it, all of them with the same result: they wait for the shares themselves, marked words (SHARE: a float or
+// a double per tile, of the width that the tile's own sums have been added in), which a kernel before has zeroed.  (Counting the tiles and having the last
 // one publish lambda took 8 us in place of 3: two trips through L2 and two fences more.)
 struct Limit { double sum; float kmat, norm, lambda; };
 
@@ -17,6 +17,7 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 // prev: the norm remembered before the step.
+template <typename SHARE>
 __device__ __forceinline__ bool wait_limit(const unsigned long long* shares, int tiles, const MatDev& mt, float prev, const Hyper& hp, volatile int* abort_flag, Limit& out) {
   const int lane = threadIdx.x & 31;
   out.kmat = 1.f;
@@ -30,8 +31,8 @@ __device__ __forceinline__ bool wait_limit(const unsigned long long* shares, int
     bool there = true;
     double acc = 0.0;
     for (int i = lane; i < tiles; i += 32) {
-      float v;
-      there = ptx::get_marked(shares + i, &v) && there;
+      SHARE v;
+      there = ptx::get_marked(shares + i * (sizeof(SHARE) / sizeof(float)), &v) && there;
       acc += (double)v;
     }
     if (__all_sync(0xffffffffu, there)) { out.sum = warp_sum(acc); break; }

@@ -65,7 +65,7 @@ struct alignas(32) TileDev {
 };
 static_assert(sizeof(TileDev) == 32, "TileDev layout");
 struct alignas(32) TileNorm {
-  unsigned long long* shares;                   // of ||S||^2: one marked word per tile of the matrix (k_part_step)
+  unsigned long long* shares;                   // of ||S||^2: a double in two marked words per tile of the matrix (k_part_step)
   int index, tiles, mat, unused;                // the tile's index among them
 };
 
@@ -621,13 +621,13 @@ k_part_step(const BackJob* __restrict__ jobs, int njobs, const TileDev* __restri
           if (!ptx::mbar_wait_cluster(ptx::smem_u32(&ctl->shared_in[b]), (firsts >> 1) & 1, abort_flag)) return false;
           ++firsts;
           const double sum = warp_sum(lane < 2 * RU_WARPS ? (double)ctl->shares[b][lane] : 0.0);
-          if (lane == 0) ptx::put_marked(tn.shares + tn.index, (float)sum);
+          if (lane == 0) ptx::put_marked(tn.shares + PART_SHARE_WORDS * tn.index, sum);
           return true;
         }
         const int b = seconds++ & 1;
         Limit lim;
         const MatDev& mt = mats[tn.mat];
-        if (!wait_limit(tn.shares, tn.tiles, mt, mt.bias->prev, hp, abort_flag, lim)) return false;
+        if (!wait_limit<double>(tn.shares, tn.tiles, mt, mt.bias->prev, hp, abort_flag, lim)) return false;
         if (lane < 2)
           ptx::st_async_f32(ptx::map_to_cta(ptx::smem_u32(&ctl->lambda[b]), lane), lim.lambda * lim.kmat, ptx::map_to_cta(ptx::smem_u32(&ctl->lambda_in[b]), lane));
         if (tn.index == 0) store_limit(mt, hp, lim, status);

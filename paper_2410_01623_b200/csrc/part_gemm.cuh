@@ -57,6 +57,8 @@ struct PartStepPlan {
 };
 constexpr int PART_STEP_MAX_RANK = 512;    // (k_moments keeps a row of R in registers)
 constexpr int PART_SUMS_PER_TILE = 16;   // partial sums of ||S||^2 that a tile leaves
+constexpr int PART_SHARE_WORDS = 2;      // or, in their place, marked words of k_part_step
+static_assert(PART_SHARE_WORDS * 8 <= PART_SUMS_PER_TILE * 4, "the words fit where the sums would be");
 inline int part_rank_pitch(int r) { return (r + 7) / 8 * 8; }
 __host__ __device__ inline int part_step_tiles(int m, int n) { return ((m + 255) / 256) * ((n + 127) / 128); }
 inline int part_project_tiles(int l, int r) { return ((l + 255) / 256) * ((r + 127) / 128); }

@@ -541,7 +541,7 @@ __device__ __forceinline__ void step_tile(const MatDev& mt, int tile, int i0, in
   for (int y = 0; y < PASSES; ++y) load_row<VEC, LANES>(W + (long long)(i0 + row0 + AT_ONCE * y) * mt.ld + j0, hl, i0 + row0 + AT_ONCE * y < mt.m ? n : 0, w[y]);
   if (warp == STEP_THREADS / 32 - 1) {           // (while the product is made)
     Limit lim;
-    const bool known = wait_limit(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, prev, hp, &ctl->abort_flag, lim);
+    const bool known = wait_limit<float>(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, prev, hp, &ctl->abort_flag, lim);
     if (lane == 0 && known) *coef = hp.a_res * lim.lambda * lim.kmat;
   }
   if (!read_back(&ctl->done[1]) || *(volatile int*)&ctl->abort_flag) return;
@@ -594,7 +594,7 @@ k_back_step(const MatDev* mats, const int* list, int nlist, const int* tile_star
     }
     if (threadIdx.x < 32) {
       Limit lim;
-      if (wait_limit(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, mt.bias->prev, hp, &waited, lim)) store_limit(mt, hp, lim, status);
+      if (wait_limit<float>(mt.shares, SIMT_TILE / COLS * simt_tiles_dev(mt.m) * simt_tiles_dev(mt.n), mt, mt.bias->prev, hp, &waited, lim)) store_limit(mt, hp, lim, status);
       else if (lane == 0) atomicOr(status, DEV_STATUS_TIMEOUT);
       if (lane == 0 && norm_out) { *norm_out = mt.sc->prev_norm; *t_out = mt.sc->t; }
     }
@@ -780,7 +780,7 @@ k_split_projection(const MatDev* __restrict__ mats, const int* __restrict__ list
       mt.bias->prev = mt.sc->prev_norm;
       mt.bias->now = step_bias(*mt.bias, mt.sc->t + 1, hp);
     }
-    for (int i = threadIdx.x; i < part_step_tiles(mt.m, mt.n); i += 256) reinterpret_cast<unsigned long long*>(mt.part)[i] = 0ull;
+    for (int i = threadIdx.x; i < PART_SHARE_WORDS * part_step_tiles(mt.m, mt.n); i += 256) reinterpret_cast<unsigned long long*>(mt.part)[i] = 0ull;
     return;
   }
   if (mt.bf16) split_units<__nv_bfloat16>(mt, block, per);

@@ -224,6 +224,17 @@ __device__ __forceinline__ bool get_marked(const unsigned long long* p, float* v
   *v = __uint_as_float((uint32_t)w);
   return w >> 32;
 }
+// A double, in two such words.
+__device__ __forceinline__ void put_marked(unsigned long long* p, double v) {
+  put_marked(p, __int_as_float(__double2hiint(v)));
+  put_marked(p + 1, __int_as_float(__double2loint(v)));
+}
+__device__ __forceinline__ bool get_marked(const unsigned long long* p, double* v) {
+  float hi, lo;
+  const bool there = get_marked(p, &hi), both = get_marked(p + 1, &lo) && there;
+  *v = __hiloint2double(__float_as_int(hi), __float_as_int(lo));
+  return both;
+}
 
 // ----------------------------------------------------------------------------- CTA pairs
 // Two CTAs of a cluster share one tcgen05.mma (cta_group::2): each holds half of the

@@ -1,5 +1,7 @@
 """GPU checks of the fp32-precision tensor-core paths at the sizes where their tilings can go wrong: long lists
 (kernels of their own), tile remainders, ranks around the tile widths, the factorisation's blocks."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -210,3 +212,42 @@ def test_long_list_with_runs_of_narrow_tiles(shapes, ranks):
         torch.cuda.synchronize()
     assert [f.poll() for f in fs] == [0, 0]
     assert all(torch.equal(w.cpu(), h) for w, h in zip(W, Wh))
+
+
+def _squares(total, count):
+    """`count` whole numbers of at most 90 whose squares add up to total."""
+    out = np.zeros(count)
+    whole, rest = divmod(total, 8100)
+    out[:whole] = 90
+    four = next((a, b, c, e) for a in range(91) for b in range(a + 1) for c in range(b + 1)
+                for e in [math.isqrt(max(0, rest - a * a - b * b - c * c))] if a * a + b * b + c * c + e * e == rest)
+    out[whole:whole + 4] = four
+    return out
+
+
+@pytest.mark.parametrize("dtype,launches", [(torch.float32, 4), (torch.bfloat16, 7)])
+def test_norm_of_long_lists_loses_nothing_between_tiles(dtype, launches):
+    """||S|| of whole numbers.  What one warp adds up in fp32 is exact (2048 squares of 90 at most: below 2^24).  A tile's sum takes 28 bits
+    and lies 7 above a multiple of 16, which rounding it to 24 bits takes off in each of 32 tiles; the whole lies 2 to 18
+    above the square of the middle between two fp32 numbers.  So the norm is the upper one only if nothing is rounded in between."""
+    shapes = [(1024, 1024)] * 6
+    f = fb.Fira(shapes, 64, dtype, fb.make_hparams(flags=fb.FLAG_NO_SCALING | fb.FLAG_FORCE_SIMT))      # P = 0: S = G
+    Gs, want = [], []
+    for i in range(len(shapes)):
+        low = np.float32(92000 + 17 * i)
+        middle = (float(low) + float(np.spacing(low)) / 2) ** 2
+        total = (int(middle) // 16 + 1) * 16
+        total += 16 * (total - middle < 2)
+        G = np.zeros((1024, 1024))
+        sums = [total // 32 // 16 * 16 + 7] * 32
+        sums[-1] += total - sum(sums)
+        for t, x in enumerate(sums):
+            assert x % 16 == 7 and 2 ** 27 < x < 2 ** 28
+            G[t // 8 * 256:t // 8 * 256 + 256, t % 8 * 128:t % 8 * 128 + 128] = _squares(x, 256 * 128).reshape(256, 128)
+        assert (G * G).sum() == total
+        Gs.append(torch.from_numpy(G).to(dtype).cuda())
+        want.append(float(np.nextafter(low, np.float32(np.inf))))
+        assert want[-1] == float(np.float32(math.sqrt(total)))
+    f.step([torch.zeros(1024, 1024, dtype=dtype, device="cuda") for _ in shapes], Gs)
+    assert f.poll() == 0 and f.last_step_launches() == launches
+    assert [f.diagnostics(i)["norm_scaled"] for i in range(len(shapes))] == want
