@@ -91,16 +91,11 @@ struct NoAllocInts { int v[6]; };
 // that a step reads there is rewritten by the step's own kernels before it is read).  The matrix
 // record and the schedule arrays travel as kernel arguments, so that no host memory is referenced
 // once the call has returned.  Also moves the two state scalars from the caller's memory into the
-// MatScalars block that the step kernels use.  One warp: the two powers of the bias factor (bias_factor's), in double the
-// kernel's longest part, by a lane each.
-__global__ void __launch_bounds__(32)
-k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, int* ints_out,
+// MatScalars block that the step kernels use.
+__global__ void k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, int* ints_out,
                                 const float* norm_prev, const long long* t, float beta1, float beta2) {
   ptx::grid_launch_next();
   const long long steps = *t;
-  const double power = pow((double)(threadIdx.x & 1 ? beta2 : beta1), (double)(steps + 1));
-  const double power2 = __shfl_sync(0xffffffffu, power, 1);
-  if (threadIdx.x) return;
   const float norm = *norm_prev;
   *mats_out = mt;
   for (int i = 0; i < 6; ++i) ints_out[i] = ints.v[i];
@@ -109,7 +104,7 @@ k_noalloc_setup(MatDev mt, NoAllocInts ints, MatDev* mats_out, int* ints_out,
   sc->lambda = 1.f; sc->norm_scaled = 0.f; sc->k_min = 0.f; sc->k_max = 0.f; sc->bias = 0.f;
   sc->t = steps;
   mt.bias->step = steps + 1;
-  mt.bias->next = (float)(sqrt(1.0 - power2) / (1.0 - power));
+  mt.bias->next = bias_factor(beta1, beta2, steps + 1);
 }
 __global__ void k_noalloc_store_scalars(const MatScalars* sc, float* norm_prev, long long* t) {
   ptx::grid_wait();
@@ -182,7 +177,7 @@ extern "C" fira_status fira_step_single_noalloc(const fira_hparams* hp, const fi
   // sticky across calls until fira_noalloc_poll() reads it (zero when the library is loaded)
   unsigned* status_dev = reinterpret_cast<unsigned*>(base + cv.off_status);
 
-  k_noalloc_setup<<<1, 32, 0, st>>>(mt, ints, reinterpret_cast<MatDev*>(base + cv.off_mats), ints_dev,
+  k_noalloc_setup<<<1, 1, 0, st>>>(mt, ints, reinterpret_cast<MatDev*>(base + cv.off_mats), ints_dev,
                                    norm_prev_dev, reinterpret_cast<const long long*>(t_dev), hp->beta1, hp->beta2);
   SimtPlan pl;
   pl.mats = reinterpret_cast<const MatDev*>(base + cv.off_mats);
