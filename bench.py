@@ -83,6 +83,7 @@ NCU_DRAM_BYTES_2_LAYERS = {"k_tc_project": 1.881e9 + 1.172e9, "k_tc_back_project
 # kernel name -> (pipe that does its arithmetic, share of the step's 4 m n r flops)
 KERNEL_PIPE = {
     "k_project": ("tensor", 0.5), "k_back_project<norm>": ("tensor", 0.5), "k_back_project<update>": ("tensor", 0.5),
+    "k_back_step": ("tensor", 1.0), "k_part_step": ("tensor", 1.0),        # the norm's product and the update's
     "k_tc_project": ("tensor", 0.5), "k_tc_back_project": ("tensor", 0.5),
 }
 
@@ -96,7 +97,7 @@ def kernel_min_bytes(name, wl):
     by = 0
     for (m, n) in wl.shapes:
         l, d = max(m, n), min(m, n)
-        if "back_project" in name:
+        if "back" in name or name == "k_part_step":
             by += 2 * e * m * n
         elif name == "k_project":          # fp32 precision: the moments are counted at k_moments
             by += e * m * n + e * wl.r * d

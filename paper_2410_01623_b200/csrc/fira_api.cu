@@ -717,7 +717,7 @@ fira_status fira_enable_phase_timing(fira_ctx* c, int32_t enable) {
   if (enable && tm.events.empty()) {
     tm.events.resize((size_t)FIRA_TIMING_MAX_STEPS * (FIRA_TIMING_MAX_PHASES + 1));
     for (auto& ev : tm.events) FIRA_CUDA(cudaEventCreate(&ev));
-    if (c->simt.nlist) for (int i = 0; i < SIMT_PHASES; ++i) tm.names.push_back(kSimtPhaseNames[i]);
+    if (c->simt.nlist) tm.names = simt_phase_names(c->simt, c->hp.flags & FIRA_FLAG_ONLY_SCALING);
     if (!c->tc_list.empty()) {
       const char* nm[8];
       const int k = tc_phase_names(nm);

@@ -950,7 +950,11 @@ k_finalize(const MatDev* __restrict__ mats, const int* __restrict__ list, int nl
   }
 }
 
-const char* const kSimtPhaseNames[SIMT_PHASES] = {"k_project", "k_moments", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"};
+std::vector<const char*> simt_phase_names(const SimtPlan& pl, bool only_scaling) {
+  if (pl.resident && !only_scaling) return {"k_project", "k_back_step"};
+  if (pl.parts.one_kernel_pairs && !only_scaling) return {"k_project", "k_moments", "k_part_step"};
+  return {"k_project", "k_moments", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"};
+}
 
 // Measured (fp32 / bf16 storage, times of a step in us, short against long): 6 matrices 512 x 1376, r = 128, 63 / 51 against 71 / 62,
 // 8 of them 102 / 72 against 82 / 69; 4 of 1024 x 1024, r = 256, 92 / 65 against 94 / 71, 6 of them 151 / 98 against 113 / 82; 24 of
@@ -1100,7 +1104,6 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
     tm->mark(st);
   }
   if (pl.resident && !only_scaling) {
-    for (int i = 0; i < 4; ++i) tm->mark(st);    // (its time counts as the update's)
     const int per = short_one_kernel(2 * pl.w_tiles, pl.nlist, pl.max_r, pl.resident) ? 2 : 1, blocks = per * (wt1 - wt0);       // (of the whole list, whatever range is stepped)
     launch_error(launch_resident(per == 2 ? k_back_step<SIMT_TILE / 2> : k_back_step<SIMT_TILE>, blocks + nq, STEP_THREADS, STEP_SMEM, st, true, 1, pl.mats, pl.list,
                                  pl.nlist, pl.w_tile_start, wt0, blocks, qa, hp, pl.norm_out, pl.t_out, status_dev));
@@ -1110,7 +1113,6 @@ int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, 
   }
   tm->mark(st);
   if (one_kernel) {
-    for (int i = 0; i < 3; ++i) tm->mark(st);    // (its time counts as the update's)
     if (part_step_run_one_kernel(pl.parts, pl.mats, qa, qe, hp, status_dev, st) != FIRA_OK) return -1;
     launch_stage(pl.mats, pl.stage_list, nstage, pl.stage_start, s0, staged, 1, st);
     tm->mark(st);

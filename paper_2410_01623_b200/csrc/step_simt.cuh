@@ -7,7 +7,6 @@ namespace fira {
 
 constexpr int SIMT_TILE = 128;              // tiles of R (l x r) and of W (m x n)
 inline int simt_tiles(long long extent) { return (int)((extent + SIMT_TILE - 1) / SIMT_TILE); }
-constexpr int SIMT_PHASES = 6;
 
 // The factor k_l from the row sums.
 __device__ __forceinline__ float row_factor(const MatDev& mt, int l, const Hyper& hp) {
@@ -80,7 +79,8 @@ void launch_stage(const MatDev* mats, const int* list, int nlist, const int* row
 // the number of launches (negative: error, message set).
 int launch_simt_step(const SimtPlan& pl, const Hyper& hp, unsigned* status_dev, cudaStream_t st,
                      PhaseTimer* tm, int qa = 0, int qb = -1);
-extern const char* const kSimtPhaseNames[SIMT_PHASES];
+// The names of the phases that a step of the list marks.
+std::vector<const char*> simt_phase_names(const SimtPlan& pl, bool only_scaling);
 
 // One block of 256 threads per matrix of the list: sums the matrix's partial sums
 // of ||S||^2 (npart_of[i] floats at mt.part) in a fixed order, applies the limiter

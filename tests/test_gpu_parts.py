@@ -251,3 +251,20 @@ def test_norm_of_long_lists_loses_nothing_between_tiles(dtype, launches):
     f.step([torch.zeros(1024, 1024, dtype=dtype, device="cuda") for _ in shapes], Gs)
     assert f.poll() == 0 and f.last_step_launches() == launches
     assert [f.diagnostics(i)["norm_scaled"] for i in range(len(shapes))] == want
+
+
+@pytest.mark.parametrize("shapes,flags,names", [
+    ([(512, 1376)], 0, ["k_project", "k_back_step"]),
+    ([(512, 1376)] * 8, 0, ["k_project", "k_moments", "k_part_step"]),
+    ([(512, 1376)], fb.FLAG_ONLY_SCALING, ["k_project", "k_moments", "k_back_project<norm>", "k_finalize", "k_form_x", "k_back_project<update>"])])
+def test_phase_times_name_the_kernels_that_ran(shapes, flags, names):
+    f = fb.Fira(shapes, 128, torch.float32, fb.make_hparams(flags=flags))
+    W, G = ([torch.randn(s, device="cuda") for s in shapes] for _ in range(2))
+    f.refresh_projection(G)
+    f.step(W, G)
+    f.enable_phase_timing()
+    for _ in range(3):
+        f.step(W, G)
+    phases, steps = f.phase_times()
+    assert [k for k, _ in phases] == names and steps == 3
+    assert flags or all(ms > 1e-3 for _, ms in phases)
