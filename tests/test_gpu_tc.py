@@ -244,31 +244,35 @@ def test_limiter_acts_on_a_list_of_long_products_with_ragged_rows():
     assert all(l < 0.5 for l in tr.lams[2])
 
 
-@pytest.mark.parametrize("shapes,r", [([(1024, 1536), (1536, 1024)], 256), ([(2048, 2304), (512, 768)], 512), ([(2048, 2304), (1024, 1536)], 512)])
-def test_x_is_the_same_whichever_kernel_forms_it(shapes, r):
+@pytest.mark.parametrize("shapes", [[(2048, 2304), (2304, 2048)], [(2048, 2309), (2309, 2048)], [(2048, 2304), (2304, 2048), (1024, 1536)]])
+def test_x_is_the_same_whichever_kernel_forms_it(shapes):
     """The projection forms X of a matrix, or leaves it to a later kernel if its limiter acted on the step before; the weights do not
-    depend on that, bit for bit.  A context that has been given the state through set_state does not know about the step before."""
+    depend on that, bit for bit.  That is for lists of d >= 2048 and several tiles of r: one matrix limited and one not, rows that
+    start on 16-byte boundaries and others, and one beside them whose X neither forms.  A context that has been given the state through set_state
+    does not know about the step before.  On the last step the matrix that was limited is so no more: its residual is a rounding error."""
     g = torch.Generator(device="cuda").manual_seed(9)
     hp = fb.make_hparams(lr=1e-2, alpha=0.25, gamma=1.01)
-    ranks = [min(r, min(s) // 2 // 128 * 128) for s in shapes]
-    a, b = fb.Fira(shapes, ranks, torch.bfloat16, hp), fb.Fira(shapes, ranks, torch.bfloat16, hp)
+    a, b = fb.Fira(shapes, 512, torch.bfloat16, hp), fb.Fira(shapes, 512, torch.bfloat16, hp)
     W = [(torch.randn(s, generator=g, device="cuda") * 0.02).to(torch.bfloat16) for s in shapes]
     for i, s in enumerate(shapes):
-        P = torch.linalg.qr(torch.randn(min(s), ranks[i], generator=g, device="cuda"))[0].to(torch.bfloat16).contiguous()
-        V = torch.rand(max(s), ranks[i], generator=g, device="cuda") + 0.5
+        P = torch.linalg.qr(torch.randn(min(s), 512, generator=g, device="cuda"))[0].to(torch.bfloat16).contiguous()
+        V = torch.rand(max(s), 512, generator=g, device="cuda") + 0.5
         for f in (a, b):
             f.set_projection(i, P)
-        a.set_state(i, 0.1 * torch.randn(V.shape, generator=g, device="cuda"), V, 1.0 if i == 0 else 1e6, 50)
-    for step in range(2):
+        a.set_state(i, 0.23 * torch.randn(V.shape, generator=g, device="cuda"), V, 50.0 if i == 0 else 1e6, 50)      # (of the size that M keeps)
+    P = a.get_projection(0).float()
+    for step in range(3):
         G = [torch.randn(s, generator=g, device="cuda").to(torch.bfloat16) for s in shapes]
-        if step == 1:
-            assert a.diagnostics(0)["lam"] < 1.0
+        if step == 2:
+            G[0] = (P @ (P.T @ G[0].float())).to(torch.bfloat16)
+        if step:
+            assert [a.diagnostics(i)["lam"] < 1.0 for i in range(len(shapes))] == [i == 0 for i in range(len(shapes))]
             Wb = [w.clone() for w in W]
             for i in range(len(shapes)):
                 M, V, norm, t = a.get_state(i)
                 b.set_state(i, M, V, norm, t)
             b.step(Wb, G)
         a.step(W, G)
-    assert a.poll() == 0 and b.poll() == 0 and a.diagnostics(0)["lam"] < 1.0
-    for i in range(len(shapes)):
-        assert torch.equal(W[i], Wb[i]), shapes[i]
+        if step:
+            assert all(torch.equal(x, y) for x, y in zip(W, Wb)), step
+    assert a.poll() == 0 and b.poll() == 0 and a.diagnostics(0)["lam"] == 1.0
