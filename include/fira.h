@@ -42,6 +42,11 @@
  *
  * Streams and errors.  All device work is enqueued on the stream given to
  * fira_init() and calls return without waiting for it unless stated otherwise.
+ * Most steps of the kernels of fp32 precision (all fp32 matrices; engine 0 in fira_diag) and fira_step_single_noalloc()
+ * hold a kernel whose blocks wait for one another: one block on every SM, or on one per 128 x 64 elements of W in short
+ * lists.  It starts only when all of them fit on the stream's SMs at once (a cooperative launch; how many SMs those are
+ * is asked at fira_init(), and by each fira_step_single_noalloc()).  Kernels of other streams that end by themselves delay
+ * it; one that holds SMs until such a step has finished would be waited for without end.
  * Host-side argument errors are returned at once and leave the state untouched.
  * Device-side conditions (a bounded wait that ran out, a non-finite norm) are
  * recorded in a status word that fira_poll() reads.  No entry point throws, aborts
@@ -285,7 +290,7 @@ FIRA_API const char* fira_phase_name(const fira_ctx* ctx, int32_t phase);
  * stay out of the driver's allocator, a process whose memory was budgeted at start
  * -- and therefore cannot provide the state and scratch buffers of fira_init().  The
  * intermediates live in a fixed array inside the library image instead:
- * fira_noalloc_max_scratch_bytes() bytes (8 MiB) and 144 KiB of row sums, held on every GPU
+ * fira_noalloc_max_scratch_bytes() bytes (8 MiB) and 147 KiB of row sums and marks, held on every GPU
  * that loads the library until the process exits.  The call allocates nothing.
  *
  * desc: the matrix (fp32 or bf16; it always runs on the kernels of fp32 precision).  Its
