@@ -896,8 +896,11 @@ fira_status part_step_prepare(const std::vector<MatDev>& mats, const std::vector
   int pairs = resident_pairs();
   if (!pairs) return FIRA_ERR_CUDA;
   pairs = std::min(pairs, stream_sms(st) / 2);
-  // One kernel for norm and update: 56 matrices 512 / 1376 fp32, step 231 us against 246 with two (210 / 256 where the limiter acts on all and
-  // a step finds its tables in L2).  bf16, where G is half of the traffic less: 28 of 640 / 1707, 189 / 185.
+  // One kernel for norm and update.  Steps with two kernels / with one, us, lists back to back, limiter acting on all: 56 matrices 512 / 1376 fp32
+  // r = 64 246 / 201, 128 256 / 210, 160 372 / 289, 192 391 / 306, 256 429 / 338; 14 of 1024 / 2736 r = 128 223 / 198, 192 319 / 260, 256 347 / 288,
+  // 384 484 / 399, 512 628 / 528; 14 of 768 / 2048 r = 64 132 / 116, 384 304 / 247; 112 of 288 / 992, r = 64, 286 / 238; 140 of 160 / 416, r = 40, 150 / 117;
+  // 28 of 640 / 1707 r = 100 (copies to an aligned pitch) 271 / 233.  Limiter acting on none, inputs not in L2: 56 of 512 / 1376, r = 128, 246 / 239.
+  // bf16, where G is half of the traffic less: 28 of 640 / 1707, 185 / 189.
   plan->one_kernel_pairs = pairs;
   BackJob* jd = reinterpret_cast<BackJob*>(plan->jobs.data());
   for (size_t q = 0; q < list.size(); ++q) {

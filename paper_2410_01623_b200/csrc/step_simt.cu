@@ -1,15 +1,20 @@
 // Kernels of the Fira step (Algorithm 1's loop body) in fp32 precision, grouped over a list of
 // matrices of any size and pitch: one launch per phase covers every matrix of the list.
 //
-// Phases (l = unprojected index, d = projected index, Pi = the d x r projection):
+// What is to be made (l = unprojected index, d = projected index, Pi = the d x r projection):
 //   1. project      R[l][j] = sum_d G(d,l) Pi[d][j]  (R = P^T G); epilogue: M, V update, N (Eq. 2-4) and the
 //                   row sums ||N_l||^2, ||R_l||^2 of which k_l = ||N_l|| / (||R_l|| + eps) is made (Eq. 11)
 //   2. norm         D = Pi R; part = sum (k_l (G - D))^2                   (||S||, literal residual)
 //   3. finalize     lambda, ||S_prev||, t                                  (Eq. 12)
-//   4. update       D = Pi X with X = a_low N - a_res lambda k_l R; W -= lr (D + a_res lambda k_l G)
-// Phase 4 uses the identity alpha (P N + lambda (G - P R) diag k) =
-// P (alpha N - alpha lambda R diag k) + alpha lambda G diag k, so that the update needs one product
-// instead of two; X is formed while the product loads N and R.
+//   4. update       W -= lr (a_low Pi N + a_res lambda S), S = k_l (G - Pi R)
+// By which kernels:
+//   k_project, k_back_step          short lists of few tiles and ranks up to 128: 2 to 4 in one kernel whose blocks keep S
+//   k_project, k_back_project<norm>, k_finalize, k_back_project<update>        other short lists.  S is not kept: the update is
+//                                   D = Pi X with X = a_low N - a_res lambda k_l R, W -= lr (D + a_res lambda k_l G), by the identity
+//                                   alpha (P N + lambda (G - P R) diag k) = P (alpha N - alpha lambda R diag k) + alpha lambda G diag k,
+//                                   which needs one product instead of two; X is formed while the product loads N and R
+//   k_split_projection, k_part_project, k_moments, then k_part_step or k_part_back<norm>, k_finalize, k_form_x, k_part_back<update>
+//                                   long lists (part_project.cu, part_back.cu), by the same two ways
 //
 // The products are the 128 x 128 tile products of split_gemm.cuh: fp32 precision on the tensor cores.  Every
 // epilogue takes the finished tile from shared memory, one warp per row, so that all traffic with
@@ -17,7 +22,7 @@
 //
 // Short lists are bound by latency, so all of their kernels are chained (launch_chained): one's set-up (tables, barriers,
 // tensor memory) runs while the one before it ends.  Step of one 512 x 1376 matrix: 74 us without that and without the
-// split projection, 35 us with both, 26.7 us with phases 2 to 4 in one kernel (k_back_step).
+// split projection, 35 us with both, 26.6 us with 2 to 4 in one kernel (k_back_step).
 #include <cuda.h>
 
 #include <algorithm>
@@ -406,6 +411,10 @@ k_back_project(const MatDev* __restrict__ mats, const int* __restrict__ list, in
 // Measured, one 512 x 1376 matrix, r = 128, the kernel's time: 22 us as two ordinary tile products in a row, 18.6 with all slabs loaded at
 // once, 15 with all of them stored before the first MMA is issued (of that 5.5 to the first product's end, 2 the second's, the rest rows
 // and conversions), 10.9 with half tiles (88 blocks).
+// Steps by the three kernels / by this one, us, whole tiles: 1280 x 1280, r = 64 (100 tiles) 38.3 / 35.2; 768 x 2048, r = 128 (96) 40.3 / 35.7;
+// 1024 x 2048, r = 128 (128) 41.3 / 37.2; 1152 x 2048, r = 128 (144) 46.0 / 41.3; 2048 x 1000, r = 100 (128, scalar loads of the factors) 47.5 / 47.1.
+// Half tiles: 7 matrices 256 / 688, r = 64, 39.2 / 31.2; bf16 600 x 1200, r = 110, 41.3 / 33.3.  The single-matrix entry point, 512 x 1376 and
+// 768 x 2304, r = 128: fp32 39.2 / 30.7 and 45.2 / 39.3, bf16 36.0 / 27.0 and 37.1 / 31.9.
 constexpr int STEP_THREADS = 512, STEP_ROWS = SIMT_TILE / (STEP_THREADS / 32);         // rows per warp
 constexpr int STEP_SLABS = 128 / split::BK;
 constexpr int STEP_X = STEP_SLABS * split::OPERAND_BYTES;       // the slabs of R, then N, behind those of the projection; the finished tile overlays them

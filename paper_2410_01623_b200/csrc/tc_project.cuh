@@ -64,8 +64,9 @@
 // leaves about 2.4 times the error.)
 // FUSE_X = 3: as 2, but the matrices that k_tc_prep has marked leave N and R instead, as without FUSE_X: those whose limiter acted on
 // the step before, and which are likely to be limited again; k_tc_fix_x makes the same X from them bit for bit.  For lists with two
-// groups of epilogue warps, where the second sweep and its exchange are on the critical path.  Measured, 1B list, limiter
-// acting on all: projection 1863 us forming X and correction 285 us; 1649 and 306 leaving N and R; step 5205 / 5065.  Not on the 350M list,
+// groups of epilogue warps, where the second sweep and its exchange are on the critical path.  Measured, 1B list, step with FUSE_X = 2 / 3 by
+// the matrices that the limiter acts on, this step and the one before: none 4502 / 4500 us, one in eight 4552 / 4512, all 4770 / 4568 (projection 1863 us
+// forming X and correction 285; 1649 and 306 leaving N and R).  Not on the 350M list,
 // whose rows of tiles need no exchange (projection + 43, correction - 51, the check itself 1 % of the step), nor on the 7B list, one group
 // (projection + 2 %).
 // (Adam only: with RMSProp or Adagrad N cannot be rebuilt from V alone, and those steps keep the
