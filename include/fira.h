@@ -42,11 +42,11 @@
  *
  * Streams and errors.  All device work is enqueued on the stream given to
  * fira_init() and calls return without waiting for it unless stated otherwise.
- * Most steps of the kernels of fp32 precision (all fp32 matrices; engine 0 in fira_diag) and fira_step_single_noalloc()
- * hold a kernel whose blocks wait for one another: one block on every SM, or on one per 128 x 64 elements of W in short
- * lists.  It starts only when all of them fit on the stream's SMs at once (a cooperative launch; how many SMs those are
- * is asked at fira_init(), and by each fira_step_single_noalloc()).  Kernels of other streams that end by themselves delay
- * it; one that holds SMs until such a step has finished would be waited for without end.
+ * Most steps in fp32 precision (engine 0 in fira_diag: all fp32 matrices) and of fira_step_single_noalloc() hold a kernel
+ * whose blocks wait for one another, one block to an SM: all SMs in long lists, in short ones a block per 128 x 64 or
+ * 128 x 128 elements of W.  It starts only when all of them fit on the stream's SMs at once (a cooperative launch; how many
+ * SMs those are is asked at fira_init(), and by each fira_step_single_noalloc()).  Kernels of other streams that end by
+ * themselves delay it; one that holds SMs until such a step has finished would be waited for without end.
  * Host-side argument errors are returned at once and leave the state untouched.
  * Device-side conditions (a bounded wait that ran out, a non-finite norm) are
  * recorded in a status word that fira_poll() reads.  No entry point throws, aborts
